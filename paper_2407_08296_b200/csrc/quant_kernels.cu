@@ -1,84 +1,112 @@
 // Stream kernels of the block-wise quantizer (Sec. 3.1, Sec. 3.3) and of the similarity
-// statistic between adjacent projection matrices (Sec. 3.2).  All are HBM-bound: one warp
-// owns one 256-element group, each lane eight consecutive elements (two 16-byte loads, one
-// 8- or 4-byte store), the group minimum/maximum come from warp shuffles.
+// statistic between adjacent projection matrices (Sec. 3.2).  All are HBM-bound.
 #include "qg_common.cuh"
 
 namespace qg {
 
+// Both quantizer streams work in runs of kRunGroups groups (512 columns) of a row, one warp each.  A lane takes four
+// consecutive columns out of every 128, so that every load and store of a warp is contiguous, and has the loads of its
+// whole run in flight before it uses the first.  Measured on 4096 x 11008 at 8 bits, against eight consecutive columns
+// per lane (two loads 32 bytes apart, scalar stores of the dequantized values) and one group per warp:
+// quantize 57 -> 52 us, dequantize 150 -> 33 us, both together 225 -> 86 us (450 MB: 5.3 TB/s of 6.55 measured).
+constexpr int kRunGroups = 2, kRunPieces = kRunGroups * 2, kStreamWarps = 8;
+
+// Row and run of this warp; false past the end.
+__device__ __forceinline__ bool stream_unit(int64_t rows, int runs, int64_t& row, int& run) {
+  const int64_t u = (int64_t)blockIdx.x * kStreamWarps + (threadIdx.x >> 5), total = rows * runs;
+  if (u >= total) return false;
+  if (total <= 0xFFFFFFFFll) {                      // the short division
+    row = (uint32_t)u / (uint32_t)runs;
+    run = (int)((uint32_t)u - (uint32_t)row * (uint32_t)runs);
+  } else {
+    row = u / runs;
+    run = (int)(u - row * runs);
+  }
+  return true;
+}
+
+__device__ __forceinline__ float redux_min(float v) {
+  float r;
+  asm("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+  return r;
+}
+__device__ __forceinline__ float redux_max(float v) {
+  float r;
+  asm("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+  return r;
+}
+
 // ------------------------------------------------------------------------ quantize (RTN)
 template <int BITS>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(kStreamWarps * 32)
 quantize_rtn_kernel(const float* __restrict__ src, int64_t ld_src, int64_t rows, int64_t cols,
                     uint8_t* __restrict__ codes, int64_t ld_code_bytes,
                     float* __restrict__ scales, float* __restrict__ zeros, int ngroups) {
   const int lane = threadIdx.x & 31;
-  const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (warp >= rows * ngroups) return;               // whole warps leave together
-  const int64_t row = warp / ngroups;
-  const int g = (int)(warp % ngroups);
-  const int64_t c0 = (int64_t)g * kGroup + lane * 8;
-  const int nvalid = (int)max((int64_t)0, min((int64_t)8, cols - c0));
+  int64_t row;
+  int run;
+  if (!stream_unit(rows, (ngroups + kRunGroups - 1) / kRunGroups, row, run)) return;      // whole warps leave together
+  const int64_t c0 = (int64_t)run * kRunGroups * kGroup + lane * 4;
   const float* p = src + row * ld_src + c0;
-
-  float v[8];
-  if (nvalid == 8) {
-    const float4 a = __ldg(reinterpret_cast<const float4*>(p));
-    const float4 b = __ldg(reinterpret_cast<const float4*>(p + 4));
-    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
-    v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
-  } else {
+  float v[kRunPieces][4];
+  int nv[kRunPieces];                               // valid columns of each piece
 #pragma unroll
-    for (int i = 0; i < 8; ++i) v[i] = (i < nvalid) ? __ldg(p + i) : 0.0f;
-  }
-  float mn = INFINITY, mx = -INFINITY;
-#pragma unroll
-  for (int i = 0; i < 8; ++i)
-    if (i < nvalid) { mn = fminf(mn, v[i]); mx = fmaxf(mx, v[i]); }
-  mn = warp_min(mn);
-  mx = warp_max(mx);
-  const GroupParams gp = group_params<BITS>(mn, mx);
-  if (lane == 0) {
-    scales[row * ngroups + g] = gp.s;
-    zeros[row * ngroups + g] = gp.z;
-  }
-  if (nvalid == 0) return;
-
-  int q[8];
-#pragma unroll
-  for (int i = 0; i < 8; ++i) q[i] = (i < nvalid) ? (int)rtn_code<BITS>(v[i], gp) : 0;
-
-  if (BITS == 8) {
-    uint8_t* out = codes + row * ld_code_bytes + c0;
-    if (nvalid == 8) {
-      uint2 w;
-      w.x = (uint32_t)(q[0] & 0xFF) | ((uint32_t)(q[1] & 0xFF) << 8) | ((uint32_t)(q[2] & 0xFF) << 16) |
-            ((uint32_t)(q[3] & 0xFF) << 24);
-      w.y = (uint32_t)(q[4] & 0xFF) | ((uint32_t)(q[5] & 0xFF) << 8) | ((uint32_t)(q[6] & 0xFF) << 16) |
-            ((uint32_t)(q[7] & 0xFF) << 24);
-      *reinterpret_cast<uint2*>(out) = w;
+  for (int i = 0; i < kRunPieces; ++i) {
+    nv[i] = (int)max((int64_t)0, min((int64_t)4, cols - (c0 + 128 * i)));
+    if (nv[i] == 4) {
+      const float4 a = __ldcs(reinterpret_cast<const float4*>(p + 128 * i));
+      v[i][0] = a.x; v[i][1] = a.y; v[i][2] = a.z; v[i][3] = a.w;
     } else {
-      for (int i = 0; i < nvalid; ++i) out[i] = (uint8_t)(q[i] & 0xFF);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) v[i][e] = (e < nv[i]) ? __ldg(p + 128 * i + e) : 0.0f;
     }
-  } else if (BITS == 4) {
-    uint8_t* out = codes + row * ld_code_bytes + (c0 >> 1);
-    uint32_t w = 0;
+  }
 #pragma unroll
-    for (int i = 0; i < 8; ++i) w |= (uint32_t)((q[i] + 8) & 0xF) << (4 * i);   // padding nibbles hold code 0
-    if (nvalid == 8) {
-      *reinterpret_cast<uint32_t*>(out) = w;
-    } else {
-      for (int i = 0; i < (nvalid + 1) / 2; ++i) out[i] = (uint8_t)((w >> (8 * i)) & 0xFF);
+  for (int h = 0; h < kRunGroups; ++h) {
+    const int g = run * kRunGroups + h;
+    if (g >= ngroups) break;
+    float mn = INFINITY, mx = -INFINITY;
+#pragma unroll
+    for (int i = 2 * h; i < 2 * h + 2; ++i)
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        if (e < nv[i]) { mn = fminf(mn, v[i][e]); mx = fmaxf(mx, v[i][e]); }
+    mn = redux_min(mn);
+    mx = redux_max(mx);
+    const GroupParams gp = group_params<BITS>(mn, mx);
+    // rint(t) + z as integers: adding 1.5 * 2^23 rounds t to the nearest integer, ties to even, and leaves it in the low
+    // mantissa bits; exact while |t| < 2^22, i.e. for all of a group whose zero point is below 2^20
+    const bool small = fabsf(gp.z) < 0x1p20f;
+    const int iz = small ? (int)gp.z - 0x4B400000 : 0;
+    if (lane == 0) {
+      scales[row * ngroups + g] = gp.s;
+      zeros[row * ngroups + g] = gp.z;
     }
-  } else {
-    uint8_t* out = codes + row * ld_code_bytes + (c0 >> 2);
-    uint32_t w = 0;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) w |= (uint32_t)(((i < nvalid ? q[i] : 0) + 2) & 0x3) << (2 * i);   // padding holds code 0
-    if (nvalid == 8) {
-      *reinterpret_cast<uint16_t*>(out) = (uint16_t)w;
-    } else {
-      for (int i = 0; i < (nvalid + 3) / 4; ++i) out[i] = (uint8_t)((w >> (8 * i)) & 0xFF);
+    for (int i = 2 * h; i < 2 * h + 2; ++i) {
+      if (nv[i] == 0) continue;
+      constexpr int kPerByte = 8 / BITS, kOffset = BITS == 8 ? 0 : 1 << (BITS - 1);
+      uint32_t w = 0;                               // unused positions hold code 0, as stored
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        int q;
+        if (small) {
+          q = __float_as_int(__fadd_rn(__fmul_rn(v[i][e], gp.inv), 12582912.0f)) + iz;
+          q = min(max(q, -(1 << (BITS - 1))), (1 << (BITS - 1)) - 1);
+        } else {
+          q = (int)rtn_code<BITS>(v[i][e], gp);
+        }
+        if (e >= nv[i]) q = 0;
+        w |= ((uint32_t)(q + kOffset) & ((1u << BITS) - 1u)) << (BITS * e);
+      }
+      uint8_t* out = codes + row * ld_code_bytes + (c0 + 128 * i) / kPerByte;
+      if (nv[i] == 4) {
+        if (BITS == 8) *reinterpret_cast<uint32_t*>(out) = w;
+        else if (BITS == 4) *reinterpret_cast<uint16_t*>(out) = (uint16_t)w;
+        else *out = (uint8_t)w;
+      } else {
+        for (int e = 0; e < (nv[i] + kPerByte - 1) / kPerByte; ++e) out[e] = (uint8_t)((w >> (8 * e)) & 0xFF);
+      }
     }
   }
 }
@@ -86,48 +114,76 @@ quantize_rtn_kernel(const float* __restrict__ src, int64_t ld_src, int64_t rows,
 int launch_quantize_rtn(int bits, const float* src, int64_t rows, int64_t cols, int64_t ld_src,
                         const qg_qtensor* dst, cudaStream_t st) {
   const int ngroups = (int)ceil_div(cols, kGroup);
-  const int64_t warps = rows * ngroups;
-  const int64_t blocks = ceil_div(warps, 8);
+  const int64_t blocks = ceil_div(rows * ceil_div(ngroups, kRunGroups), kStreamWarps);
   if (blocks > 0x7FFFFFFFll) return QG_UNSUPPORTED_SHAPE;
-  if (bits == 8) {
-    quantize_rtn_kernel<8><<<(unsigned)blocks, 256, 0, st>>>(src, ld_src, rows, cols, (uint8_t*)dst->codes, dst->ld,
-                                                             dst->scales, dst->zeros, ngroups);
-  } else if (bits == 4) {
-    quantize_rtn_kernel<4><<<(unsigned)blocks, 256, 0, st>>>(src, ld_src, rows, cols, (uint8_t*)dst->codes,
-                                                             dst->ld / 2, dst->scales, dst->zeros, ngroups);
-  } else {
-    quantize_rtn_kernel<2><<<(unsigned)blocks, 256, 0, st>>>(src, ld_src, rows, cols, (uint8_t*)dst->codes,
-                                                             dst->ld / 4, dst->scales, dst->zeros, ngroups);
-  }
+  auto kern = bits == 8 ? quantize_rtn_kernel<8> : bits == 4 ? quantize_rtn_kernel<4> : quantize_rtn_kernel<2>;
+  kern<<<(unsigned)blocks, kStreamWarps * 32, 0, st>>>(src, ld_src, rows, cols, (uint8_t*)dst->codes, dst->ld * bits / 8,
+                                                       dst->scales, dst->zeros, ngroups);
   QG_LAUNCH_CHECK();
   return QG_OK;
 }
 
 // ------------------------------------------------------------------------ dequantize
-__global__ void __launch_bounds__(256)
-dequantize_kernel(qg_qtensor T, int ngroups, float* __restrict__ dst, int64_t ld_dst) {
-  const int64_t chunks_per_row = ceil_div(T.cols, 8);
-  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= T.rows * chunks_per_row) return;
-  const int64_t row = idx / chunks_per_row;
-  const int64_t c0 = (idx % chunks_per_row) * 8;
-  const int nvalid = (int)min((int64_t)8, T.cols - c0);
-  const int g = (int)(c0 / kGroup);
-  const float s = __ldg(T.scales + row * ngroups + g), z = __ldg(T.zeros + row * ngroups + g);
-  float q[8];
-  load_codes8(T, row, c0, nvalid, q);
+template <int BITS>
+__global__ void __launch_bounds__(kStreamWarps * 32)
+dequantize_kernel(const uint8_t* __restrict__ codes, int64_t ld_code_bytes, const float* __restrict__ scales,
+                  const float* __restrict__ zeros, int64_t rows, int64_t cols, int ngroups, float* __restrict__ dst, int64_t ld_dst) {
+  const int lane = threadIdx.x & 31;
+  int64_t row;
+  int run;
+  if (!stream_unit(rows, (ngroups + kRunGroups - 1) / kRunGroups, row, run)) return;
+  constexpr int kPerByte = 8 / BITS, kOffset = BITS == 8 ? 0 : 1 << (BITS - 1);
+  const int64_t c0 = (int64_t)run * kRunGroups * kGroup + lane * 4;
+  const uint8_t* p = codes + row * ld_code_bytes + c0 / kPerByte;
   float* out = dst + row * ld_dst + c0;
+  uint32_t w[kRunPieces];
+  int nv[kRunPieces];
 #pragma unroll
-  for (int i = 0; i < 8; ++i)
-    if (i < nvalid) out[i] = __fmul_rn(__fsub_rn(q[i], z), s);
+  for (int i = 0; i < kRunPieces; ++i) {
+    nv[i] = (int)max((int64_t)0, min((int64_t)4, cols - (c0 + 128 * i)));
+    const uint8_t* pi = p + 128 * i / kPerByte;
+    w[i] = 0;
+    if (nv[i] == 4) {
+      if (BITS == 8) w[i] = __ldcs(reinterpret_cast<const uint32_t*>(pi));
+      else if (BITS == 4) w[i] = __ldcs(reinterpret_cast<const uint16_t*>(pi));
+      else w[i] = *pi;
+    } else {
+      for (int e = 0; e < (nv[i] + kPerByte - 1) / kPerByte; ++e) w[i] |= (uint32_t)pi[e] << (8 * e);
+    }
+  }
+  float s[kRunGroups], z[kRunGroups];
+#pragma unroll
+  for (int h = 0; h < kRunGroups; ++h) {
+    const int g = min(run * kRunGroups + h, ngroups - 1);
+    s[h] = __ldg(scales + row * ngroups + g);
+    z[h] = __ldg(zeros + row * ngroups + g);
+  }
+#pragma unroll
+  for (int i = 0; i < kRunPieces; ++i) {
+    float v[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const uint32_t bits = (w[i] >> (BITS * e)) & ((1u << BITS) - 1u);
+      const int q = BITS == 8 ? (int)(int8_t)bits : (int)bits - kOffset;
+      v[e] = __fmul_rn(__fsub_rn((float)q, z[i / 2]), s[i / 2]);
+    }
+    if (nv[i] == 4) {
+      *reinterpret_cast<float4*>(out + 128 * i) = make_float4(v[0], v[1], v[2], v[3]);
+    } else {
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        if (e < nv[i]) out[128 * i + e] = v[e];
+    }
+  }
 }
 
 int launch_dequantize(const qg_qtensor* src, float* dst, int64_t ld_dst, cudaStream_t st) {
   const int ngroups = (int)ceil_div(src->cols, kGroup);
-  const int64_t threads = src->rows * ceil_div(src->cols, 8);
-  const int64_t blocks = ceil_div(threads, 256);
+  const int64_t blocks = ceil_div(src->rows * ceil_div(ngroups, kRunGroups), kStreamWarps);
   if (blocks > 0x7FFFFFFFll) return QG_UNSUPPORTED_SHAPE;
-  dequantize_kernel<<<(unsigned)blocks, 256, 0, st>>>(*src, ngroups, dst, ld_dst);
+  auto kern = src->bits == 8 ? dequantize_kernel<8> : src->bits == 4 ? dequantize_kernel<4> : dequantize_kernel<2>;
+  kern<<<(unsigned)blocks, kStreamWarps * 32, 0, st>>>((const uint8_t*)src->codes, src->ld * src->bits / 8, src->scales, src->zeros,
+                                                       src->rows, src->cols, ngroups, dst, ld_dst);
   QG_LAUNCH_CHECK();
   return QG_OK;
 }
