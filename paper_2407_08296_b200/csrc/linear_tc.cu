@@ -593,6 +593,7 @@ int launch_mode(const LinArgs& args, int32_t* status, cudaStream_t st) {
 int launch_int8_linear(int mode, const uint16_t* act, int64_t ld_act, const uint16_t* act2, int64_t ld_act2,
                        const qg_qtensor* W, int64_t T, int64_t m, int64_t n, uint16_t* D, int64_t ldd,
                        int32_t* status, cudaStream_t st) {
+  if (mode == kForward && T <= kSkinnyTokens) return launch_int8_linear_skinny(act, ld_act, W, T, D, ldd, st);
   LinArgs a;
   memset(&a, 0, sizeof(a));
   a.D = D;

@@ -265,4 +265,8 @@ int launch_int8_linear(int mode, const uint16_t* act, int64_t ld_act, const uint
                        const qg_qtensor* W, int64_t T, int64_t m, int64_t n, uint16_t* D, int64_t ldd,
                        int32_t* status, cudaStream_t st);
 
+// linear_skinny.cu: the forward product for at most kSkinnyTokens rows of X
+constexpr int64_t kSkinnyTokens = 16;
+int launch_int8_linear_skinny(const uint16_t* X, int64_t ldx, const qg_qtensor* W, int64_t T, uint16_t* Y, int64_t ldy, cudaStream_t st);
+
 }  // namespace qg

@@ -1,0 +1,42 @@
+"""The INT8 linear layer where its kernels change: the few-token forward product at the ends of its range and of its rule
+for warps per CTA, against torch's fp32 product of the same operands."""
+import pytest
+import torch
+
+from paper_2407_08296_b200 import binding as B
+
+pytestmark = pytest.mark.gpu
+
+
+def _operands(T, m, n, seed=0):
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(seed)
+    w = B.zeros_matrix(m, n, torch.float32)
+    w.copy_(0.02 * torch.randn(m, n, device="cuda", generator=gen) + 0.01)
+    W = B.quantize_int8(w)
+    # what lies past a row may be anything: NaN here
+    X, dY = B.empty_matrix(T, n, torch.bfloat16), B.empty_matrix(T, m, torch.bfloat16)
+    for t in (X, dY):
+        (t._base if t._base is not None else t).fill_(float("nan"))
+        t.copy_(torch.randn(t.shape, device="cuda", generator=gen))
+    return X, dY, W, B.dequantize(W).to(torch.bfloat16).float()
+
+
+def _check(got, a, b, status):
+    """Products are exact and sums binary32: the error is that of a binary32 sum of K terms in another order (both sides),
+    K * 2^-24 of the sum of magnitudes to first order (that bound holds for any order), plus the rounding to bfloat16."""
+    want, mag = a @ b, a.abs() @ b.abs()
+    tol = 2 * a.shape[1] * 2.0 ** -24 * mag + 2.0 ** -8 * want.abs()
+    assert got.shape == want.shape and int(status.item()) == 0
+    assert bool(((got.float() - want).abs() <= tol).all())
+    assert float((got == want.to(torch.bfloat16)).float().mean()) > 0.98     # rounded the same but for near-ties
+
+
+@pytest.mark.parametrize("T", [1, 7, 8, 9, 16, 17])
+@pytest.mark.parametrize("m,n", [(1, 1), (17, 255), (40, 1025), (2369, 4096), (2368, 4096), (15, 11001)])
+def test_forward_of_a_few_tokens(T, m, n):
+    torch.backends.cuda.matmul.allow_tf32 = False
+    X, _, W, Wd = _operands(T, m, n, seed=m + n)
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    Y = B.int8_linear_forward(X, W, status=status)
+    _check(Y, X.float(), Wd.T, status)
