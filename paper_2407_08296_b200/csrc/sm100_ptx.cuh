@@ -308,6 +308,12 @@ __device__ __forceinline__ void umma_commit_pair(uint64_t* bar) {
                : "memory");
 }
 
+// ----------------------------------------------------------------------------- programmatic dependent launch
+// A launch made with programmatic stream serialization may begin once every CTA of the launch before it has called
+// grid_launch_dependents (or left); grid_dependency_wait then waits until that launch is complete and its writes visible.
+__device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 __device__ __forceinline__ void named_bar_sync(int id, int nthreads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
 }

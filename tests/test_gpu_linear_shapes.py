@@ -40,3 +40,25 @@ def test_forward_of_a_few_tokens(T, m, n):
     status = torch.zeros(1, dtype=torch.int32, device="cuda")
     Y = B.int8_linear_forward(X, W, status=status)
     _check(Y, X.float(), Wd.T, status)
+
+
+# Tiles of 128 x 256 (256 x 256 for the input gradient): a few of them shared by clusters of 2 .. 8 CTAs along K, a whole
+# round of persistent CTAs followed by a remainder in clusters, extents that end inside a tile, a K that ends inside a block.
+@pytest.mark.parametrize("T,m,n", [(40, 200, 1500), (300, 1159, 3001), (257, 515, 2100), (4200, 1100, 700), (129, 2100, 4500), (1000, 3001, 640)])
+def test_products_whose_tiles_are_split_along_k(T, m, n):
+    torch.backends.cuda.matmul.allow_tf32 = False
+    X, dY, W, Wd = _operands(T, m, n, seed=T)
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    x, d = X.float(), dY.float()
+    Y = B.int8_linear_forward(X, W, status=status)
+    _check(Y, x, Wd.T, status)
+    dX = B.int8_linear_backward_input(dY, W, status=status)
+    _check(dX, d, Wd, status)
+    # the weight gradient reads whole 64-column slabs: give it zeros past the row
+    Xz, dYz = B.zeros_matrix(T, n, torch.bfloat16), B.zeros_matrix(T, m, torch.bfloat16)
+    Xz.copy_(X)
+    dYz.copy_(dY)
+    G = B.int8_linear_backward_weight(dYz, Xz, status=status)
+    _check(G, d.T, x, status)
+    for again, first in ((B.int8_linear_forward(X, W), Y), (B.int8_linear_backward_input(dY, W), dX), (B.int8_linear_backward_weight(dYz, Xz), G)):
+        assert torch.equal(again, first)
