@@ -136,13 +136,13 @@ def _check(status: int, what: str) -> None:
 
 
 def _stream_ptr(stream) -> int:
-    if stream is None:
-        stream = torch.cuda.current_stream()
+    if stream is None:          # the current stream's handle, without building a Stream object around it
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
     return int(stream.cuda_stream)
 
 
 def _ptr(t) -> int:
-    return 0 if t is None else int(t.data_ptr())
+    return 0 if t is None else t.data_ptr()
 
 
 def round_up(x: int, mult: int) -> int:
@@ -152,7 +152,8 @@ def round_up(x: int, mult: int) -> int:
 def empty_matrix(rows: int, cols: int, dtype, device="cuda", pitch_multiple: int = 64) -> torch.Tensor:
     """A rows x cols view of a buffer whose row pitch is cols rounded up to ``pitch_multiple`` elements."""
     ld = round_up(cols, pitch_multiple)
-    return torch.empty((rows, ld), dtype=dtype, device=device)[:, :cols]
+    buf = torch.empty((rows, ld), dtype=dtype, device=device)
+    return buf if ld == cols else buf[:, :cols]
 
 
 def zeros_matrix(rows: int, cols: int, dtype, device="cuda", pitch_multiple: int = 64) -> torch.Tensor:
@@ -161,9 +162,10 @@ def zeros_matrix(rows: int, cols: int, dtype, device="cuda", pitch_multiple: int
 
 
 def _matrix_ld(t: torch.Tensor, what: str) -> int:
-    if t.dim() != 2 or (t.shape[1] > 1 and t.stride(1) != 1):
+    shape, stride = t.shape, t.stride()
+    if len(shape) != 2 or (shape[1] > 1 and stride[1] != 1):
         raise ValueError(f"{what}: expected a 2-D tensor with unit column stride")
-    return int(t.stride(0)) if t.shape[0] > 1 else max(int(t.stride(0)), int(t.shape[1]))
+    return stride[0] if shape[0] > 1 else max(stride[0], shape[1])
 
 
 @dataclass
@@ -283,8 +285,18 @@ def dequantize(q: QTensor, out: torch.Tensor | None = None, stream=None) -> torc
     return out
 
 
+def _bf16_out(like: torch.Tensor, rows: int, cols: int) -> torch.Tensor:
+    """``empty_matrix`` on the device of ``like`` (new_empty costs half of torch.empty)."""
+    if like.dtype is not torch.bfloat16:
+        return empty_matrix(rows, cols, torch.bfloat16, like.device, 64)
+    ld = round_up(cols, 64)
+    buf = like.new_empty((rows, ld))
+    return buf if ld == cols else buf[:, :cols]
+
+
 def _bf16_arg(t: torch.Tensor, what: str) -> torch.Tensor:
-    if t.dtype not in (torch.bfloat16, torch.int16, torch.uint16):
+    dt = t.dtype
+    if dt is not torch.bfloat16 and dt is not torch.int16 and dt is not torch.uint16:
         raise ValueError(f"{what} must hold bfloat16 values (bfloat16 / int16 / uint16 storage)")
     return t
 
@@ -294,7 +306,7 @@ def int8_linear_forward(X: torch.Tensor, W: QTensor, out: torch.Tensor | None = 
     """App. A, forward: Y (T x m) = X (T x n) W~^T with the INT8 weight dequantized inside the GEMM."""
     T = X.shape[0]
     if out is None:
-        out = empty_matrix(T, W.rows, torch.bfloat16, X.device, 64)
+        out = _bf16_out(X, T, W.rows)
     cs = W.c_struct()
     _check(lib().qgalore_int8_linear_forward(_ptr(_bf16_arg(X, "X")), T, _matrix_ld(X, "X"), C.byref(cs),
                                              _ptr(_bf16_arg(out, "out")), _matrix_ld(out, "out"),
@@ -308,7 +320,7 @@ def int8_linear_backward_input(dY: torch.Tensor, W: QTensor, out: torch.Tensor |
     """App. A, backward: grad_input (T x n) = dY (T x m) W~."""
     T = dY.shape[0]
     if out is None:
-        out = empty_matrix(T, W.cols, torch.bfloat16, dY.device, 64)
+        out = _bf16_out(dY, T, W.cols)
     cs = W.c_struct()
     _check(lib().qgalore_int8_linear_backward_input(_ptr(_bf16_arg(dY, "dY")), T, _matrix_ld(dY, "dY"), C.byref(cs),
                                                     _ptr(_bf16_arg(out, "out")), _matrix_ld(out, "out"),
@@ -326,7 +338,7 @@ def int8_linear_backward_weight(dY: torch.Tensor, X: torch.Tensor, out: torch.Te
     if X.shape[0] != T:
         raise ValueError("dY and X must have the same number of rows")
     if out is None:
-        out = empty_matrix(m, n, torch.bfloat16, dY.device, 64)
+        out = _bf16_out(dY, m, n)
     _check(lib().qgalore_int8_linear_backward_weight(_ptr(_bf16_arg(dY, "dY")), T, _matrix_ld(dY, "dY"),
                                                      _ptr(_bf16_arg(X, "X")), _matrix_ld(X, "X"), m, n,
                                                      _ptr(_bf16_arg(out, "out")), _matrix_ld(out, "out"),
