@@ -5,6 +5,8 @@
 // A 32 x 256 output tile per block of 256 threads: warp w owns rows 4w..4w+3, lane l the eight
 // columns 8l..8l+7, so one warp holds one whole quantization group of a row and the group
 // minimum/maximum are warp-shuffle reductions.  fp32 accumulation of bf16 products.
+#include "launch.cuh"
+#include "sm100_ptx.cuh"
 #include "step_epilogue.cuh"
 
 namespace qg {
@@ -15,6 +17,8 @@ constexpr int kTM = 32, kTN = 256, kTK = 32;
 
 __global__ void __launch_bounds__(256)
 dequant_p_bf16_kernel(qg_qtensor P, uint16_t* __restrict__ out, int64_t ld_out) {
+  ptx::grid_launch_dependents();
+  ptx::grid_dependency_wait();
   const int ngroups = (int)((P.cols + kGroup - 1) / kGroup);
   const int64_t chunks = P.cols / 8;                 // r % 32 == 0
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -164,9 +168,7 @@ struct RequantEpilogue {
 
 int launch_dequant_p(const qg_qtensor& P, uint16_t* out, int64_t ld_out, cudaStream_t st) {
   const int64_t threads = P.rows * (P.cols / 8);
-  dequant_p_bf16_kernel<<<(unsigned)ceil_div(threads, 256), 256, 0, st>>>(P, out, ld_out);
-  QG_LAUNCH_CHECK();
-  return QG_OK;
+  return launch_overlapping(dequant_p_bf16_kernel, (unsigned)ceil_div(threads, 256), 256, 0, st, 1, P, out, ld_out);
 }
 
 size_t simt_workspace_bytes(int64_t m, int64_t n, int64_t r) {

@@ -30,6 +30,7 @@
 #include "sm100_ptx.cuh"
 #include "tensor_map.cuh"
 #include "step_epilogue.cuh"
+#include "launch.cuh"
 
 namespace qg {
 
@@ -261,6 +262,7 @@ project_adam_kernel(const __grid_constant__ TcProblem single, const TcProblem* _
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const TcProblem* probs = SINGLE ? &single : table;
+  grid_launch_dependents();
 
   if (threadIdx.x == 0) {
     // a stage is full once the producer's copies have landed and, in a launch some matrix of which has its A tile
@@ -284,6 +286,7 @@ project_adam_kernel(const __grid_constant__ TcProblem single, const TcProblem* _
   if (CTAS == 2) cluster_sync_all();              // the peer's barriers exist before anything signals them
   tc_fence_after_sync();
   const uint32_t tmem_base = *tmem_slot;
+  grid_dependency_wait();                         // everything up to here overlaps the end of the launch before
 
   // tile -> (r block, n block) of its problem; consecutive tiles share the n block, so that the G tile
   // one of them brings from HBM serves the others from L2.  A pair takes two adjacent r blocks (this CTA the
@@ -1026,6 +1029,7 @@ backproject_sr_kernel(const __grid_constant__ TcProblem single, const TcProblem*
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const TcProblem* probs = SINGLE ? &single : table;
+  grid_launch_dependents();
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < S::kStages; ++i) { mbar_init(&full[i], 1); mbar_init(&empty[i], 1); }
@@ -1043,6 +1047,7 @@ backproject_sr_kernel(const __grid_constant__ TcProblem single, const TcProblem*
   if (CTAS == 2) cluster_sync_all();              // the peer's barriers exist before anything signals them
   tc_fence_after_sync();
   const uint32_t tmem_base = *tmem_slot;
+  grid_dependency_wait();                         // everything up to here overlaps the end of the launch before
 
   // tile -> (m block, n block) of its problem; consecutive tiles share the n block of N_b.  A pair takes two
   // adjacent m blocks, this CTA the one of its rank; the leader's `full` barriers count the loads of both CTAs
@@ -1452,23 +1457,8 @@ int launch_k1(const TcProblem* single, const TcProblem* table, const TileSchedul
   const int sms = sm_count();
   const int grid = SINGLE ? (total_tiles < sms ? total_tiles : sms) : grid_planned;
   static const TcProblem dummy{};
-  if (CTAS == 1) {
-    kern<<<grid, S::kThreads, S::kBytes, st>>>(single ? *single : dummy, table, sched, total_tiles, sc, status, conv_active);
-  } else {
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3(S::kThreads);
-    cfg.dynamicSmemBytes = S::kBytes;
-    cfg.stream = st;
-    cudaLaunchAttribute attr{};
-    attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim.x = 2; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    QG_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, dummy, table, sched, total_tiles, sc, status, conv_active));
-  }
-  QG_LAUNCH_CHECK();
-  return QG_OK;
+  return launch_overlapping(kern, (unsigned)grid, S::kThreads, S::kBytes, st, CTAS, single ? *single : dummy, table, sched, total_tiles, sc, status,
+                            conv_active);
 }
 
 template <bool SINGLE, int CTAS>
@@ -1482,23 +1472,7 @@ int launch_k2(const TcProblem* single, const TcProblem* table, const TileSchedul
   const int sms = sm_count();
   const int grid = SINGLE ? (total_tiles < sms ? total_tiles : sms) : grid_planned;
   static const TcProblem dummy{};
-  if (CTAS == 1) {
-    kern<<<grid, S::kThreads, S::kBytes, st>>>(single ? *single : dummy, table, sched, total_tiles, sc, status);
-  } else {
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3(S::kThreads);
-    cfg.dynamicSmemBytes = S::kBytes;
-    cfg.stream = st;
-    cudaLaunchAttribute attr{};
-    attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim.x = 2; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    QG_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, dummy, table, sched, total_tiles, sc, status));
-  }
-  QG_LAUNCH_CHECK();
-  return QG_OK;
+  return launch_overlapping(kern, (unsigned)grid, S::kThreads, S::kBytes, st, CTAS, single ? *single : dummy, table, sched, total_tiles, sc, status);
 }
 
 // ---- P~ = bf16(dequant(P)) for a list of matrices in one launch
@@ -1540,7 +1514,9 @@ constexpr int kDqUnits = 8;
 
 __global__ void __launch_bounds__(256)
 dequant_p_grouped_kernel(const DequantItem* __restrict__ items, const int32_t* __restrict__ block_item) {
+  grid_launch_dependents();
   const DequantItem& it = items[__ldg(block_item + blockIdx.x)];   // host-made map: block -> matrix of the chunk
+  grid_dependency_wait();
   const uint32_t cols = (uint32_t)it.P.cols, rows = (uint32_t)it.P.rows;
   const uint32_t per_row = cols / 8, ngroups = (cols + kGroup - 1) / kGroup, total = rows * per_row;   // r % 32 == 0
   const uint32_t base = (blockIdx.x - (uint32_t)it.block0) * (kDqUnits * 256u) + threadIdx.x;
@@ -1807,8 +1783,9 @@ int plan_step(const Plan* plan, const StepScalars& sc, int32_t* status, cudaStre
   for (const PlanChunk& ch : plan->chunks) {
     if (ev) QG_CUDA_TRY(cudaEventRecord(ev[4 * c + 0], st));
     if (ch.dq_blocks > 0) {                              // matrices whose projection the first kernel does not convert itself
-      dequant_p_grouped_kernel<<<ch.dq_blocks, 256, 0, st>>>(plan->dq_dev + ch.first, plan->sched_dev + ch.dq_map_off);
-      QG_LAUNCH_CHECK();
+      const int rc = launch_overlapping(dequant_p_grouped_kernel, (unsigned)ch.dq_blocks, 256, 0, st, 1, plan->dq_dev + ch.first,
+                                        plan->sched_dev + ch.dq_map_off);
+      if (rc != QG_OK) return rc;
     }
     if (ev) QG_CUDA_TRY(cudaEventRecord(ev[4 * c + 1], st));
     const TcProblem* tab = plan->table_dev + ch.first;
