@@ -168,7 +168,7 @@ struct RequantEpilogue {
 
 int launch_dequant_p(const qg_qtensor& P, uint16_t* out, int64_t ld_out, cudaStream_t st) {
   const int64_t threads = P.rows * (P.cols / 8);
-  return launch_overlapping(dequant_p_bf16_kernel, (unsigned)ceil_div(threads, 256), 256, 0, st, 1, P, out, ld_out);
+  return launch_overlapping(dequant_p_bf16_kernel, (unsigned)ceil_div(threads, 256), 256, 0, st, 1, true, P, out, ld_out);
 }
 
 size_t simt_workspace_bytes(int64_t m, int64_t n, int64_t r) {

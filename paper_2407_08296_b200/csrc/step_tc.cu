@@ -1442,6 +1442,12 @@ int set_smem_once(K kernel, int bytes, bool* done) {
   return QG_OK;
 }
 
+// Whether a launch of the step overlaps the one before it.  Short launches are latency: 512 x 1376 at r = 128 28.7 -> 22.7 us
+// per step, 5461 x 2048 at r = 512 67.6 -> 63.2, the first pass over a LLaMA-130M stack (5 tiles per CTA) 285 -> 267.  Long
+// ones run at the power cap, where closing a gap saves nothing and waiting CTAs cost a little: a LLaMA-1B stack (30 tiles
+// per CTA) 3.68-3.70 ms a step with ordinary launches, 3.73-3.79 with overlapping ones.
+bool overlaps(int64_t tiles, int64_t grid) { return tiles <= 8 * grid; }
+
 // The projection's column-tile width: 256 halves the operand traffic per flop of the 128-wide tile,
 // but only pays once there are enough tiles to occupy every SM.
 int choose_bn(int64_t tiles_at_256) { return tiles_at_256 >= 2 * (int64_t)sm_count() ? 256 : 128; }
@@ -1457,7 +1463,7 @@ int launch_k1(const TcProblem* single, const TcProblem* table, const TileSchedul
   const int sms = sm_count();
   const int grid = SINGLE ? (total_tiles < sms ? total_tiles : sms) : grid_planned;
   static const TcProblem dummy{};
-  return launch_overlapping(kern, (unsigned)grid, S::kThreads, S::kBytes, st, CTAS, single ? *single : dummy, table, sched, total_tiles, sc, status,
+  return launch_overlapping(kern, (unsigned)grid, S::kThreads, S::kBytes, st, CTAS, overlaps(total_tiles * CTAS, grid), single ? *single : dummy, table, sched, total_tiles, sc, status,
                             conv_active);
 }
 
@@ -1472,7 +1478,7 @@ int launch_k2(const TcProblem* single, const TcProblem* table, const TileSchedul
   const int sms = sm_count();
   const int grid = SINGLE ? (total_tiles < sms ? total_tiles : sms) : grid_planned;
   static const TcProblem dummy{};
-  return launch_overlapping(kern, (unsigned)grid, S::kThreads, S::kBytes, st, CTAS, single ? *single : dummy, table, sched, total_tiles, sc, status);
+  return launch_overlapping(kern, (unsigned)grid, S::kThreads, S::kBytes, st, CTAS, overlaps(total_tiles * CTAS, grid), single ? *single : dummy, table, sched, total_tiles, sc, status);
 }
 
 // ---- P~ = bf16(dequant(P)) for a list of matrices in one launch
@@ -1783,7 +1789,7 @@ int plan_step(const Plan* plan, const StepScalars& sc, int32_t* status, cudaStre
   for (const PlanChunk& ch : plan->chunks) {
     if (ev) QG_CUDA_TRY(cudaEventRecord(ev[4 * c + 0], st));
     if (ch.dq_blocks > 0) {                              // matrices whose projection the first kernel does not convert itself
-      const int rc = launch_overlapping(dequant_p_grouped_kernel, (unsigned)ch.dq_blocks, 256, 0, st, 1, plan->dq_dev + ch.first,
+      const int rc = launch_overlapping(dequant_p_grouped_kernel, (unsigned)ch.dq_blocks, 256, 0, st, 1, overlaps(ch.k2_tiles, ch.k2_grid), plan->dq_dev + ch.first,
                                         plan->sched_dev + ch.dq_map_off);
       if (rc != QG_OK) return rc;
     }
