@@ -1,0 +1,777 @@
+// Leading eigenvectors of symmetric matrices, several of one size at a time, for the subspace refresh (Sec. 3.5).
+//
+//   1. Householder reduction to tridiagonal form, A = H T H^T, H = H_0 H_1 ... (binary32)
+//   2. the r largest eigenvalues of T by multisection on Sturm counts (binary64)
+//   3. their eigenvectors by one twisted factorisation of T - lambda each (binary64)
+//   4. X = H Z (binary32)
+//
+// The reduction is a chain of N dependent steps whatever runs it, so it is laid out for the shortest step: the matrix
+// stays on the SMs (columns dealt out to the CTAs, in registers and shared memory), one pass over it per step applies the
+// previous rank-2 update and multiplies by the new Householder vector, and ONE exchange through L2 per step carries what
+// every CTA needs of the others.  That exchange has no barrier: every value travels in a word of its own with the step's
+// number beside it, and the reader polls the word itself.
+#include <algorithm>
+#include <cmath>
+#include <mutex>
+
+#include "refresh_common.cuh"
+#include "sm100_ptx.cuh"
+
+namespace qg {
+
+namespace {
+
+using ptx::fma2;
+using ptx::mul2;
+
+// ------------------------------------------------------------------------------------------ 1. tridiagonal form
+// Column j of a matrix belongs to CTA j mod C of its C; row and column indices below the step are dead, so a cyclic deal
+// keeps the CTAs level to the end.  Both triangles are kept: column j then yields (A v)_j by itself, with no sum over
+// CTAs, and element k + 1 of column j is element j of the next pivot column, so the owner of column j publishes both
+// values the next step wants at index j.  Of step k (v, tau: the Householder vector of step k - 1, its update pending):
+//     P_j = (A v)_j, R_j = A_kj                      received for j >= k
+//     w = tau P - kappa v, kappa = tau^2 (P . v) / 2
+//     x = R - w - v w_k = (R - tau P) + v mu          (column k with the pending update; mu = 2 kappa - tau P_k, v_k = 1)
+//     d_k = x_k;  v', tau', e_k annihilate x below k + 1
+//     A <- A - v w^T - w v^T,  P' = A v'              one pass over the columns j > k
+//     publish P'_j and A_{k+1, j}
+// What bounds a step is latency: the trip through L2, two CTA barriers and the reductions.  |x|^2 is therefore taken
+// from sums over R - tau P and v that are reduced together with P . v (one barrier less); where the two terms of x
+// cancel the sum is taken again over x itself.
+// A thread keeps rows tid + 512 q of every column, the last columns in registers, those before in shared memory and,
+// past that, in global memory (L2): the row's v, w, v' are then registers too, and the pass reads nothing but two
+// scalars per column.
+constexpr int kTriThreads = 512, kTriWarps = kTriThreads / 32;
+constexpr uint32_t kPollLimit = 1u << 20;
+constexpr int kTriSmem = 225 * 1024;
+
+__device__ __forceinline__ uint4 ld_relaxed_v4(const uint4* p) {
+  uint4 v;
+  asm volatile("ld.relaxed.gpu.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
+  return v;
+}
+// Two values, each in an 8-byte word with the tag of its step.
+__device__ __forceinline__ void st_relaxed_v4(uint4* p, float a, float b, uint32_t tag) {
+  asm volatile("st.relaxed.gpu.global.v4.u32 [%0], {%1, %2, %3, %4};" ::"l"(p), "r"(__float_as_uint(a)), "r"(tag), "r"(__float_as_uint(b)), "r"(tag)
+               : "memory");
+}
+
+struct TriArgs {
+  Ptrs<float> A, V, tau, d, e;
+  Ptrs<uint4> xchg;
+  int N, Np, C;
+  int in_smem;               // columns per CTA that shared memory holds
+};
+
+__device__ __forceinline__ float2 both(float x) { return make_float2(x, x); }
+// Sums of several values over the lanes of a warp, by halving the values and the lanes together.
+__device__ __forceinline__ float halve(float lo, float hi, int bit, int lane) {
+  const bool up = lane & bit;
+  return (up ? hi : lo) + __shfl_xor_sync(0xFFFFFFFFu, up ? lo : hi, bit);
+}
+// lane 8 i: the sum of value i
+__device__ __forceinline__ float warp_sums4(const float (&v)[4], int lane) {
+  const float a = halve(v[0], v[2], 16, lane), b = halve(v[1], v[3], 16, lane);
+  float s = halve(a, b, 8, lane);
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
+  return s;
+}
+// lane 4 i: the sum of value i
+__device__ __forceinline__ float warp_sums8(const float2 (&v)[4], int lane) {
+  const float a = halve(v[0].x, v[2].x, 16, lane), b = halve(v[0].y, v[2].y, 16, lane);
+  const float c = halve(v[1].x, v[3].x, 16, lane), d = halve(v[1].y, v[3].y, 16, lane);
+  const float e = halve(a, c, 8, lane), f = halve(b, d, 8, lane);
+  float s = halve(e, f, 4, lane);
+  s += __shfl_xor_sync(0xFFFFFFFFu, s, 2);
+  s += __shfl_xor_sync(0xFFFFFFFFu, s, 1);
+  return s;
+}
+
+template <int NQ>                              // rows per thread: N <= NQ * kTriThreads
+__global__ void __launch_bounds__(kTriThreads, 1)
+tridiagonal_kernel(const __grid_constant__ TriArgs a, int32_t* __restrict__ status) {
+  constexpr int RC = 64 / NQ;                  // columns in registers
+  extern __shared__ __align__(16) float tri_smem[];
+  __shared__ __align__(16) float4 red1[kTriWarps];
+  __shared__ float red_x[kTriWarps];
+  __shared__ float s_pk, s_a1, s_v1;
+  __shared__ int s_fail;
+  const int N = a.N, Np = a.Np, C = a.C;
+  const int mat = blockIdx.x / C, cta = blockIdx.x % C;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  float* const A = a.A.p[mat];
+  float* const Vg = a.V.p[mat];
+  uint4* const xchg = a.xchg.p[mat];
+  const int ncols = (N - cta + C - 1) / C;     // this CTA's columns: cta + l C, l = 0 .. ncols - 1
+  const int nr = min(ncols, RC), ns = min(ncols - nr, a.in_smem), ng = ncols - nr - ns;   // registers, shared, global (these retire first)
+  const int nc8 = ((N + C - 1) / C + 8) & ~7;  // pitch of the per-column arrays: groups of eight may reach past the end
+  float* const colP = tri_smem;                // P_j and v_j of this CTA's columns
+  float* const colV = colP + 2 * nc8;          // (twice the room: a group starts anywhere)
+  float* const pivot = colV + 2 * nc8;         // A_{k+1, j}
+  float* const part = pivot + 2 * nc8;         // [warp][column] partial sums of P'_j
+  float* const scols = part + kTriWarps * 2 * nc8;   // [column][Np]
+
+  float2 ar[NQ][RC / 2];
+  float v[NQ], w[NQ], vn[NQ], r[NQ];
+  int slot[NQ];                                // the row's own column, if it is this CTA's, else -1
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) {
+    const int j = tid + q * kTriThreads;
+    v[q] = w[q] = 0.f;
+    r[q] = j < N ? Vg[(int64_t)(N - 1) * Np + j] : 0.f;   // row 0 as eig_scale_kernel put it aside
+    slot[q] = j < N && j % C == cta ? j / C : -1;
+#pragma unroll
+    for (int c = 0; c < RC; c += 2) {
+      const int l = ng + ns + c;
+      ar[q][c / 2].x = (l < ncols && j < Np) ? A[(int64_t)(cta + l * C) * Np + j] : 0.f;
+      ar[q][c / 2].y = (l + 1 < ncols && j < Np) ? A[(int64_t)(cta + (l + 1) * C) * Np + j] : 0.f;
+    }
+  }
+  for (int l = 0; l < ns; ++l)
+    for (int i = tid; i < Np; i += kTriThreads) scols[l * Np + i] = A[(int64_t)(cta + (ng + l) * C) * Np + i];
+  for (int i = tid; i < 6 * nc8; i += kTriThreads) tri_smem[i] = 0.f;
+  if (tid == 0) { s_fail = 0; s_pk = 0.f; }
+  __syncthreads();
+
+  // A CTA works while it owns a column beyond the step's, i.e. while it has something to publish: whoever has received a
+  // step's values then knows that everybody who will ever read the step before has done so, and may overwrite them (the
+  // exchange is double buffered by the step's parity).  The owner of column k + 1 records what step k yields.
+  const int last = cta + (ncols - 1) * C;
+  float tau = 0.f;
+  for (int k = 0; k < N && (last > k || last == N - 1); ++k) {
+    const bool writer = k == N - 1 || cta == (k + 1) % C;
+    // ---- receive; sums over P . v, and over a = R - tau P and v below row k + 1
+    float sums[4] = {0.f, 0.f, 0.f, 0.f};
+    bool ok = true;
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) {
+      const int j = tid + q * kTriThreads;
+      float p = 0.f;
+      if (j >= k && j < N) {
+        if (k > 0) {
+          const uint4* in = xchg + (k & 1) * Np + j;
+          uint4 got = ld_relaxed_v4(in);
+          uint32_t polls = 0;
+          while ((got.y != (uint32_t)k || got.w != (uint32_t)k) && ++polls < kPollLimit) got = ld_relaxed_v4(in);
+          ok = ok && polls < kPollLimit;
+          p = __uint_as_float(got.x);
+          r[q] = __uint_as_float(got.z);
+        }
+        if (j == k) s_pk = p;
+      } else {
+        r[q] = 0.f;
+      }
+      if (slot[q] >= 0) { colP[slot[q]] = p; colV[slot[q]] = v[q]; }
+      w[q] = p;
+      r[q] = fmaf(-tau, p, r[q]);
+      if (j == k + 1) { s_a1 = r[q]; s_v1 = v[q]; }
+      sums[0] = fmaf(p, v[q], sums[0]);
+      if (j > k + 1) {
+        sums[1] = fmaf(r[q], r[q], sums[1]);
+        sums[2] = fmaf(r[q], v[q], sums[2]);
+        sums[3] = fmaf(v[q], v[q], sums[3]);
+      }
+    }
+    if (!ok) s_fail = 1;
+    {
+      const float s = warp_sums4(sums, lane);
+      if ((lane & 7) == 0) reinterpret_cast<float*>(&red1[warp])[lane >> 3] = s;
+    }
+    __syncthreads();
+    if (s_fail) {                              // somebody's values never came: every CTA runs into the same limit
+      if (tid == 0 && status) atomicOr(status, QG_DEV_WAIT_EXPIRED);
+      return;
+    }
+    float s_pv, s_aa, s_av, s_vv;
+    {
+      const float4 t = red1[lane & 15];
+      const float e = halve(t.x, t.z, 8, lane), f = halve(t.y, t.w, 8, lane);
+      float s = halve(e, f, 4, lane);
+      s += __shfl_xor_sync(0xFFFFFFFFu, s, 2);
+      s += __shfl_xor_sync(0xFFFFFFFFu, s, 1);
+      s_pv = __shfl_sync(0xFFFFFFFFu, s, 0);
+      s_aa = __shfl_sync(0xFFFFFFFFu, s, 4);
+      s_av = __shfl_sync(0xFFFFFFFFu, s, 8);
+      s_vv = __shfl_sync(0xFFFFFFFFu, s, 12);
+    }
+    const float kappa = 0.5f * tau * tau * s_pv, mu = fmaf(-tau, s_pk, 2.f * kappa);
+    const float alpha = fmaf(mu, s_v1, s_a1);
+    float sig = fmaf(mu, fmaf(mu, s_vv, 2.f * s_av), s_aa);
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) {
+      const int j = tid + q * kTriThreads;
+      w[q] = fmaf(tau, w[q], -kappa * v[q]);
+      r[q] = fmaf(mu, v[q], r[q]);             // x
+      if (j == k && writer) a.d.p[mat][k] = r[q];
+    }
+    if (k == N - 1) break;
+    if (!(sig >= 0.25f * s_aa)) {              // the same in every thread of every CTA
+      sig = 0.f;
+#pragma unroll
+      for (int q = 0; q < NQ; ++q)
+        if (tid + q * kTriThreads > k + 1) sig = fmaf(r[q], r[q], sig);
+      sig = warp_sum(sig);
+      if (lane == 0) red_x[warp] = sig;
+      __syncthreads();
+      sig = 0.f;
+      for (int i = 0; i < kTriWarps; ++i) sig += red_x[i];
+    }
+    const float tau_old = tau;
+    float beta = alpha, scl = 0.f;
+    tau = 0.f;
+    if (sig > 1e-36f) {
+      beta = -copysignf(sqrtf(fmaf(alpha, alpha, sig)), alpha);
+      tau = (beta - alpha) / beta;
+      scl = 1.f / (alpha - beta);
+    }
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) {
+      const int j = tid + q * kTriThreads;
+      vn[q] = j > k + 1 ? r[q] * scl : (j == k + 1 ? 1.f : 0.f);
+      if (writer && j < Np) Vg[(int64_t)k * Np + j] = vn[q];
+    }
+    if (writer && tid == 0) { a.tau.p[mat][k] = tau; a.e.p[mat][k] = beta; }
+
+    // ---- the pass, eight columns at a time
+    const int k1 = k + 1, qk = k1 / kTriThreads;
+    const bool pivot_thread = tid == k1 % kTriThreads;
+    const float2 tau2 = both(tau_old), kap2 = both(-kappa);
+    auto scalars = [&](int l, float2 (&wj)[4], float2 (&vj)[4]) {      // w_j, v_j of columns l .. l + 7
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        vj[c] = make_float2(colV[l + 2 * c], colV[l + 2 * c + 1]);
+        wj[c] = fma2(tau2, make_float2(colP[l + 2 * c], colP[l + 2 * c + 1]), mul2(kap2, vj[c]));
+      }
+    };
+    auto partial = [&](int l, const float2 (&acc)[4]) {
+      const float s = warp_sums8(acc, lane);
+      if ((lane & 3) == 0) part[warp * 2 * nc8 + l + (lane >> 2)] = s;
+    };
+    // columns in memory: element (row, l) at at(l)[row]
+    auto memory_columns = [&](int l0, int l1, auto at) {
+      for (int l = l0; l < l1; l += 8) {
+        if (cta + min(l + 7, l1 - 1) * C <= k) continue;               // all of them retired
+        float2 wj[4], vj[4], acc[4] = {};
+        scalars(l, wj, vj);
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) {
+          const int row = tid + q * kTriThreads;
+          if (q * kTriThreads + kTriThreads - 1 <= k || row >= Np) continue;
+          const float2 nv = both(-v[q]), nw = both(-w[q]), n2 = both(vn[q]);
+#pragma unroll
+          for (int c = 0; c < 4; ++c) {
+            const int la = l + 2 * c, lb = min(la + 1, l1 - 1);
+            if (la >= l1) break;
+            float2 x = make_float2(at(la)[row], at(lb)[row]);
+            x = fma2(nw, vj[c], fma2(nv, wj[c], x));
+            at(la)[row] = x.x;
+            if (la + 1 < l1) at(lb)[row] = x.y;
+            acc[c] = fma2(x, n2, acc[c]);
+            if (pivot_thread && q == qk) { pivot[la] = x.x; if (la + 1 < l1) pivot[la + 1] = x.y; }
+          }
+        }
+        partial(l, acc);
+      }
+    };
+    if (ng > 0) memory_columns(0, ng, [&](int l) { return A + (int64_t)(cta + l * C) * Np; });
+    if (ns > 0) memory_columns(ng, ng + ns, [&](int l) { return scols + (l - ng) * Np; });
+#pragma unroll
+    for (int g = 0; g < RC / 8; ++g) {
+      const int l = ng + ns + 8 * g;
+      if (l < ncols && cta + min(l + 7, ncols - 1) * C > k) {
+        float2 wj[4], vj[4], acc[4] = {};
+        scalars(l, wj, vj);
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) {
+          if (q * kTriThreads + kTriThreads - 1 <= k) continue;
+          const float2 nv = both(-v[q]), nw = both(-w[q]), n2 = both(vn[q]);
+#pragma unroll
+          for (int c = 0; c < 4; ++c) {
+            float2& x = ar[q][4 * g + c];
+            x = fma2(nw, vj[c], fma2(nv, wj[c], x));
+            acc[c] = fma2(x, n2, acc[c]);
+            if (pivot_thread && q == qk) { pivot[l + 2 * c] = x.x; pivot[l + 2 * c + 1] = x.y; }
+          }
+        }
+        partial(l, acc);
+      }
+    }
+    __syncthreads();
+    // ---- publish
+    for (int l = tid; l < ncols; l += kTriThreads) {
+      const int j = cta + l * C;
+      if (j <= k) continue;
+      float s = 0.f;
+#pragma unroll
+      for (int i = 0; i < kTriWarps; ++i) s += part[i * 2 * nc8 + l];
+      st_relaxed_v4(xchg + (k1 & 1) * Np + j, s, pivot[l], (uint32_t)k1);
+    }
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) v[q] = vn[q];
+  }
+}
+
+// The power of two that brings the largest diagonal element of a positive semi-definite A into [1, 2), so that squares
+// in the reduction neither over- nor underflow.
+__global__ void __launch_bounds__(256)
+eig_scale_factor_kernel(const Ptrs<const float> Ab, int N, int Np, const Ptrs<float> scaleb) {
+  const float* A = Ab.p[blockIdx.x];
+  __shared__ float red[8];
+  float top = 0.f;
+  for (int i = threadIdx.x; i < N; i += 256) top = fmaxf(top, fabsf(A[(int64_t)i * Np + i]));
+  top = warp_max(top);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = top;
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  for (int i = 0; i < 8; ++i) top = fmaxf(top, red[i]);
+  const int ex = (int)(__float_as_uint(top) >> 23) - 127;
+  scaleb.p[blockIdx.x][0] = !(top >= FLT_MIN) || !isfinite(top) ? 1.f : ex >= 127 ? 0x1p-126f : __uint_as_float((uint32_t)(127 - ex) << 23);
+}
+
+// Applies it, zeroes the padding columns, and puts row 0 aside (in the last row of V, which holds no Householder vector):
+// every CTA of the reduction starts from it, while their owners already write the columns.
+__global__ void __launch_bounds__(256)
+eig_scale_kernel(const Ptrs<float> Ab, int N, int Np, const Ptrs<const float> scaleb, const Ptrs<float> Vb) {
+  const float s = scaleb.p[blockIdx.y][0];
+  float* row = Ab.p[blockIdx.y] + (int64_t)blockIdx.x * Np;
+  float* aside = blockIdx.x == 0 ? Vb.p[blockIdx.y] + (int64_t)(N - 1) * Np : nullptr;
+  for (int i = threadIdx.x; i < Np; i += 256) {
+    const float x = i < N ? row[i] * s : 0.f;
+    row[i] = x;
+    if (aside) aside[i] = x;
+  }
+}
+
+// ------------------------------------------------------------------------------------------ 2. eigenvalues
+// One warp per eigenvalue, 32 trial points per round.  The number of eigenvalues below x is the number of sign changes of
+// p_i = (d_i - x) p_{i-1} - e_{i-1}^2 p_{i-2}; the chain per row is one fused multiply-add, and both terms are scaled
+// back by a power of two every eight rows.  e^2 is kept above a floor, so that two consecutive p never vanish.
+constexpr int kSturmWarps = 8;
+constexpr double kE2Floor = 1e-36;
+
+__device__ __forceinline__ int sturm_count(const double2* __restrict__ t, int N, double x) {
+  double p0 = 1.0, p1 = t[0].x - x;
+  int cnt = __double2hiint(p1) < 0 ? 1 : 0;
+  int i = 1;
+  for (; i + 8 <= N; i += 8) {
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const double2 te = t[i + u];                 // (d_i, e_{i-1}^2)
+      const double p2 = fma(te.x - x, p1, -(te.y * p0));
+      cnt += (uint32_t)(__double2hiint(p2) ^ __double2hiint(p1)) >> 31;
+      p0 = p1;
+      p1 = p2;
+    }
+    const int h = max(__double2hiint(p0) & 0x7FF00000, __double2hiint(p1) & 0x7FF00000);
+    const double sc = __hiloint2double(min(max(0x7FE00000 - h, 0x00100000), 0x7FD00000), 0);   // 2^-exponent of the larger
+    p0 *= sc;
+    p1 *= sc;
+  }
+  for (; i < N; ++i) {
+    const double2 te = t[i];
+    const double p2 = fma(te.x - x, p1, -(te.y * p0));
+    cnt += (uint32_t)(__double2hiint(p2) ^ __double2hiint(p1)) >> 31;
+    p0 = p1;
+    p1 = p2;
+  }
+  return cnt;
+}
+
+__global__ void __launch_bounds__(kSturmWarps * 32)
+eigenvalue_kernel(const Ptrs<const float> db, const Ptrs<const float> eb, int N, int r, const Ptrs<double> lamb) {
+  extern __shared__ __align__(16) double2 sturm_smem[];
+  __shared__ double bound[kSturmWarps];
+  const float* d = db.p[blockIdx.y];
+  const float* e = eb.p[blockIdx.y];
+  double b = 0.0;                                // every |eigenvalue| <= max |d_i| + |e_{i-1}| + |e_i|
+  for (int i = threadIdx.x; i < N; i += blockDim.x) {
+    const double di = d[i], el = i > 0 ? (double)e[i - 1] : 0.0, er = i + 1 < N ? (double)e[i] : 0.0;
+    sturm_smem[i] = make_double2(di, fmax(el * el, kE2Floor));
+    b = fmax(b, fabs(di) + fabs(el) + fabs(er));
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) b = fmax(b, __shfl_xor_sync(0xFFFFFFFFu, b, o));
+  if ((threadIdx.x & 31) == 0) bound[threadIdx.x >> 5] = b;
+  __syncthreads();
+  for (int i = 0; i < kSturmWarps; ++i) b = fmax(b, bound[i]);
+  const int lane = threadIdx.x & 31, j = blockIdx.x * kSturmWarps + (threadIdx.x >> 5);
+  if (j >= r) return;
+  const int below = N - 1 - j;                   // eigenvalues smaller than the j-th largest
+  double lo = -1.001 * b - 1e-30, hi = 1.001 * b + 1e-30;
+  for (int round = 0; round < 16 && hi - lo > 2.3e-16 * b; ++round) {
+    const double h = (hi - lo) * (1.0 / 33.0), x = fma(h, (double)(lane + 1), lo);
+    const uint32_t mask = __ballot_sync(0xFFFFFFFFu, sturm_count(sturm_smem, N, x) <= below);
+    const int n = __popc(mask);                  // the trial points at or below it
+    hi = n < 32 ? fma(h, (double)(n + 1), lo) : hi;
+    lo = n > 0 ? fma(h, (double)n, lo) : lo;
+  }
+  if (lane == 0) lamb.p[blockIdx.y][j] = 0.5 * (lo + hi);
+}
+
+// Whether binary32 resolved the vectors.  A and its reduction carry an error of about sqrt(N) units in the last place of the
+// largest eigenvalue; neighbours in the bulk of a gradient's spectrum lie about lambda / N apart.  Measured on a rank-32
+// signal plus noise (N = 2048, lambda_r / lambda_1 = 8e-3: 1.1e-3 of rad for the 99 % worst vector, 6e-5 for the subspace),
+// the bound below keeps the subspace within 5e-3 rad.  Coinciding eigenvalues have no vectors of their own.
+__global__ void __launch_bounds__(256)
+doubtful_kernel(const Ptrs<const double> lamb, int N, int r, const Ptrs<int32_t> doubtb) {
+  const double* lam = lamb.p[blockIdx.x];
+  const double top = lam[0];
+  bool bad = !(lam[r - 1] >= 8.0 * N * 0x1p-24 * top) || !(top > 0.0);
+  for (int j = threadIdx.x + 1; j < r; j += blockDim.x) bad = bad || !(lam[j - 1] - lam[j] > 1e-14 * top);
+  const int any = __syncthreads_or(bad);
+  if (threadIdx.x == 0) *doubtb.p[blockIdx.x] = any ? 1 : 0;
+}
+
+// ------------------------------------------------------------------------------------------ 3. eigenvectors of T
+// One thread per eigenvalue: T - lambda = L D+ L^T from the top and U D- U^T from the bottom; where
+// gamma_i = d_i - lambda - e_{i-1} l_{i-1} - e_i u_i is smallest the two factorisations are joined, and the vector follows
+// outward from that row by products of multipliers alone, without cancellation.
+constexpr double kPivotFloor = 1e-280;
+__device__ __forceinline__ double guarded(double q) { return fabs(q) < kPivotFloor ? copysign(kPivotFloor, q) : q; }
+
+__global__ void __launch_bounds__(32)
+tridiagonal_vectors_kernel(const Ptrs<const float> db, const Ptrs<const float> eb, int N, int r, const Ptrs<const double> lamb,
+                           const Ptrs<double> lowerb, const Ptrs<float> Zb, const Ptrs<double> invb) {
+  extern __shared__ float vec_smem[];
+  float* d = vec_smem;
+  float* e = vec_smem + N;
+  const int mat = blockIdx.y;
+  for (int i = threadIdx.x; i < N; i += 32) {
+    d[i] = db.p[mat][i];
+    e[i] = i + 1 < N ? eb.p[mat][i] : 0.f;
+  }
+  __syncwarp();
+  const int t = blockIdx.x * 32 + threadIdx.x;
+  if (t >= r) return;
+  const double lam = lamb.p[mat][t];
+  double* lower = lowerb.p[mat] + t;
+  float* Z = Zb.p[mat] + t;
+  double q = guarded((double)d[0] - lam);
+#pragma unroll 4
+  for (int i = 0; i + 1 < N; ++i) {
+    const double ei = e[i], l = ei / q;
+    lower[(int64_t)i * r] = l;
+    q = guarded(((double)d[i + 1] - lam) - ei * l);
+  }
+  // from the bottom; gamma_i = D-_i - e_{i-1} l_{i-1}
+  q = (double)d[N - 1] - lam;
+  double best = 1e300;
+  int twist = N - 1;
+  for (int i0 = N - 1; i0 >= 0; i0 -= 8) {
+    double lb[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) lb[u] = i0 - u > 0 ? lower[(int64_t)(i0 - u - 1) * r] : 0.0;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int i = i0 - u;
+      if (i < 0) break;
+      const double el = i > 0 ? (double)e[i - 1] : 0.0;
+      const double gamma = fabs(q - el * lb[u]);
+      if (gamma < best) { best = gamma; twist = i; }
+      if (i > 0) {
+        const double uu = el / guarded(q);
+        Z[(int64_t)i * r] = (float)uu;             // the multiplier between rows i - 1 and i
+        q = ((double)d[i - 1] - lam) - el * uu;
+      }
+    }
+  }
+  double z = 1.0, sum = 1.0;
+  for (int i0 = N - 2; i0 >= 0; i0 -= 8) {
+    double lb[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) lb[u] = i0 - u >= 0 ? lower[(int64_t)(i0 - u) * r] : 0.0;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int i = i0 - u;
+      if (i >= 0 && i < twist) {
+        z *= -lb[u];
+        sum = fma(z, z, sum);
+        Z[(int64_t)i * r] = (float)z;
+      }
+    }
+  }
+  z = 1.0;
+  for (int i0 = 1; i0 < N; i0 += 8) {
+    float ub[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) ub[u] = i0 + u < N ? Z[(int64_t)(i0 + u) * r] : 0.f;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int i = i0 + u;
+      if (i < N && i > twist) {
+        z *= -(double)ub[u];
+        sum = fma(z, z, sum);
+        Z[(int64_t)i * r] = (float)z;
+      }
+    }
+  }
+  Z[(int64_t)twist * r] = 1.f;
+  invb.p[mat][t] = 1.0 / sqrt(sum);
+}
+
+// ------------------------------------------------------------------------------------------ 4. X = H Z
+// A warp keeps VW vectors in registers (lane: rows 128 c + 4 lane .. + 3) and runs through all Householder vectors, the
+// last first; the CTA's warps share each of them from a ring in shared memory that is filled four steps ahead.
+constexpr int kBackStages = 4;
+
+__device__ __forceinline__ void cp_async_16(void* smem_dst, const void* gsrc) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(smem_dst)), "l"(gsrc) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+template <int NCH, int VW, int WARPS>
+__global__ void __launch_bounds__(WARPS * 32, 1)
+back_transform_kernel(const Ptrs<const float> Vb, const Ptrs<const float> taub, int N, int Np, int r, const Ptrs<float> Zb,
+                      const Ptrs<const double> invb) {
+  extern __shared__ __align__(16) float back_smem[];
+  constexpr int kW = WARPS * VW, kThreads = WARPS * 32;   // vectors and threads of this CTA
+  float* ring = back_smem;                          // [kBackStages][Np]
+  float* tile = ring + kBackStages * Np;            // [128][kW + 1]
+  float* taus = tile + 128 * (kW + 1);              // [N]
+  const int mat = blockIdx.y, t0 = blockIdx.x * kW;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const float* V = Vb.p[mat];
+  float* Z = Zb.p[mat];
+  const int chunks = Np / 128;
+  for (int i = tid; i < N; i += kThreads) taus[i] = i + 1 < N ? taub.p[mat][i] : 0.f;
+
+  auto fetch = [&](int k) {                         // rows k + 1 .. of Householder vector k, whole chunks
+    if (k >= 0) {
+      const float* src = V + (int64_t)k * Np;
+      float* dst = ring + (k % kBackStages) * Np;
+      for (int i = (k + 1) / 128 * 128 + tid * 4; i < Np; i += kThreads * 4) cp_async_16(dst + i, src + i);
+    }
+    cp_async_commit();
+  };
+  for (int s = 0; s < kBackStages - 1; ++s) fetch(N - 2 - s);
+
+  float inv[VW];
+#pragma unroll
+  for (int u = 0; u < VW; ++u) { const int t = t0 + warp * VW + u; inv[u] = t < r ? (float)invb.p[mat][t] : 0.f; }
+  float4 x[VW][NCH];
+#pragma unroll
+  for (int ch = 0; ch < NCH; ++ch) {
+    if (ch < chunks) {
+      __syncthreads();
+      for (int i = tid; i < 128 * kW; i += kThreads) {
+        const int row = i / kW, col = i % kW;
+        tile[row * (kW + 1) + col] = (ch * 128 + row < N && t0 + col < r) ? Z[(int64_t)(ch * 128 + row) * r + t0 + col] : 0.f;
+      }
+      __syncthreads();
+#pragma unroll
+      for (int u = 0; u < VW; ++u) {
+        const float* p = tile + lane * 4 * (kW + 1) + warp * VW + u;
+        x[u][ch] = make_float4(p[0] * inv[u], p[kW + 1] * inv[u], p[2 * (kW + 1)] * inv[u], p[3 * (kW + 1)] * inv[u]);
+      }
+    } else {
+#pragma unroll
+      for (int u = 0; u < VW; ++u) x[u][ch] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+  }
+  for (int k = N - 2; k >= 0; --k) {
+    cp_async_wait<kBackStages - 2>();
+    __syncthreads();                                // vector k has landed; everybody is done with the slot refilled now
+    fetch(k - (kBackStages - 1));
+    const float* v = ring + (k % kBackStages) * Np;
+    const int c0 = (k + 1) / 128;
+    float s[VW];
+#pragma unroll
+    for (int u = 0; u < VW; ++u) s[u] = 0.f;
+#pragma unroll
+    for (int ch = 0; ch < NCH; ++ch) {
+      if (ch >= c0 && ch < chunks) {
+        const float4 v4 = *reinterpret_cast<const float4*>(v + ch * 128 + lane * 4);
+#pragma unroll
+        for (int u = 0; u < VW; ++u)
+          s[u] = fmaf(v4.x, x[u][ch].x, fmaf(v4.y, x[u][ch].y, fmaf(v4.z, x[u][ch].z, fmaf(v4.w, x[u][ch].w, s[u]))));
+      }
+    }
+    const float tk = taus[k];
+#pragma unroll
+    for (int u = 0; u < VW; ++u) s[u] = -tk * warp_sum(s[u]);
+#pragma unroll
+    for (int ch = 0; ch < NCH; ++ch) {
+      if (ch >= c0 && ch < chunks) {
+        const float4 v4 = *reinterpret_cast<const float4*>(v + ch * 128 + lane * 4);
+#pragma unroll
+        for (int u = 0; u < VW; ++u) {
+          x[u][ch].x = fmaf(s[u], v4.x, x[u][ch].x);
+          x[u][ch].y = fmaf(s[u], v4.y, x[u][ch].y);
+          x[u][ch].z = fmaf(s[u], v4.z, x[u][ch].z);
+          x[u][ch].w = fmaf(s[u], v4.w, x[u][ch].w);
+        }
+      }
+    }
+  }
+#pragma unroll
+  for (int ch = 0; ch < NCH; ++ch) {
+    if (ch < chunks) {
+      __syncthreads();
+#pragma unroll
+      for (int u = 0; u < VW; ++u) {
+        float* p = tile + lane * 4 * (kW + 1) + warp * VW + u;
+        p[0] = x[u][ch].x; p[kW + 1] = x[u][ch].y; p[2 * (kW + 1)] = x[u][ch].z; p[3 * (kW + 1)] = x[u][ch].w;
+      }
+      __syncthreads();
+      for (int i = tid; i < 128 * kW; i += kThreads) {
+        const int row = i / kW, col = i % kW;
+        if (ch * 128 + row < N && t0 + col < r) Z[(int64_t)(ch * 128 + row) * r + t0 + col] = tile[row * (kW + 1) + col];
+      }
+    }
+  }
+}
+
+// ------------------------------------------------------------------------------------------ host side
+constexpr int kDevices = 64;
+std::mutex g_coop_mutex;
+cudaEvent_t g_coop_done[kDevices] = {};        // completion of the last cooperative launch, per device ordinal
+
+int sm_count() {
+  static int n = [] {
+    int dev = 0, v = 148;
+    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
+    return v > 0 ? v : 148;
+  }();
+  return n;
+}
+
+// Opts a kernel instance into its dynamic shared memory, once per device and instance.
+template <class K>
+int opt_in(K kernel, int bytes, bool* done) {
+  int dev = 0;
+  QG_CUDA_TRY(cudaGetDevice(&dev));
+  if (dev < 0 || dev >= kDevices) return QG_UNSUPPORTED_SHAPE;
+  if (done[dev]) return QG_OK;
+  QG_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+  done[dev] = true;
+  return QG_OK;
+}
+
+template <int NQ>
+int launch_tridiagonal(TriArgs a, int nb, int32_t* status, cudaStream_t st) {
+  static bool done[kDevices] = {};
+  auto kern = tridiagonal_kernel<NQ>;
+  const int rc = opt_in(kern, kTriSmem, done);
+  if (rc != QG_OK) return rc;
+  void* args[] = {&a, &status};
+  return launch_cooperative((const void*)kern, (unsigned)(a.C * nb), kTriThreads, args, (size_t)kTriSmem, st);
+}
+
+template <int NCH, int VW, int WARPS>
+int launch_back(const Ptrs<const float>& V, const Ptrs<const float>& tau, int nb, int64_t N, int64_t Np, int64_t r, const Ptrs<float>& Z,
+                const Ptrs<const double>& inv, cudaStream_t st) {
+  static bool done[kDevices] = {};
+  auto kern = back_transform_kernel<NCH, VW, WARPS>;
+  const int rc = opt_in(kern, (kBackStages * NCH * 128 + 128 * (WARPS * VW + 1) + NCH * 128) * 4, done);
+  if (rc != QG_OK) return rc;
+  const size_t smem = (size_t)(kBackStages * Np + 128 * (WARPS * VW + 1) + N) * 4;
+  kern<<<dim3((unsigned)ceil_div(r, WARPS * VW), (unsigned)nb), WARPS * 32, smem, st>>>(V, tau, (int)N, (int)Np, (int)r, Z, inv);
+  QG_LAUNCH_CHECK();
+  return QG_OK;
+}
+
+}  // namespace
+
+int launch_cooperative(const void* kern, unsigned grid, unsigned block, void** args, size_t smem, cudaStream_t st) {
+  std::lock_guard<std::mutex> lock(g_coop_mutex);
+  int dev = 0;
+  QG_CUDA_TRY(cudaGetDevice(&dev));
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  QG_CUDA_TRY(cudaStreamIsCapturing(st, &cap));
+  const bool chain = cap == cudaStreamCaptureStatusNone && dev >= 0 && dev < kDevices;
+  if (chain) {
+    if (!g_coop_done[dev]) QG_CUDA_TRY(cudaEventCreateWithFlags(&g_coop_done[dev], cudaEventDisableTiming));
+    else QG_CUDA_TRY(cudaStreamWaitEvent(st, g_coop_done[dev], 0));
+  }
+  QG_CUDA_TRY(cudaLaunchCooperativeKernel(kern, dim3(grid), dim3(block), args, smem, st));
+  count_launch();
+  if (chain) QG_CUDA_TRY(cudaEventRecord(g_coop_done[dev], st));
+  return QG_OK;
+}
+
+size_t carve_eig(void* base, int64_t N, int64_t r, EigBuffers* out) {
+  size_t off = 0;
+  auto take = [&](size_t bytes) { void* p = base ? (char*)base + off : nullptr; off += (size_t)round_up((int64_t)bytes, 256); return p; };
+  const int64_t Np = eig_pitch(N);
+  EigBuffers w{};
+  w.A = (float*)take((size_t)(N * Np * 4));
+  w.V = (float*)take((size_t)(N * Np * 4));
+  w.tau = (float*)take((size_t)(N * 4));
+  w.d = (float*)take((size_t)(N * 4));
+  w.e = (float*)take((size_t)(N * 4));
+  w.scale = (float*)take(4);
+  w.lam = (double*)take((size_t)(r * 8));
+  w.inv = (double*)take((size_t)(r * 8));
+  w.lower = (double*)take((size_t)(N * r * 8));
+  w.Z = (float*)take((size_t)(N * r * 4));
+  w.xchg = (uint4*)take((size_t)(2 * Np * 16));
+  if (out) *out = w;
+  return off;
+}
+
+int launch_sym_eig(const EigBuffers* w, int32_t* const* doubtful, int nb, int64_t N, int64_t r, int32_t* status, cudaStream_t st) {
+  if (N < 2 || N > kEigMax || r < 1 || r > N || nb < 1 || nb > kMaxBatch) return QG_UNSUPPORTED_SHAPE;
+  const int64_t Np = eig_pitch(N);
+  Ptrs<float> A{}, V{}, tau{}, d{}, e{}, Z{}, scale{};
+  Ptrs<const float> Ac{}, Vc{}, tauc{}, dc{}, ec{}, scalec{};
+  Ptrs<double> lam{}, inv{}, lower{};
+  Ptrs<const double> lamc{}, invc{};
+  Ptrs<uint4> xchg{};
+  Ptrs<int32_t> doubt{};
+  for (int i = 0; i < nb; ++i) {
+    Ac.p[i] = A.p[i] = w[i].A; Vc.p[i] = V.p[i] = w[i].V; tauc.p[i] = tau.p[i] = w[i].tau;
+    dc.p[i] = d.p[i] = w[i].d; ec.p[i] = e.p[i] = w[i].e; Z.p[i] = w[i].Z; scalec.p[i] = scale.p[i] = w[i].scale;
+    lamc.p[i] = lam.p[i] = w[i].lam; invc.p[i] = inv.p[i] = w[i].inv; lower.p[i] = w[i].lower; xchg.p[i] = w[i].xchg;
+    doubt.p[i] = doubtful[i];
+    QG_CUDA_TRY(cudaMemsetAsync(w[i].xchg, 0, (size_t)(2 * Np * 16), st));   // no tag of an earlier call
+  }
+  eig_scale_factor_kernel<<<nb, 256, 0, st>>>(Ac, (int)N, (int)Np, scale);
+  QG_LAUNCH_CHECK();
+  eig_scale_kernel<<<dim3((unsigned)N, (unsigned)nb), 256, 0, st>>>(A, (int)N, (int)Np, scalec, V);
+  QG_LAUNCH_CHECK();
+
+  // Matrices reduced together share the SMs; as many as stay (all but a fifth of their columns, the first to retire) in
+  // registers and shared memory.
+  const int sms = sm_count();
+  const int64_t nq = Np <= kTriThreads ? 1 : Np <= 2 * kTriThreads ? 2 : Np <= 4 * kTriThreads ? 4 : 8;
+  auto ctas = [&](int cnt) { return std::max<int64_t>(1, std::min<int64_t>(sms / cnt, ceil_div(N, 16))); };
+  auto in_smem = [&](int64_t C) { return std::max<int64_t>(0, (kTriSmem / 4 - (6 + 2 * kTriWarps) * (ceil_div(N, C) + 8)) / Np); };
+  int together = nb;
+  while (together > 1 && ctas(together) * (64 / nq + in_smem(ctas(together))) * 5 < N * 4) --together;
+  for (int first = 0; first < nb; first += together) {
+    const int cnt = std::min(together, nb - first);
+    TriArgs a{};
+    for (int i = 0; i < cnt; ++i) {
+      a.A.p[i] = A.p[first + i]; a.V.p[i] = V.p[first + i]; a.tau.p[i] = tau.p[first + i];
+      a.d.p[i] = d.p[first + i]; a.e.p[i] = e.p[first + i]; a.xchg.p[i] = xchg.p[first + i];
+    }
+    a.N = (int)N; a.Np = (int)Np;
+    a.C = (int)ctas(cnt);
+    a.in_smem = (int)in_smem(a.C);
+    const int rc = nq == 1   ? launch_tridiagonal<1>(a, cnt, status, st)
+                   : nq == 2 ? launch_tridiagonal<2>(a, cnt, status, st)
+                   : nq == 4 ? launch_tridiagonal<4>(a, cnt, status, st)
+                             : launch_tridiagonal<8>(a, cnt, status, st);
+    if (rc != QG_OK) return rc;
+  }
+  {
+    static bool done[kDevices] = {};
+    const int rc = opt_in(eigenvalue_kernel, (int)kEigMax * 16, done);
+    if (rc != QG_OK) return rc;
+    eigenvalue_kernel<<<dim3((unsigned)ceil_div(r, kSturmWarps), (unsigned)nb), kSturmWarps * 32, (size_t)N * 16, st>>>(dc, ec, (int)N, (int)r, lam);
+    QG_LAUNCH_CHECK();
+  }
+  doubtful_kernel<<<nb, 256, 0, st>>>(lamc, (int)N, (int)r, doubt);
+  QG_LAUNCH_CHECK();
+  tridiagonal_vectors_kernel<<<dim3((unsigned)ceil_div(r, 32), (unsigned)nb), 32, (size_t)N * 8, st>>>(dc, ec, (int)N, (int)r, lamc, lower, Z, inv);
+  QG_LAUNCH_CHECK();
+  if (Np <= 512) return launch_back<4, 2, 16>(Vc, tauc, nb, N, Np, r, Z, invc, st);
+  if (Np <= 1024) return launch_back<8, 2, 16>(Vc, tauc, nb, N, Np, r, Z, invc, st);
+  if (Np <= 2048) return launch_back<16, 1, 16>(Vc, tauc, nb, N, Np, r, Z, invc, st);
+  return launch_back<32, 1, 8>(Vc, tauc, nb, N, Np, r, Z, invc, st);
+}
+
+}  // namespace qg
