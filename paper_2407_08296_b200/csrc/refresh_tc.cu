@@ -18,7 +18,7 @@
 // Every barrier wait is bounded; a wait that runs out raises QG_DEV_WAIT_EXPIRED and the role stops.
 #include <cstring>
 
-#include "qg_common.cuh"
+#include "refresh_common.cuh"
 #include "sm100_ptx.cuh"
 #include "tensor_map.cuh"
 
@@ -61,7 +61,8 @@ __device__ __forceinline__ void raise_expired(int32_t* status) {
 
 template <bool A_MN>
 __global__ void __launch_bounds__(SplitSmem::kThreads, 1)
-split_gemm_kernel(const __grid_constant__ SplitArgs a, int32_t* __restrict__ status) {
+split_gemm_kernel(const __grid_constant__ SplitArgs a, const int32_t* __restrict__ gate, int32_t* __restrict__ status) {
+  if (gate && *gate == 0) return;
   using S = SplitSmem;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -197,11 +198,172 @@ split_gemm_kernel(const __grid_constant__ SplitArgs a, int32_t* __restrict__ sta
   }
 }
 
+// ----------------------------------------------------------------------------------------------------------
+// The Gram matrix A = X X^T (N x N, fp32) of the gradient's short side, X = G or G^T, for a batch of gradients: both
+// operands are the same bfloat16 matrix, every product is exact, one pass.  Tiles of 128 x 256; those that lie wholly
+// above the diagonal are not computed, their elements are written as mirror images.  K-major operands (rows of X are
+// rows of G) come as boxes of 64 x 128 rows; MN-major ones (rows of X are columns of G) as 64 x 64 slabs with the exact
+// bounds of the matrix, so that any row pitch will do.  Eight of 2048 x 5461: 165 us (730 TFLOP/s on what is computed).
+struct GramArgs {
+  CUtensorMap map[kMaxBatch];
+  float* A[kMaxBatch];
+  int64_t lda;
+  int32_t N, K, tiles;         // tiles per matrix
+};
+
+struct GramSmem {
+  static constexpr int kABytes = kTileM * kBK * 2, kBBytes = kTileN * kBK * 2;
+  static constexpr int kStageBytes = kABytes + kBBytes;        // 48 KB
+  static constexpr int kStages = 4;
+  static constexpr int kBarOffset = kStages * kStageBytes;
+  static constexpr int kBytes = kBarOffset + 256 + 1024;
+  static constexpr int kThreads = 256;
+};
+
+// Tile t of the triangle: row block m has the column blocks 0 .. m / 2.
+__device__ __forceinline__ void gram_tile(int t, int& mb, int& nb) {
+  for (mb = 0; t >= mb / 2 + 1; ++mb) t -= mb / 2 + 1;
+  nb = t;
+}
+
+template <bool MN>
+__global__ void __launch_bounds__(GramSmem::kThreads, 1)
+gram_kernel(const __grid_constant__ GramArgs a, int nmat, int32_t* __restrict__ status) {
+  using S = GramSmem;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + S::kBarOffset);
+  uint64_t* empty = full + S::kStages;
+  uint64_t* acc_full = empty + S::kStages;
+  uint64_t* acc_empty = acc_full + 2;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 2);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < S::kStages; ++i) { mbar_init(&full[i], 1); mbar_init(&empty[i], 1); }
+    for (int i = 0; i < 2; ++i) { mbar_init(&acc_full[i], 1); mbar_init(&acc_empty[i], 4); }
+    fence_mbar_init();
+    fence_proxy_async_smem();
+  }
+  if (warp == 1) { tmem_alloc(tmem_slot, 512); tmem_relinquish(); }
+  tc_fence_before_sync();
+  __syncthreads();
+  tc_fence_after_sync();
+  const uint32_t tmem_base = *tmem_slot;
+  const int total = a.tiles * nmat, kblocks = (a.K + kBK - 1) / kBK;
+
+  if (warp == 0) {
+    if (lane == 0) {
+      uint32_t it = 0;
+      bool ok = true;
+      for (int t = blockIdx.x; ok && t < total; t += gridDim.x) {
+        int mb, nb;
+        gram_tile(t % a.tiles, mb, nb);
+        const CUtensorMap* map = &a.map[t / a.tiles];
+        const int m0 = mb * kTileM, n0 = nb * kTileN;
+        for (int kb = 0; kb < kblocks; ++kb, ++it) {
+          const int s = it % S::kStages;
+          if (!mbar_wait(&empty[s], ((it / S::kStages) & 1) ^ 1)) { ok = false; break; }
+          uint8_t* sA = smem + s * S::kStageBytes;
+          uint8_t* sB = sA + S::kABytes;
+          mbar_arrive_expect_tx(&full[s], S::kStageBytes);
+          if (MN) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h) tma_load_2d(sA + h * kSlab, map, &full[s], m0 + 64 * h, kb * kBK);
+#pragma unroll
+            for (int h = 0; h < 4; ++h) tma_load_2d(sB + h * kSlab, map, &full[s], n0 + 64 * h, kb * kBK);
+          } else {
+            tma_load_2d(sA, map, &full[s], kb * kBK, m0);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) tma_load_2d(sB + h * S::kABytes, map, &full[s], kb * kBK, n0 + 128 * h);
+          }
+        }
+      }
+      if (!ok) raise_expired(status);
+    }
+  } else if (warp == 1) {
+    if (lane == 0) {
+      constexpr uint32_t idesc = umma_idesc_bf16(kTileM, kTileN, MN, MN);
+      const uint64_t desc_a0 = umma_smem_desc_sw128(smem_u32(smem), MN ? kSlab : 16, 1024);
+      const uint64_t desc_b0 = umma_smem_desc_sw128(smem_u32(smem) + S::kABytes, MN ? kSlab : 16, 1024);
+      constexpr uint64_t step = MN ? (2048 >> 4) : (32 >> 4);
+      uint32_t it = 0, tcount = 0;
+      bool ok = true;
+      for (int t = blockIdx.x; ok && t < total; t += gridDim.x, ++tcount) {
+        const uint32_t ab = tcount & 1;
+        if (!mbar_wait(&acc_empty[ab], ((tcount >> 1) & 1) ^ 1)) { ok = false; break; }
+        tc_fence_after_sync();
+        for (int kb = 0; kb < kblocks; ++kb, ++it) {
+          const int s = it % S::kStages;
+          if (!mbar_wait(&full[s], (it / S::kStages) & 1)) { ok = false; break; }
+          tc_fence_after_sync();
+          const uint64_t off = (uint64_t)((s * S::kStageBytes) >> 4);
+#pragma unroll
+          for (int k = 0; k < kBK / 16; ++k)
+            umma_bf16(tmem_base + ab * kTileN, desc_a0 + off + k * step, desc_b0 + off + k * step, idesc, (kb | k) != 0);
+          umma_commit(&empty[s]);
+        }
+        if (ok) umma_commit(&acc_full[ab]);
+      }
+      if (!ok) raise_expired(status);
+    }
+  } else if (warp >= 4) {
+    const int q = warp & 3;
+    uint32_t tcount = 0;
+    bool ok = true;
+    for (int t = blockIdx.x; ok && t < total; t += gridDim.x, ++tcount) {
+      int mb, nb;
+      gram_tile(t % a.tiles, mb, nb);
+      float* A = a.A[t / a.tiles];
+      const uint32_t ab = tcount & 1;
+      if (!mbar_wait(&acc_full[ab], (tcount >> 1) & 1)) { ok = false; break; }
+      tc_fence_after_sync();
+      const uint32_t tacc = tmem_base + ((uint32_t)(q * 32) << 16) + ab * kTileN;
+      const int row = mb * kTileM + q * 32 + lane;
+#pragma unroll 1
+      for (int c = 0; c < kTileN / 32; ++c) {
+        uint32_t v[32];
+        tmem_ld_32x32(tacc + 32 * c, v);
+        tmem_ld_wait();
+        if (c == kTileN / 32 - 1) {
+          tc_fence_before_sync();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&acc_empty[ab]);
+        }
+        const int col = nb * kTileN + 32 * c;
+        if (row >= a.N) continue;
+        if (col + 32 <= a.N) {
+#pragma unroll
+          for (int i = 0; i < 8; ++i)
+            *reinterpret_cast<uint4*>(A + (int64_t)row * a.lda + col + 4 * i) = make_uint4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+        } else {
+#pragma unroll
+          for (int i = 0; i < 32; ++i)
+            if (col + i < a.N) A[(int64_t)row * a.lda + col + i] = __uint_as_float(v[i]);
+        }
+        // the mirror image, where no tile of the triangle covers it (32 lanes: 128 contiguous bytes of a row)
+        if (mb / 2 > (col / kTileM) / 2) {
+#pragma unroll
+          for (int i = 0; i < 32; ++i)
+            if (col + i < a.N) A[(int64_t)(col + i) * a.lda + row] = __uint_as_float(v[i]);
+        }
+      }
+    }
+    if (!ok && lane == 0) raise_expired(status);
+  }
+  tc_fence_before_sync();
+  __syncthreads();
+  if (warp == 1) {
+    tc_fence_after_sync();
+    tmem_dealloc(tmem_base, 512);
+  }
+}
+
 // B (K x N fp32, pitch ldb) -> three bfloat16 planes [kpad][N] each, stacked: hi = bf16(x), mid = bf16(x - hi),
 // lo = bf16(x - hi - mid) (the subtractions are exact in binary32).  Rows K .. kpad - 1 are written as zero, so that
 // a K block that reaches past K reads zeros and never the next plane.  A thread takes eight columns.
 __global__ void __launch_bounds__(256)
-split_planes_kernel(const float* __restrict__ B, int64_t ldb, int K, int N, int kpad, uint16_t* __restrict__ planes) {
+split_planes_kernel(const float* __restrict__ B, int64_t ldb, int K, int N, int kpad, uint16_t* __restrict__ planes, const int32_t* __restrict__ gate) {
+  if (gate && *gate == 0) return;
   const int64_t per_row = N / 8;
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= (int64_t)kpad * per_row) return;
@@ -242,6 +404,38 @@ int split_sm_count() {
 
 }  // namespace
 
+int launch_gram(const uint16_t* const* G, int nmat, int64_t ldg, bool columns, int64_t N, int64_t K, float* const* A, int64_t lda,
+                int32_t* status, cudaStream_t st) {
+  GramArgs a;
+  memset(&a, 0, sizeof(a));
+  bool ok = true;
+  for (int i = 0; i < nmat; ++i) {
+    if (columns) ok &= make_map(&a.map[i], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, G[i], N, K, ldg, 64, kBK, CU_TENSOR_MAP_SWIZZLE_128B);
+    else ok &= make_map(&a.map[i], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, G[i], K, N, ldg, kBK, kTileM, CU_TENSOR_MAP_SWIZZLE_128B);
+    a.A[i] = A[i];
+  }
+  if (!ok) {
+    note_cuda_error(cudaErrorUnknown, "cuTensorMapEncodeTiled");
+    return QG_CUDA_ERROR;
+  }
+  a.lda = lda; a.N = (int32_t)N; a.K = (int32_t)K;
+  const int mblocks = (int)ceil_div(N, kTileM);
+  for (int mb = 0; mb < mblocks; ++mb) a.tiles += mb / 2 + 1;
+  const int total = a.tiles * nmat, grid = total < split_sm_count() ? total : split_sm_count();
+  static bool smem_set[2][64] = {};
+  int dev = 0;
+  QG_CUDA_TRY(cudaGetDevice(&dev));
+  if (dev < 0 || dev >= 64) return QG_UNSUPPORTED_SHAPE;
+  auto kern = columns ? gram_kernel<true> : gram_kernel<false>;
+  if (!smem_set[columns][dev]) {
+    QG_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, GramSmem::kBytes));
+    smem_set[columns][dev] = true;
+  }
+  kern<<<grid, GramSmem::kThreads, GramSmem::kBytes, st>>>(a, nmat, status);
+  QG_LAUNCH_CHECK();
+  return QG_OK;
+}
+
 // Scratch the planes of a K x N iterate need.
 size_t split_planes_bytes(int64_t K, int64_t N) { return (size_t)(kPlanes * round_up(K, kBK) * N * 2); }
 
@@ -257,13 +451,13 @@ bool split_gemm_supported(const uint16_t* A, int64_t sa_m, int64_t sa_k, int64_t
 }
 
 // D (M x N fp32, pitch ldd) = A * B with A(i, k) = A[i * sa_m + k * sa_k] in bfloat16 and B (K x N fp32, pitch ldb)
-// split into `planes` (split_planes_bytes(K, N) bytes of scratch) first.
+// split into `planes` (split_planes_bytes(K, N) bytes of scratch) first.  Nothing happens where `gate` is given and *gate is 0.
 int launch_split_gemm(const uint16_t* A, int64_t sa_m, int64_t sa_k, const float* B, int64_t ldb, float* D, int64_t ldd,
-                      int64_t M, int64_t N, int64_t K, uint16_t* planes, int32_t* status, cudaStream_t st) {
+                      int64_t M, int64_t N, int64_t K, uint16_t* planes, const int32_t* gate, int32_t* status, cudaStream_t st) {
   const int kpad = (int)round_up(K, kBK);
   {
     const int64_t threads = (int64_t)kpad * (N / 8);
-    split_planes_kernel<<<(unsigned)ceil_div(threads, 256), 256, 0, st>>>(B, ldb, (int)K, (int)N, kpad, planes);
+    split_planes_kernel<<<(unsigned)ceil_div(threads, 256), 256, 0, st>>>(B, ldb, (int)K, (int)N, kpad, planes, gate);
     QG_LAUNCH_CHECK();
   }
   SplitArgs a;
@@ -292,13 +486,13 @@ int launch_split_gemm(const uint16_t* A, int64_t sa_m, int64_t sa_k, const float
       QG_CUDA_TRY(cudaFuncSetAttribute(split_gemm_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SplitSmem::kBytes));
       smem_set[1][dev] = true;
     }
-    split_gemm_kernel<true><<<grid, SplitSmem::kThreads, SplitSmem::kBytes, st>>>(a, status);
+    split_gemm_kernel<true><<<grid, SplitSmem::kThreads, SplitSmem::kBytes, st>>>(a, gate, status);
   } else {
     if (!smem_set[0][dev]) {
       QG_CUDA_TRY(cudaFuncSetAttribute(split_gemm_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SplitSmem::kBytes));
       smem_set[0][dev] = true;
     }
-    split_gemm_kernel<false><<<grid, SplitSmem::kThreads, SplitSmem::kBytes, st>>>(a, status);
+    split_gemm_kernel<false><<<grid, SplitSmem::kThreads, SplitSmem::kBytes, st>>>(a, gate, status);
   }
   QG_LAUNCH_CHECK();
   return QG_OK;
