@@ -26,9 +26,8 @@
 // and resolving that subspace to 1e-2 rad needs fp32-faithful products: plain bf16 tensor-core products of the
 // iterate do not get there, the three-plane split does.
 #include <cmath>
-#include <mutex>
 
-#include "qg_common.cuh"
+#include "refresh_common.cuh"
 
 namespace qg {
 
@@ -36,17 +35,16 @@ namespace qg {
 size_t split_planes_bytes(int64_t K, int64_t N);
 bool split_gemm_supported(const uint16_t* A, int64_t sa_m, int64_t sa_k, int64_t M, int64_t N, int64_t K);
 int launch_split_gemm(const uint16_t* A, int64_t sa_m, int64_t sa_k, const float* B, int64_t ldb, float* D, int64_t ldd,
-                      int64_t M, int64_t N, int64_t K, uint16_t* planes, int32_t* status, cudaStream_t st);
+                      int64_t M, int64_t N, int64_t K, uint16_t* planes, const int32_t* gate, int32_t* status, cudaStream_t st);
 
 namespace {
 
 constexpr int kCoopDevices = 64;
-std::mutex g_coop_mutex;
-cudaEvent_t g_coop_done[kCoopDevices] = {};   // completion of the last cooperative launch, per device ordinal
 
 // Test aid: 0 keeps every product of the refresh on the CUDA cores.
 int g_refresh_tc = 1;
-// Test aid: 0 rotates the rows of the Rayleigh-Ritz matrix pair by pair through L2 for every shape.
+// Test aid: 0 takes the iterative route for every shape, and rotates the rows of its Rayleigh-Ritz matrix pair by pair
+// through L2.
 int g_jacobi_blocks = 1;
 
 constexpr int kPanel = 64;    // columns orthonormalised together
@@ -55,18 +53,17 @@ constexpr int64_t kJacobiBytes = 64ll << 20;   // Rayleigh-Ritz matrices rotated
 constexpr int kGT = 64;       // GEMM tile (square), 16 x 16 threads, 4 x 4 outputs each
 constexpr int kGK = 16;
 
-constexpr int kMaxBatch = 8;  // matrices refreshed together
-// One pointer per matrix of a batch, passed to the kernels by value.
-template <class T>
-struct Ptrs {
-  T* p[kMaxBatch];
-};
 template <class T, class U>
 Ptrs<T> offset_ptrs(const Ptrs<U>& src, int nb, int64_t off) {
   Ptrs<T> out{};
   for (int i = 0; i < nb; ++i) out.p[i] = src.p[i] + off;
   return out;
 }
+
+// Kernels of the iterative route take a gate per matrix: where it is given and reads 0, the matrix has its vectors from the
+// direct route already and nothing happens.
+using Gates = Ptrs<const int32_t>;
+__device__ __forceinline__ bool closed(const Gates& gate, int mat) { return gate.p[mat] != nullptr && *gate.p[mat] == 0; }
 
 __device__ __forceinline__ float ld_as_float(const uint16_t* p, int64_t i) { return bf16_bits_to_float(p[i]); }
 __device__ __forceinline__ float ld_as_float(const float* p, int64_t i) { return p[i]; }
@@ -81,8 +78,9 @@ template <class TA, class ACC, class TC>
 __global__ void __launch_bounds__(256)
 gemm_kernel(const Ptrs<const TA> Ab, int64_t sa_m, int64_t sa_k, const Ptrs<const float> Bb, int64_t sb_k, int64_t sb_n,
             const Ptrs<TC> Cb, int64_t ldc, int M, int N, int K, ACC alpha, ACC beta, int k_slice, int slices,
-            const Ptrs<ACC> partb) {
+            const Ptrs<ACC> partb, const Gates gate) {
   const int mat = (int)blockIdx.z / slices, slice = (int)blockIdx.z % slices;
+  if (closed(gate, mat)) return;
   const TA* __restrict__ A = Ab.p[mat];
   const float* __restrict__ B = Bb.p[mat];
   TC* __restrict__ C = Cb.p[mat];
@@ -166,7 +164,9 @@ gemm_kernel(const Ptrs<const TA> Ab, int64_t sa_m, int64_t sa_k, const Ptrs<cons
 // C = alpha * (sum of the slices' partial sums, in slice order) + beta * C
 template <class ACC, class TC>
 __global__ void __launch_bounds__(256)
-gemm_reduce_kernel(const Ptrs<ACC> partb, int slices, const Ptrs<TC> Cb, int64_t ldc, int M, int N, ACC alpha, ACC beta) {
+gemm_reduce_kernel(const Ptrs<ACC> partb, int slices, const Ptrs<TC> Cb, int64_t ldc, int M, int N, ACC alpha, ACC beta,
+                   const Gates gate) {
+  if (closed(gate, blockIdx.y)) return;
   const ACC* __restrict__ part = partb.p[blockIdx.y];
   TC* __restrict__ C = Cb.p[blockIdx.y];
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -196,7 +196,7 @@ constexpr int64_t kSplitScratch = 32 << 20;  // bytes of partial sums a product 
 template <class TA, class ACC, class TC>
 int gemm(int nb, const Ptrs<const TA>& A, int64_t sa_m, int64_t sa_k, const Ptrs<const float>& B, int64_t sb_k, int64_t sb_n,
          const Ptrs<TC>& C, int64_t ldc, int64_t M, int64_t N, int64_t K, ACC alpha, ACC beta, cudaStream_t st,
-         const Ptrs<void>* part = nullptr) {
+         const Ptrs<void>* part = nullptr, const Gates& gate = Gates{}) {
   if (M <= 0 || N <= 0) return QG_OK;
   dim3 grid((unsigned)ceil_div(N, kGT), (unsigned)ceil_div(M, kGT));
   const int64_t tiles = (int64_t)grid.x * grid.y * nb;
@@ -211,7 +211,7 @@ int gemm(int nb, const Ptrs<const TA>& A, int64_t sa_m, int64_t sa_k, const Ptrs
   if (slices <= 1) {
     grid.z = (unsigned)nb;
     gemm_kernel<TA, ACC, TC><<<grid, 256, 0, st>>>(A, sa_m, sa_k, B, sb_k, sb_n, C, ldc, (int)M, (int)N, (int)K, alpha, beta,
-                                                   (int)K, 1, pt);
+                                                   (int)K, 1, pt, gate);
     QG_LAUNCH_CHECK();
     return QG_OK;
   }
@@ -220,17 +220,18 @@ int gemm(int nb, const Ptrs<const TA>& A, int64_t sa_m, int64_t sa_k, const Ptrs
   const int nslices = (int)ceil_div(K, k_slice);
   grid.z = (unsigned)(nslices * nb);
   gemm_kernel<TA, ACC, TC><<<grid, 256, 0, st>>>(A, sa_m, sa_k, B, sb_k, sb_n, C, ldc, (int)M, (int)N, (int)K, alpha, beta,
-                                                 (int)k_slice, nslices, pt);
+                                                 (int)k_slice, nslices, pt, gate);
   QG_LAUNCH_CHECK();
   gemm_reduce_kernel<ACC, TC><<<dim3((unsigned)ceil_div(M * N, 256), (unsigned)nb), 256, 0, st>>>(pt, nslices, C, ldc, (int)M, (int)N,
-                                                                                                  alpha, beta);
+                                                                                                  alpha, beta, gate);
   QG_LAUNCH_CHECK();
   return QG_OK;
 }
 
 // ---- Gaussian start block: Q[i][j] ~ N(0, 1) from Philox4x32-10 (counter (j / 4, i, 0, 0x51)) and Box-Muller
 __global__ void __launch_bounds__(256)
-gaussian_kernel(const Ptrs<float> Qb, int64_t ld, int64_t rows, int64_t cols, const Ptrs<const void> seeds) {
+gaussian_kernel(const Ptrs<float> Qb, int64_t ld, int64_t rows, int64_t cols, const Ptrs<const void> seeds, const Gates gate) {
+  if (closed(gate, blockIdx.y)) return;
   float* __restrict__ Q = Qb.p[blockIdx.y];
   // the seed of matrix y travels in the pointer table's slot (a 64-bit value, not an address)
   const uint64_t seed = (uint64_t)reinterpret_cast<uintptr_t>(seeds.p[blockIdx.y]);
@@ -259,7 +260,8 @@ gaussian_kernel(const Ptrs<float> Qb, int64_t ld, int64_t rows, int64_t cols, co
 // memory.  Binary32 is enough here: S itself comes from a binary32 product, and where the basis has to be
 // orthonormal to rounding the panel goes through this twice.
 __global__ void __launch_bounds__(32)
-chol64_inverse_kernel(const Ptrs<const float> Sb, const Ptrs<float> Linvb, int32_t* __restrict__ status) {
+chol64_inverse_kernel(const Ptrs<const float> Sb, const Ptrs<float> Linvb, int32_t* __restrict__ status, const Gates gate) {
+  if (closed(gate, blockIdx.x)) return;
   static_assert(kPanel == 64, "two rows and two columns per lane");
   const float* __restrict__ S = Sb.p[blockIdx.x];
   float* __restrict__ Linv = Linvb.p[blockIdx.x];
@@ -373,13 +375,14 @@ constexpr int kTeam = 128, kTeamsPerCta = 4;
 template <int NE>
 __global__ void __launch_bounds__(kTeam * kTeamsPerCta, NE <= 16 ? 2 : 1)   // two CTAs per SM while the rows fit 64 registers
 jacobi_sweeps_kernel(const Ptrs<float> Tb, int nb, int b, int sweeps, double tol, const Ptrs<unsigned long long> offb,
-                     unsigned int* __restrict__ sync_words, int32_t* __restrict__ status) {
+                     unsigned int* __restrict__ sync_words, int32_t* __restrict__ status, const Gates gate) {
   __shared__ double red[kTeamsPerCta][3][kTeam / 32];
   __shared__ double s_worst[kTeamsPerCta][kMaxBatch];
   const int team = threadIdx.x / kTeam, tt = threadIdx.x % kTeam, tw = tt >> 5, lane = threadIdx.x & 31;
   const int pairs = b / 2, jobs = pairs * nb, batch = (int)gridDim.x * kTeamsPerCta;
   unsigned int gen = 0;
-  uint32_t active = (1u << nb) - 1u;                // matrices still rotating
+  uint32_t active = 0;                              // matrices still rotating
+  for (int i = 0; i < nb; ++i) active |= closed(gate, i) ? 0u : 1u << i;
   for (int sw = 0; sw < sweeps && active != 0u; ++sw) {
     if (tt < kMaxBatch) s_worst[team][tt] = 0.0;
     for (int rnd = 0; rnd < b - 1; ++rnd) {
@@ -455,7 +458,7 @@ jacobi_sweeps_kernel(const Ptrs<float> Tb, int nb, int b, int sweeps, double tol
 
 template <int NE>
 int launch_jacobi(const Ptrs<float>& T, int nb, int64_t b, int sweeps, double tol, const Ptrs<unsigned long long>& off,
-                  unsigned int* sync_words, int32_t* status, cudaStream_t st) {
+                  unsigned int* sync_words, int32_t* status, const Gates& gate, cudaStream_t st) {
   // one cooperative launch, never more CTAs than are resident at once
   int per_sm = 0;
   QG_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, jacobi_sweeps_kernel<NE>, kTeam * kTeamsPerCta, 0));
@@ -466,11 +469,9 @@ int launch_jacobi(const Ptrs<float>& T, int nb, int64_t b, int sweeps, double to
   int bi = (int)b;
   Ptrs<float> Tc = T;
   Ptrs<unsigned long long> offc = off;
-  void* args[] = {&Tc, &nb, &bi, &sweeps, &tol, &offc, &sync_words, &status};
-  QG_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)jacobi_sweeps_kernel<NE>, dim3((unsigned)grid), dim3(kTeam * kTeamsPerCta),
-                                          args, 0, st));
-  count_launch();
-  return QG_OK;
+  Gates gatec = gate;
+  void* args[] = {&Tc, &nb, &bi, &sweeps, &tol, &offc, &sync_words, &status, &gatec};
+  return launch_cooperative((const void*)jacobi_sweeps_kernel<NE>, (unsigned)grid, kTeam * kTeamsPerCta, args, 0, st);
 }
 
 // ---- the same iteration with the rows in blocks of eight.  A sweep first rotates the pairs INSIDE every block
@@ -541,7 +542,7 @@ __device__ __forceinline__ double team_rotate(float (&x)[NE], float (&y)[NE], bo
 template <int NE>
 __global__ void __launch_bounds__(kBlkThreads, NE <= 16 ? 2 : 1)
 jacobi_block_kernel(const Ptrs<float> Tb, int nb, int b, int sweeps, double tol, const Ptrs<unsigned long long> offb,
-                    unsigned int* __restrict__ sync_words, int32_t* __restrict__ status) {
+                    unsigned int* __restrict__ sync_words, int32_t* __restrict__ status, const Gates gate) {
   // three sets of eight rows of b floats: the rows of block J of this job and of the next one (the copy engine brings
   // the next job's rows in while this one rotates), and the rows of block I of the next job
   extern __shared__ __align__(16) float blk_smem[];
@@ -553,7 +554,8 @@ jacobi_block_kernel(const Ptrs<float> Tb, int nb, int b, int sweeps, double tol,
   const int set = kBlkRows * b;
   float* const rows_i_next = blk_smem + 2 * set;
   unsigned int gen = 0;
-  uint32_t active = (1u << nb) - 1u;                 // matrices still rotating
+  uint32_t active = 0;                               // matrices still rotating
+  for (int i = 0; i < nb; ++i) active |= closed(gate, i) ? 0u : 1u << i;
   for (int sw = 0; sw < sweeps && active != 0u; ++sw) {
     if (tt < kMaxBatch) s_worst[team][tt] = 0.0;
     __syncthreads();
@@ -706,7 +708,7 @@ jacobi_block_kernel(const Ptrs<float> Tb, int nb, int b, int sweeps, double tol,
 // Opts the instance into its dynamic shared memory once per device.
 template <int NE>
 int launch_jacobi_block(const Ptrs<float>& T, int nb, int64_t b, int sweeps, double tol, const Ptrs<unsigned long long>& off,
-                        unsigned int* sync_words, int32_t* status, cudaStream_t st) {
+                        unsigned int* sync_words, int32_t* status, const Gates& gate, cudaStream_t st) {
   const int smem = (int)(3 * kBlkRows * b * sizeof(float));
   static bool smem_set[kCoopDevices] = {};
   int dev = 0;
@@ -726,16 +728,15 @@ int launch_jacobi_block(const Ptrs<float>& T, int nb, int64_t b, int sweeps, dou
   int bi = (int)b;
   Ptrs<float> Tc = T;
   Ptrs<unsigned long long> offc = off;
-  void* args[] = {&Tc, &nb, &bi, &sweeps, &tol, &offc, &sync_words, &status};
-  QG_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)jacobi_block_kernel<NE>, dim3((unsigned)grid), dim3(kBlkThreads), args,
-                                          (size_t)smem, st));
-  count_launch();
-  return QG_OK;
+  Gates gatec = gate;
+  void* args[] = {&Tc, &nb, &bi, &sweeps, &tol, &offc, &sync_words, &status, &gatec};
+  return launch_cooperative((const void*)jacobi_block_kernel<NE>, (unsigned)grid, kBlkThreads, args, (size_t)smem, st);
 }
 
 // lambda_j = norm of row j of the rotated T (= |eigenvalue j|); rank_j = its position in descending order
 __global__ void __launch_bounds__(128)
-row_norm_kernel(const Ptrs<const float> Tb, int b, const Ptrs<double> lamb) {
+row_norm_kernel(const Ptrs<const float> Tb, int b, const Ptrs<double> lamb, const Gates gate) {
+  if (closed(gate, blockIdx.y)) return;
   const float* row = Tb.p[blockIdx.y] + (int64_t)blockIdx.x * b;
   double* __restrict__ lam = lamb.p[blockIdx.y];
   double s = 0.0;
@@ -750,7 +751,8 @@ row_norm_kernel(const Ptrs<const float> Tb, int b, const Ptrs<double> lamb) {
 
 // Xsel[i][rank_j] = X[i][j] = T[j][i] / lambda_j for the r largest lambda_j
 __global__ void __launch_bounds__(256)
-select_top_kernel(const Ptrs<const float> Tb, const Ptrs<const double> lamb, int b, int r, const Ptrs<float> Xselb) {
+select_top_kernel(const Ptrs<const float> Tb, const Ptrs<const double> lamb, int b, int r, const Ptrs<float> Xselb, const Gates gate) {
+  if (closed(gate, blockIdx.y)) return;
   const float* __restrict__ T = Tb.p[blockIdx.y];
   const double* __restrict__ lam = lamb.p[blockIdx.y];
   float* __restrict__ Xsel = Xselb.p[blockIdx.y];
@@ -772,34 +774,56 @@ select_top_kernel(const Ptrs<const float> Tb, const Ptrs<const double> lamb, int
   for (int i = threadIdx.x; i < b; i += blockDim.x) Xsel[(int64_t)i * r + rank] = (float)((double)T[(int64_t)j * b + i] * inv);
 }
 
-// Each column of P gets the sign that makes its largest-magnitude entry positive; optional copy to P_out.
-__global__ void __launch_bounds__(256)
-sign_fix_kernel(const Ptrs<float> Pb, int64_t m, int r, const Ptrs<float> P_outb) {
-  float* __restrict__ P = Pb.p[blockIdx.y];
+// The last pass over the vectors: column j of S (rows x r, pitch lds) is given unit length (if `normalise`) and the sign
+// that makes its largest-magnitude entry positive; P (pitch r) and, if given, P_out receive it (S may be P).  A CTA takes
+// 32 columns and reads 32 rows of them at a time, so that every access is a whole line.
+__global__ void __launch_bounds__(1024)
+finish_vectors_kernel(const Ptrs<const float> Sb, int64_t lds, int64_t rows, int r, bool normalise, const Ptrs<float> Pb,
+                      const Ptrs<float> P_outb, const Gates gate) {
+  if (closed(gate, blockIdx.y)) return;
+  __shared__ float s_big[32][33], s_sum[32][33];
+  const float* S = Sb.p[blockIdx.y];
+  float* P = Pb.p[blockIdx.y];
   float* __restrict__ P_out = P_outb.p[blockIdx.y];
-  const int j = blockIdx.x;
-  float best = 0.f, bestv = 0.f;
-  for (int64_t i = threadIdx.x; i < m; i += blockDim.x) {
-    const float v = P[i * r + j];
-    if (fabsf(v) > best) { best = fabsf(v); bestv = v; }
+  const int lane = threadIdx.x & 31, y = threadIdx.x >> 5, j = blockIdx.x * 32 + lane;
+  float big = 0.f, sum = 0.f;                       // the entry of largest magnitude, with its sign
+  if (j < r) {
+    for (int64_t i = y; i < rows; i += 32) {
+      const float v = S[i * lds + j];
+      if (fabsf(v) > fabsf(big)) big = v;
+      sum = fmaf(v, v, sum);
+    }
   }
-  __shared__ float sb[256], sv[256];
-  sb[threadIdx.x] = best; sv[threadIdx.x] = bestv;
+  s_big[y][lane] = big;
+  s_sum[y][lane] = sum;
   __syncthreads();
-  for (int o = 128; o > 0; o >>= 1) {
-    if (threadIdx.x < o && sb[threadIdx.x + o] > sb[threadIdx.x]) { sb[threadIdx.x] = sb[threadIdx.x + o]; sv[threadIdx.x] = sv[threadIdx.x + o]; }
-    __syncthreads();
+  if (y == 0) {
+    for (int k = 1; k < 32; ++k) {
+      if (fabsf(s_big[k][lane]) > fabsf(big)) big = s_big[k][lane];
+      sum += s_sum[k][lane];
+    }
+    const float len = normalise && sum > 0.f ? 1.f / sqrtf(sum) : 1.f;
+    s_sum[0][lane] = big < 0.f ? -len : len;
   }
-  const float sgn = sv[0] < 0.f ? -1.f : 1.f;
-  for (int64_t i = threadIdx.x; i < m; i += blockDim.x) {
-    const float v = P[i * r + j] * sgn;
+  __syncthreads();
+  if (j >= r) return;
+  const float f = s_sum[0][lane];
+  for (int64_t i = y; i < rows; i += 32) {
+    const float v = S[i * lds + j] * f;
     P[i * r + j] = v;
     if (P_out) P_out[i * r + j] = v;
   }
 }
 
 struct RefreshWs {
-  float *Q, *Y, *Z, *Wp, *Cb, *S, *Linv, *Xsel, *P32;
+  float* P32;      // the vectors before quantization
+  int32_t* gate;   // 1: the direct route has not resolved them
+  // direct route
+  EigBuffers eig;  // of the Gram matrix of the short side
+  float* XV;       // X V, for vectors on the long side
+  uint16_t* planes_v;
+  // iterative route (in the same memory: it begins when the direct one has ended)
+  float *Q, *Y, *Z, *Wp, *Cb, *S, *Linv, *Xsel;
   void* part;      // partial sums of sliced products
   uint16_t* planes;  // the three bfloat16 planes of an iterate, for the tensor-core products
   float* T;        // the Rayleigh-Ritz matrix, then its rotated rows
@@ -807,10 +831,22 @@ struct RefreshWs {
   int32_t* done;
 };
 
-size_t carve_refresh(void* base, int64_t m, int64_t n, int64_t b, int64_t r, RefreshWs* w) {
+// Scratch of one matrix (left singular vectors of X, m x n; a block of b columns, at most as many vectors).
+size_t carve_refresh(void* base, int64_t m, int64_t n, int64_t b, RefreshWs* w) {
   size_t off = 0;
   auto take = [&](size_t bytes) { void* p = base ? (char*)base + off : nullptr; off += (size_t)round_up((int64_t)bytes, 256); return p; };
   RefreshWs t{};
+  t.P32 = (float*)take((size_t)m * b * 4);
+  t.gate = (int32_t*)take(4);
+  const size_t routes = off;
+  const int64_t s = m < n ? m : n;
+  if (s <= kEigMax) {
+    take(carve_eig(base ? (char*)base + off : nullptr, s, b, &t.eig));
+    t.XV = (float*)take((size_t)m * b * 4);
+    t.planes_v = (uint16_t*)take(split_planes_bytes(s, b));
+  }
+  const size_t direct = off;
+  off = routes;
   t.T = (float*)take((size_t)b * b * 4);
   t.lam = (double*)take((size_t)b * 8);
   t.off = (double*)take(kMaxSweeps * 8);     // largest normalised inner product of each sweep
@@ -822,12 +858,11 @@ size_t carve_refresh(void* base, int64_t m, int64_t n, int64_t b, int64_t r, Ref
   t.Cb = (float*)take((size_t)b * kPanel * 4);
   t.S = (float*)take((size_t)kPanel * kPanel * 4);
   t.Linv = (float*)take((size_t)kPanel * kPanel * 4);
-  t.Xsel = (float*)take((size_t)b * r * 4);
-  t.P32 = (float*)take((size_t)m * r * 4);
+  t.Xsel = (float*)take((size_t)b * b * 4);
   t.part = take((size_t)kSplitScratch);
   t.planes = (uint16_t*)take(split_planes_bytes(m > n ? m : n, b));
   if (w) *w = t;
-  return off;
+  return off > direct ? off : direct;
 }
 
 // The workspaces of the matrices of one batch, and pointer tables into them.
@@ -850,7 +885,7 @@ struct Batch {
 // about 1e-2 (fp32 Gram matrices of panels with a condition number of several hundred), which is all an
 // intermediate subspace iteration asks of it: the next multiplication by G G^T and the next orthonormalisation
 // start from that basis, they do not inherit its error.
-int orthonormalize(const Batch& bt, int64_t m, int64_t b, int32_t* status, cudaStream_t st, bool full) {
+int orthonormalize(const Batch& bt, int64_t m, int64_t b, const Gates& gate, int32_t* status, cudaStream_t st, bool full) {
   const int passes = full ? 2 : 1;
   const int nb = bt.nb;
   Ptrs<void> part{};
@@ -865,9 +900,9 @@ int orthonormalize(const Batch& bt, int64_t m, int64_t b, int32_t* status, cudaS
     int rc;
     for (int pass = 0; pass < passes && j0 > 0; ++pass) {
       // C = Q[:, :j0]^T Yj   (j0 x 64);   Yj -= Q[:, :j0] C
-      rc = gemm<float, float, float>(nb, Q, 1, b, Yjc, b, 1, Cb, kPanel, j0, kPanel, m, 1.f, 0.f, st, &part);
+      rc = gemm<float, float, float>(nb, Q, 1, b, Yjc, b, 1, Cb, kPanel, j0, kPanel, m, 1.f, 0.f, st, &part, gate);
       if (rc != QG_OK) return rc;
-      rc = gemm<float, float, float>(nb, Q, b, 1, Cbc, kPanel, 1, Yj, b, m, kPanel, j0, -1.f, 1.f, st, &part);
+      rc = gemm<float, float, float>(nb, Q, b, 1, Cbc, kPanel, 1, Yj, b, m, kPanel, j0, -1.f, 1.f, st, &part, gate);
       if (rc != QG_OK) return rc;
     }
     // Cholesky QR on the panel, two rounds (Yj -> Wp -> Qj) or one (Yj -> Qj)
@@ -877,12 +912,12 @@ int orthonormalize(const Batch& bt, int64_t m, int64_t b, int32_t* status, cudaS
       const int64_t lds = pass == 0 ? b : kPanel;
       const Ptrs<float>& dst = last ? Qj : Wp;
       const int64_t ldd = last ? b : kPanel;
-      rc = gemm<float, float, float>(nb, src, 1, lds, src, lds, 1, S, kPanel, kPanel, kPanel, m, 1.f, 0.f, st, &part);
+      rc = gemm<float, float, float>(nb, src, 1, lds, src, lds, 1, S, kPanel, kPanel, kPanel, m, 1.f, 0.f, st, &part, gate);
       if (rc != QG_OK) return rc;
-      chol64_inverse_kernel<<<nb, 32, 0, st>>>(Sc, Linv, status);
+      chol64_inverse_kernel<<<nb, 32, 0, st>>>(Sc, Linv, status, gate);
       QG_LAUNCH_CHECK();
       // dst = src * Linv^T:  B(k, j) = Linv[j][k]
-      rc = gemm<float, float, float>(nb, src, lds, 1, Linvc, 1, kPanel, dst, ldd, m, kPanel, kPanel, 1.f, 0.f, st);
+      rc = gemm<float, float, float>(nb, src, lds, 1, Linvc, 1, kPanel, dst, ldd, m, kPanel, kPanel, 1.f, 0.f, st, nullptr, gate);
       if (rc != QG_OK) return rc;
     }
   }
@@ -891,24 +926,70 @@ int orthonormalize(const Batch& bt, int64_t m, int64_t b, int32_t* status, cudaS
 
 }  // namespace
 
-size_t refresh_workspace_bytes(int64_t m, int64_t n, int64_t b) { return carve_refresh(nullptr, m, n, b, b, nullptr); }
+size_t refresh_workspace_bytes(int64_t m, int64_t n, int64_t b) { return carve_refresh(nullptr, m, n, b, nullptr); }
 
-// One batch (at most kMaxBatch matrices of one shape).  `transposed`: the singular vectors wanted are the RIGHT ones
+// Unit length (if asked for) and sign of the vectors in S (pitch lds): P32, P_fp32.
+static int finish_vectors(const RefreshJob* jobs, const Batch& bt, const Ptrs<const float>& S, int64_t lds, int64_t rows, int64_t r,
+                          bool normalise, const Gates& gate, cudaStream_t st) {
+  Ptrs<float> P_out{};
+  for (int i = 0; i < bt.nb; ++i) P_out.p[i] = jobs[i].P_fp32;
+  finish_vectors_kernel<<<dim3((unsigned)ceil_div(r, 32), (unsigned)bt.nb), 1024, 0, st>>>(S, lds, rows, (int)r, normalise, QG_TAB(float, P32), P_out,
+                                                                                           gate);
+  QG_LAUNCH_CHECK();
+  return QG_OK;
+}
+
+// The direct route: X X^T or X^T X, whichever is smaller, on the tensor cores (bfloat16 operands, exact products, fp32
+// accumulation), its leading eigenvectors, and for vectors on the long side X V at unit length.
+static int refresh_direct(const RefreshJob* jobs, const Batch& bt, int64_t m, int64_t n, int64_t r, int32_t* status, cudaStream_t st,
+                          bool transposed) {
+  const int nb = bt.nb;
+  const uint16_t* G[kMaxBatch];
+  float* A[kMaxBatch];
+  int32_t* doubtful[kMaxBatch];
+  EigBuffers eig[kMaxBatch];
+  const int64_t ldg = jobs[0].ldg;
+  const bool long_side = m > n;
+  const int64_t s = long_side ? n : m, l = long_side ? m : n;
+  const int64_t re = long_side ? round_up(r, 64) : r;      // the product X V wants whole 64-column slabs; re <= b
+  for (int i = 0; i < nb; ++i) {
+    G[i] = jobs[i].G;
+    eig[i] = bt.w[i].eig;
+    A[i] = eig[i].A;
+    doubtful[i] = bt.w[i].gate;
+  }
+  int rc = launch_gram(G, nb, ldg, transposed != long_side, s, l, A, eig_pitch(s), status, st);
+  if (rc != QG_OK) return rc;
+  rc = launch_sym_eig(eig, doubtful, nb, s, re, status, st);
+  if (rc != QG_OK) return rc;
+  const Ptrs<const float> V = bt.tab<const float>([](const RefreshWs& x) { return x.eig.Z; });
+  if (!long_side) return finish_vectors(jobs, bt, V, re, m, r, false, Gates{}, st);
+  const int64_t rs = transposed ? 1 : ldg, cs = transposed ? ldg : 1;
+  if (split_gemm_supported(G[0], rs, cs, m, re, s)) {
+    for (int i = 0; i < nb; ++i) {
+      rc = launch_split_gemm(G[i], rs, cs, eig[i].Z, re, bt.w[i].XV, re, m, re, s, bt.w[i].planes_v, nullptr, status, st);
+      if (rc != QG_OK) return rc;
+    }
+  } else {
+    Ptrs<const uint16_t> Gp{};
+    for (int i = 0; i < nb; ++i) Gp.p[i] = G[i];
+    rc = gemm<uint16_t, float, float>(nb, Gp, rs, cs, V, re, 1, QG_TAB(float, XV), re, m, re, s, 1.f, 0.f, st);
+    if (rc != QG_OK) return rc;
+  }
+  return finish_vectors(jobs, bt, QG_TAB(const float, XV), re, m, r, true, Gates{}, st);
+}
+
+// The iterative route, for the matrices whose gate is open.  `transposed`: the singular vectors wanted are the RIGHT ones
 // of G, i.e. the left ones of G^T; G is then read with its two strides swapped and (m, n) are the extents of G^T.
-static int refresh_batch(const RefreshJob* jobs, int nb, int64_t m, int64_t n, int64_t r, int64_t b, int iters, int sweeps,
-                         char* ws, size_t ws_stride, int32_t* status, cudaStream_t st, bool transposed) {
-  Batch bt{};
-  bt.nb = nb;
+static int refresh_iterative(const RefreshJob* jobs, const Batch& bt, const Gates& gate, int64_t m, int64_t n, int64_t r, int64_t b, int iters,
+                             int sweeps, int32_t* status, cudaStream_t st, bool transposed) {
+  const int nb = bt.nb;
   Ptrs<const uint16_t> G{};
   Ptrs<const void> seeds{};
-  Ptrs<float> P_out{};
-  int64_t ldg = jobs[0].ldg;
+  const int64_t ldg = jobs[0].ldg;
   for (int i = 0; i < nb; ++i) {
-    carve_refresh(ws + (size_t)i * ws_stride, m, n, b, r, &bt.w[i]);
     G.p[i] = jobs[i].G;
     seeds.p[i] = reinterpret_cast<const void*>((uintptr_t)jobs[i].seed);
-    P_out.p[i] = jobs[i].P_fp32;
-    if (jobs[i].ldg != ldg) return QG_INVALID_ARGUMENT;          // one pitch per batch (the caller groups by it)
   }
   const int64_t rs = transposed ? 1 : ldg, cs = transposed ? ldg : 1;   // strides between rows / columns of the matrix
   const Ptrs<const float> Q = QG_TAB(const float, Q), Z = QG_TAB(const float, Z), Xsel = QG_TAB(const float, Xsel);
@@ -917,9 +998,9 @@ static int refresh_batch(const RefreshJob* jobs, int nb, int64_t m, int64_t n, i
   // start block
   {
     const int64_t threads = m * (b / 4);
-    gaussian_kernel<<<dim3((unsigned)ceil_div(threads, 256), (unsigned)nb), 256, 0, st>>>(Y, b, m, b, seeds);
+    gaussian_kernel<<<dim3((unsigned)ceil_div(threads, 256), (unsigned)nb), 256, 0, st>>>(Y, b, m, b, seeds, gate);
     QG_LAUNCH_CHECK();
-    rc = orthonormalize(bt, m, b, status, st, iters < 2);          // in full only if no later iteration will be
+    rc = orthonormalize(bt, m, b, gate, status, st, iters < 2);          // in full only if no later iteration will be
     if (rc != QG_OK) return rc;
   }
   // The two products with the gradient go to the tensor cores (bfloat16 gradient times an iterate split into three
@@ -934,31 +1015,31 @@ static int refresh_batch(const RefreshJob* jobs, int nb, int64_t m, int64_t n, i
     // Z = G^T Q
     if (tc_z && it < iters) {
       for (int i = 0; i < nb; ++i) {
-        rc = launch_split_gemm(G.p[i], cs, rs, bt.w[i].Q, b, bt.w[i].Z, b, n, b, m, bt.w[i].planes, status, st);
+        rc = launch_split_gemm(G.p[i], cs, rs, bt.w[i].Q, b, bt.w[i].Z, b, n, b, m, bt.w[i].planes, gate.p[i], status, st);
         if (rc != QG_OK) return rc;
       }
     } else {
-      rc = gemm<uint16_t, float, float>(nb, G, cs, rs, Q, b, 1, Zw, b, n, b, m, 1.f, 0.f, st);
+      rc = gemm<uint16_t, float, float>(nb, G, cs, rs, Q, b, 1, Zw, b, n, b, m, 1.f, 0.f, st, nullptr, gate);
       if (rc != QG_OK) return rc;
     }
     if (it == iters) break;
     // Y = G Z
     if (tc_y) {
       for (int i = 0; i < nb; ++i) {
-        rc = launch_split_gemm(G.p[i], rs, cs, bt.w[i].Z, b, bt.w[i].Y, b, m, b, n, bt.w[i].planes, status, st);
+        rc = launch_split_gemm(G.p[i], rs, cs, bt.w[i].Z, b, bt.w[i].Y, b, m, b, n, bt.w[i].planes, gate.p[i], status, st);
         if (rc != QG_OK) return rc;
       }
     } else {
-      rc = gemm<uint16_t, float, float>(nb, G, rs, cs, Z, b, 1, Y, b, m, b, n, 1.f, 0.f, st);
+      rc = gemm<uint16_t, float, float>(nb, G, rs, cs, Z, b, 1, Y, b, m, b, n, 1.f, 0.f, st, nullptr, gate);
       if (rc != QG_OK) return rc;
     }
-    rc = orthonormalize(bt, m, b, status, st, it + 2 >= iters);   // the last two in full
+    rc = orthonormalize(bt, m, b, gate, status, st, it + 2 >= iters);   // the last two in full
     if (rc != QG_OK) return rc;
   }
   // Rayleigh-Ritz: T = Z^T Z (accumulated in binary64, kept in binary32), eigenvectors by one-sided Jacobi
   const Ptrs<float> T = QG_TAB(float, T);
   const Ptrs<double> lam = QG_TAB(double, lam);
-  rc = gemm<float, double, float>(nb, Z, 1, b, Z, b, 1, T, b, b, b, n, 1.0, 0.0, st);
+  rc = gemm<float, double, float>(nb, Z, 1, b, Z, b, 1, T, b, b, b, n, 1.0, 0.0, st, nullptr, gate);
   if (rc != QG_OK) return rc;
   if (sweeps > kMaxSweeps) sweeps = kMaxSweeps;
   for (int i = 0; i < nb; ++i) QG_CUDA_TRY(cudaMemsetAsync(bt.w[i].off, 0, kMaxSweeps * 8, st));
@@ -972,47 +1053,59 @@ static int refresh_batch(const RefreshJob* jobs, int nb, int64_t m, int64_t n, i
     const int cnt = std::min(per_launch, nb - first);
     Ptrs<float> Tsub{};
     Ptrs<unsigned long long> off{};
+    Gates gate_sub{};
     for (int i = 0; i < cnt; ++i) {
       Tsub.p[i] = bt.w[first + i].T;
       off.p[i] = reinterpret_cast<unsigned long long*>(bt.w[first + i].off);
+      gate_sub.p[i] = gate.p[first + i];
     }
     QG_CUDA_TRY(cudaMemsetAsync(bt.w[0].done, 0, 8, st));
     unsigned int* sync_words = reinterpret_cast<unsigned int*>(bt.w[0].done);
     // the iteration converges quadratically at the end: a sweep that met nothing above 1e-5 leaves ~1e-10
     constexpr double kTol = 1e-5;
-    // Refreshes may run on several streams at once (their many small kernels overlap well), but two grids whose
-    // CTAs wait for one another must never be half resident together: each cooperative launch waits for the
-    // previous one of this process on the device, whatever its stream.
-    std::lock_guard<std::mutex> lock(g_coop_mutex);
-    int dev = 0;
-    QG_CUDA_TRY(cudaGetDevice(&dev));
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    QG_CUDA_TRY(cudaStreamIsCapturing(st, &cap));
-    const bool chain = cap == cudaStreamCaptureStatusNone && dev >= 0 && dev < kCoopDevices;
-    if (chain) {
-      if (!g_coop_done[dev]) QG_CUDA_TRY(cudaEventCreateWithFlags(&g_coop_done[dev], cudaEventDisableTiming));
-      else QG_CUDA_TRY(cudaStreamWaitEvent(st, g_coop_done[dev], 0));
-    }
     // rows in blocks of eight where the block count is even and a block fits shared memory; else row by row
-    if (blocks && b <= 16 * kBlkTeam) rc = launch_jacobi_block<16>(Tsub, cnt, b, sweeps, kTol, off, sync_words, status, st);
-    else if (blocks) rc = launch_jacobi_block<32>(Tsub, cnt, b, sweeps, kTol, off, sync_words, status, st);
-    else if (b <= 8 * kTeam) rc = launch_jacobi<8>(Tsub, cnt, b, sweeps, kTol, off, sync_words, status, st);
-    else if (b <= 16 * kTeam) rc = launch_jacobi<16>(Tsub, cnt, b, sweeps, kTol, off, sync_words, status, st);
-    else rc = launch_jacobi<32>(Tsub, cnt, b, sweeps, kTol, off, sync_words, status, st);
+    if (blocks && b <= 16 * kBlkTeam) rc = launch_jacobi_block<16>(Tsub, cnt, b, sweeps, kTol, off, sync_words, status, gate_sub, st);
+    else if (blocks) rc = launch_jacobi_block<32>(Tsub, cnt, b, sweeps, kTol, off, sync_words, status, gate_sub, st);
+    else if (b <= 8 * kTeam) rc = launch_jacobi<8>(Tsub, cnt, b, sweeps, kTol, off, sync_words, status, gate_sub, st);
+    else if (b <= 16 * kTeam) rc = launch_jacobi<16>(Tsub, cnt, b, sweeps, kTol, off, sync_words, status, gate_sub, st);
+    else rc = launch_jacobi<32>(Tsub, cnt, b, sweeps, kTol, off, sync_words, status, gate_sub, st);
     if (rc != QG_OK) return rc;
-    if (chain) QG_CUDA_TRY(cudaEventRecord(g_coop_done[dev], st));
   }
   const Ptrs<const float> Tc = QG_TAB(const float, T);
   const Ptrs<const double> lamc = QG_TAB(const double, lam);
-  row_norm_kernel<<<dim3((unsigned)b, (unsigned)nb), 128, 0, st>>>(Tc, (int)b, lam);
+  row_norm_kernel<<<dim3((unsigned)b, (unsigned)nb), 128, 0, st>>>(Tc, (int)b, lam, gate);
   QG_LAUNCH_CHECK();
-  select_top_kernel<<<dim3((unsigned)b, (unsigned)nb), 256, 0, st>>>(Tc, lamc, (int)b, (int)r, QG_TAB(float, Xsel));
+  select_top_kernel<<<dim3((unsigned)b, (unsigned)nb), 256, 0, st>>>(Tc, lamc, (int)b, (int)r, QG_TAB(float, Xsel), gate);
   QG_LAUNCH_CHECK();
   // P = Q Xsel
-  rc = gemm<float, float, float>(nb, Q, b, 1, Xsel, r, 1, P32, r, m, r, b, 1.f, 0.f, st);
+  rc = gemm<float, float, float>(nb, Q, b, 1, Xsel, r, 1, P32, r, m, r, b, 1.f, 0.f, st, nullptr, gate);
   if (rc != QG_OK) return rc;
-  sign_fix_kernel<<<dim3((unsigned)r, (unsigned)nb), 256, 0, st>>>(P32, m, (int)r, P_out);
-  QG_LAUNCH_CHECK();
+  return finish_vectors(jobs, bt, QG_TAB(const float, P32), r, m, r, false, gate, st);
+}
+
+// The route of a shape.  Direct: all of the short side's Gram matrix is reduced, ~4 us a row up to 1024 rows and 6 to 18
+// beyond.  Iterative: the cost goes with the block.
+static bool direct_route(int64_t m, int64_t n, int64_t b) {
+  const int64_t s = m < n ? m : n;
+  return g_jacobi_blocks && s <= kEigMax && s <= 8 * b;
+}
+
+// One batch (at most kMaxBatch matrices of one shape).
+static int refresh_batch(const RefreshJob* jobs, int nb, int64_t m, int64_t n, int64_t r, int64_t b, int iters, int sweeps,
+                         char* ws, size_t ws_stride, int32_t* status, cudaStream_t st, bool transposed) {
+  Batch bt{};
+  bt.nb = nb;
+  Gates gate{};
+  const bool direct = direct_route(m, n, b);
+  for (int i = 0; i < nb; ++i) {
+    carve_refresh(ws + (size_t)i * ws_stride, m, n, b, &bt.w[i]);
+    if (jobs[i].ldg != jobs[0].ldg) return QG_INVALID_ARGUMENT;          // one pitch per batch (the caller groups by it)
+    if (direct) gate.p[i] = bt.w[i].gate;
+  }
+  int rc = direct ? refresh_direct(jobs, bt, m, n, r, status, st, transposed) : QG_OK;
+  if (rc != QG_OK) return rc;
+  rc = refresh_iterative(jobs, bt, gate, m, n, r, b, iters, sweeps, status, st, transposed);
+  if (rc != QG_OK) return rc;
   for (int i = 0; i < nb; ++i) {
     rc = launch_quantize_rtn(jobs[i].P_new->bits, bt.w[i].P32, m, r, r, jobs[i].P_new, st);
     if (rc != QG_OK) return rc;
