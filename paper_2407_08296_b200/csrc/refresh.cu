@@ -1,7 +1,20 @@
-// Subspace refresh (Sec. 3.5: "obtain the projection matrix using SVD"; Sec. 3.3: INT4 storage).
+// Subspace refresh (Sec. 3.5: "obtain the projection matrix using SVD"; Sec. 3.3: INT4 storage): the top-r left singular
+// vectors of the gradient G (m x n, bf16), without a full SVD, by one of two routes.
 //
-// The top-r left singular vectors of the gradient G (m x n, bf16) are found without a full SVD:
-// block subspace iteration on G G^T with a block of b = r + oversample columns, followed by a
+// Direct, where the short side has at most kEigMax rows and the block is not a small part of it:
+//
+//   A = G G^T or G^T G, whichever is smaller (refresh_tc.cu: every product of two bfloat16 values is exact, sums in fp32)
+//   X <- its r leading eigenvectors (sym_eig.cu: tridiagonal reduction, bisection, twisted factorisations)
+//   P = X, or G X at unit length where the vectors wanted are those of the long side
+//
+// Its error is that of a symmetric eigenproblem in binary32: measured against an exact SVD the subspace is off by 4e-5 ..
+// 3e-4 rad on rank-32 signals with noise at 1e-3 (the iterative route: 1e-4 .. 5e-3, and up to 0.4 at r = s / 8, where its
+// block of 2 r columns does not converge in 12 iterations).  It grows with lambda_1 / lambda_r; where that leaves the r-th
+// vector unresolved QG_DEV_BAD_FACTOR is raised (the iterative route met a bad pivot there and returned NaN).
+// Time (one matrix, then a batch of eight, per matrix): 768 x 2048 r 256 17.2 -> 4.0 ms; 1024 x 1024 r 256 x 8 3.7 -> 1.0;
+// 2048 x 5461 r 512 42.8 -> 12.5 and 15.3 -> 6.1; 4096 x 11008 r 1024 139 -> 73.
+//
+// Iterative, for the rest: block subspace iteration on G G^T with a block of b = r + oversample columns, followed by a
 // Rayleigh-Ritz step that rotates the converged block onto the singular vectors.
 //
 //   Q <- orth(Gaussian m x b)
@@ -14,17 +27,12 @@
 // projection twice and two rounds of Cholesky QR in the last iterations, one of each before.  The eigenvectors of T
 // come from a one-sided (Hestenes) Jacobi iteration (rows kept in fp32, every sum in fp64: the result is INT4 in the
 // end) over blocks of eight rows held on the SM, all sweeps in one cooperative launch with a grid barrier between the
-// rounds of the tournament of blocks.  Each column of P is then given the sign that makes its largest entry positive,
-// and P is quantized to INT4 (Quant_4).
+// rounds of the tournament of blocks.
 //
-// Several matrices of one shape are refreshed together (a "batch", up to kMaxBatch): every launch carries a matrix
-// index beside its tile index and reads its operands from small pointer tables passed by value, so the few
-// thousand small launches and the grid barriers of the eigen-iteration (about 1200) are paid once per batch instead of
-// once per matrix.
-//
-// The singular values next to the r-th one sit in the noise bulk of the gradient with relative gaps of 1e-4..1e-3,
-// and resolving that subspace to 1e-2 rad needs fp32-faithful products: plain bf16 tensor-core products of the
-// iterate do not get there, the three-plane split does.
+// Either way each column of P is then given the sign that makes its largest entry positive, and P is quantized to INT4
+// (Quant_4).  Several matrices of one shape are refreshed together (a "batch", up to kMaxBatch): every launch carries a
+// matrix index beside its tile index and reads its operands from small pointer tables passed by value, so launches and
+// barriers are paid once per batch instead of once per matrix.
 #include <cmath>
 
 #include "refresh_common.cuh"
@@ -35,7 +43,7 @@ namespace qg {
 size_t split_planes_bytes(int64_t K, int64_t N);
 bool split_gemm_supported(const uint16_t* A, int64_t sa_m, int64_t sa_k, int64_t M, int64_t N, int64_t K);
 int launch_split_gemm(const uint16_t* A, int64_t sa_m, int64_t sa_k, const float* B, int64_t ldb, float* D, int64_t ldd,
-                      int64_t M, int64_t N, int64_t K, uint16_t* planes, const int32_t* gate, int32_t* status, cudaStream_t st);
+                      int64_t M, int64_t N, int64_t K, uint16_t* planes, int32_t* status, cudaStream_t st);
 
 namespace {
 
@@ -60,11 +68,6 @@ Ptrs<T> offset_ptrs(const Ptrs<U>& src, int nb, int64_t off) {
   return out;
 }
 
-// Kernels of the iterative route take a gate per matrix: where it is given and reads 0, the matrix has its vectors from the
-// direct route already and nothing happens.
-using Gates = Ptrs<const int32_t>;
-__device__ __forceinline__ bool closed(const Gates& gate, int mat) { return gate.p[mat] != nullptr && *gate.p[mat] == 0; }
-
 __device__ __forceinline__ float ld_as_float(const uint16_t* p, int64_t i) { return bf16_bits_to_float(p[i]); }
 __device__ __forceinline__ float ld_as_float(const float* p, int64_t i) { return p[i]; }
 
@@ -78,9 +81,8 @@ template <class TA, class ACC, class TC>
 __global__ void __launch_bounds__(256)
 gemm_kernel(const Ptrs<const TA> Ab, int64_t sa_m, int64_t sa_k, const Ptrs<const float> Bb, int64_t sb_k, int64_t sb_n,
             const Ptrs<TC> Cb, int64_t ldc, int M, int N, int K, ACC alpha, ACC beta, int k_slice, int slices,
-            const Ptrs<ACC> partb, const Gates gate) {
+            const Ptrs<ACC> partb) {
   const int mat = (int)blockIdx.z / slices, slice = (int)blockIdx.z % slices;
-  if (closed(gate, mat)) return;
   const TA* __restrict__ A = Ab.p[mat];
   const float* __restrict__ B = Bb.p[mat];
   TC* __restrict__ C = Cb.p[mat];
@@ -164,9 +166,7 @@ gemm_kernel(const Ptrs<const TA> Ab, int64_t sa_m, int64_t sa_k, const Ptrs<cons
 // C = alpha * (sum of the slices' partial sums, in slice order) + beta * C
 template <class ACC, class TC>
 __global__ void __launch_bounds__(256)
-gemm_reduce_kernel(const Ptrs<ACC> partb, int slices, const Ptrs<TC> Cb, int64_t ldc, int M, int N, ACC alpha, ACC beta,
-                   const Gates gate) {
-  if (closed(gate, blockIdx.y)) return;
+gemm_reduce_kernel(const Ptrs<ACC> partb, int slices, const Ptrs<TC> Cb, int64_t ldc, int M, int N, ACC alpha, ACC beta) {
   const ACC* __restrict__ part = partb.p[blockIdx.y];
   TC* __restrict__ C = Cb.p[blockIdx.y];
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -196,7 +196,7 @@ constexpr int64_t kSplitScratch = 32 << 20;  // bytes of partial sums a product 
 template <class TA, class ACC, class TC>
 int gemm(int nb, const Ptrs<const TA>& A, int64_t sa_m, int64_t sa_k, const Ptrs<const float>& B, int64_t sb_k, int64_t sb_n,
          const Ptrs<TC>& C, int64_t ldc, int64_t M, int64_t N, int64_t K, ACC alpha, ACC beta, cudaStream_t st,
-         const Ptrs<void>* part = nullptr, const Gates& gate = Gates{}) {
+         const Ptrs<void>* part = nullptr) {
   if (M <= 0 || N <= 0) return QG_OK;
   dim3 grid((unsigned)ceil_div(N, kGT), (unsigned)ceil_div(M, kGT));
   const int64_t tiles = (int64_t)grid.x * grid.y * nb;
@@ -211,7 +211,7 @@ int gemm(int nb, const Ptrs<const TA>& A, int64_t sa_m, int64_t sa_k, const Ptrs
   if (slices <= 1) {
     grid.z = (unsigned)nb;
     gemm_kernel<TA, ACC, TC><<<grid, 256, 0, st>>>(A, sa_m, sa_k, B, sb_k, sb_n, C, ldc, (int)M, (int)N, (int)K, alpha, beta,
-                                                   (int)K, 1, pt, gate);
+                                                   (int)K, 1, pt);
     QG_LAUNCH_CHECK();
     return QG_OK;
   }
@@ -220,18 +220,17 @@ int gemm(int nb, const Ptrs<const TA>& A, int64_t sa_m, int64_t sa_k, const Ptrs
   const int nslices = (int)ceil_div(K, k_slice);
   grid.z = (unsigned)(nslices * nb);
   gemm_kernel<TA, ACC, TC><<<grid, 256, 0, st>>>(A, sa_m, sa_k, B, sb_k, sb_n, C, ldc, (int)M, (int)N, (int)K, alpha, beta,
-                                                 (int)k_slice, nslices, pt, gate);
+                                                 (int)k_slice, nslices, pt);
   QG_LAUNCH_CHECK();
   gemm_reduce_kernel<ACC, TC><<<dim3((unsigned)ceil_div(M * N, 256), (unsigned)nb), 256, 0, st>>>(pt, nslices, C, ldc, (int)M, (int)N,
-                                                                                                  alpha, beta, gate);
+                                                                                                  alpha, beta);
   QG_LAUNCH_CHECK();
   return QG_OK;
 }
 
 // ---- Gaussian start block: Q[i][j] ~ N(0, 1) from Philox4x32-10 (counter (j / 4, i, 0, 0x51)) and Box-Muller
 __global__ void __launch_bounds__(256)
-gaussian_kernel(const Ptrs<float> Qb, int64_t ld, int64_t rows, int64_t cols, const Ptrs<const void> seeds, const Gates gate) {
-  if (closed(gate, blockIdx.y)) return;
+gaussian_kernel(const Ptrs<float> Qb, int64_t ld, int64_t rows, int64_t cols, const Ptrs<const void> seeds) {
   float* __restrict__ Q = Qb.p[blockIdx.y];
   // the seed of matrix y travels in the pointer table's slot (a 64-bit value, not an address)
   const uint64_t seed = (uint64_t)reinterpret_cast<uintptr_t>(seeds.p[blockIdx.y]);
@@ -260,8 +259,7 @@ gaussian_kernel(const Ptrs<float> Qb, int64_t ld, int64_t rows, int64_t cols, co
 // memory.  Binary32 is enough here: S itself comes from a binary32 product, and where the basis has to be
 // orthonormal to rounding the panel goes through this twice.
 __global__ void __launch_bounds__(32)
-chol64_inverse_kernel(const Ptrs<const float> Sb, const Ptrs<float> Linvb, int32_t* __restrict__ status, const Gates gate) {
-  if (closed(gate, blockIdx.x)) return;
+chol64_inverse_kernel(const Ptrs<const float> Sb, const Ptrs<float> Linvb, int32_t* __restrict__ status) {
   static_assert(kPanel == 64, "two rows and two columns per lane");
   const float* __restrict__ S = Sb.p[blockIdx.x];
   float* __restrict__ Linv = Linvb.p[blockIdx.x];
@@ -375,14 +373,13 @@ constexpr int kTeam = 128, kTeamsPerCta = 4;
 template <int NE>
 __global__ void __launch_bounds__(kTeam * kTeamsPerCta, NE <= 16 ? 2 : 1)   // two CTAs per SM while the rows fit 64 registers
 jacobi_sweeps_kernel(const Ptrs<float> Tb, int nb, int b, int sweeps, double tol, const Ptrs<unsigned long long> offb,
-                     unsigned int* __restrict__ sync_words, int32_t* __restrict__ status, const Gates gate) {
+                     unsigned int* __restrict__ sync_words, int32_t* __restrict__ status) {
   __shared__ double red[kTeamsPerCta][3][kTeam / 32];
   __shared__ double s_worst[kTeamsPerCta][kMaxBatch];
   const int team = threadIdx.x / kTeam, tt = threadIdx.x % kTeam, tw = tt >> 5, lane = threadIdx.x & 31;
   const int pairs = b / 2, jobs = pairs * nb, batch = (int)gridDim.x * kTeamsPerCta;
   unsigned int gen = 0;
-  uint32_t active = 0;                              // matrices still rotating
-  for (int i = 0; i < nb; ++i) active |= closed(gate, i) ? 0u : 1u << i;
+  uint32_t active = (1u << nb) - 1u;                // matrices still rotating
   for (int sw = 0; sw < sweeps && active != 0u; ++sw) {
     if (tt < kMaxBatch) s_worst[team][tt] = 0.0;
     for (int rnd = 0; rnd < b - 1; ++rnd) {
@@ -458,7 +455,7 @@ jacobi_sweeps_kernel(const Ptrs<float> Tb, int nb, int b, int sweeps, double tol
 
 template <int NE>
 int launch_jacobi(const Ptrs<float>& T, int nb, int64_t b, int sweeps, double tol, const Ptrs<unsigned long long>& off,
-                  unsigned int* sync_words, int32_t* status, const Gates& gate, cudaStream_t st) {
+                  unsigned int* sync_words, int32_t* status, cudaStream_t st) {
   // one cooperative launch, never more CTAs than are resident at once
   int per_sm = 0;
   QG_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, jacobi_sweeps_kernel<NE>, kTeam * kTeamsPerCta, 0));
@@ -469,8 +466,7 @@ int launch_jacobi(const Ptrs<float>& T, int nb, int64_t b, int sweeps, double to
   int bi = (int)b;
   Ptrs<float> Tc = T;
   Ptrs<unsigned long long> offc = off;
-  Gates gatec = gate;
-  void* args[] = {&Tc, &nb, &bi, &sweeps, &tol, &offc, &sync_words, &status, &gatec};
+  void* args[] = {&Tc, &nb, &bi, &sweeps, &tol, &offc, &sync_words, &status};
   return launch_cooperative((const void*)jacobi_sweeps_kernel<NE>, (unsigned)grid, kTeam * kTeamsPerCta, args, 0, st);
 }
 
@@ -542,7 +538,7 @@ __device__ __forceinline__ double team_rotate(float (&x)[NE], float (&y)[NE], bo
 template <int NE>
 __global__ void __launch_bounds__(kBlkThreads, NE <= 16 ? 2 : 1)
 jacobi_block_kernel(const Ptrs<float> Tb, int nb, int b, int sweeps, double tol, const Ptrs<unsigned long long> offb,
-                    unsigned int* __restrict__ sync_words, int32_t* __restrict__ status, const Gates gate) {
+                    unsigned int* __restrict__ sync_words, int32_t* __restrict__ status) {
   // three sets of eight rows of b floats: the rows of block J of this job and of the next one (the copy engine brings
   // the next job's rows in while this one rotates), and the rows of block I of the next job
   extern __shared__ __align__(16) float blk_smem[];
@@ -554,8 +550,7 @@ jacobi_block_kernel(const Ptrs<float> Tb, int nb, int b, int sweeps, double tol,
   const int set = kBlkRows * b;
   float* const rows_i_next = blk_smem + 2 * set;
   unsigned int gen = 0;
-  uint32_t active = 0;                               // matrices still rotating
-  for (int i = 0; i < nb; ++i) active |= closed(gate, i) ? 0u : 1u << i;
+  uint32_t active = (1u << nb) - 1u;                 // matrices still rotating
   for (int sw = 0; sw < sweeps && active != 0u; ++sw) {
     if (tt < kMaxBatch) s_worst[team][tt] = 0.0;
     __syncthreads();
@@ -708,7 +703,7 @@ jacobi_block_kernel(const Ptrs<float> Tb, int nb, int b, int sweeps, double tol,
 // Opts the instance into its dynamic shared memory once per device.
 template <int NE>
 int launch_jacobi_block(const Ptrs<float>& T, int nb, int64_t b, int sweeps, double tol, const Ptrs<unsigned long long>& off,
-                        unsigned int* sync_words, int32_t* status, const Gates& gate, cudaStream_t st) {
+                        unsigned int* sync_words, int32_t* status, cudaStream_t st) {
   const int smem = (int)(3 * kBlkRows * b * sizeof(float));
   static bool smem_set[kCoopDevices] = {};
   int dev = 0;
@@ -728,15 +723,13 @@ int launch_jacobi_block(const Ptrs<float>& T, int nb, int64_t b, int sweeps, dou
   int bi = (int)b;
   Ptrs<float> Tc = T;
   Ptrs<unsigned long long> offc = off;
-  Gates gatec = gate;
-  void* args[] = {&Tc, &nb, &bi, &sweeps, &tol, &offc, &sync_words, &status, &gatec};
+  void* args[] = {&Tc, &nb, &bi, &sweeps, &tol, &offc, &sync_words, &status};
   return launch_cooperative((const void*)jacobi_block_kernel<NE>, (unsigned)grid, kBlkThreads, args, (size_t)smem, st);
 }
 
 // lambda_j = norm of row j of the rotated T (= |eigenvalue j|); rank_j = its position in descending order
 __global__ void __launch_bounds__(128)
-row_norm_kernel(const Ptrs<const float> Tb, int b, const Ptrs<double> lamb, const Gates gate) {
-  if (closed(gate, blockIdx.y)) return;
+row_norm_kernel(const Ptrs<const float> Tb, int b, const Ptrs<double> lamb) {
   const float* row = Tb.p[blockIdx.y] + (int64_t)blockIdx.x * b;
   double* __restrict__ lam = lamb.p[blockIdx.y];
   double s = 0.0;
@@ -751,8 +744,7 @@ row_norm_kernel(const Ptrs<const float> Tb, int b, const Ptrs<double> lamb, cons
 
 // Xsel[i][rank_j] = X[i][j] = T[j][i] / lambda_j for the r largest lambda_j
 __global__ void __launch_bounds__(256)
-select_top_kernel(const Ptrs<const float> Tb, const Ptrs<const double> lamb, int b, int r, const Ptrs<float> Xselb, const Gates gate) {
-  if (closed(gate, blockIdx.y)) return;
+select_top_kernel(const Ptrs<const float> Tb, const Ptrs<const double> lamb, int b, int r, const Ptrs<float> Xselb) {
   const float* __restrict__ T = Tb.p[blockIdx.y];
   const double* __restrict__ lam = lamb.p[blockIdx.y];
   float* __restrict__ Xsel = Xselb.p[blockIdx.y];
@@ -779,8 +771,7 @@ select_top_kernel(const Ptrs<const float> Tb, const Ptrs<const double> lamb, int
 // 32 columns and reads 32 rows of them at a time, so that every access is a whole line.
 __global__ void __launch_bounds__(1024)
 finish_vectors_kernel(const Ptrs<const float> Sb, int64_t lds, int64_t rows, int r, bool normalise, const Ptrs<float> Pb,
-                      const Ptrs<float> P_outb, const Gates gate) {
-  if (closed(gate, blockIdx.y)) return;
+                      const Ptrs<float> P_outb) {
   __shared__ float s_big[32][33], s_sum[32][33];
   const float* S = Sb.p[blockIdx.y];
   float* P = Pb.p[blockIdx.y];
@@ -817,12 +808,11 @@ finish_vectors_kernel(const Ptrs<const float> Sb, int64_t lds, int64_t rows, int
 
 struct RefreshWs {
   float* P32;      // the vectors before quantization
-  int32_t* gate;   // 1: the direct route has not resolved them
   // direct route
   EigBuffers eig;  // of the Gram matrix of the short side
   float* XV;       // X V, for vectors on the long side
   uint16_t* planes_v;
-  // iterative route (in the same memory: it begins when the direct one has ended)
+  // iterative route (in the same memory)
   float *Q, *Y, *Z, *Wp, *Cb, *S, *Linv, *Xsel;
   void* part;      // partial sums of sliced products
   uint16_t* planes;  // the three bfloat16 planes of an iterate, for the tensor-core products
@@ -837,7 +827,6 @@ size_t carve_refresh(void* base, int64_t m, int64_t n, int64_t b, RefreshWs* w) 
   auto take = [&](size_t bytes) { void* p = base ? (char*)base + off : nullptr; off += (size_t)round_up((int64_t)bytes, 256); return p; };
   RefreshWs t{};
   t.P32 = (float*)take((size_t)m * b * 4);
-  t.gate = (int32_t*)take(4);
   const size_t routes = off;
   const int64_t s = m < n ? m : n;
   if (s <= kEigMax) {
@@ -885,7 +874,7 @@ struct Batch {
 // about 1e-2 (fp32 Gram matrices of panels with a condition number of several hundred), which is all an
 // intermediate subspace iteration asks of it: the next multiplication by G G^T and the next orthonormalisation
 // start from that basis, they do not inherit its error.
-int orthonormalize(const Batch& bt, int64_t m, int64_t b, const Gates& gate, int32_t* status, cudaStream_t st, bool full) {
+int orthonormalize(const Batch& bt, int64_t m, int64_t b, int32_t* status, cudaStream_t st, bool full) {
   const int passes = full ? 2 : 1;
   const int nb = bt.nb;
   Ptrs<void> part{};
@@ -900,9 +889,9 @@ int orthonormalize(const Batch& bt, int64_t m, int64_t b, const Gates& gate, int
     int rc;
     for (int pass = 0; pass < passes && j0 > 0; ++pass) {
       // C = Q[:, :j0]^T Yj   (j0 x 64);   Yj -= Q[:, :j0] C
-      rc = gemm<float, float, float>(nb, Q, 1, b, Yjc, b, 1, Cb, kPanel, j0, kPanel, m, 1.f, 0.f, st, &part, gate);
+      rc = gemm<float, float, float>(nb, Q, 1, b, Yjc, b, 1, Cb, kPanel, j0, kPanel, m, 1.f, 0.f, st, &part);
       if (rc != QG_OK) return rc;
-      rc = gemm<float, float, float>(nb, Q, b, 1, Cbc, kPanel, 1, Yj, b, m, kPanel, j0, -1.f, 1.f, st, &part, gate);
+      rc = gemm<float, float, float>(nb, Q, b, 1, Cbc, kPanel, 1, Yj, b, m, kPanel, j0, -1.f, 1.f, st, &part);
       if (rc != QG_OK) return rc;
     }
     // Cholesky QR on the panel, two rounds (Yj -> Wp -> Qj) or one (Yj -> Qj)
@@ -912,12 +901,12 @@ int orthonormalize(const Batch& bt, int64_t m, int64_t b, const Gates& gate, int
       const int64_t lds = pass == 0 ? b : kPanel;
       const Ptrs<float>& dst = last ? Qj : Wp;
       const int64_t ldd = last ? b : kPanel;
-      rc = gemm<float, float, float>(nb, src, 1, lds, src, lds, 1, S, kPanel, kPanel, kPanel, m, 1.f, 0.f, st, &part, gate);
+      rc = gemm<float, float, float>(nb, src, 1, lds, src, lds, 1, S, kPanel, kPanel, kPanel, m, 1.f, 0.f, st, &part);
       if (rc != QG_OK) return rc;
-      chol64_inverse_kernel<<<nb, 32, 0, st>>>(Sc, Linv, status, gate);
+      chol64_inverse_kernel<<<nb, 32, 0, st>>>(Sc, Linv, status);
       QG_LAUNCH_CHECK();
       // dst = src * Linv^T:  B(k, j) = Linv[j][k]
-      rc = gemm<float, float, float>(nb, src, lds, 1, Linvc, 1, kPanel, dst, ldd, m, kPanel, kPanel, 1.f, 0.f, st, nullptr, gate);
+      rc = gemm<float, float, float>(nb, src, lds, 1, Linvc, 1, kPanel, dst, ldd, m, kPanel, kPanel, 1.f, 0.f, st);
       if (rc != QG_OK) return rc;
     }
   }
@@ -930,11 +919,10 @@ size_t refresh_workspace_bytes(int64_t m, int64_t n, int64_t b) { return carve_r
 
 // Unit length (if asked for) and sign of the vectors in S (pitch lds): P32, P_fp32.
 static int finish_vectors(const RefreshJob* jobs, const Batch& bt, const Ptrs<const float>& S, int64_t lds, int64_t rows, int64_t r,
-                          bool normalise, const Gates& gate, cudaStream_t st) {
+                          bool normalise, cudaStream_t st) {
   Ptrs<float> P_out{};
   for (int i = 0; i < bt.nb; ++i) P_out.p[i] = jobs[i].P_fp32;
-  finish_vectors_kernel<<<dim3((unsigned)ceil_div(r, 32), (unsigned)bt.nb), 1024, 0, st>>>(S, lds, rows, (int)r, normalise, QG_TAB(float, P32), P_out,
-                                                                                           gate);
+  finish_vectors_kernel<<<dim3((unsigned)ceil_div(r, 32), (unsigned)bt.nb), 1024, 0, st>>>(S, lds, rows, (int)r, normalise, QG_TAB(float, P32), P_out);
   QG_LAUNCH_CHECK();
   return QG_OK;
 }
@@ -946,7 +934,6 @@ static int refresh_direct(const RefreshJob* jobs, const Batch& bt, int64_t m, in
   const int nb = bt.nb;
   const uint16_t* G[kMaxBatch];
   float* A[kMaxBatch];
-  int32_t* doubtful[kMaxBatch];
   EigBuffers eig[kMaxBatch];
   const int64_t ldg = jobs[0].ldg;
   const bool long_side = m > n;
@@ -956,18 +943,17 @@ static int refresh_direct(const RefreshJob* jobs, const Batch& bt, int64_t m, in
     G[i] = jobs[i].G;
     eig[i] = bt.w[i].eig;
     A[i] = eig[i].A;
-    doubtful[i] = bt.w[i].gate;
   }
   int rc = launch_gram(G, nb, ldg, transposed != long_side, s, l, A, eig_pitch(s), status, st);
   if (rc != QG_OK) return rc;
-  rc = launch_sym_eig(eig, doubtful, nb, s, re, status, st);
+  rc = launch_sym_eig(eig, nb, s, re, status, st);
   if (rc != QG_OK) return rc;
   const Ptrs<const float> V = bt.tab<const float>([](const RefreshWs& x) { return x.eig.Z; });
-  if (!long_side) return finish_vectors(jobs, bt, V, re, m, r, false, Gates{}, st);
+  if (!long_side) return finish_vectors(jobs, bt, V, re, m, r, false, st);
   const int64_t rs = transposed ? 1 : ldg, cs = transposed ? ldg : 1;
   if (split_gemm_supported(G[0], rs, cs, m, re, s)) {
     for (int i = 0; i < nb; ++i) {
-      rc = launch_split_gemm(G[i], rs, cs, eig[i].Z, re, bt.w[i].XV, re, m, re, s, bt.w[i].planes_v, nullptr, status, st);
+      rc = launch_split_gemm(G[i], rs, cs, eig[i].Z, re, bt.w[i].XV, re, m, re, s, bt.w[i].planes_v, status, st);
       if (rc != QG_OK) return rc;
     }
   } else {
@@ -976,13 +962,13 @@ static int refresh_direct(const RefreshJob* jobs, const Batch& bt, int64_t m, in
     rc = gemm<uint16_t, float, float>(nb, Gp, rs, cs, V, re, 1, QG_TAB(float, XV), re, m, re, s, 1.f, 0.f, st);
     if (rc != QG_OK) return rc;
   }
-  return finish_vectors(jobs, bt, QG_TAB(const float, XV), re, m, r, true, Gates{}, st);
+  return finish_vectors(jobs, bt, QG_TAB(const float, XV), re, m, r, true, st);
 }
 
-// The iterative route, for the matrices whose gate is open.  `transposed`: the singular vectors wanted are the RIGHT ones
+// The iterative route.  `transposed`: the singular vectors wanted are the RIGHT ones
 // of G, i.e. the left ones of G^T; G is then read with its two strides swapped and (m, n) are the extents of G^T.
-static int refresh_iterative(const RefreshJob* jobs, const Batch& bt, const Gates& gate, int64_t m, int64_t n, int64_t r, int64_t b, int iters,
-                             int sweeps, int32_t* status, cudaStream_t st, bool transposed) {
+static int refresh_iterative(const RefreshJob* jobs, const Batch& bt, int64_t m, int64_t n, int64_t r, int64_t b, int iters, int sweeps,
+                             int32_t* status, cudaStream_t st, bool transposed) {
   const int nb = bt.nb;
   Ptrs<const uint16_t> G{};
   Ptrs<const void> seeds{};
@@ -998,9 +984,9 @@ static int refresh_iterative(const RefreshJob* jobs, const Batch& bt, const Gate
   // start block
   {
     const int64_t threads = m * (b / 4);
-    gaussian_kernel<<<dim3((unsigned)ceil_div(threads, 256), (unsigned)nb), 256, 0, st>>>(Y, b, m, b, seeds, gate);
+    gaussian_kernel<<<dim3((unsigned)ceil_div(threads, 256), (unsigned)nb), 256, 0, st>>>(Y, b, m, b, seeds);
     QG_LAUNCH_CHECK();
-    rc = orthonormalize(bt, m, b, gate, status, st, iters < 2);          // in full only if no later iteration will be
+    rc = orthonormalize(bt, m, b, status, st, iters < 2);          // in full only if no later iteration will be
     if (rc != QG_OK) return rc;
   }
   // The two products with the gradient go to the tensor cores (bfloat16 gradient times an iterate split into three
@@ -1015,31 +1001,31 @@ static int refresh_iterative(const RefreshJob* jobs, const Batch& bt, const Gate
     // Z = G^T Q
     if (tc_z && it < iters) {
       for (int i = 0; i < nb; ++i) {
-        rc = launch_split_gemm(G.p[i], cs, rs, bt.w[i].Q, b, bt.w[i].Z, b, n, b, m, bt.w[i].planes, gate.p[i], status, st);
+        rc = launch_split_gemm(G.p[i], cs, rs, bt.w[i].Q, b, bt.w[i].Z, b, n, b, m, bt.w[i].planes, status, st);
         if (rc != QG_OK) return rc;
       }
     } else {
-      rc = gemm<uint16_t, float, float>(nb, G, cs, rs, Q, b, 1, Zw, b, n, b, m, 1.f, 0.f, st, nullptr, gate);
+      rc = gemm<uint16_t, float, float>(nb, G, cs, rs, Q, b, 1, Zw, b, n, b, m, 1.f, 0.f, st);
       if (rc != QG_OK) return rc;
     }
     if (it == iters) break;
     // Y = G Z
     if (tc_y) {
       for (int i = 0; i < nb; ++i) {
-        rc = launch_split_gemm(G.p[i], rs, cs, bt.w[i].Z, b, bt.w[i].Y, b, m, b, n, bt.w[i].planes, gate.p[i], status, st);
+        rc = launch_split_gemm(G.p[i], rs, cs, bt.w[i].Z, b, bt.w[i].Y, b, m, b, n, bt.w[i].planes, status, st);
         if (rc != QG_OK) return rc;
       }
     } else {
-      rc = gemm<uint16_t, float, float>(nb, G, rs, cs, Z, b, 1, Y, b, m, b, n, 1.f, 0.f, st, nullptr, gate);
+      rc = gemm<uint16_t, float, float>(nb, G, rs, cs, Z, b, 1, Y, b, m, b, n, 1.f, 0.f, st);
       if (rc != QG_OK) return rc;
     }
-    rc = orthonormalize(bt, m, b, gate, status, st, it + 2 >= iters);   // the last two in full
+    rc = orthonormalize(bt, m, b, status, st, it + 2 >= iters);   // the last two in full
     if (rc != QG_OK) return rc;
   }
   // Rayleigh-Ritz: T = Z^T Z (accumulated in binary64, kept in binary32), eigenvectors by one-sided Jacobi
   const Ptrs<float> T = QG_TAB(float, T);
   const Ptrs<double> lam = QG_TAB(double, lam);
-  rc = gemm<float, double, float>(nb, Z, 1, b, Z, b, 1, T, b, b, b, n, 1.0, 0.0, st, nullptr, gate);
+  rc = gemm<float, double, float>(nb, Z, 1, b, Z, b, 1, T, b, b, b, n, 1.0, 0.0, st);
   if (rc != QG_OK) return rc;
   if (sweeps > kMaxSweeps) sweeps = kMaxSweeps;
   for (int i = 0; i < nb; ++i) QG_CUDA_TRY(cudaMemsetAsync(bt.w[i].off, 0, kMaxSweeps * 8, st));
@@ -1053,38 +1039,37 @@ static int refresh_iterative(const RefreshJob* jobs, const Batch& bt, const Gate
     const int cnt = std::min(per_launch, nb - first);
     Ptrs<float> Tsub{};
     Ptrs<unsigned long long> off{};
-    Gates gate_sub{};
     for (int i = 0; i < cnt; ++i) {
       Tsub.p[i] = bt.w[first + i].T;
       off.p[i] = reinterpret_cast<unsigned long long*>(bt.w[first + i].off);
-      gate_sub.p[i] = gate.p[first + i];
     }
     QG_CUDA_TRY(cudaMemsetAsync(bt.w[0].done, 0, 8, st));
     unsigned int* sync_words = reinterpret_cast<unsigned int*>(bt.w[0].done);
     // the iteration converges quadratically at the end: a sweep that met nothing above 1e-5 leaves ~1e-10
     constexpr double kTol = 1e-5;
     // rows in blocks of eight where the block count is even and a block fits shared memory; else row by row
-    if (blocks && b <= 16 * kBlkTeam) rc = launch_jacobi_block<16>(Tsub, cnt, b, sweeps, kTol, off, sync_words, status, gate_sub, st);
-    else if (blocks) rc = launch_jacobi_block<32>(Tsub, cnt, b, sweeps, kTol, off, sync_words, status, gate_sub, st);
-    else if (b <= 8 * kTeam) rc = launch_jacobi<8>(Tsub, cnt, b, sweeps, kTol, off, sync_words, status, gate_sub, st);
-    else if (b <= 16 * kTeam) rc = launch_jacobi<16>(Tsub, cnt, b, sweeps, kTol, off, sync_words, status, gate_sub, st);
-    else rc = launch_jacobi<32>(Tsub, cnt, b, sweeps, kTol, off, sync_words, status, gate_sub, st);
+    if (blocks && b <= 16 * kBlkTeam) rc = launch_jacobi_block<16>(Tsub, cnt, b, sweeps, kTol, off, sync_words, status, st);
+    else if (blocks) rc = launch_jacobi_block<32>(Tsub, cnt, b, sweeps, kTol, off, sync_words, status, st);
+    else if (b <= 8 * kTeam) rc = launch_jacobi<8>(Tsub, cnt, b, sweeps, kTol, off, sync_words, status, st);
+    else if (b <= 16 * kTeam) rc = launch_jacobi<16>(Tsub, cnt, b, sweeps, kTol, off, sync_words, status, st);
+    else rc = launch_jacobi<32>(Tsub, cnt, b, sweeps, kTol, off, sync_words, status, st);
     if (rc != QG_OK) return rc;
   }
   const Ptrs<const float> Tc = QG_TAB(const float, T);
   const Ptrs<const double> lamc = QG_TAB(const double, lam);
-  row_norm_kernel<<<dim3((unsigned)b, (unsigned)nb), 128, 0, st>>>(Tc, (int)b, lam, gate);
+  row_norm_kernel<<<dim3((unsigned)b, (unsigned)nb), 128, 0, st>>>(Tc, (int)b, lam);
   QG_LAUNCH_CHECK();
-  select_top_kernel<<<dim3((unsigned)b, (unsigned)nb), 256, 0, st>>>(Tc, lamc, (int)b, (int)r, QG_TAB(float, Xsel), gate);
+  select_top_kernel<<<dim3((unsigned)b, (unsigned)nb), 256, 0, st>>>(Tc, lamc, (int)b, (int)r, QG_TAB(float, Xsel));
   QG_LAUNCH_CHECK();
   // P = Q Xsel
-  rc = gemm<float, float, float>(nb, Q, b, 1, Xsel, r, 1, P32, r, m, r, b, 1.f, 0.f, st, nullptr, gate);
+  rc = gemm<float, float, float>(nb, Q, b, 1, Xsel, r, 1, P32, r, m, r, b, 1.f, 0.f, st);
   if (rc != QG_OK) return rc;
-  return finish_vectors(jobs, bt, QG_TAB(const float, P32), r, m, r, false, gate, st);
+  return finish_vectors(jobs, bt, QG_TAB(const float, P32), r, m, r, false, st);
 }
 
-// The route of a shape.  Direct: all of the short side's Gram matrix is reduced, ~4 us a row up to 1024 rows and 6 to 18
-// beyond.  Iterative: the cost goes with the block.
+// The route of a shape.  Direct: the whole of the short side's Gram matrix is reduced, 4 us a row up to 1024 rows, 6 to 18
+// beyond.  Iterative: the cost goes with the block, whose accuracy at a small part of the spectrum is poor (above):
+// 2048 x 2048, b = 256 9.3 ms at 0.2 rad against 12.4 ms at 2e-5; 1024 x 2048, b = 64 2.5 ms against 5.
 static bool direct_route(int64_t m, int64_t n, int64_t b) {
   const int64_t s = m < n ? m : n;
   return g_jacobi_blocks && s <= kEigMax && s <= 8 * b;
@@ -1095,16 +1080,12 @@ static int refresh_batch(const RefreshJob* jobs, int nb, int64_t m, int64_t n, i
                          char* ws, size_t ws_stride, int32_t* status, cudaStream_t st, bool transposed) {
   Batch bt{};
   bt.nb = nb;
-  Gates gate{};
-  const bool direct = direct_route(m, n, b);
   for (int i = 0; i < nb; ++i) {
     carve_refresh(ws + (size_t)i * ws_stride, m, n, b, &bt.w[i]);
     if (jobs[i].ldg != jobs[0].ldg) return QG_INVALID_ARGUMENT;          // one pitch per batch (the caller groups by it)
-    if (direct) gate.p[i] = bt.w[i].gate;
   }
-  int rc = direct ? refresh_direct(jobs, bt, m, n, r, status, st, transposed) : QG_OK;
-  if (rc != QG_OK) return rc;
-  rc = refresh_iterative(jobs, bt, gate, m, n, r, b, iters, sweeps, status, st, transposed);
+  int rc = direct_route(m, n, b) ? refresh_direct(jobs, bt, m, n, r, status, st, transposed)
+                                 : refresh_iterative(jobs, bt, m, n, r, b, iters, sweeps, status, st, transposed);
   if (rc != QG_OK) return rc;
   for (int i = 0; i < nb; ++i) {
     rc = launch_quantize_rtn(jobs[i].P_new->bits, bt.w[i].P32, m, r, r, jobs[i].P_new, st);

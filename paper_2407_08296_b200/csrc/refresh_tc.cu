@@ -61,8 +61,7 @@ __device__ __forceinline__ void raise_expired(int32_t* status) {
 
 template <bool A_MN>
 __global__ void __launch_bounds__(SplitSmem::kThreads, 1)
-split_gemm_kernel(const __grid_constant__ SplitArgs a, const int32_t* __restrict__ gate, int32_t* __restrict__ status) {
-  if (gate && *gate == 0) return;
+split_gemm_kernel(const __grid_constant__ SplitArgs a, int32_t* __restrict__ status) {
   using S = SplitSmem;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -203,7 +202,11 @@ split_gemm_kernel(const __grid_constant__ SplitArgs a, const int32_t* __restrict
 // operands are the same bfloat16 matrix, every product is exact, one pass.  Tiles of 128 x 256; those that lie wholly
 // above the diagonal are not computed, their elements are written as mirror images.  K-major operands (rows of X are
 // rows of G) come as boxes of 64 x 128 rows; MN-major ones (rows of X are columns of G) as 64 x 64 slabs with the exact
-// bounds of the matrix, so that any row pitch will do.  Eight of 2048 x 5461: 165 us (730 TFLOP/s on what is computed).
+// bounds of the matrix, so that any row pitch will do.
+// The tensor core truncates each aligned sum, which biases an accumulator by half a unit in its last place per instruction.
+// Every 256 columns of K the accumulator is therefore handed to the epilogue, whose threads add the parts up in registers
+// (rounded to nearest, each part with the bias of its own size): on 768 x 2048, noise at 1e-4, the subspace error falls
+// from 1.3e-2 to GRAM_NOW.  Eight of 2048 x 5461: GRAM_TIME us.
 struct GramArgs {
   CUtensorMap map[kMaxBatch];
   float* A[kMaxBatch];
@@ -217,7 +220,8 @@ struct GramSmem {
   static constexpr int kStages = 4;
   static constexpr int kBarOffset = kStages * kStageBytes;
   static constexpr int kBytes = kBarOffset + 256 + 1024;
-  static constexpr int kThreads = 256;
+  static constexpr int kSegment = 4;                           // K blocks per handed-over accumulator
+  static constexpr int kThreads = (4 + 8) * 32;
 };
 
 // Tile t of the triangle: row block m has the column blocks 0 .. m / 2.
@@ -240,7 +244,7 @@ gram_kernel(const __grid_constant__ GramArgs a, int nmat, int32_t* __restrict__ 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     for (int i = 0; i < S::kStages; ++i) { mbar_init(&full[i], 1); mbar_init(&empty[i], 1); }
-    for (int i = 0; i < 2; ++i) { mbar_init(&acc_full[i], 1); mbar_init(&acc_empty[i], 4); }
+    for (int i = 0; i < 2; ++i) { mbar_init(&acc_full[i], 1); mbar_init(&acc_empty[i], 8); }
     fence_mbar_init();
     fence_proxy_async_smem();
   }
@@ -286,65 +290,77 @@ gram_kernel(const __grid_constant__ GramArgs a, int nmat, int32_t* __restrict__ 
       const uint64_t desc_a0 = umma_smem_desc_sw128(smem_u32(smem), MN ? kSlab : 16, 1024);
       const uint64_t desc_b0 = umma_smem_desc_sw128(smem_u32(smem) + S::kABytes, MN ? kSlab : 16, 1024);
       constexpr uint64_t step = MN ? (2048 >> 4) : (32 >> 4);
-      uint32_t it = 0, tcount = 0;
+      uint32_t it = 0, seg = 0;
       bool ok = true;
-      for (int t = blockIdx.x; ok && t < total; t += gridDim.x, ++tcount) {
-        const uint32_t ab = tcount & 1;
-        if (!mbar_wait(&acc_empty[ab], ((tcount >> 1) & 1) ^ 1)) { ok = false; break; }
-        tc_fence_after_sync();
-        for (int kb = 0; kb < kblocks; ++kb, ++it) {
+      for (int t = blockIdx.x; ok && t < total; t += gridDim.x) {
+        for (int kb = 0; ok && kb < kblocks; ++kb, ++it) {
+          const int in_seg = kb % S::kSegment;
+          const uint32_t ab = seg & 1;
+          if (in_seg == 0) {
+            if (!mbar_wait(&acc_empty[ab], ((seg >> 1) & 1) ^ 1)) { ok = false; break; }
+            tc_fence_after_sync();
+          }
           const int s = it % S::kStages;
           if (!mbar_wait(&full[s], (it / S::kStages) & 1)) { ok = false; break; }
           tc_fence_after_sync();
           const uint64_t off = (uint64_t)((s * S::kStageBytes) >> 4);
 #pragma unroll
           for (int k = 0; k < kBK / 16; ++k)
-            umma_bf16(tmem_base + ab * kTileN, desc_a0 + off + k * step, desc_b0 + off + k * step, idesc, (kb | k) != 0);
+            umma_bf16(tmem_base + ab * kTileN, desc_a0 + off + k * step, desc_b0 + off + k * step, idesc, (in_seg | k) != 0);
           umma_commit(&empty[s]);
+          if (in_seg == S::kSegment - 1 || kb == kblocks - 1) { umma_commit(&acc_full[ab]); ++seg; }
         }
-        if (ok) umma_commit(&acc_full[ab]);
       }
       if (!ok) raise_expired(status);
     }
   } else if (warp >= 4) {
-    const int q = warp & 3;
-    uint32_t tcount = 0;
+    // warps 4-7: columns 0 .. 127 of the tile, 8-11: 128 .. 255; a thread sums up 128 elements of its row
+    const int q = warp & 3, half = (warp - 4) >> 2;
+    uint32_t seg = 0;
     bool ok = true;
-    for (int t = blockIdx.x; ok && t < total; t += gridDim.x, ++tcount) {
+    for (int t = blockIdx.x; ok && t < total; t += gridDim.x) {
       int mb, nb;
       gram_tile(t % a.tiles, mb, nb);
       float* A = a.A[t / a.tiles];
-      const uint32_t ab = tcount & 1;
-      if (!mbar_wait(&acc_full[ab], (tcount >> 1) & 1)) { ok = false; break; }
-      tc_fence_after_sync();
-      const uint32_t tacc = tmem_base + ((uint32_t)(q * 32) << 16) + ab * kTileN;
-      const int row = mb * kTileM + q * 32 + lane;
-#pragma unroll 1
-      for (int c = 0; c < kTileN / 32; ++c) {
-        uint32_t v[32];
-        tmem_ld_32x32(tacc + 32 * c, v);
-        tmem_ld_wait();
-        if (c == kTileN / 32 - 1) {
-          tc_fence_before_sync();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(&acc_empty[ab]);
+      float sum[128];
+#pragma unroll
+      for (int i = 0; i < 128; ++i) sum[i] = 0.f;
+      for (int kb = 0; kb < kblocks; kb += S::kSegment, ++seg) {
+        const uint32_t ab = seg & 1;
+        if (!mbar_wait(&acc_full[ab], (seg >> 1) & 1)) { ok = false; break; }
+        tc_fence_after_sync();
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          uint32_t v[32];
+          tmem_ld_32x32(tmem_base + ((uint32_t)(q * 32) << 16) + ab * kTileN + half * 128 + 32 * c, v);
+          tmem_ld_wait();
+#pragma unroll
+          for (int i = 0; i < 32; ++i) sum[32 * c + i] += __uint_as_float(v[i]);
         }
-        const int col = nb * kTileN + 32 * c;
-        if (row >= a.N) continue;
+        tc_fence_before_sync();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&acc_empty[ab]);
+      }
+      const int row = mb * kTileM + q * 32 + lane;
+      if (!ok || row >= a.N) continue;
+      const bool mirror = mb / 2 > nb;                 // no tile of the triangle covers the mirror image
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const int col = nb * kTileN + half * 128 + 32 * c;
         if (col + 32 <= a.N) {
 #pragma unroll
           for (int i = 0; i < 8; ++i)
-            *reinterpret_cast<uint4*>(A + (int64_t)row * a.lda + col + 4 * i) = make_uint4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+            *reinterpret_cast<float4*>(A + (int64_t)row * a.lda + col + 4 * i) =
+                make_float4(sum[32 * c + 4 * i], sum[32 * c + 4 * i + 1], sum[32 * c + 4 * i + 2], sum[32 * c + 4 * i + 3]);
         } else {
 #pragma unroll
           for (int i = 0; i < 32; ++i)
-            if (col + i < a.N) A[(int64_t)row * a.lda + col + i] = __uint_as_float(v[i]);
+            if (col + i < a.N) A[(int64_t)row * a.lda + col + i] = sum[32 * c + i];
         }
-        // the mirror image, where no tile of the triangle covers it (32 lanes: 128 contiguous bytes of a row)
-        if (mb / 2 > (col / kTileM) / 2) {
+        if (mirror) {                                  // 32 lanes: 128 contiguous bytes of a row
 #pragma unroll
           for (int i = 0; i < 32; ++i)
-            if (col + i < a.N) A[(int64_t)(col + i) * a.lda + row] = __uint_as_float(v[i]);
+            if (col + i < a.N) A[(int64_t)(col + i) * a.lda + row] = sum[32 * c + i];
         }
       }
     }
@@ -362,8 +378,7 @@ gram_kernel(const __grid_constant__ GramArgs a, int nmat, int32_t* __restrict__ 
 // lo = bf16(x - hi - mid) (the subtractions are exact in binary32).  Rows K .. kpad - 1 are written as zero, so that
 // a K block that reaches past K reads zeros and never the next plane.  A thread takes eight columns.
 __global__ void __launch_bounds__(256)
-split_planes_kernel(const float* __restrict__ B, int64_t ldb, int K, int N, int kpad, uint16_t* __restrict__ planes, const int32_t* __restrict__ gate) {
-  if (gate && *gate == 0) return;
+split_planes_kernel(const float* __restrict__ B, int64_t ldb, int K, int N, int kpad, uint16_t* __restrict__ planes) {
   const int64_t per_row = N / 8;
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= (int64_t)kpad * per_row) return;
@@ -451,13 +466,13 @@ bool split_gemm_supported(const uint16_t* A, int64_t sa_m, int64_t sa_k, int64_t
 }
 
 // D (M x N fp32, pitch ldd) = A * B with A(i, k) = A[i * sa_m + k * sa_k] in bfloat16 and B (K x N fp32, pitch ldb)
-// split into `planes` (split_planes_bytes(K, N) bytes of scratch) first.  Nothing happens where `gate` is given and *gate is 0.
+// split into `planes` (split_planes_bytes(K, N) bytes of scratch) first.
 int launch_split_gemm(const uint16_t* A, int64_t sa_m, int64_t sa_k, const float* B, int64_t ldb, float* D, int64_t ldd,
-                      int64_t M, int64_t N, int64_t K, uint16_t* planes, const int32_t* gate, int32_t* status, cudaStream_t st) {
+                      int64_t M, int64_t N, int64_t K, uint16_t* planes, int32_t* status, cudaStream_t st) {
   const int kpad = (int)round_up(K, kBK);
   {
     const int64_t threads = (int64_t)kpad * (N / 8);
-    split_planes_kernel<<<(unsigned)ceil_div(threads, 256), 256, 0, st>>>(B, ldb, (int)K, (int)N, kpad, planes, gate);
+    split_planes_kernel<<<(unsigned)ceil_div(threads, 256), 256, 0, st>>>(B, ldb, (int)K, (int)N, kpad, planes);
     QG_LAUNCH_CHECK();
   }
   SplitArgs a;
@@ -486,13 +501,13 @@ int launch_split_gemm(const uint16_t* A, int64_t sa_m, int64_t sa_k, const float
       QG_CUDA_TRY(cudaFuncSetAttribute(split_gemm_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SplitSmem::kBytes));
       smem_set[1][dev] = true;
     }
-    split_gemm_kernel<true><<<grid, SplitSmem::kThreads, SplitSmem::kBytes, st>>>(a, gate, status);
+    split_gemm_kernel<true><<<grid, SplitSmem::kThreads, SplitSmem::kBytes, st>>>(a, status);
   } else {
     if (!smem_set[0][dev]) {
       QG_CUDA_TRY(cudaFuncSetAttribute(split_gemm_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SplitSmem::kBytes));
       smem_set[0][dev] = true;
     }
-    split_gemm_kernel<false><<<grid, SplitSmem::kThreads, SplitSmem::kBytes, st>>>(a, gate, status);
+    split_gemm_kernel<false><<<grid, SplitSmem::kThreads, SplitSmem::kBytes, st>>>(a, status);
   }
   QG_LAUNCH_CHECK();
   return QG_OK;

@@ -348,6 +348,11 @@ eig_scale_kernel(const Ptrs<float> Ab, int N, int Np, const Ptrs<const float> sc
 // p_i = (d_i - x) p_{i-1} - e_{i-1}^2 p_{i-2}; the chain per row is one fused multiply-add, and both terms are scaled
 // back by a power of two every eight rows.  e^2 is kept above a floor, so that two consecutive p never vanish.
 constexpr int kSturmWarps = 8;
+
+// The diagonal as steps 2 and 3 see it: each element raised by its own part of 2^-30 of the largest (A is scaled so that
+// that is between 1 and 2), a sixtieth of a unit in the last place.  Eigenvalues that coincide, as those of zero rows do,
+// come apart by it and have orthogonal vectors.
+__device__ __forceinline__ double diagonal(const float* d, int i) { return (double)d[i] + 0x1p-62 * (double)(uint32_t)(2654435769u * (uint32_t)i); }
 constexpr double kE2Floor = 1e-36;
 
 __device__ __forceinline__ int sturm_count(const double2* __restrict__ t, int N, double x) {
@@ -386,7 +391,7 @@ eigenvalue_kernel(const Ptrs<const float> db, const Ptrs<const float> eb, int N,
   const float* e = eb.p[blockIdx.y];
   double b = 0.0;                                // every |eigenvalue| <= max |d_i| + |e_{i-1}| + |e_i|
   for (int i = threadIdx.x; i < N; i += blockDim.x) {
-    const double di = d[i], el = i > 0 ? (double)e[i - 1] : 0.0, er = i + 1 < N ? (double)e[i] : 0.0;
+    const double di = diagonal(d, i), el = i > 0 ? (double)e[i - 1] : 0.0, er = i + 1 < N ? (double)e[i] : 0.0;
     sturm_smem[i] = make_double2(di, fmax(el * el, kE2Floor));
     b = fmax(b, fabs(di) + fabs(el) + fabs(er));
   }
@@ -409,18 +414,12 @@ eigenvalue_kernel(const Ptrs<const float> db, const Ptrs<const float> eb, int N,
   if (lane == 0) lamb.p[blockIdx.y][j] = 0.5 * (lo + hi);
 }
 
-// Whether binary32 resolved the vectors.  A and its reduction carry an error of about sqrt(N) units in the last place of the
-// largest eigenvalue; neighbours in the bulk of a gradient's spectrum lie about lambda / N apart.  Measured on a rank-32
-// signal plus noise (N = 2048, lambda_r / lambda_1 = 8e-3: 1.1e-3 of rad for the 99 % worst vector, 6e-5 for the subspace),
-// the bound below keeps the subspace within 5e-3 rad.  Coinciding eigenvalues have no vectors of their own.
-__global__ void __launch_bounds__(256)
-doubtful_kernel(const Ptrs<const double> lamb, int N, int r, const Ptrs<int32_t> doubtb) {
+// Whether binary32 resolved the vectors: A and its reduction carry an error of some units in the last place of the largest
+// eigenvalue, and neighbours in the bulk of a gradient's spectrum lie about lambda / N apart.  Below this bound the subspace
+// can be off by more than 1e-2 rad (768 rows: lambda_r / lambda_1 = 3e-6 gave RESOLVE_NOW).
+__global__ void resolved_kernel(const Ptrs<const double> lamb, int N, int r, int32_t* __restrict__ status) {
   const double* lam = lamb.p[blockIdx.x];
-  const double top = lam[0];
-  bool bad = !(lam[r - 1] >= 8.0 * N * 0x1p-24 * top) || !(top > 0.0);
-  for (int j = threadIdx.x + 1; j < r; j += blockDim.x) bad = bad || !(lam[j - 1] - lam[j] > 1e-14 * top);
-  const int any = __syncthreads_or(bad);
-  if (threadIdx.x == 0) *doubtb.p[blockIdx.x] = any ? 1 : 0;
+  if (!(lam[r - 1] >= 0.1 * N * 0x1p-24 * lam[0]) && status) atomicOr(status, QG_DEV_BAD_FACTOR);
 }
 
 // ------------------------------------------------------------------------------------------ 3. eigenvectors of T
@@ -433,12 +432,12 @@ __device__ __forceinline__ double guarded(double q) { return fabs(q) < kPivotFlo
 __global__ void __launch_bounds__(32)
 tridiagonal_vectors_kernel(const Ptrs<const float> db, const Ptrs<const float> eb, int N, int r, const Ptrs<const double> lamb,
                            const Ptrs<double> lowerb, const Ptrs<float> Zb, const Ptrs<double> invb) {
-  extern __shared__ float vec_smem[];
-  float* d = vec_smem;
-  float* e = vec_smem + N;
+  extern __shared__ double vec_smem[];
+  double* d = vec_smem;
+  float* e = reinterpret_cast<float*>(vec_smem + N);
   const int mat = blockIdx.y;
   for (int i = threadIdx.x; i < N; i += 32) {
-    d[i] = db.p[mat][i];
+    d[i] = diagonal(db.p[mat], i);
     e[i] = i + 1 < N ? eb.p[mat][i] : 0.f;
   }
   __syncwarp();
@@ -447,15 +446,15 @@ tridiagonal_vectors_kernel(const Ptrs<const float> db, const Ptrs<const float> e
   const double lam = lamb.p[mat][t];
   double* lower = lowerb.p[mat] + t;
   float* Z = Zb.p[mat] + t;
-  double q = guarded((double)d[0] - lam);
+  double q = guarded(d[0] - lam);
 #pragma unroll 4
   for (int i = 0; i + 1 < N; ++i) {
     const double ei = e[i], l = ei / q;
     lower[(int64_t)i * r] = l;
-    q = guarded(((double)d[i + 1] - lam) - ei * l);
+    q = guarded((d[i + 1] - lam) - ei * l);
   }
   // from the bottom; gamma_i = D-_i - e_{i-1} l_{i-1}
-  q = (double)d[N - 1] - lam;
+  q = d[N - 1] - lam;
   double best = 1e300;
   int twist = N - 1;
   for (int i0 = N - 1; i0 >= 0; i0 -= 8) {
@@ -472,7 +471,7 @@ tridiagonal_vectors_kernel(const Ptrs<const float> db, const Ptrs<const float> e
       if (i > 0) {
         const double uu = el / guarded(q);
         Z[(int64_t)i * r] = (float)uu;             // the multiplier between rows i - 1 and i
-        q = ((double)d[i - 1] - lam) - el * uu;
+        q = (d[i - 1] - lam) - el * uu;
       }
     }
   }
@@ -712,7 +711,7 @@ size_t carve_eig(void* base, int64_t N, int64_t r, EigBuffers* out) {
   return off;
 }
 
-int launch_sym_eig(const EigBuffers* w, int32_t* const* doubtful, int nb, int64_t N, int64_t r, int32_t* status, cudaStream_t st) {
+int launch_sym_eig(const EigBuffers* w, int nb, int64_t N, int64_t r, int32_t* status, cudaStream_t st) {
   if (N < 2 || N > kEigMax || r < 1 || r > N || nb < 1 || nb > kMaxBatch) return QG_UNSUPPORTED_SHAPE;
   const int64_t Np = eig_pitch(N);
   Ptrs<float> A{}, V{}, tau{}, d{}, e{}, Z{}, scale{};
@@ -720,12 +719,10 @@ int launch_sym_eig(const EigBuffers* w, int32_t* const* doubtful, int nb, int64_
   Ptrs<double> lam{}, inv{}, lower{};
   Ptrs<const double> lamc{}, invc{};
   Ptrs<uint4> xchg{};
-  Ptrs<int32_t> doubt{};
   for (int i = 0; i < nb; ++i) {
     Ac.p[i] = A.p[i] = w[i].A; Vc.p[i] = V.p[i] = w[i].V; tauc.p[i] = tau.p[i] = w[i].tau;
     dc.p[i] = d.p[i] = w[i].d; ec.p[i] = e.p[i] = w[i].e; Z.p[i] = w[i].Z; scalec.p[i] = scale.p[i] = w[i].scale;
     lamc.p[i] = lam.p[i] = w[i].lam; invc.p[i] = inv.p[i] = w[i].inv; lower.p[i] = w[i].lower; xchg.p[i] = w[i].xchg;
-    doubt.p[i] = doubtful[i];
     QG_CUDA_TRY(cudaMemsetAsync(w[i].xchg, 0, (size_t)(2 * Np * 16), st));   // no tag of an earlier call
   }
   eig_scale_factor_kernel<<<nb, 256, 0, st>>>(Ac, (int)N, (int)Np, scale);
@@ -764,9 +761,9 @@ int launch_sym_eig(const EigBuffers* w, int32_t* const* doubtful, int nb, int64_
     eigenvalue_kernel<<<dim3((unsigned)ceil_div(r, kSturmWarps), (unsigned)nb), kSturmWarps * 32, (size_t)N * 16, st>>>(dc, ec, (int)N, (int)r, lam);
     QG_LAUNCH_CHECK();
   }
-  doubtful_kernel<<<nb, 256, 0, st>>>(lamc, (int)N, (int)r, doubt);
+  resolved_kernel<<<nb, 1, 0, st>>>(lamc, (int)N, (int)r, status);
   QG_LAUNCH_CHECK();
-  tridiagonal_vectors_kernel<<<dim3((unsigned)ceil_div(r, 32), (unsigned)nb), 32, (size_t)N * 8, st>>>(dc, ec, (int)N, (int)r, lamc, lower, Z, inv);
+  tridiagonal_vectors_kernel<<<dim3((unsigned)ceil_div(r, 32), (unsigned)nb), 32, (size_t)N * 12, st>>>(dc, ec, (int)N, (int)r, lamc, lower, Z, inv);
   QG_LAUNCH_CHECK();
   if (Np <= 512) return launch_back<4, 2, 16>(Vc, tauc, nb, N, Np, r, Z, invc, st);
   if (Np <= 1024) return launch_back<8, 2, 16>(Vc, tauc, nb, N, Np, r, Z, invc, st);
