@@ -416,7 +416,7 @@ eigenvalue_kernel(const Ptrs<const float> db, const Ptrs<const float> eb, int N,
 
 // Whether binary32 resolved the vectors: A and its reduction carry an error of some units in the last place of the largest
 // eigenvalue, and neighbours in the bulk of a gradient's spectrum lie about lambda / N apart.  Below this bound the subspace
-// can be off by more than 1e-2 rad (768 rows: lambda_r / lambda_1 = 3e-6 gave RESOLVE_NOW).
+// can be off by more than 1e-2 rad (768 rows: lambda_r / lambda_1 = 3e-6 gave 3.5e-2).
 __global__ void resolved_kernel(const Ptrs<const double> lamb, int N, int r, int32_t* __restrict__ status) {
   const double* lam = lamb.p[blockIdx.x];
   if (!(lam[r - 1] >= 0.1 * N * 0x1p-24 * lam[0]) && status) atomicOr(status, QG_DEV_BAD_FACTOR);

@@ -1,0 +1,68 @@
+"""The direct route of the subspace refresh where its kernels change: the row counts at which the tridiagonal reduction and
+the back-transformation take another instance, a batch that is reduced in several launches, vectors on the long side,
+odd extents, and gradients whose eigenvalues coincide."""
+import pytest
+import torch
+
+from paper_2407_08296_b200 import binding as B
+
+pytestmark = pytest.mark.gpu
+
+
+def _gradient(m, n, seed):
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(seed)
+    k = 16
+    u = torch.randn(m, k, device="cuda", generator=gen) / m ** 0.5 / torch.arange(1, k + 1, device="cuda")
+    v = torch.randn(n, k, device="cuda", generator=gen) / n ** 0.5
+    G = B.zeros_matrix(m, n, torch.bfloat16)
+    G.copy_(u @ v.T + 1e-3 * torch.randn(m, n, device="cuda", generator=gen))
+    return G
+
+
+def _check(G, P, side):
+    """Backward error: P holds the leading eigenvectors of a matrix within s * 2^-24 * lambda_1 (s the short side: the
+    first-order bound of a Householder reduction in binary32, which also covers the sums of the Gram matrix) of G G^T."""
+    X = G.double() if side == "left" else G.double().T
+    A, Z = X @ X.T, P.double()
+    s, r = min(G.shape), P.shape[1]
+    lam = torch.linalg.eigvalsh(A if A.shape[0] == s else X.T @ X).flip(0)
+    eps = s * 2.0 ** -24
+    assert float((Z.T @ Z - torch.eye(r, device="cuda")).abs().max()) <= max(eps, 1e-5)
+    q = (Z * (A @ Z)).sum(0)
+    assert float((A @ Z - Z * q).norm(dim=0).max()) <= eps * float(lam[0])
+    assert float((q - lam[:r]).abs().max()) <= eps * float(lam[0])
+    assert bool((Z.gather(0, Z.abs().argmax(0, keepdim=True)) > 0).all())
+
+
+@pytest.mark.parametrize("m,n,r,side", [(64, 700, 32, "left"), (130, 128, 32, "left"), (511, 640, 64, "left"), (513, 1025, 128, "left"),
+                                        (1025, 1030, 160, "right"), (1100, 769, 96, "left"), (2049, 2100, 288, "left"), (2500, 2047, 256, "left")])
+def test_vectors_are_those_of_a_nearby_matrix(m, n, r, side):
+    G = _gradient(m, n, seed=m)
+    P = torch.zeros((m if side == "left" else n, r), device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    B.refresh_subspace(G, r, P_fp32=P, status=status, side=side)
+    assert int(status.item()) == 0
+    _check(G, P, side)
+
+
+def test_a_batch_reduced_in_several_launches():
+    m, n, r = 1400, 1600, 352               # eight matrices do not fit the SMs at once
+    items = [{"G": _gradient(m, n, seed=i), "seed": i, "P_fp32": torch.zeros((m, r), device="cuda")} for i in range(8)]
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    B.refresh_subspace_batched(items, r, status=status)
+    assert int(status.item()) == 0
+    for it in (items[0], items[5], items[7]):
+        _check(it["G"], it["P_fp32"], "left")
+
+
+@pytest.mark.parametrize("kind", ["zero", "identity", "zero_rows"])
+def test_coinciding_eigenvalues_have_orthogonal_vectors(kind):
+    G = B.zeros_matrix(256, 384, torch.bfloat16)
+    if kind == "identity":
+        G.copy_(torch.eye(256, 384))
+    elif kind == "zero_rows":
+        G[::5].copy_(torch.randn(52, 384))
+    P = torch.zeros((256, 64), device="cuda")
+    B.refresh_subspace(G, 64, P_fp32=P)
+    assert float((P.T @ P - torch.eye(64, device="cuda")).abs().max()) <= 1e-5
