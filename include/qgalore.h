@@ -61,7 +61,8 @@ typedef enum {
 /* flags OR-ed into the optional device status word */
 #define QG_DEV_WAIT_EXPIRED 1   /* a bounded barrier wait ran out; the tile was abandoned */
 #define QG_DEV_NOT_CONVERGED 2  /* eigen-iteration of the refresh hit its sweep limit     */
-#define QG_DEV_BAD_FACTOR 4     /* Cholesky factor of the refresh met a non-positive pivot */
+#define QG_DEV_BAD_FACTOR 4     /* refresh: the gradient's r-th singular value is so small against the first that its
+                                   vector is lost in rounding (or a Cholesky factor met a non-positive pivot)   */
 
 /* A block-wise quantized matrix (Sec. 3.1; App. A: W = (codes - zeros) * scales). */
 typedef struct {
@@ -211,10 +212,13 @@ QG_API int qgalore_plan_step_timed(const qg_plan* plan, const qg_hyper* h, int32
                             float* kernel_ms, int32_t* kernel_launches);
 
 /* --- Sec. 3.5 "obtain the projection matrix using SVD" + Sec. 3.3 INT4 storage ------------
- * Top-r left singular vectors of G (bf16, m x n, pitch ldg) by block subspace iteration on G G^T with a
- * block of b = r + oversample_cols columns (`iters` multiplications by G G^T, each followed by a block
- * Gram-Schmidt orthonormalisation) and a Rayleigh-Ritz step (eigenvectors of the projected b x b matrix by
- * a Jacobi iteration on binary32 rows with binary64 sums), then Quant_4 into P_new.  Each column carries the sign that makes its
+ * Top-r left singular vectors of G (bf16, m x n, pitch ldg), then Quant_4 into P_new.  Where the short side s = min(m, n)
+ * has at most 4096 rows and s <= 8 b, b = r + oversample_cols: the r leading eigenvectors of the Gram matrix of the short
+ * side (tridiagonal reduction in binary32, eigenvalues and their vectors in binary64), and G times them for vectors on the
+ * long side; iters and seed do not enter.  Else: block subspace iteration on G G^T with a block of b columns (`iters`
+ * multiplications by G G^T, each followed by a block Gram-Schmidt orthonormalisation) and a Rayleigh-Ritz step
+ * (eigenvectors of the projected b x b matrix by a Jacobi iteration on binary32 rows with binary64 sums), the random start
+ * block drawn from Philox keyed by `seed`.  Each column carries the sign that makes its
  * largest-magnitude entry positive.
  *   P_new      INT4, m x r, ld == r; written
  *   P_fp32     optional (may be NULL): m x r fp32, pitch r, receives the vectors before quantization
@@ -223,8 +227,7 @@ QG_API int qgalore_plan_step_timed(const qg_plan* plan, const qg_hyper* h, int32
  *   workspace  qgalore_workspace_bytes(QG_OP_REFRESH, m, n, b) bytes, 256-byte aligned
  *   status_dev optional; receives QG_DEV_NOT_CONVERGED / QG_DEV_BAD_FACTOR
  * Shape rules: r % 32 == 0, b % 64 == 0, b <= min(m, n), b <= 4096.  Typical use: b = 2 r, iters = 12.
- * The Adam moments and the step count are not touched.  The random start block is drawn from Philox
- * keyed by `seed`. */
+ * The Adam moments and the step count are not touched. */
 QG_API int qgalore_refresh_subspace(const uint16_t* G, int64_t ldg, int64_t m, int64_t n, int64_t r,
                              int32_t iters, int32_t oversample_cols, uint64_t seed,
                              const qg_qtensor* P_new, float* P_fp32,
@@ -243,8 +246,8 @@ QG_API int qgalore_refresh_subspace_right(const uint16_t* G, int64_t ldg, int64_
 
 /* --- Sec. 3.5, the refresh of several matrices of ONE shape in one call (with a fixed interval every matrix of a
  * stack is due in the same step; under the adaptive schedule of Sec. 3.2, those whose interval has run out).
- * The matrices are refreshed in batches: every kernel launch, and every grid barrier of the eigen-iteration,
- * serves all matrices of a batch, so that a stack costs far less than its matrices one after the other.
+ * The matrices are refreshed in batches: every kernel launch serves all matrices of a batch, so that a stack costs far
+ * less than its matrices one after the other.
  *   items      HOST; per matrix: the gradient and its pitch, the seed of its start block, where the new
  *              projection goes (P_new, ld == r) and optionally the fp32 vectors (P_fp32), the previous projection
  *              (P_prev, may be NULL) and the device word that receives the similarity to it (sim_dev, may be NULL)
@@ -357,9 +360,10 @@ QG_API int qgalore_debug_set_fused_dequant(int on);
 /* 1 (the default): the early iterations of a refresh take their two products with the gradient on the tensor cores
  * (the iterate split into three bfloat16 planes); 0: every product on the CUDA cores. */
 QG_API int qgalore_debug_set_refresh_tensor_cores(int on);
-/* 1 (the default): the eigen-iteration of a refresh handles the rows of the projected matrix in blocks of eight
- * kept in shared memory and registers (block widths up to 2048); 0: row by row through L2, the form wider blocks
- * take.  Applies to calls made afterwards; both meet the same accuracy bound, their results differ in the last bits. */
+/* 1 (the default): a refresh takes the direct route where the shape allows it, and the eigen-iteration of the iterative
+ * route handles the rows of the projected matrix in blocks of eight kept in shared memory and registers (block widths up
+ * to 2048); 0: the iterative route for every shape, row by row through L2, the form wider blocks take.  Applies to calls
+ * made afterwards; all meet the same accuracy bound. */
 QG_API int qgalore_debug_set_jacobi_blocks(int on);
 /* Scratch bytes a chunk of a plan may use (plans created afterwards; at least 1 MiB).  Larger chunks mean
  * fewer, longer launches; smaller ones keep the bf16 direction between the two kernels inside L2. */
