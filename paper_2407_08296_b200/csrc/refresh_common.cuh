@@ -32,8 +32,8 @@ struct EigBuffers {
   float *tau, *d, *e;  // N floats each: the reflectors' factors, the tridiagonal matrix
   float* scale;        // the power of two A is scaled by
   double *lam, *inv;   // r doubles each: the leading eigenvalues (of the scaled matrix), 1 / norm of the vectors of step 3
-  double* lower;       // N x r doubles: multipliers of the forward factorisation
-  float* Z;            // N x r (pitch r): backward multipliers, eigenvectors of the tridiagonal matrix, then of A
+  double *plus, *minus;  // N x r doubles each: pivots of the two factorisations of step 3
+  float* Z;            // N x r (pitch r): eigenvectors of the tridiagonal matrix, then of A
   uint4* xchg;         // 2 x eig_pitch(N): exchange between the CTAs of a matrix
 };
 size_t carve_eig(void* base, int64_t N, int64_t r, EigBuffers* out);

@@ -423,95 +423,97 @@ __global__ void resolved_kernel(const Ptrs<const double> lamb, int N, int r, int
 }
 
 // ------------------------------------------------------------------------------------------ 3. eigenvectors of T
-// One thread per eigenvalue: T - lambda = L D+ L^T from the top and U D- U^T from the bottom; where
-// gamma_i = d_i - lambda - e_{i-1} l_{i-1} - e_i u_i is smallest the two factorisations are joined, and the vector follows
-// outward from that row by products of multipliers alone, without cancellation.
+// T - lambda = L D+ L^T from the top and U D- U^T from the bottom; where gamma_i = D+_i + D-_i - (d_i - lambda) is smallest
+// the two factorisations are joined, and the vector follows outward from that row by products of multipliers alone, without
+// cancellation.  Bound: the chain of binary64 divisions, so a pair of threads takes an eigenvalue, one from each end (warp 0
+// and warp 1 of a CTA): 768 rows 320 -> 298 us.
 constexpr double kPivotFloor = 1e-280;
 __device__ __forceinline__ double guarded(double q) { return fabs(q) < kPivotFloor ? copysign(kPivotFloor, q) : q; }
 
-__global__ void __launch_bounds__(32)
+__global__ void __launch_bounds__(64)
 tridiagonal_vectors_kernel(const Ptrs<const float> db, const Ptrs<const float> eb, int N, int r, const Ptrs<const double> lamb,
-                           const Ptrs<double> lowerb, const Ptrs<float> Zb, const Ptrs<double> invb) {
+                           const Ptrs<double> plusb, const Ptrs<double> minusb, const Ptrs<float> Zb, const Ptrs<double> invb) {
   extern __shared__ double vec_smem[];
+  __shared__ double s_best[2][32], s_sum[32];
+  __shared__ int s_at[2][32];
   double* d = vec_smem;
   float* e = reinterpret_cast<float*>(vec_smem + N);
-  const int mat = blockIdx.y;
-  for (int i = threadIdx.x; i < N; i += 32) {
+  const int mat = blockIdx.y, lane = threadIdx.x & 31, side = threadIdx.x >> 5;
+  for (int i = threadIdx.x; i < N; i += 64) {
     d[i] = diagonal(db.p[mat], i);
     e[i] = i + 1 < N ? eb.p[mat][i] : 0.f;
   }
-  __syncwarp();
-  const int t = blockIdx.x * 32 + threadIdx.x;
-  if (t >= r) return;
-  const double lam = lamb.p[mat][t];
-  double* lower = lowerb.p[mat] + t;
-  float* Z = Zb.p[mat] + t;
-  double q = guarded(d[0] - lam);
+  __syncthreads();
+  const int t = blockIdx.x * 32 + lane;
+  const bool live = t < r;
+  const double lam = live ? lamb.p[mat][t] : 0.0;
+  double* plus = plusb.p[mat] + min(t, r - 1);      // D+_i, D-_i
+  double* minus = minusb.p[mat] + min(t, r - 1);
+  if (live && side == 0) {
+    double q = guarded(d[0] - lam);
+    plus[0] = q;
 #pragma unroll 4
-  for (int i = 0; i + 1 < N; ++i) {
-    const double ei = e[i], l = ei / q;
-    lower[(int64_t)i * r] = l;
-    q = guarded((d[i + 1] - lam) - ei * l);
-  }
-  // from the bottom; gamma_i = D-_i - e_{i-1} l_{i-1}
-  q = d[N - 1] - lam;
-  double best = 1e300;
-  int twist = N - 1;
-  for (int i0 = N - 1; i0 >= 0; i0 -= 8) {
-    double lb[8];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) lb[u] = i0 - u > 0 ? lower[(int64_t)(i0 - u - 1) * r] : 0.0;
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      const int i = i0 - u;
-      if (i < 0) break;
-      const double el = i > 0 ? (double)e[i - 1] : 0.0;
-      const double gamma = fabs(q - el * lb[u]);
-      if (gamma < best) { best = gamma; twist = i; }
-      if (i > 0) {
-        const double uu = el / guarded(q);
-        Z[(int64_t)i * r] = (float)uu;             // the multiplier between rows i - 1 and i
-        q = (d[i - 1] - lam) - el * uu;
-      }
+    for (int i = 1; i < N; ++i) {
+      const double ei = e[i - 1];
+      q = guarded((d[i] - lam) - ei * (ei / q));
+      plus[(int64_t)i * r] = q;
+    }
+  } else if (live) {
+    double q = guarded(d[N - 1] - lam);
+    minus[(int64_t)(N - 1) * r] = q;
+#pragma unroll 4
+    for (int i = N - 2; i >= 0; --i) {
+      const double ei = e[i];
+      q = guarded((d[i] - lam) - ei * (ei / q));
+      minus[(int64_t)i * r] = q;
     }
   }
-  double z = 1.0, sum = 1.0;
-  for (int i0 = N - 2; i0 >= 0; i0 -= 8) {
-    double lb[8];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) lb[u] = i0 - u >= 0 ? lower[(int64_t)(i0 - u) * r] : 0.0;
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      const int i = i0 - u;
-      if (i >= 0 && i < twist) {
-        z *= -lb[u];
-        sum = fma(z, z, sum);
-        Z[(int64_t)i * r] = (float)z;
+  __syncthreads();
+  // the row with the smallest gamma: each thread looks through half of them
+  {
+    double best = 1e300;
+    int at = 0;
+    const int i0 = side * (N / 2), i1 = side ? N : N / 2;
+    if (live)
+#pragma unroll 8
+      for (int i = i0; i < i1; ++i) {
+        const double gamma = fabs(plus[(int64_t)i * r] + (minus[(int64_t)i * r] - (d[i] - lam)));
+        if (gamma < best) { best = gamma; at = i; }
       }
+    s_best[side][lane] = best;
+    s_at[side][lane] = at;
+  }
+  __syncthreads();
+  const int twist = s_best[1][lane] < s_best[0][lane] ? s_at[1][lane] : s_at[0][lane];
+  float* Z = Zb.p[mat] + min(t, r - 1);
+  double z = 1.0, sum = 0.0;
+  if (live && side == 0) {                          // z_i = -(e_i / D+_i) z_{i+1} above the twist
+#pragma unroll 4
+    for (int i = twist - 1; i >= 0; --i) {
+      z *= -((double)e[i] / plus[(int64_t)i * r]);
+      sum = fma(z, z, sum);
+      Z[(int64_t)i * r] = (float)z;
+    }
+    Z[(int64_t)twist * r] = 1.f;
+    s_sum[lane] = sum + 1.0;
+  } else if (live) {                                // z_i = -(e_{i-1} / D-_i) z_{i-1} below
+#pragma unroll 4
+    for (int i = twist + 1; i < N; ++i) {
+      z *= -((double)e[i - 1] / minus[(int64_t)i * r]);
+      sum = fma(z, z, sum);
+      Z[(int64_t)i * r] = (float)z;
     }
   }
-  z = 1.0;
-  for (int i0 = 1; i0 < N; i0 += 8) {
-    float ub[8];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) ub[u] = i0 + u < N ? Z[(int64_t)(i0 + u) * r] : 0.f;
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      const int i = i0 + u;
-      if (i < N && i > twist) {
-        z *= -(double)ub[u];
-        sum = fma(z, z, sum);
-        Z[(int64_t)i * r] = (float)z;
-      }
-    }
-  }
-  Z[(int64_t)twist * r] = 1.f;
-  invb.p[mat][t] = 1.0 / sqrt(sum);
+  __syncthreads();
+  if (live && side == 1) invb.p[mat][t] = 1.0 / sqrt(s_sum[lane] + sum);
 }
 
 // ------------------------------------------------------------------------------------------ 4. X = H Z
 // A warp keeps VW vectors in registers (lane: rows 128 c + 4 lane .. + 3) and runs through all Householder vectors, the
-// last first; the CTA's warps share each of them from a ring in shared memory that is filled four steps ahead.
+// last first; the CTA's warps share each of them from a ring in shared memory that is filled four steps ahead.  Bound: the
+// chain of one dot product and one update per reflector where there are few vectors (so few warps per CTA, more CTAs), and
+// else shared-memory reads of the reflector (so two vectors per warp, and one read for dot product and update).
+// 768 rows, 256 vectors 605 -> 242 us; 2048 rows, eight times 512 vectors 4180 -> 4090.
 constexpr int kBackStages = 4;
 
 __device__ __forceinline__ void cp_async_16(void* smem_dst, const void* gsrc) {
@@ -576,31 +578,35 @@ back_transform_kernel(const Ptrs<const float> Vb, const Ptrs<const float> taub, 
     fetch(k - (kBackStages - 1));
     const float* v = ring + (k % kBackStages) * Np;
     const int c0 = (k + 1) / 128;
-    float s[VW];
+    constexpr bool kKeep = NCH * 4 * (VW + 1) <= 200;       // the reflector fits the registers beside the vectors
+    float4 vk[kKeep ? NCH : 1];
+    float s[VW][2];
 #pragma unroll
-    for (int u = 0; u < VW; ++u) s[u] = 0.f;
+    for (int u = 0; u < VW; ++u) s[u][0] = s[u][1] = 0.f;
 #pragma unroll
     for (int ch = 0; ch < NCH; ++ch) {
       if (ch >= c0 && ch < chunks) {
         const float4 v4 = *reinterpret_cast<const float4*>(v + ch * 128 + lane * 4);
+        if (kKeep) vk[kKeep ? ch : 0] = v4;
 #pragma unroll
         for (int u = 0; u < VW; ++u)
-          s[u] = fmaf(v4.x, x[u][ch].x, fmaf(v4.y, x[u][ch].y, fmaf(v4.z, x[u][ch].z, fmaf(v4.w, x[u][ch].w, s[u]))));
+          s[u][ch & 1] = fmaf(v4.x, x[u][ch].x, fmaf(v4.y, x[u][ch].y, fmaf(v4.z, x[u][ch].z, fmaf(v4.w, x[u][ch].w, s[u][ch & 1]))));
       }
     }
     const float tk = taus[k];
+    float f[VW];
 #pragma unroll
-    for (int u = 0; u < VW; ++u) s[u] = -tk * warp_sum(s[u]);
+    for (int u = 0; u < VW; ++u) f[u] = -tk * warp_sum(s[u][0] + s[u][1]);
 #pragma unroll
     for (int ch = 0; ch < NCH; ++ch) {
       if (ch >= c0 && ch < chunks) {
-        const float4 v4 = *reinterpret_cast<const float4*>(v + ch * 128 + lane * 4);
+        const float4 v4 = kKeep ? vk[kKeep ? ch : 0] : *reinterpret_cast<const float4*>(v + ch * 128 + lane * 4);
 #pragma unroll
         for (int u = 0; u < VW; ++u) {
-          x[u][ch].x = fmaf(s[u], v4.x, x[u][ch].x);
-          x[u][ch].y = fmaf(s[u], v4.y, x[u][ch].y);
-          x[u][ch].z = fmaf(s[u], v4.z, x[u][ch].z);
-          x[u][ch].w = fmaf(s[u], v4.w, x[u][ch].w);
+          x[u][ch].x = fmaf(f[u], v4.x, x[u][ch].x);
+          x[u][ch].y = fmaf(f[u], v4.y, x[u][ch].y);
+          x[u][ch].z = fmaf(f[u], v4.z, x[u][ch].z);
+          x[u][ch].w = fmaf(f[u], v4.w, x[u][ch].w);
         }
       }
     }
@@ -704,7 +710,8 @@ size_t carve_eig(void* base, int64_t N, int64_t r, EigBuffers* out) {
   w.scale = (float*)take(4);
   w.lam = (double*)take((size_t)(r * 8));
   w.inv = (double*)take((size_t)(r * 8));
-  w.lower = (double*)take((size_t)(N * r * 8));
+  w.plus = (double*)take((size_t)(N * r * 8));
+  w.minus = (double*)take((size_t)(N * r * 8));
   w.Z = (float*)take((size_t)(N * r * 4));
   w.xchg = (uint4*)take((size_t)(2 * Np * 16));
   if (out) *out = w;
@@ -716,13 +723,13 @@ int launch_sym_eig(const EigBuffers* w, int nb, int64_t N, int64_t r, int32_t* s
   const int64_t Np = eig_pitch(N);
   Ptrs<float> A{}, V{}, tau{}, d{}, e{}, Z{}, scale{};
   Ptrs<const float> Ac{}, Vc{}, tauc{}, dc{}, ec{}, scalec{};
-  Ptrs<double> lam{}, inv{}, lower{};
+  Ptrs<double> lam{}, inv{}, plus{}, minus{};
   Ptrs<const double> lamc{}, invc{};
   Ptrs<uint4> xchg{};
   for (int i = 0; i < nb; ++i) {
     Ac.p[i] = A.p[i] = w[i].A; Vc.p[i] = V.p[i] = w[i].V; tauc.p[i] = tau.p[i] = w[i].tau;
     dc.p[i] = d.p[i] = w[i].d; ec.p[i] = e.p[i] = w[i].e; Z.p[i] = w[i].Z; scalec.p[i] = scale.p[i] = w[i].scale;
-    lamc.p[i] = lam.p[i] = w[i].lam; invc.p[i] = inv.p[i] = w[i].inv; lower.p[i] = w[i].lower; xchg.p[i] = w[i].xchg;
+    lamc.p[i] = lam.p[i] = w[i].lam; invc.p[i] = inv.p[i] = w[i].inv; plus.p[i] = w[i].plus; minus.p[i] = w[i].minus; xchg.p[i] = w[i].xchg;
     QG_CUDA_TRY(cudaMemsetAsync(w[i].xchg, 0, (size_t)(2 * Np * 16), st));   // no tag of an earlier call
   }
   eig_scale_factor_kernel<<<nb, 256, 0, st>>>(Ac, (int)N, (int)Np, scale);
@@ -763,11 +770,18 @@ int launch_sym_eig(const EigBuffers* w, int nb, int64_t N, int64_t r, int32_t* s
   }
   resolved_kernel<<<nb, 1, 0, st>>>(lamc, (int)N, (int)r, status);
   QG_LAUNCH_CHECK();
-  tridiagonal_vectors_kernel<<<dim3((unsigned)ceil_div(r, 32), (unsigned)nb), 32, (size_t)N * 12, st>>>(dc, ec, (int)N, (int)r, lamc, lower, Z, inv);
+  {
+    static bool done[kDevices] = {};
+    const int rc = opt_in(tridiagonal_vectors_kernel, (int)kEigMax * 12, done);
+    if (rc != QG_OK) return rc;
+  }
+  tridiagonal_vectors_kernel<<<dim3((unsigned)ceil_div(r, 32), (unsigned)nb), 64, (size_t)N * 12, st>>>(dc, ec, (int)N, (int)r, lamc, plus, minus, Z, inv);
   QG_LAUNCH_CHECK();
-  if (Np <= 512) return launch_back<4, 2, 16>(Vc, tauc, nb, N, Np, r, Z, invc, st);
-  if (Np <= 1024) return launch_back<8, 2, 16>(Vc, tauc, nb, N, Np, r, Z, invc, st);
-  if (Np <= 2048) return launch_back<16, 1, 16>(Vc, tauc, nb, N, Np, r, Z, invc, st);
+  const bool few = nb * r <= 4 * sms;                // a CTA of two warps per SM
+  if (Np <= 512) return few ? launch_back<4, 1, 2>(Vc, tauc, nb, N, Np, r, Z, invc, st) : launch_back<4, 2, 8>(Vc, tauc, nb, N, Np, r, Z, invc, st);
+  if (Np <= 768) return few ? launch_back<6, 1, 2>(Vc, tauc, nb, N, Np, r, Z, invc, st) : launch_back<6, 2, 8>(Vc, tauc, nb, N, Np, r, Z, invc, st);
+  if (Np <= 1024) return few ? launch_back<8, 1, 2>(Vc, tauc, nb, N, Np, r, Z, invc, st) : launch_back<8, 2, 8>(Vc, tauc, nb, N, Np, r, Z, invc, st);
+  if (Np <= 2048) return few ? launch_back<16, 1, 4>(Vc, tauc, nb, N, Np, r, Z, invc, st) : launch_back<16, 2, 8>(Vc, tauc, nb, N, Np, r, Z, invc, st);
   return launch_back<32, 1, 8>(Vc, tauc, nb, N, Np, r, Z, invc, st);
 }
 
