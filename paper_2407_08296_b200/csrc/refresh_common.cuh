@@ -30,6 +30,7 @@ struct EigBuffers {
   float* A;            // N rows of eig_pitch(N) floats, symmetric: the matrix, destroyed
   float* V;            // same extents: row k holds Householder vector v_k
   float *tau, *d, *e;  // N floats each: the reflectors' factors, the tridiagonal matrix
+  float* cross;        // N floats: v_k . v_{k-1}
   float* scale;        // the power of two A is scaled by
   double *lam, *inv;   // r doubles each: the leading eigenvalues (of the scaled matrix), 1 / norm of the vectors of step 3
   double *plus, *minus;  // N x r doubles each: pivots of the two factorisations of step 3

@@ -483,16 +483,27 @@ tridiagonal_vectors_kernel(const Ptrs<const float> db, const Ptrs<const float> e
     }
   }
   __syncthreads();
-  // the row with the smallest gamma: each thread looks through half of them
+  // the row with the smallest gamma: each thread looks through half of them (loads in batches: they come from L2)
+  constexpr int kBatch = 16;
   {
     double best = 1e300;
     int at = 0;
     const int i0 = side * (N / 2), i1 = side ? N : N / 2;
     if (live)
-#pragma unroll 8
-      for (int i = i0; i < i1; ++i) {
-        const double gamma = fabs(plus[(int64_t)i * r] + (minus[(int64_t)i * r] - (d[i] - lam)));
-        if (gamma < best) { best = gamma; at = i; }
+      for (int b = i0; b < i1; b += kBatch) {
+        double p[kBatch], m[kBatch];
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u) {
+          const int64_t i = min(b + u, N - 1);
+          p[u] = plus[i * r];
+          m[u] = minus[i * r];
+        }
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u) {
+          if (b + u >= i1) break;
+          const double gamma = fabs(p[u] + (m[u] - (d[b + u] - lam)));
+          if (gamma < best) { best = gamma; at = b + u; }
+        }
       }
     s_best[side][lane] = best;
     s_at[side][lane] = at;
@@ -502,20 +513,36 @@ tridiagonal_vectors_kernel(const Ptrs<const float> db, const Ptrs<const float> e
   float* Z = Zb.p[mat] + min(t, r - 1);
   double z = 1.0, sum = 0.0;
   if (live && side == 0) {                          // z_i = -(e_i / D+_i) z_{i+1} above the twist
-#pragma unroll 4
-    for (int i = twist - 1; i >= 0; --i) {
-      z *= -((double)e[i] / plus[(int64_t)i * r]);
-      sum = fma(z, z, sum);
-      Z[(int64_t)i * r] = (float)z;
+    for (int b = twist - 1; b >= 0; b -= kBatch) {
+      double l[kBatch];
+#pragma unroll
+      for (int u = 0; u < kBatch; ++u) { const int64_t i = max(b - u, 0); l[u] = plus[i * r]; }
+#pragma unroll
+      for (int u = 0; u < kBatch; ++u) l[u] = (double)e[max(b - u, 0)] / l[u];
+#pragma unroll
+      for (int u = 0; u < kBatch; ++u) {
+        if (b - u < 0) break;
+        z *= -l[u];
+        sum = fma(z, z, sum);
+        Z[(int64_t)(b - u) * r] = (float)z;
+      }
     }
     Z[(int64_t)twist * r] = 1.f;
     s_sum[lane] = sum + 1.0;
   } else if (live) {                                // z_i = -(e_{i-1} / D-_i) z_{i-1} below
-#pragma unroll 4
-    for (int i = twist + 1; i < N; ++i) {
-      z *= -((double)e[i - 1] / minus[(int64_t)i * r]);
-      sum = fma(z, z, sum);
-      Z[(int64_t)i * r] = (float)z;
+    for (int b = twist + 1; b < N; b += kBatch) {
+      double l[kBatch];
+#pragma unroll
+      for (int u = 0; u < kBatch; ++u) { const int64_t i = min(b + u, N - 1); l[u] = minus[i * r]; }
+#pragma unroll
+      for (int u = 0; u < kBatch; ++u) l[u] = (double)e[min(b + u, N - 1) - 1] / l[u];
+#pragma unroll
+      for (int u = 0; u < kBatch; ++u) {
+        if (b + u >= N) break;
+        z *= -l[u];
+        sum = fma(z, z, sum);
+        Z[(int64_t)(b + u) * r] = (float)z;
+      }
     }
   }
   __syncthreads();
@@ -524,44 +551,77 @@ tridiagonal_vectors_kernel(const Ptrs<const float> db, const Ptrs<const float> e
 
 // ------------------------------------------------------------------------------------------ 4. X = H Z
 // A warp keeps VW vectors in registers (lane: rows 128 c + 4 lane .. + 3) and runs through all Householder vectors, the
-// last first; the CTA's warps share each of them from a ring in shared memory that is filled four steps ahead.  Bound: the
-// chain of one dot product and one update per reflector where there are few vectors (so few warps per CTA, more CTAs), and
-// else shared-memory reads of the reflector (so two vectors per warp, and one read for dot product and update).
+// last first; the CTA's warps share them from a ring in shared memory that is filled several pairs ahead.  Bound: the chain of
+// dot product and update.  So the reflectors are applied two at a time, with one reduction for both,
+//     s_k = v_k . x,  s_{k-1} = v_{k-1} . x - tau_k s_k (v_{k-1} . v_k),  x <- x - tau_k s_k v_k - tau_{k-1} s_{k-1} v_{k-1},
+// and few vectors are spread over many CTAs of two warps.
 // 768 rows, 256 vectors 605 -> 242 us; 2048 rows, eight times 512 vectors 4180 -> 4090.
-constexpr int kBackStages = 4;
+constexpr int back_stages(int nch) { return nch <= 16 ? 6 : 4; }   // pairs of reflectors in the ring
 
-__device__ __forceinline__ void cp_async_16(void* smem_dst, const void* gsrc) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(smem_dst)), "l"(gsrc) : "memory");
+// `bytes` (a multiple of 16) consecutive bytes to shared memory by the copy engine.
+__device__ __forceinline__ void bulk_load(void* smem_dst, const void* gsrc, uint32_t bytes, uint64_t* bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(ptx::smem_u32(smem_dst)), "l"(gsrc),
+               "r"(bytes), "r"(ptx::smem_u32(bar))
+               : "memory");
 }
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+// cross_k = v_k . v_{k-1} for k = N - 1, N - 3, ... (v_{N-1} counts as zero): a warp each
+__global__ void __launch_bounds__(128)
+reflector_pairs_kernel(const Ptrs<const float> Vb, int N, int Np, const Ptrs<float> crossb) {
+  const int k = N - 1 - 2 * (int)(blockIdx.x * 4 + (threadIdx.x >> 5)), lane = threadIdx.x & 31;
+  if (k < 1) return;
+  const float* v = Vb.p[blockIdx.y] + (int64_t)k * Np;
+  float s = 0.f;
+  if (k < N - 1)
+    for (int i = (k + 1) / 4 * 4 + 4 * lane; i < Np; i += 128) {
+      const float4 x = *reinterpret_cast<const float4*>(v + i), y = *reinterpret_cast<const float4*>(v - Np + i);
+      s = fmaf(x.x, y.x, fmaf(x.y, y.y, fmaf(x.z, y.z, fmaf(x.w, y.w, s))));
+    }
+  s = warp_sum(s);
+  if (lane == 0) crossb.p[blockIdx.y][k] = s;
+}
 
 template <int NCH, int VW, int WARPS>
 __global__ void __launch_bounds__(WARPS * 32, 1)
-back_transform_kernel(const Ptrs<const float> Vb, const Ptrs<const float> taub, int N, int Np, int r, const Ptrs<float> Zb,
-                      const Ptrs<const double> invb) {
+back_transform_kernel(const Ptrs<const float> Vb, const Ptrs<const float> taub, const Ptrs<const float> crossb, int N, int Np, int r,
+                      const Ptrs<float> Zb, const Ptrs<const double> invb, int32_t* __restrict__ status) {
   extern __shared__ __align__(16) float back_smem[];
+  constexpr int kBackStages = back_stages(NCH);
+  __shared__ __align__(8) uint64_t landed[kBackStages];
   constexpr int kW = WARPS * VW, kThreads = WARPS * 32;   // vectors and threads of this CTA
-  float* ring = back_smem;                          // [kBackStages][Np]
-  float* tile = ring + kBackStages * Np;            // [128][kW + 1]
+  float* ring = back_smem;                          // [kBackStages][2][Np]
+  float* tile = ring + 2 * kBackStages * Np;        // [128][kW + 1]
   float* taus = tile + 128 * (kW + 1);              // [N]
+  float* cross = taus + N;                          // [N]
   const int mat = blockIdx.y, t0 = blockIdx.x * kW;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const float* V = Vb.p[mat];
   float* Z = Zb.p[mat];
   const int chunks = Np / 128;
-  for (int i = tid; i < N; i += kThreads) taus[i] = i + 1 < N ? taub.p[mat][i] : 0.f;
+  for (int i = tid; i < N; i += kThreads) {
+    taus[i] = i + 1 < N ? taub.p[mat][i] : 0.f;
+    cross[i] = crossb.p[mat][i];
+  }
 
-  auto fetch = [&](int k) {                         // rows k + 1 .. of Householder vector k, whole chunks
-    if (k >= 0) {
-      const float* src = V + (int64_t)k * Np;
-      float* dst = ring + (k % kBackStages) * Np;
-      for (int i = (k + 1) / 128 * 128 + tid * 4; i < Np; i += kThreads * 4) cp_async_16(dst + i, src + i);
-    }
-    cp_async_commit();
+  if (tid == 0) {
+    for (int i = 0; i < kBackStages; ++i) ptx::mbar_init(&landed[i], 1);
+    ptx::fence_mbar_init();
+  }
+  auto fetch = [&](int step) {                      // one thread: reflectors k = N - 1 - 2 step and k - 1, rows k .. on in whole chunks
+    const int k = N - 1 - 2 * step;
+    if (tid != 0 || k < 0) return;
+    uint64_t* bar = &landed[step % kBackStages];
+    float* dst = ring + (step % kBackStages) * 2 * Np;
+    const float* src = V + (int64_t)k * Np;
+    const int i = k / 128 * 128;
+    const uint32_t bytes = (uint32_t)(Np - i) * 4u;
+    ptx::fence_proxy_async_smem();
+    ptx::mbar_arrive_expect_tx(bar, k > 0 ? 2 * bytes : bytes);
+    bulk_load(dst + i, src + i, bytes, bar);
+    if (k > 0) bulk_load(dst + Np + i, src - Np + i, bytes, bar);
   };
-  for (int s = 0; s < kBackStages - 1; ++s) fetch(N - 2 - s);
+  __syncthreads();
+  for (int s = 0; s < kBackStages - 1; ++s) fetch(s);
 
   float inv[VW];
 #pragma unroll
@@ -586,41 +646,56 @@ back_transform_kernel(const Ptrs<const float> Vb, const Ptrs<const float> taub, 
       for (int u = 0; u < VW; ++u) x[u][ch] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
   }
-  for (int k = N - 2; k >= 0; --k) {
-    cp_async_wait<kBackStages - 2>();
-    __syncthreads();                                // vector k has landed; everybody is done with the slot refilled now
-    fetch(k - (kBackStages - 1));
-    const float* v = ring + (k % kBackStages) * Np;
-    const int c0 = (k + 1) / 128;
-    constexpr bool kKeep = NCH * 4 * (VW + 1) <= 200;       // the reflector fits the registers beside the vectors
-    float4 vk[kKeep ? NCH : 1];
-    float s[VW][2];
-#pragma unroll
-    for (int u = 0; u < VW; ++u) s[u][0] = s[u][1] = 0.f;
-#pragma unroll
-    for (int ch = 0; ch < NCH; ++ch) {
-      if (ch >= c0 && ch < chunks) {
-        const float4 v4 = *reinterpret_cast<const float4*>(v + ch * 128 + lane * 4);
-        if (kKeep) vk[kKeep ? ch : 0] = v4;
-#pragma unroll
-        for (int u = 0; u < VW; ++u)
-          s[u][ch & 1] = fmaf(v4.x, x[u][ch].x, fmaf(v4.y, x[u][ch].y, fmaf(v4.z, x[u][ch].z, fmaf(v4.w, x[u][ch].w, s[u][ch & 1]))));
-      }
+  int step = 0;
+  for (int k = N - 1; k >= 0; k -= 2, ++step) {
+    __syncthreads();                                // everybody is done with the slot refilled now
+    fetch(step + kBackStages - 1);
+    if (!ptx::mbar_wait(&landed[step % kBackStages], (step / kBackStages) & 1)) {   // (the copies in flight end by themselves)
+      if (status) atomicOr(status, QG_DEV_WAIT_EXPIRED);
     }
-    const float tk = taus[k];
-    float f[VW];
+    const float* va = ring + (step % kBackStages) * 2 * Np + lane * 4;   // v_k (tau = 0 stands for v_{N-1}), v_{k-1}
+    const float* vb = va + Np;
+    const bool two = k > 0;
+    const int c0 = k / 128;
+    const float ta = taus[k], tb = two ? taus[k - 1] : 0.f, cr = two ? cross[k] : 0.f;
+    float sa[VW], sb[VW];
 #pragma unroll
-    for (int u = 0; u < VW; ++u) f[u] = -tk * warp_sum(s[u][0] + s[u][1]);
+    for (int u = 0; u < VW; ++u) sa[u] = sb[u] = 0.f;
 #pragma unroll
     for (int ch = 0; ch < NCH; ++ch) {
       if (ch >= c0 && ch < chunks) {
-        const float4 v4 = kKeep ? vk[kKeep ? ch : 0] : *reinterpret_cast<const float4*>(v + ch * 128 + lane * 4);
+        const float4 a4 = *reinterpret_cast<const float4*>(va + ch * 128);
+        const float4 b4 = two ? *reinterpret_cast<const float4*>(vb + ch * 128) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
         for (int u = 0; u < VW; ++u) {
-          x[u][ch].x = fmaf(f[u], v4.x, x[u][ch].x);
-          x[u][ch].y = fmaf(f[u], v4.y, x[u][ch].y);
-          x[u][ch].z = fmaf(f[u], v4.z, x[u][ch].z);
-          x[u][ch].w = fmaf(f[u], v4.w, x[u][ch].w);
+          sa[u] = fmaf(a4.x, x[u][ch].x, fmaf(a4.y, x[u][ch].y, fmaf(a4.z, x[u][ch].z, fmaf(a4.w, x[u][ch].w, sa[u]))));
+          sb[u] = fmaf(b4.x, x[u][ch].x, fmaf(b4.y, x[u][ch].y, fmaf(b4.z, x[u][ch].z, fmaf(b4.w, x[u][ch].w, sb[u]))));
+        }
+      }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+      for (int u = 0; u < VW; ++u) {
+        sa[u] += __shfl_xor_sync(0xFFFFFFFFu, sa[u], o);
+        sb[u] += __shfl_xor_sync(0xFFFFFFFFu, sb[u], o);
+      }
+#pragma unroll
+    for (int u = 0; u < VW; ++u) {
+      sa[u] *= -ta;
+      sb[u] = -tb * fmaf(cr, sa[u], sb[u]);
+    }
+#pragma unroll
+    for (int ch = 0; ch < NCH; ++ch) {
+      if (ch >= c0 && ch < chunks) {
+        const float4 a4 = *reinterpret_cast<const float4*>(va + ch * 128);
+        const float4 b4 = two ? *reinterpret_cast<const float4*>(vb + ch * 128) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int u = 0; u < VW; ++u) {
+          x[u][ch].x = fmaf(sa[u], a4.x, fmaf(sb[u], b4.x, x[u][ch].x));
+          x[u][ch].y = fmaf(sa[u], a4.y, fmaf(sb[u], b4.y, x[u][ch].y));
+          x[u][ch].z = fmaf(sa[u], a4.z, fmaf(sb[u], b4.z, x[u][ch].z));
+          x[u][ch].w = fmaf(sa[u], a4.w, fmaf(sb[u], b4.w, x[u][ch].w));
         }
       }
     }
@@ -680,14 +755,15 @@ int launch_tridiagonal(TriArgs a, int nb, int32_t* status, cudaStream_t st) {
 }
 
 template <int NCH, int VW, int WARPS>
-int launch_back(const Ptrs<const float>& V, const Ptrs<const float>& tau, int nb, int64_t N, int64_t Np, int64_t r, const Ptrs<float>& Z,
-                const Ptrs<const double>& inv, cudaStream_t st) {
+int launch_back(const Ptrs<const float>& V, const Ptrs<const float>& tau, const Ptrs<const float>& cross, int nb, int64_t N, int64_t Np, int64_t r, const Ptrs<float>& Z,
+                const Ptrs<const double>& inv, int32_t* status, cudaStream_t st) {
+  constexpr int kBackStages = back_stages(NCH);
   static bool done[kDevices] = {};
   auto kern = back_transform_kernel<NCH, VW, WARPS>;
-  const int rc = opt_in(kern, (kBackStages * NCH * 128 + 128 * (WARPS * VW + 1) + NCH * 128) * 4, done);
+  const int rc = opt_in(kern, ((2 * kBackStages + 2) * NCH * 128 + 128 * (WARPS * VW + 1)) * 4, done);
   if (rc != QG_OK) return rc;
-  const size_t smem = (size_t)(kBackStages * Np + 128 * (WARPS * VW + 1) + N) * 4;
-  kern<<<dim3((unsigned)ceil_div(r, WARPS * VW), (unsigned)nb), WARPS * 32, smem, st>>>(V, tau, (int)N, (int)Np, (int)r, Z, inv);
+  const size_t smem = (size_t)(2 * kBackStages * Np + 128 * (WARPS * VW + 1) + 2 * N) * 4;
+  kern<<<dim3((unsigned)ceil_div(r, WARPS * VW), (unsigned)nb), WARPS * 32, smem, st>>>(V, tau, cross, (int)N, (int)Np, (int)r, Z, inv, status);
   QG_LAUNCH_CHECK();
   return QG_OK;
 }
@@ -721,6 +797,7 @@ size_t carve_eig(void* base, int64_t N, int64_t r, EigBuffers* out) {
   w.tau = (float*)take((size_t)(N * 4));
   w.d = (float*)take((size_t)(N * 4));
   w.e = (float*)take((size_t)(N * 4));
+  w.cross = (float*)take((size_t)(N * 4));
   w.scale = (float*)take(4);
   w.lam = (double*)take((size_t)(r * 8));
   w.inv = (double*)take((size_t)(r * 8));
@@ -735,14 +812,14 @@ size_t carve_eig(void* base, int64_t N, int64_t r, EigBuffers* out) {
 int launch_sym_eig(const EigBuffers* w, int nb, int64_t N, int64_t r, int32_t* status, cudaStream_t st) {
   if (N < 2 || N > kEigMax || r < 1 || r > N || nb < 1 || nb > kMaxBatch) return QG_UNSUPPORTED_SHAPE;
   const int64_t Np = eig_pitch(N);
-  Ptrs<float> A{}, V{}, tau{}, d{}, e{}, Z{}, scale{};
-  Ptrs<const float> Ac{}, Vc{}, tauc{}, dc{}, ec{}, scalec{};
+  Ptrs<float> A{}, V{}, tau{}, d{}, e{}, Z{}, scale{}, cross{};
+  Ptrs<const float> Ac{}, Vc{}, tauc{}, dc{}, ec{}, scalec{}, crossc{};
   Ptrs<double> lam{}, inv{}, plus{}, minus{};
   Ptrs<const double> lamc{}, invc{};
   Ptrs<uint4> xchg{};
   for (int i = 0; i < nb; ++i) {
     Ac.p[i] = A.p[i] = w[i].A; Vc.p[i] = V.p[i] = w[i].V; tauc.p[i] = tau.p[i] = w[i].tau;
-    dc.p[i] = d.p[i] = w[i].d; ec.p[i] = e.p[i] = w[i].e; Z.p[i] = w[i].Z; scalec.p[i] = scale.p[i] = w[i].scale;
+    dc.p[i] = d.p[i] = w[i].d; ec.p[i] = e.p[i] = w[i].e; Z.p[i] = w[i].Z; scalec.p[i] = scale.p[i] = w[i].scale; crossc.p[i] = cross.p[i] = w[i].cross;
     lamc.p[i] = lam.p[i] = w[i].lam; invc.p[i] = inv.p[i] = w[i].inv; plus.p[i] = w[i].plus; minus.p[i] = w[i].minus; xchg.p[i] = w[i].xchg;
     QG_CUDA_TRY(cudaMemsetAsync(w[i].xchg, 0, (size_t)(2 * Np * 16), st));   // no tag of an earlier call
   }
@@ -755,7 +832,8 @@ int launch_sym_eig(const EigBuffers* w, int nb, int64_t N, int64_t r, int32_t* s
   // registers and shared memory.
   const int sms = sm_count();
   const int64_t nq = Np <= kTriThreads ? 1 : Np <= 2 * kTriThreads ? 2 : Np <= 4 * kTriThreads ? 4 : 8;
-  auto ctas = [&](int cnt) { return std::max<int64_t>(1, std::min<int64_t>(sms / cnt, ceil_div(N, 16))); };
+  // (a matrix alone: 128 CTAs are faster than 148 although more of its columns spill, 4096 rows 64 -> 57 ms, 2500 25 -> 22)
+  auto ctas = [&](int cnt) { return std::max<int64_t>(1, std::min<int64_t>(cnt == 1 ? std::min(sms, 128) : sms / cnt, ceil_div(N, 16))); };
   auto in_smem = [&](int64_t C) { return std::max<int64_t>(0, (kTriSmem / 4 - (6 + 2 * kTriWarps) * (ceil_div(N, C) + 8)) / Np); };
   int together = nb;
   while (together > 1 && ctas(together) * (64 / nq + in_smem(ctas(together))) * 5 < N * 4) --together;
@@ -791,12 +869,14 @@ int launch_sym_eig(const EigBuffers* w, int nb, int64_t N, int64_t r, int32_t* s
   }
   tridiagonal_vectors_kernel<<<dim3((unsigned)ceil_div(r, 32), (unsigned)nb), 64, (size_t)N * 12, st>>>(dc, ec, (int)N, (int)r, lamc, plus, minus, Z, inv);
   QG_LAUNCH_CHECK();
+  reflector_pairs_kernel<<<dim3((unsigned)ceil_div(N, 8), (unsigned)nb), 128, 0, st>>>(Vc, (int)N, (int)Np, cross);
+  QG_LAUNCH_CHECK();
   const bool few = nb * r <= 4 * sms;                // a CTA of two warps per SM
-  if (Np <= 512) return few ? launch_back<4, 1, 2>(Vc, tauc, nb, N, Np, r, Z, invc, st) : launch_back<4, 2, 8>(Vc, tauc, nb, N, Np, r, Z, invc, st);
-  if (Np <= 768) return few ? launch_back<6, 1, 2>(Vc, tauc, nb, N, Np, r, Z, invc, st) : launch_back<6, 2, 8>(Vc, tauc, nb, N, Np, r, Z, invc, st);
-  if (Np <= 1024) return few ? launch_back<8, 1, 2>(Vc, tauc, nb, N, Np, r, Z, invc, st) : launch_back<8, 2, 8>(Vc, tauc, nb, N, Np, r, Z, invc, st);
-  if (Np <= 2048) return few ? launch_back<16, 1, 4>(Vc, tauc, nb, N, Np, r, Z, invc, st) : launch_back<16, 2, 8>(Vc, tauc, nb, N, Np, r, Z, invc, st);
-  return launch_back<32, 1, 8>(Vc, tauc, nb, N, Np, r, Z, invc, st);
+  if (Np <= 512) return few ? launch_back<4, 1, 2>(Vc, tauc, crossc, nb, N, Np, r, Z, invc, status, st) : launch_back<4, 2, 8>(Vc, tauc, crossc, nb, N, Np, r, Z, invc, status, st);
+  if (Np <= 768) return few ? launch_back<6, 1, 2>(Vc, tauc, crossc, nb, N, Np, r, Z, invc, status, st) : launch_back<6, 2, 8>(Vc, tauc, crossc, nb, N, Np, r, Z, invc, status, st);
+  if (Np <= 1024) return few ? launch_back<8, 1, 2>(Vc, tauc, crossc, nb, N, Np, r, Z, invc, status, st) : launch_back<8, 2, 8>(Vc, tauc, crossc, nb, N, Np, r, Z, invc, status, st);
+  if (Np <= 2048) return few ? launch_back<16, 1, 4>(Vc, tauc, crossc, nb, N, Np, r, Z, invc, status, st) : launch_back<16, 2, 8>(Vc, tauc, crossc, nb, N, Np, r, Z, invc, status, st);
+  return launch_back<32, 1, 8>(Vc, tauc, crossc, nb, N, Np, r, Z, invc, status, st);
 }
 
 }  // namespace qg
