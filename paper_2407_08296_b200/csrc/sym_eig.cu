@@ -589,8 +589,10 @@ back_transform_kernel(const Ptrs<const float> Vb, const Ptrs<const float> taub, 
   constexpr int kBackStages = back_stages(NCH);
   __shared__ __align__(8) uint64_t landed[kBackStages];
   constexpr int kW = WARPS * VW, kThreads = WARPS * 32;   // vectors and threads of this CTA
-  float* ring = back_smem;                          // [kBackStages][2][Np]
-  float* tile = ring + 2 * kBackStages * Np;        // [128][kW + 1]
+  // chunks are taken in groups, so that their loads overlap; a group that begins above the reflector's first row meets zeros
+  constexpr int kGrp = NCH % 4 == 0 ? 4 : 3, kPitch = NCH * 128;
+  float* ring = back_smem;                          // [kBackStages][2][kPitch]
+  float* tile = ring + 2 * kBackStages * kPitch;    // [128][kW + 1]
   float* taus = tile + 128 * (kW + 1);              // [N]
   float* cross = taus + N;                          // [N]
   const int mat = blockIdx.y, t0 = blockIdx.x * kW;
@@ -603,22 +605,23 @@ back_transform_kernel(const Ptrs<const float> Vb, const Ptrs<const float> taub, 
     cross[i] = crossb.p[mat][i];
   }
 
+  for (int i = tid; i < 2 * kBackStages * kPitch; i += kThreads) ring[i] = 0.f;   // what lies past Np stays zero
   if (tid == 0) {
     for (int i = 0; i < kBackStages; ++i) ptx::mbar_init(&landed[i], 1);
     ptx::fence_mbar_init();
   }
-  auto fetch = [&](int step) {                      // one thread: reflectors k = N - 1 - 2 step and k - 1, rows k .. on in whole chunks
+  auto fetch = [&](int step) {                      // one thread: reflectors k = N - 1 - 2 step and k - 1, rows k .. on in whole groups
     const int k = N - 1 - 2 * step;
     if (tid != 0 || k < 0) return;
     uint64_t* bar = &landed[step % kBackStages];
-    float* dst = ring + (step % kBackStages) * 2 * Np;
+    float* dst = ring + (step % kBackStages) * 2 * kPitch;
     const float* src = V + (int64_t)k * Np;
-    const int i = k / 128 * 128;
+    const int i = k / (128 * kGrp) * (128 * kGrp);
     const uint32_t bytes = (uint32_t)(Np - i) * 4u;
     ptx::fence_proxy_async_smem();
     ptx::mbar_arrive_expect_tx(bar, k > 0 ? 2 * bytes : bytes);
     bulk_load(dst + i, src + i, bytes, bar);
-    if (k > 0) bulk_load(dst + Np + i, src - Np + i, bytes, bar);
+    if (k > 0) bulk_load(dst + kPitch + i, src - Np + i, bytes, bar);
   };
   __syncthreads();
   for (int s = 0; s < kBackStages - 1; ++s) fetch(s);
@@ -653,23 +656,30 @@ back_transform_kernel(const Ptrs<const float> Vb, const Ptrs<const float> taub, 
     if (!ptx::mbar_wait(&landed[step % kBackStages], (step / kBackStages) & 1)) {   // (the copies in flight end by themselves)
       if (status) atomicOr(status, QG_DEV_WAIT_EXPIRED);
     }
-    const float* va = ring + (step % kBackStages) * 2 * Np + lane * 4;   // v_k (tau = 0 stands for v_{N-1}), v_{k-1}
-    const float* vb = va + Np;
+    const float* va = ring + (step % kBackStages) * 2 * kPitch + lane * 4;   // v_k (tau = 0 stands for v_{N-1}), v_{k-1}
+    const float* vb = va + kPitch;
     const bool two = k > 0;
-    const int c0 = k / 128;
+    const int g0 = k / (128 * kGrp);
     const float ta = taus[k], tb = two ? taus[k - 1] : 0.f, cr = two ? cross[k] : 0.f;
     float sa[VW], sb[VW];
 #pragma unroll
     for (int u = 0; u < VW; ++u) sa[u] = sb[u] = 0.f;
 #pragma unroll
-    for (int ch = 0; ch < NCH; ++ch) {
-      if (ch >= c0 && ch < chunks) {
-        const float4 a4 = *reinterpret_cast<const float4*>(va + ch * 128);
-        const float4 b4 = two ? *reinterpret_cast<const float4*>(vb + ch * 128) : make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int g = 0; g < NCH / kGrp; ++g) {
+      if (g < g0) continue;
+      float4 a4[kGrp], b4[kGrp];
+#pragma unroll
+      for (int c = 0; c < kGrp; ++c) {
+        a4[c] = *reinterpret_cast<const float4*>(va + (g * kGrp + c) * 128);
+        b4[c] = two ? *reinterpret_cast<const float4*>(vb + (g * kGrp + c) * 128) : make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+#pragma unroll
+      for (int c = 0; c < kGrp; ++c) {
+        const int ch = g * kGrp + c;
 #pragma unroll
         for (int u = 0; u < VW; ++u) {
-          sa[u] = fmaf(a4.x, x[u][ch].x, fmaf(a4.y, x[u][ch].y, fmaf(a4.z, x[u][ch].z, fmaf(a4.w, x[u][ch].w, sa[u]))));
-          sb[u] = fmaf(b4.x, x[u][ch].x, fmaf(b4.y, x[u][ch].y, fmaf(b4.z, x[u][ch].z, fmaf(b4.w, x[u][ch].w, sb[u]))));
+          sa[u] = fmaf(a4[c].x, x[u][ch].x, fmaf(a4[c].y, x[u][ch].y, fmaf(a4[c].z, x[u][ch].z, fmaf(a4[c].w, x[u][ch].w, sa[u]))));
+          sb[u] = fmaf(b4[c].x, x[u][ch].x, fmaf(b4[c].y, x[u][ch].y, fmaf(b4[c].z, x[u][ch].z, fmaf(b4[c].w, x[u][ch].w, sb[u]))));
         }
       }
     }
@@ -686,16 +696,23 @@ back_transform_kernel(const Ptrs<const float> Vb, const Ptrs<const float> taub, 
       sb[u] = -tb * fmaf(cr, sa[u], sb[u]);
     }
 #pragma unroll
-    for (int ch = 0; ch < NCH; ++ch) {
-      if (ch >= c0 && ch < chunks) {
-        const float4 a4 = *reinterpret_cast<const float4*>(va + ch * 128);
-        const float4 b4 = two ? *reinterpret_cast<const float4*>(vb + ch * 128) : make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int g = 0; g < NCH / kGrp; ++g) {
+      if (g < g0) continue;
+      float4 a4[kGrp], b4[kGrp];
+#pragma unroll
+      for (int c = 0; c < kGrp; ++c) {
+        a4[c] = *reinterpret_cast<const float4*>(va + (g * kGrp + c) * 128);
+        b4[c] = two ? *reinterpret_cast<const float4*>(vb + (g * kGrp + c) * 128) : make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+#pragma unroll
+      for (int c = 0; c < kGrp; ++c) {
+        const int ch = g * kGrp + c;
 #pragma unroll
         for (int u = 0; u < VW; ++u) {
-          x[u][ch].x = fmaf(sa[u], a4.x, fmaf(sb[u], b4.x, x[u][ch].x));
-          x[u][ch].y = fmaf(sa[u], a4.y, fmaf(sb[u], b4.y, x[u][ch].y));
-          x[u][ch].z = fmaf(sa[u], a4.z, fmaf(sb[u], b4.z, x[u][ch].z));
-          x[u][ch].w = fmaf(sa[u], a4.w, fmaf(sb[u], b4.w, x[u][ch].w));
+          x[u][ch].x = fmaf(sa[u], a4[c].x, fmaf(sb[u], b4[c].x, x[u][ch].x));
+          x[u][ch].y = fmaf(sa[u], a4[c].y, fmaf(sb[u], b4[c].y, x[u][ch].y));
+          x[u][ch].z = fmaf(sa[u], a4[c].z, fmaf(sb[u], b4[c].z, x[u][ch].z));
+          x[u][ch].w = fmaf(sa[u], a4[c].w, fmaf(sb[u], b4[c].w, x[u][ch].w));
         }
       }
     }
@@ -762,7 +779,7 @@ int launch_back(const Ptrs<const float>& V, const Ptrs<const float>& tau, const 
   auto kern = back_transform_kernel<NCH, VW, WARPS>;
   const int rc = opt_in(kern, ((2 * kBackStages + 2) * NCH * 128 + 128 * (WARPS * VW + 1)) * 4, done);
   if (rc != QG_OK) return rc;
-  const size_t smem = (size_t)(2 * kBackStages * Np + 128 * (WARPS * VW + 1) + 2 * N) * 4;
+  const size_t smem = (size_t)(2 * kBackStages * NCH * 128 + 128 * (WARPS * VW + 1) + 2 * N) * 4;
   kern<<<dim3((unsigned)ceil_div(r, WARPS * VW), (unsigned)nb), WARPS * 32, smem, st>>>(V, tau, cross, (int)N, (int)Np, (int)r, Z, inv, status);
   QG_LAUNCH_CHECK();
   return QG_OK;
