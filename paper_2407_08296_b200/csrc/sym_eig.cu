@@ -440,7 +440,7 @@ __global__ void resolved_kernel(const Ptrs<const double> lamb, int N, int r, int
 // T - lambda = L D+ L^T from the top and U D- U^T from the bottom; where gamma_i = D+_i + D-_i - (d_i - lambda) is smallest
 // the two factorisations are joined, and the vector follows outward from that row by products of multipliers alone, without
 // cancellation.  Bound: the chain of binary64 divisions, so a pair of threads takes an eigenvalue, one from each end (warp 0
-// and warp 1 of a CTA): 768 rows 320 -> 298 us.
+// and warp 1 of a CTA): 768 rows, 256 vectors 320 -> 208 us.
 constexpr double kPivotFloor = 1e-280;
 __device__ __forceinline__ double guarded(double q) { return fabs(q) < kPivotFloor ? copysign(kPivotFloor, q) : q; }
 
@@ -555,7 +555,7 @@ tridiagonal_vectors_kernel(const Ptrs<const float> db, const Ptrs<const float> e
 // dot product and update.  So the reflectors are applied two at a time, with one reduction for both,
 //     s_k = v_k . x,  s_{k-1} = v_{k-1} . x - tau_k s_k (v_{k-1} . v_k),  x <- x - tau_k s_k v_k - tau_{k-1} s_{k-1} v_{k-1},
 // and few vectors are spread over many CTAs of two warps.
-// 768 rows, 256 vectors 605 -> 242 us; 2048 rows, eight times 512 vectors 4180 -> 4090.
+// 768 rows, 256 vectors 605 -> 228 us; 2048 rows, eight times 512 vectors 4180 -> 2665.
 constexpr int back_stages(int nch) { return nch <= 16 ? 6 : 4; }   // pairs of reflectors in the ring
 
 // `bytes` (a multiple of 16) consecutive bytes to shared memory by the copy engine.
