@@ -149,25 +149,34 @@ tridiagonal_kernel(const __grid_constant__ TriArgs a, int32_t* __restrict__ stat
 #pragma unroll
       for (int q = 0; q < NQ; ++q)
         if ((tid | 31) + q * kTriThreads >= k && (tid | 31) + q * kTriThreads < N) jq = (tid | 31) + q * kTriThreads;
-      if (lane == 0 && jq >= 0) {
-        uint32_t polls = 0;
-        while (ld_relaxed_v4(xchg + (k & 1) * Np + jq).y != (uint32_t)k && ++polls < kPollLimit) __nanosleep(32);
-      }
-      __syncwarp();
+      if (jq >= 0)
+        for (uint32_t polls = 0; polls < kPollLimit; ++polls) {
+          bool here = true;
+          if (lane == 0) here = ld_relaxed_v4(xchg + (k & 1) * Np + jq).y == (uint32_t)k;
+          if (__all_sync(0xFFFFFFFFu, here)) break;
+          __nanosleep(32);
+        }
     }
     float sums[4] = {0.f, 0.f, 0.f, 0.f};
     bool ok = true;
 #pragma unroll
     for (int q = 0; q < NQ; ++q) {
       const int j = tid + q * kTriThreads;
+      // (the whole warp stays in the loop: lanes that left it one by one would run on by themselves, and a CTA barrier counts
+      // a warp as arrived with the first of them)
+      const bool wanted = k > 0 && j >= k && j < N;
+      const uint4* const in = xchg + (k & 1) * Np + j;
+      uint4 got = make_uint4(0, 0, 0, 0);
+      bool here = !wanted;
+      for (uint32_t polls = 0; polls < kPollLimit && !__all_sync(0xFFFFFFFFu, here); ++polls)
+        if (!here) {
+          got = ld_relaxed_v4(in);
+          here = got.y == (uint32_t)k && got.w == (uint32_t)k;
+        }
+      ok = ok && here;
       float p = 0.f;
       if (j >= k && j < N) {
-        if (k > 0) {
-          const uint4* in = xchg + (k & 1) * Np + j;
-          uint4 got = ld_relaxed_v4(in);
-          uint32_t polls = 0;
-          while ((got.y != (uint32_t)k || got.w != (uint32_t)k) && ++polls < kPollLimit) got = ld_relaxed_v4(in);
-          ok = ok && polls < kPollLimit;
+        if (wanted) {
           p = __uint_as_float(got.x);
           r[q] = __uint_as_float(got.z);
         }
@@ -321,6 +330,7 @@ tridiagonal_kernel(const __grid_constant__ TriArgs a, int32_t* __restrict__ stat
       for (int i = 0; i < kTriWarps; ++i) s += part[i * 2 * nc8 + l];
       st_relaxed_v4(xchg + (k1 & 1) * Np + j, s, pivot[l], (uint32_t)k1);
     }
+    __syncwarp();
 #pragma unroll
     for (int q = 0; q < NQ; ++q) v[q] = vn[q];
   }
