@@ -134,16 +134,6 @@ __device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t a_desc, uint
       ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"((uint32_t)accumulate)
       : "memory");
 }
-// The same with A read from tensor memory: 128 lanes (rows of A), the K elements of a row packed two per
-// 32-bit column in order (element 2c in the low half of column c), so one instruction (K = 16) reads 8 columns.
-__device__ __forceinline__ void umma_bf16_tmem_a(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc, bool accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
-      ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"((uint32_t)accumulate)
-      : "memory");
-}
 // The barrier receives one arrival once every tcgen05.mma issued so far by this thread has completed.
 __device__ __forceinline__ void umma_commit(uint64_t* bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
@@ -181,18 +171,7 @@ __device__ __forceinline__ void tmem_st_32x16(uint32_t taddr, const uint32_t v[1
         "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15]), "r"(taddr)
       : "memory");
 }
-// The store counterpart of tmem_ld_32x32, and the wait that orders it before later tcgen05.ld of the thread.
-__device__ __forceinline__ void tmem_st_32x32(uint32_t taddr, const uint32_t v[32]) {
-  asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%32], "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31};"
-      ::"r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]), "r"(v[8]), "r"(v[9]),
-        "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15]), "r"(v[16]), "r"(v[17]), "r"(v[18]),
-        "r"(v[19]), "r"(v[20]), "r"(v[21]), "r"(v[22]), "r"(v[23]), "r"(v[24]), "r"(v[25]), "r"(v[26]), "r"(v[27]),
-        "r"(v[28]), "r"(v[29]), "r"(v[30]), "r"(v[31]), "r"(taddr)
-      : "memory");
-}
+// Orders a thread's tcgen05.st before its later tcgen05.ld.
 __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
 // 16 lanes x 32 columns in the 16x256b shape: thread t receives, for k = 0..3, a = 0..1, b = 0..1,
@@ -251,6 +230,13 @@ __device__ __forceinline__ uint32_t mapa_u32(uint32_t local_addr, uint32_t rank)
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
+// The same, ordering this thread's writes for its own CTA only.  Enough for an operand that the tensor core of THIS SM reads
+// (shared memory behind a proxy fence) whoever issues the MMA, and for an accumulator handed back (tensor memory behind
+// tcgen05.wait::ld); the arrival above holds its thread up for 900 to 1300 clocks, until all of its loads and stores, global
+// ones too, are done.
+__device__ __forceinline__ void mbar_arrive_remote(uint32_t cluster_addr) {
+  asm volatile("mbarrier.arrive.release.cta.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
+}
 // Bounded wait on a barrier of this CTA that is also signalled from the peer CTA (acquire at cluster scope).
 __device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity) {
   for (uint32_t i = 0; i < kWaitPollLimit; ++i) {
@@ -301,10 +287,10 @@ __device__ __forceinline__ void umma_bf16_pair(uint32_t d_tmem, uint64_t a_desc,
       : "memory");
 }
 // One arrival on the barrier at this shared-memory offset in BOTH CTAs of the pair once the MMAs issued so
-// far have completed.
-__device__ __forceinline__ void umma_commit_pair(uint64_t* bar) {
+// far have completed (`leader`: the cluster rank of the first of the two, which issues).
+__device__ __forceinline__ void umma_commit_pair(uint64_t* bar, uint32_t leader = 0) {
   asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
-               ::"r"(smem_u32(bar)), "h"((uint16_t)3)
+               ::"r"(smem_u32(bar)), "h"((uint16_t)(3u << leader))
                : "memory");
 }
 

@@ -42,9 +42,11 @@ def test_forward_of_a_few_tokens(T, m, n):
     _check(Y, X.float(), Wd.T, status)
 
 
-# Tiles of 128 x 256 (256 x 256 for the input gradient): a few of them shared by clusters of 2 .. 8 CTAs along K, a whole
-# round of persistent CTAs followed by a remainder in clusters, extents that end inside a tile, a K that ends inside a block.
-@pytest.mark.parametrize("T,m,n", [(40, 200, 1500), (300, 1159, 3001), (257, 515, 2100), (4200, 1100, 700), (129, 2100, 4500), (1000, 3001, 640)])
+# Tiles of 256 or 512 x 256, one per CTA pair: a few of them shared by clusters of 2 .. 4 pairs along K, whole rounds of persistent
+# pairs alone or followed by a remainder in clusters, a tile part of whose rows are empty, extents that end inside a tile, a K
+# that ends inside a block.  The last takes 512 rows for all three products.
+@pytest.mark.parametrize("T,m,n", [(40, 200, 1500), (300, 1159, 3001), (257, 515, 2100), (4200, 1100, 700), (129, 2100, 4500), (1000, 3001, 640),
+                                   (2817, 2100, 1800), (600, 4300, 5000), (257, 256, 65), (4500, 4096, 4090)])
 def test_products_whose_tiles_are_split_along_k(T, m, n):
     torch.backends.cuda.matmul.allow_tf32 = False
     X, dY, W, Wd = _operands(T, m, n, seed=T)
