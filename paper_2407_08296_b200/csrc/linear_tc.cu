@@ -534,17 +534,17 @@ int resident_clusters(int split, int dev) {
 }
 
 // CTA pairs that share a tile of the last, unfilled round (`tiles` of them for `pairs` pairs): as many as keep every tile's
-// cluster resident, each with at least four K blocks.  1 (the round as it is) where that saves fewer than 16 K blocks: adding
-// up the accumulators takes 4 to 8 us, a K block 0.35 (weight gradient) to 0.5 us.
+// cluster resident, each with at least four K blocks.  1 (the round as it is) where that saves fewer than `saves` K blocks:
+// adding up the accumulators takes 4 to 8 us, a K block 0.35 (weight gradient, 1024 x 1376 x 512: 12.6 us as it is, 14.5
+// shared) to 0.5 us (input gradient 18 x 1137 x 163: 16.5 and 12.6).
 // Measured, against whole tiles by single CTAs: forward 310 x 1159 x 5993 53 -> 27 us, 512 x 2048 x 5461 51 -> 31; input
 // gradient 904 x 6535 x 4003 120 -> 57, 64 x 4096 x 4096 74 -> 27; weight gradient 2000 x 600 x 900 22 -> 18.
-constexpr int kSplitSaves = 16;
 template <auto KERN, int THREADS, int SMEM>
-int choose_split(int tiles, int kblocks, int pairs, int dev) {
+int choose_split(int tiles, int kblocks, int pairs, int saves, int dev) {
   int split = tiles > 0 ? pairs / tiles : 1;
   split = std::min(std::min(split, kMaxSplit), kblocks / 4);
   while (split > 1 && resident_clusters<KERN, THREADS, SMEM>(split, dev) < tiles) --split;
-  return split > 1 && kblocks - (kblocks + split - 1) / split >= kSplitSaves ? split : 1;
+  return split > 1 && kblocks - (kblocks + split - 1) / split >= saves ? split : 1;
 }
 
 // How a kernel takes a product: whole rounds of one tile per pair by persistent CTAs, and the remainder, where that pays, by a
@@ -569,7 +569,7 @@ int plan_rounds(const LinArgs& a, int dev, Rounds& r) {
   r.mblocks = (a.rows + rows - 1) / rows;
   const int total = r.mblocks * a.nblocks;
   r.rest = total % r.pairs;
-  r.split = choose_split<kern, S::kThreads, S::kBytes>(r.rest, kblocks, r.pairs, dev);
+  r.split = choose_split<kern, S::kThreads, S::kBytes>(r.rest, kblocks, r.pairs, MODE == kWeightGrad ? 16 : 8, dev);
   r.whole = total - r.rest;
   // A K block of a 512-row tile takes 1.57 of a 256-row tile's time with a converted operand (16384 x 4096 x 4096 forward 498
   // us for 14 rounds, 382 for 7), 1.9 without (365 and 344, weight gradient); its epilogue, which nothing overlaps, and the
