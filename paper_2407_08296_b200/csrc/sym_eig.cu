@@ -110,7 +110,7 @@ tridiagonal_kernel(const __grid_constant__ TriArgs a, int32_t* __restrict__ stat
   float* const colV = colP + 2 * nc8;          // (twice the room: a group starts anywhere)
   float* const pivot = colV + 2 * nc8;         // A_{k+1, j}
   float* const part = pivot + 2 * nc8;         // [warp][column] partial sums of P'_j
-  float* const scols = part + kTriWarps * 2 * nc8;   // [column][Np]
+  float4* const scols = reinterpret_cast<float4*>(part + kTriWarps * 2 * nc8);   // [group of four columns][Np]
 
   float2 ar[NQ][RC / 2];
   float v[NQ], w[NQ], vn[NQ], r[NQ];
@@ -128,8 +128,13 @@ tridiagonal_kernel(const __grid_constant__ TriArgs a, int32_t* __restrict__ stat
       ar[q][c / 2].y = (l + 1 < ncols && j < Np) ? A[(int64_t)(cta + (l + 1) * C) * Np + j] : 0.f;
     }
   }
-  for (int l = 0; l < ns; ++l)
-    for (int i = tid; i < Np; i += kTriThreads) scols[l * Np + i] = A[(int64_t)(cta + (ng + l) * C) * Np + i];
+  for (int l = 0; l < ns; l += 4)
+    for (int i = tid; i < Np; i += kTriThreads) {
+      float x[4];
+#pragma unroll
+      for (int c = 0; c < 4; ++c) x[c] = l + c < ns ? A[(int64_t)(cta + (ng + l + c) * C) * Np + i] : 0.f;
+      scols[(l >> 2) * Np + i] = make_float4(x[0], x[1], x[2], x[3]);
+    }
   for (int i = tid; i < 6 * nc8; i += kTriThreads) tri_smem[i] = 0.f;
   if (tid == 0) { s_fail = 0; s_pk = 0.f; }
   __syncthreads();
@@ -271,34 +276,52 @@ tridiagonal_kernel(const __grid_constant__ TriArgs a, int32_t* __restrict__ stat
       const float s = warp_sums8(acc, lane);
       if ((lane & 3) == 0) part[warp * 2 * nc8 + l + (lane >> 2)] = s;
     };
-    // columns in memory: element (row, l) at at(l)[row]
-    auto memory_columns = [&](int l0, int l1, auto at) {
-      for (int l = l0; l < l1; l += 8) {
-        if (cta + min(l + 7, l1 - 1) * C <= k) continue;               // all of them retired
-        float2 wj[4], vj[4], acc[4] = {};
-        scalars(l, wj, vj);
+    // columns in memory, four to a load (get(l, row), put(l, row, x): columns l .. l + 3), the next row's on its way
+    auto memory_columns = [&](int l0, int l1, auto get, auto put) {
+      const int q0 = k1 / kTriThreads;
+      for (int l = l0; l < l1; l += 4) {
+        if (cta + min(l + 3, l1 - 1) * C <= k) continue;               // all of them retired
+        float2 wj[2], vj[2], acc[2] = {};
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+          vj[c] = make_float2(colV[l + 2 * c], colV[l + 2 * c + 1]);
+          wj[c] = fma2(tau2, make_float2(colP[l + 2 * c], colP[l + 2 * c + 1]), mul2(kap2, vj[c]));
+        }
+        float4 next = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (tid + q0 * kTriThreads < Np) next = get(l, tid + q0 * kTriThreads);
 #pragma unroll
         for (int q = 0; q < NQ; ++q) {
           const int row = tid + q * kTriThreads;
           if (q * kTriThreads + kTriThreads - 1 <= k || row >= Np) continue;
+          float2 lo = make_float2(next.x, next.y), hi = make_float2(next.z, next.w);
+          if (q + 1 < NQ && row + kTriThreads < Np) next = get(l, row + kTriThreads);
           const float2 nv = both(-v[q]), nw = both(-w[q]), n2 = both(vn[q]);
-#pragma unroll
-          for (int c = 0; c < 4; ++c) {
-            const int la = l + 2 * c, lb = min(la + 1, l1 - 1);
-            if (la >= l1) break;
-            float2 x = make_float2(at(la)[row], at(lb)[row]);
-            x = fma2(nw, vj[c], fma2(nv, wj[c], x));
-            at(la)[row] = x.x;
-            if (la + 1 < l1) at(lb)[row] = x.y;
-            acc[c] = fma2(x, n2, acc[c]);
-            if (pivot_thread && q == qk) { pivot[la] = x.x; if (la + 1 < l1) pivot[la + 1] = x.y; }
-          }
+          lo = fma2(nw, vj[0], fma2(nv, wj[0], lo));
+          hi = fma2(nw, vj[1], fma2(nv, wj[1], hi));
+          put(l, row, make_float4(lo.x, lo.y, hi.x, hi.y));
+          acc[0] = fma2(lo, n2, acc[0]);
+          acc[1] = fma2(hi, n2, acc[1]);
+          if (pivot_thread && q == qk) { pivot[l] = lo.x; pivot[l + 1] = lo.y; pivot[l + 2] = hi.x; pivot[l + 3] = hi.y; }
         }
-        partial(l, acc);
+        const float sums[4] = {acc[0].x, acc[0].y, acc[1].x, acc[1].y};
+        const float s = warp_sums4(sums, lane);
+        if ((lane & 7) == 0 && l + (lane >> 3) < l1) part[warp * 2 * nc8 + l + (lane >> 3)] = s;
       }
     };
-    if (ng > 0) memory_columns(0, ng, [&](int l) { return A + (int64_t)(cta + l * C) * Np; });
-    if (ns > 0) memory_columns(ng, ng + ns, [&](int l) { return scols + (l - ng) * Np; });
+    if (ng > 0) {
+      auto at = [&](int l, int row) -> float& { return A[(int64_t)(cta + min(l, ng - 1) * C) * Np + row]; };
+      memory_columns(0, ng, [&](int l, int row) { return make_float4(at(l, row), at(l + 1, row), at(l + 2, row), at(l + 3, row)); },
+                     [&](int l, int row, const float4& x) {
+                       at(l, row) = x.x;
+                       if (l + 1 < ng) at(l + 1, row) = x.y;
+                       if (l + 2 < ng) at(l + 2, row) = x.z;
+                       if (l + 3 < ng) at(l + 3, row) = x.w;
+                     });
+    }
+    if (ns > 0) {
+      auto at = [&](int l, int row) -> float4& { return scols[((l - ng) >> 2) * Np + row]; };
+      memory_columns(ng, ng + ns, at, [&](int l, int row, const float4& x) { at(l, row) = x; });
+    }
 #pragma unroll
     for (int g = 0; g < RC / 8; ++g) {
       const int l = ng + ns + 8 * g;
@@ -861,7 +884,7 @@ int launch_sym_eig(const EigBuffers* w, int nb, int64_t N, int64_t r, int32_t* s
   const int64_t nq = Np <= kTriThreads ? 1 : Np <= 2 * kTriThreads ? 2 : Np <= 4 * kTriThreads ? 4 : 8;
   // (a matrix alone: 128 CTAs are faster than 148 although more of its columns spill, 4096 rows 64 -> 57 ms, 2500 25 -> 22)
   auto ctas = [&](int cnt) { return std::max<int64_t>(1, std::min<int64_t>(cnt == 1 ? std::min(sms, 128) : sms / cnt, ceil_div(N, 16))); };
-  auto in_smem = [&](int64_t C) { return std::max<int64_t>(0, (kTriSmem / 4 - (6 + 2 * kTriWarps) * (ceil_div(N, C) + 8)) / Np); };
+  auto in_smem = [&](int64_t C) { return std::max<int64_t>(0, (kTriSmem / 4 - (6 + 2 * kTriWarps) * (ceil_div(N, C) + 8)) / Np) & ~3ll; };
   int together = nb;
   while (together > 1 && ctas(together) * (64 / nq + in_smem(ctas(together))) * 5 < N * 4) --together;
   for (int first = 0; first < nb; first += together) {
