@@ -11,8 +11,8 @@
 // 3e-4 rad on rank-32 signals with noise at 1e-3 (the iterative route: 1e-4 .. 5e-3, and up to 0.4 at r = s / 8, where its
 // block of 2 r columns does not converge in 12 iterations).  It grows with lambda_1 / lambda_r; where that leaves the r-th
 // vector unresolved QG_DEV_BAD_FACTOR is raised (the iterative route met a bad pivot there and returned NaN).
-// Time (one matrix, then a batch of eight, per matrix): 768 x 2048 r 256 17.2 -> 3.0 ms; 1024 x 1024 r 256 x 8 3.7 -> 0.84;
-// 2048 x 5461 r 512 42.8 -> 9.8 and 15.3 -> 5.1; 4096 x 11008 r 1024 139 -> 56.
+// Time (one matrix, then a batch of eight, per matrix): 768 x 2048 r 256 17.2 -> 2.4 ms; 1024 x 1024 r 256 x 8 3.7 -> 0.80;
+// 2048 x 5461 r 512 42.8 -> 9.4 and 15.3 -> 4.5; 4096 x 4608 r 512 46.
 //
 // Iterative, for the rest: block subspace iteration on G G^T with a block of b = r + oversample columns, followed by a
 // Rayleigh-Ritz step that rotates the converged block onto the singular vectors.
@@ -1067,9 +1067,9 @@ static int refresh_iterative(const RefreshJob* jobs, const Batch& bt, int64_t m,
   return finish_vectors(jobs, bt, QG_TAB(const float, P32), r, m, r, false, st);
 }
 
-// The route of a shape.  Direct: the whole of the short side's Gram matrix is reduced, 4 us a row up to 1024 rows, 5 at
-// 2048, 14 at 4096.  Iterative: the cost goes with the block, whose accuracy at a small part of the spectrum is poor (above):
-// 2048 x 2048, b = 256 9.3 ms at 0.2 rad against 9.8 ms at 2e-5; 1024 x 2048, b = 64 2.5 ms against 4.
+// The route of a shape.  Direct: the whole of the short side's Gram matrix is reduced, 3 us a row up to 1024 rows, 4.5
+// at 2048, 11 at 4096.  Iterative: the cost goes with the block, whose accuracy at a small part of the spectrum is poor (above):
+// 2048 x 2048, b = 256 9.3 ms at 0.2 rad against 9.4 ms at 2e-5; 1024 x 2048, b = 64 2.5 ms against 4.
 static bool direct_route(int64_t m, int64_t n, int64_t b) {
   const int64_t s = m < n ? m : n;
   return g_jacobi_blocks && s <= kEigMax && s <= 8 * b;

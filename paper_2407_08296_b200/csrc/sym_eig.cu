@@ -41,7 +41,6 @@ using ptx::mul2;
 // A thread keeps rows tid + 512 q of every column, the last columns in registers, those before in shared memory and,
 // past that, in global memory (L2): the row's v, w, v' are then registers too, and the pass reads nothing but two
 // scalars per column.
-constexpr int kTriThreads = 512, kTriWarps = kTriThreads / 32;
 constexpr uint32_t kPollLimit = 1u << 20;
 constexpr int kTriSmem = 225 * 1024;
 
@@ -88,13 +87,13 @@ __device__ __forceinline__ float warp_sums8(const float2 (&v)[4], int lane) {
   return s;
 }
 
-template <int NQ>                              // rows per thread: N <= NQ * kTriThreads
-__global__ void __launch_bounds__(kTriThreads, 1)
+template <int NQ, int THREADS, int RC>         // rows per thread (N <= NQ * THREADS), columns in registers
+__global__ void __launch_bounds__(THREADS, 1)
 tridiagonal_kernel(const __grid_constant__ TriArgs a, int32_t* __restrict__ status) {
-  constexpr int RC = 64 / NQ;                  // columns in registers
+  constexpr int WARPS = THREADS / 32;
   extern __shared__ __align__(16) float tri_smem[];
-  __shared__ __align__(16) float4 red1[kTriWarps];
-  __shared__ float red_x[kTriWarps];
+  __shared__ __align__(16) float4 red1[16];
+  __shared__ float red_x[WARPS];
   __shared__ float s_pk, s_a1, s_v1;
   __shared__ int s_fail;
   const int N = a.N, Np = a.Np, C = a.C;
@@ -110,14 +109,14 @@ tridiagonal_kernel(const __grid_constant__ TriArgs a, int32_t* __restrict__ stat
   float* const colV = colP + 2 * nc8;          // (twice the room: a group starts anywhere)
   float* const pivot = colV + 2 * nc8;         // A_{k+1, j}
   float* const part = pivot + 2 * nc8;         // [warp][column] partial sums of P'_j
-  float4* const scols = reinterpret_cast<float4*>(part + kTriWarps * 2 * nc8);   // [group of four columns][Np]
+  float4* const scols = reinterpret_cast<float4*>(part + WARPS * 2 * nc8);   // [group of four columns][Np]
 
   float2 ar[NQ][RC / 2];
   float v[NQ], w[NQ], vn[NQ], r[NQ];
   int slot[NQ];                                // the row's own column, if it is this CTA's, else -1
 #pragma unroll
   for (int q = 0; q < NQ; ++q) {
-    const int j = tid + q * kTriThreads;
+    const int j = tid + q * THREADS;
     v[q] = w[q] = 0.f;
     r[q] = j < N ? Vg[(int64_t)(N - 1) * Np + j] : 0.f;   // row 0 as eig_scale_kernel put it aside
     slot[q] = j < N && j % C == cta ? j / C : -1;
@@ -129,13 +128,14 @@ tridiagonal_kernel(const __grid_constant__ TriArgs a, int32_t* __restrict__ stat
     }
   }
   for (int l = 0; l < ns; l += 4)
-    for (int i = tid; i < Np; i += kTriThreads) {
+    for (int i = tid; i < Np; i += THREADS) {
       float x[4];
 #pragma unroll
       for (int c = 0; c < 4; ++c) x[c] = l + c < ns ? A[(int64_t)(cta + (ng + l + c) * C) * Np + i] : 0.f;
       scols[(l >> 2) * Np + i] = make_float4(x[0], x[1], x[2], x[3]);
     }
-  for (int i = tid; i < 6 * nc8; i += kTriThreads) tri_smem[i] = 0.f;
+  for (int i = tid; i < 6 * nc8; i += THREADS) tri_smem[i] = 0.f;
+  if (tid < 16) red1[tid] = make_float4(0.f, 0.f, 0.f, 0.f);
   if (tid == 0) { s_fail = 0; s_pk = 0.f; }
   __syncthreads();
 
@@ -147,28 +147,15 @@ tridiagonal_kernel(const __grid_constant__ TriArgs a, int32_t* __restrict__ stat
   for (int k = 0; k < N && (last > k || last == N - 1); ++k) {
     const bool writer = k == N - 1 || cta == (k + 1) % C;
     // ---- receive; sums over P . v, and over a = R - tau P and v below row k + 1
-    if (k > 0) {
-      // One lane per warp waits for one of the warp's values before all of them ask for theirs: with every thread polling,
-      // the polls hold up the values themselves (768 rows 3.47 -> 3.10 ms for the whole refresh, eight of 2048 49 -> 42.5).
-      int jq = -1;
-#pragma unroll
-      for (int q = 0; q < NQ; ++q)
-        if ((tid | 31) + q * kTriThreads >= k && (tid | 31) + q * kTriThreads < N) jq = (tid | 31) + q * kTriThreads;
-      if (jq >= 0)
-        for (uint32_t polls = 0; polls < kPollLimit; ++polls) {
-          bool here = true;
-          if (lane == 0) here = ld_relaxed_v4(xchg + (k & 1) * Np + jq).y == (uint32_t)k;
-          if (__all_sync(0xFFFFFFFFu, here)) break;
-          __nanosleep(32);
-        }
-    }
     float sums[4] = {0.f, 0.f, 0.f, 0.f};
     bool ok = true;
 #pragma unroll
     for (int q = 0; q < NQ; ++q) {
-      const int j = tid + q * kTriThreads;
-      // (the whole warp stays in the loop: lanes that left it one by one would run on by themselves, and a CTA barrier counts
-      // a warp as arrived with the first of them)
+      const int j = tid + q * THREADS;
+      // The whole warp stays in the loop: lanes that left it one by one would run on by themselves, and a CTA barrier counts a
+      // warp as arrived with the first of them.  Row after row: with all of a thread's words asked for at once the polls hold
+      // up the words themselves (2048 x 5461: 9.4 ms as it is, 14.3 at once); a lane that waits alone for the rest of its warp
+      // adds a trip (10.3).
       const bool wanted = k > 0 && j >= k && j < N;
       const uint4* const in = xchg + (k & 1) * Np + j;
       uint4 got = make_uint4(0, 0, 0, 0);
@@ -227,7 +214,7 @@ tridiagonal_kernel(const __grid_constant__ TriArgs a, int32_t* __restrict__ stat
     float sig = fmaf(mu, fmaf(mu, s_vv, 2.f * s_av), s_aa);
 #pragma unroll
     for (int q = 0; q < NQ; ++q) {
-      const int j = tid + q * kTriThreads;
+      const int j = tid + q * THREADS;
       w[q] = fmaf(tau, w[q], -kappa * v[q]);
       r[q] = fmaf(mu, v[q], r[q]);             // x
       if (j == k && writer) a.d.p[mat][k] = r[q];
@@ -237,12 +224,12 @@ tridiagonal_kernel(const __grid_constant__ TriArgs a, int32_t* __restrict__ stat
       sig = 0.f;
 #pragma unroll
       for (int q = 0; q < NQ; ++q)
-        if (tid + q * kTriThreads > k + 1) sig = fmaf(r[q], r[q], sig);
+        if (tid + q * THREADS > k + 1) sig = fmaf(r[q], r[q], sig);
       sig = warp_sum(sig);
       if (lane == 0) red_x[warp] = sig;
       __syncthreads();
       sig = 0.f;
-      for (int i = 0; i < kTriWarps; ++i) sig += red_x[i];
+      for (int i = 0; i < WARPS; ++i) sig += red_x[i];
     }
     const float tau_old = tau;
     float beta = alpha, scl = 0.f;
@@ -255,15 +242,15 @@ tridiagonal_kernel(const __grid_constant__ TriArgs a, int32_t* __restrict__ stat
     }
 #pragma unroll
     for (int q = 0; q < NQ; ++q) {
-      const int j = tid + q * kTriThreads;
+      const int j = tid + q * THREADS;
       vn[q] = j > k + 1 ? r[q] * scl : (j == k + 1 ? 1.f : 0.f);
       if (writer && j < Np) Vg[(int64_t)k * Np + j] = vn[q];
     }
     if (writer && tid == 0) { a.tau.p[mat][k] = tau; a.e.p[mat][k] = beta; }
 
     // ---- the pass, eight columns at a time
-    const int k1 = k + 1, qk = k1 / kTriThreads;
-    const bool pivot_thread = tid == k1 % kTriThreads;
+    const int k1 = k + 1, qk = k1 / THREADS;
+    const bool pivot_thread = tid == k1 % THREADS;
     const float2 tau2 = both(tau_old), kap2 = both(-kappa);
     auto scalars = [&](int l, float2 (&wj)[4], float2 (&vj)[4]) {      // w_j, v_j of columns l .. l + 7
 #pragma unroll
@@ -278,7 +265,7 @@ tridiagonal_kernel(const __grid_constant__ TriArgs a, int32_t* __restrict__ stat
     };
     // columns in memory, four to a load (get(l, row), put(l, row, x): columns l .. l + 3), the next row's on its way
     auto memory_columns = [&](int l0, int l1, auto get, auto put) {
-      const int q0 = k1 / kTriThreads;
+      const int q0 = k1 / THREADS;
       for (int l = l0; l < l1; l += 4) {
         if (cta + min(l + 3, l1 - 1) * C <= k) continue;               // all of them retired
         float2 wj[2], vj[2], acc[2] = {};
@@ -288,13 +275,13 @@ tridiagonal_kernel(const __grid_constant__ TriArgs a, int32_t* __restrict__ stat
           wj[c] = fma2(tau2, make_float2(colP[l + 2 * c], colP[l + 2 * c + 1]), mul2(kap2, vj[c]));
         }
         float4 next = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (tid + q0 * kTriThreads < Np) next = get(l, tid + q0 * kTriThreads);
+        if (tid + q0 * THREADS < Np) next = get(l, tid + q0 * THREADS);
 #pragma unroll
         for (int q = 0; q < NQ; ++q) {
-          const int row = tid + q * kTriThreads;
-          if (q * kTriThreads + kTriThreads - 1 <= k || row >= Np) continue;
+          const int row = tid + q * THREADS;
+          if (q * THREADS + THREADS - 1 <= k || row >= Np) continue;
           float2 lo = make_float2(next.x, next.y), hi = make_float2(next.z, next.w);
-          if (q + 1 < NQ && row + kTriThreads < Np) next = get(l, row + kTriThreads);
+          if (q + 1 < NQ && row + THREADS < Np) next = get(l, row + THREADS);
           const float2 nv = both(-v[q]), nw = both(-w[q]), n2 = both(vn[q]);
           lo = fma2(nw, vj[0], fma2(nv, wj[0], lo));
           hi = fma2(nw, vj[1], fma2(nv, wj[1], hi));
@@ -330,7 +317,7 @@ tridiagonal_kernel(const __grid_constant__ TriArgs a, int32_t* __restrict__ stat
         scalars(l, wj, vj);
 #pragma unroll
         for (int q = 0; q < NQ; ++q) {
-          if (q * kTriThreads + kTriThreads - 1 <= k) continue;
+          if (q * THREADS + THREADS - 1 <= k) continue;
           const float2 nv = both(-v[q]), nw = both(-w[q]), n2 = both(vn[q]);
 #pragma unroll
           for (int c = 0; c < 4; ++c) {
@@ -345,12 +332,12 @@ tridiagonal_kernel(const __grid_constant__ TriArgs a, int32_t* __restrict__ stat
     }
     __syncthreads();
     // ---- publish
-    for (int l = tid; l < ncols; l += kTriThreads) {
+    for (int l = tid; l < ncols; l += THREADS) {
       const int j = cta + l * C;
       if (j <= k) continue;
       float s = 0.f;
 #pragma unroll
-      for (int i = 0; i < kTriWarps; ++i) s += part[i * 2 * nc8 + l];
+      for (int i = 0; i < WARPS; ++i) s += part[i * 2 * nc8 + l];
       st_relaxed_v4(xchg + (k1 & 1) * Np + j, s, pivot[l], (uint32_t)k1);
     }
     __syncwarp();
@@ -794,14 +781,14 @@ int opt_in(K kernel, int bytes, bool* done) {
   return QG_OK;
 }
 
-template <int NQ>
+template <int NQ, int THREADS, int RC>
 int launch_tridiagonal(TriArgs a, int nb, int32_t* status, cudaStream_t st) {
   static bool done[kDevices] = {};
-  auto kern = tridiagonal_kernel<NQ>;
+  auto kern = tridiagonal_kernel<NQ, THREADS, RC>;
   const int rc = opt_in(kern, kTriSmem, done);
   if (rc != QG_OK) return rc;
   void* args[] = {&a, &status};
-  return launch_cooperative((const void*)kern, (unsigned)(a.C * nb), kTriThreads, args, (size_t)kTriSmem, st);
+  return launch_cooperative((const void*)kern, (unsigned)(a.C * nb), THREADS, args, (size_t)kTriSmem, st);
 }
 
 template <int NCH, int VW, int WARPS>
@@ -881,12 +868,24 @@ int launch_sym_eig(const EigBuffers* w, int nb, int64_t N, int64_t r, int32_t* s
   // Matrices reduced together share the SMs; as many as stay (all but a fifth of their columns, the first to retire) in
   // registers and shared memory.
   const int sms = sm_count();
-  const int64_t nq = Np <= kTriThreads ? 1 : Np <= 2 * kTriThreads ? 2 : Np <= 4 * kTriThreads ? 4 : 8;
+  // Threads: as few rows without a column's element as may be, every warp repeats the step's scalars and reductions (768 rows:
+  // 3.0 ms with 512 threads, 2.8 with 384).  Columns in registers: the loop should stay in the instruction cache, so only 16
+  // where a CTA has no more (768 rows 2.9 -> 2.7 ms against 40).
+  using Launch = int (*)(TriArgs, int, int32_t*, cudaStream_t);
+  struct Shape { int threads, columns; Launch few, many; };                // columns in registers: 16 if that is all, or `columns`
+  const Shape f = Np <= 256    ? Shape{256, 32, launch_tridiagonal<1, 256, 16>, launch_tridiagonal<1, 256, 32>}
+                  : Np <= 512  ? Shape{256, 32, launch_tridiagonal<2, 256, 16>, launch_tridiagonal<2, 256, 32>}
+                  : Np <= 768  ? Shape{384, 32, launch_tridiagonal<2, 384, 16>, launch_tridiagonal<2, 384, 32>}
+                  : Np <= 1024 ? Shape{512, 32, launch_tridiagonal<2, 512, 16>, launch_tridiagonal<2, 512, 32>}
+                  : Np <= 1536 ? Shape{384, 16, launch_tridiagonal<4, 384, 16>, launch_tridiagonal<4, 384, 16>}
+                  : Np <= 2048 ? Shape{512, 16, launch_tridiagonal<4, 512, 16>, launch_tridiagonal<4, 512, 16>}
+                  : Np <= 3072 ? Shape{384, 8, launch_tridiagonal<8, 384, 8>, launch_tridiagonal<8, 384, 8>}
+                               : Shape{512, 8, launch_tridiagonal<8, 512, 8>, launch_tridiagonal<8, 512, 8>};
   // (a matrix alone: 128 CTAs are faster than 148 although more of its columns spill, 4096 rows 64 -> 57 ms, 2500 25 -> 22)
   auto ctas = [&](int cnt) { return std::max<int64_t>(1, std::min<int64_t>(cnt == 1 ? std::min(sms, 128) : sms / cnt, ceil_div(N, 16))); };
-  auto in_smem = [&](int64_t C) { return std::max<int64_t>(0, (kTriSmem / 4 - (6 + 2 * kTriWarps) * (ceil_div(N, C) + 8)) / Np) & ~3ll; };
+  auto in_smem = [&](int64_t C) { return std::max<int64_t>(0, (kTriSmem / 4 - (6 + f.threads / 16) * (ceil_div(N, C) + 8)) / Np) & ~3ll; };
   int together = nb;
-  while (together > 1 && ctas(together) * (64 / nq + in_smem(ctas(together))) * 5 < N * 4) --together;
+  while (together > 1 && ctas(together) * (f.columns + in_smem(ctas(together))) * 5 < N * 4) --together;
   for (int first = 0; first < nb; first += together) {
     const int cnt = std::min(together, nb - first);
     TriArgs a{};
@@ -897,10 +896,7 @@ int launch_sym_eig(const EigBuffers* w, int nb, int64_t N, int64_t r, int32_t* s
     a.N = (int)N; a.Np = (int)Np;
     a.C = (int)ctas(cnt);
     a.in_smem = (int)in_smem(a.C);
-    const int rc = nq == 1   ? launch_tridiagonal<1>(a, cnt, status, st)
-                   : nq == 2 ? launch_tridiagonal<2>(a, cnt, status, st)
-                   : nq == 4 ? launch_tridiagonal<4>(a, cnt, status, st)
-                             : launch_tridiagonal<8>(a, cnt, status, st);
+    const int rc = (ceil_div(N, a.C) <= 16 ? f.few : f.many)(a, cnt, status, st);
     if (rc != QG_OK) return rc;
   }
   {
