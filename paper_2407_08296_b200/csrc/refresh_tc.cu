@@ -327,7 +327,8 @@ gram_kernel(const __grid_constant__ GramArgs a, int nmat, int32_t* __restrict__ 
       for (int i = 0; i < 128; ++i) sum[i] = 0.f;
       for (int kb = 0; kb < kblocks; kb += S::kSegment, ++seg) {
         const uint32_t ab = seg & 1;
-        if (!mbar_wait(&acc_full[ab], (seg >> 1) & 1)) { ok = false; break; }
+        ok = mbar_wait_warp(&acc_full[ab], (seg >> 1) & 1);
+        if (!ok) break;
         tc_fence_after_sync();
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
@@ -342,30 +343,33 @@ gram_kernel(const __grid_constant__ GramArgs a, int nmat, int32_t* __restrict__ 
         if (lane == 0) mbar_arrive(&acc_empty[ab]);
       }
       const int row = mb * kTileM + q * 32 + lane;
-      if (!ok || row >= a.N) continue;
       const bool mirror = mb / 2 > nb;                 // no tile of the triangle covers the mirror image
+      if (ok && row < a.N) {
 #pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        const int col = nb * kTileN + half * 128 + 32 * c;
-        if (col + 32 <= a.N) {
+        for (int c = 0; c < 4; ++c) {
+          const int col = nb * kTileN + half * 128 + 32 * c;
+          if (col + 32 <= a.N) {
 #pragma unroll
-          for (int i = 0; i < 8; ++i)
-            *reinterpret_cast<float4*>(A + (int64_t)row * a.lda + col + 4 * i) =
-                make_float4(sum[32 * c + 4 * i], sum[32 * c + 4 * i + 1], sum[32 * c + 4 * i + 2], sum[32 * c + 4 * i + 3]);
-        } else {
+            for (int i = 0; i < 8; ++i)
+              *reinterpret_cast<float4*>(A + (int64_t)row * a.lda + col + 4 * i) =
+                  make_float4(sum[32 * c + 4 * i], sum[32 * c + 4 * i + 1], sum[32 * c + 4 * i + 2], sum[32 * c + 4 * i + 3]);
+          } else {
 #pragma unroll
-          for (int i = 0; i < 32; ++i)
-            if (col + i < a.N) A[(int64_t)row * a.lda + col + i] = sum[32 * c + i];
-        }
-        if (mirror) {                                  // 32 lanes: 128 contiguous bytes of a row
+            for (int i = 0; i < 32; ++i)
+              if (col + i < a.N) A[(int64_t)row * a.lda + col + i] = sum[32 * c + i];
+          }
+          if (mirror) {                                // 32 lanes: 128 contiguous bytes of a row
 #pragma unroll
-          for (int i = 0; i < 32; ++i)
-            if (col + i < a.N) A[(int64_t)(col + i) * a.lda + row] = sum[32 * c + i];
+            for (int i = 0; i < 32; ++i)
+              if (col + i < a.N) A[(int64_t)(col + i) * a.lda + row] = sum[32 * c + i];
+          }
         }
       }
+      __syncwarp();                                    // the next tile's loads from tensor memory are the whole warp's
     }
     if (!ok && lane == 0) raise_expired(status);
   }
+  __syncwarp();                                        // also the warps of which one lane had a role
   tc_fence_before_sync();
   __syncthreads();
   if (warp == 1) {

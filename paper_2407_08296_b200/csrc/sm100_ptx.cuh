@@ -50,6 +50,10 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
   return false;
 }
 
+// The same by a whole warp, which leaves the wait together and with one answer: what follows may be warp-collective (the
+// .aligned instructions below).  Lanes that left a loop one by one need not have met again.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity) { return __all_sync(0xFFFFFFFFu, mbar_wait(bar, parity)); }
+
 // ----------------------------------------------------------------------------- packed fp32
 // Packed fp32 pairs (one instruction for two lanes of a float2).
 __device__ __forceinline__ float2 mul2(float2 a, float2 b) {

@@ -66,3 +66,17 @@ def test_coinciding_eigenvalues_have_orthogonal_vectors(kind):
     P = torch.zeros((256, 64), device="cuda")
     B.refresh_subspace(G, 64, P_fp32=P)
     assert float((P.T @ P - torch.eye(64, device="cuda")).abs().max()) <= 1e-5
+
+
+# More tiles of the Gram matrix than CTAs, its last rows inside a warp (1400 = 10 * 128 + 120, 2000 = 15 * 128 + 80), read along
+# the gradient's rows (m < n) and along its columns, for vectors of the short side and of the long one.
+@pytest.mark.parametrize("m,n,r", [(1400, 1600, 192), (1600, 1400, 192), (2000, 2300, 256), (2300, 2000, 256)])
+@pytest.mark.parametrize("side", ["left", "right"])
+def test_batches_of_odd_gradients_from_both_sides(m, n, r, side):
+    rows = m if side == "left" else n
+    items = [{"G": _gradient(m, n, seed=40 + i), "seed": i, "P_fp32": torch.zeros((rows, r), device="cuda")} for i in range(8)]
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    B.refresh_subspace_batched(items, r, status=status, side=side)
+    assert int(status.item()) == 0
+    for it in items[::3]:
+        _check(it["G"], it["P_fp32"], side)
