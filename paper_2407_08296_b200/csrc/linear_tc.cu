@@ -344,7 +344,8 @@ int8_linear_kernel(const __grid_constant__ LinArgs a, int32_t* __restrict__ stat
     for (int t = wk.first; ok && t < wk.end; t += wk.stride, ++tcount) {
       const int m0 = (t % a.mblocks) * (MT * 2 * kTileM) + (int)wk.half * kTileM, n0 = (t / a.mblocks) * kTileN;
       const uint32_t ab = MT == 1 ? (tcount & 1) : 0u, use = MT == 1 ? (tcount >> 1) : tcount;
-      if (!mbar_wait(&acc_full[ab], use & 1)) { ok = false; break; }
+      ok = mbar_wait_warp(&acc_full[ab], use & 1);
+      if (!ok) break;
       tc_fence_after_sync();
       if (a.split > 1) break;                          // see the end of the kernel
 #pragma unroll 1
@@ -371,11 +372,10 @@ int8_linear_kernel(const __grid_constant__ LinArgs a, int32_t* __restrict__ stat
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
             const int row = m0 + h * 2 * kTileM + q * 32 + (lane & ~3) + i;
-            if (row >= a.rows || col >= a.cols) continue;
             uint16_t* d = a.D + (int64_t)row * a.ldd + col;
-            if (col + 8 <= a.cols) {
+            if (row < a.rows && col + 8 <= a.cols) {
               *reinterpret_cast<uint4*>(d) = pk[i];
-            } else {
+            } else if (row < a.rows && col < a.cols) {
               const uint32_t u[4] = {pk[i].x, pk[i].y, pk[i].z, pk[i].w};
 #pragma unroll
               for (int e = 0; e < 8; ++e)
@@ -383,6 +383,7 @@ int8_linear_kernel(const __grid_constant__ LinArgs a, int32_t* __restrict__ stat
             }
           }
         }
+        __syncwarp();                                  // the next loads from tensor memory are the whole warp's
       }
     }
     if (!ok && lane == 0) raise_expired(status);
@@ -418,7 +419,8 @@ int8_linear_kernel(const __grid_constant__ LinArgs a, int32_t* __restrict__ stat
         bw.advance(S::kGroups);
         fetch(bw);
         const int rs = it % S::kRawStages, s = it % S::kStages;
-        if (!mbar_wait(&raw_full[rs], (it / S::kRawStages) & 1) || !mbar_wait(&empty[s], ((it / S::kStages) & 1) ^ 1)) { ok = false; break; }
+        ok = mbar_wait_warp(&raw_full[rs], (it / S::kRawStages) & 1) && mbar_wait_warp(&empty[s], ((it / S::kStages) & 1) ^ 1);
+        if (!ok) break;
         const uint8_t* raw = raw_base + rs * S::kRawBytes;
         uint8_t* sB = stage_base + s * S::kStageBytes + S::kABytes;
         if (MODE == kForward) {
@@ -460,10 +462,11 @@ int8_linear_kernel(const __grid_constant__ LinArgs a, int32_t* __restrict__ stat
     if (!ok && lane == 0) raise_expired(status);
   }
 
+  __syncwarp();                                        // one lane of the warps 0 to 2 had a role: the warp goes on together
   if (a.split > 1) {
     // Every MMA of the tile is complete, so the operand stages are free: they hold the sums on their way.  All warps but the
-    // first four add up and store, sixteen columns at a time, whatever share of the tile this CTA has.
-    __syncwarp();
+    // first four add up and store, sixteen columns at a time, whatever share of the tile this CTA has.  The cluster barriers
+    // count warps: only stores are under a condition of the lane, and every warp joins before each of them.
     const int q = warp & 3, row = q * 32 + lane;
     const int m0 = (wk.first % a.mblocks) * (MT * 2 * kTileM) + (int)wk.half * kTileM, n0 = (wk.first / a.mblocks) * kTileN;
 #pragma unroll 1
@@ -478,6 +481,7 @@ int8_linear_kernel(const __grid_constant__ LinArgs a, int32_t* __restrict__ stat
           dump_piece(stage_base, c, row, v);
         }
       }
+      __syncwarp();
       cluster_sync_all();
       if (some && warp >= 4) {
 #pragma unroll 1
@@ -485,18 +489,18 @@ int8_linear_kernel(const __grid_constant__ LinArgs a, int32_t* __restrict__ stat
           uint32_t pk[8];
           sum_columns16(stage_base, j, row, wk.half, a.split, pk);
           const int gr = m0 + h * 2 * kTileM + row, col = n0 + 16 * j;
-          if (gr >= a.rows) continue;
           uint16_t* d = a.D + (int64_t)gr * a.ldd + col;
-          if (col + 16 <= a.cols) {
+          if (gr < a.rows && col + 16 <= a.cols) {
             *reinterpret_cast<uint4*>(d) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
             *reinterpret_cast<uint4*>(d + 8) = make_uint4(pk[4], pk[5], pk[6], pk[7]);
-          } else {
+          } else if (gr < a.rows) {
 #pragma unroll
             for (int i = 0; i < 16; ++i)
               if (col + i < a.cols) d[i] = (uint16_t)((i & 1) ? (pk[i >> 1] >> 16) : (pk[i >> 1] & 0xFFFFu));
           }
         }
       }
+      __syncwarp();
       if (h + 1 < MT) cluster_sync_all();          // nobody refills its sums before all have read them
     }
     grid_dependency_wait();                            // the launch before this one, which it may have overtaken

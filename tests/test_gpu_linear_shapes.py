@@ -64,3 +64,11 @@ def test_products_whose_tiles_are_split_along_k(T, m, n):
     _check(G, d.T, x, status)
     for again, first in ((B.int8_linear_forward(X, W), Y), (B.int8_linear_backward_input(dY, W), dX), (B.int8_linear_backward_weight(dYz, Xz), G)):
         assert torch.equal(again, first)
+
+
+# Tiles shared by clusters whose last row ends inside a warp: 1337 = 5 * 256 + 57 rows leave one CTA of a pair 57 and the other
+# none; 3001 = 5 * 512 + 441, of which 57 in the second CTA's second row block, after whole rounds of persistent pairs (the forward
+# product and the input gradient; the weight gradient of either shape ends its columns and K inside a tile).
+@pytest.mark.parametrize("T,m,n", [(1337, 4096, 4096), (3001, 11008, 4096)])
+def test_split_products_whose_rows_end_inside_a_warp(T, m, n):
+    test_products_whose_tiles_are_split_along_k(T, m, n)
