@@ -157,7 +157,8 @@ split_gemm_kernel(const __grid_constant__ SplitArgs a, int32_t* __restrict__ sta
     for (int t = blockIdx.x; ok && t < total; t += gridDim.x, ++tcount) {
       const int m0 = (t % a.mblocks) * kTileM, n0 = (t / a.mblocks) * kTileN;
       const uint32_t ab = tcount & 1;
-      if (!mbar_wait(&acc_full[ab], (tcount >> 1) & 1)) { ok = false; break; }
+      ok = mbar_wait_warp(&acc_full[ab], (tcount >> 1) & 1);
+      if (!ok) break;
       tc_fence_after_sync();
       const uint32_t tacc = tmem_base + ((uint32_t)(q * 32) << 16) + ab * kTileN;
       const int row = m0 + q * 32 + lane;
@@ -184,11 +185,13 @@ split_gemm_kernel(const __grid_constant__ SplitArgs a, int32_t* __restrict__ sta
               if (col + i < a.N) drow[col + i] = __uint_as_float(v[i]);
           }
         }
+        __syncwarp();                                  // the next loads from tensor memory are the whole warp's
       }
     }
     if (!ok && lane == 0) raise_expired(status);
   }
 
+  __syncwarp();                                        // also the warps of which one lane had a role
   tc_fence_before_sync();
   __syncthreads();
   if (warp == 1) {

@@ -820,6 +820,7 @@ project_adam_kernel(const __grid_constant__ TcProblem single, const TcProblem* _
     if (!ok && lane == 0) raise_wait_expired(status);
   }
 
+  __syncwarp();                                   // also the warps of which one lane had a role
   tc_fence_before_sync();
   __syncthreads();
   if (CTAS == 2) cluster_sync_all();              // neither CTA leaves while the other may still signal it
@@ -1181,7 +1182,7 @@ backproject_sr_kernel(const __grid_constant__ TcProblem single, const TcProblem*
       float s_old = 1.f, z_old = 0.f;
       if (row_ok) { s_old = __ldg(g_scale); z_old = __ldg(g_zero); }
       const uint32_t ab = tcount & 1;                // == grp: a group always drains the same accumulator buffer
-      ok = mbar_wait(&code_full[grp], (tcount >> 1) & 1) && mbar_wait(&acc_full[ab], (tcount >> 1) & 1);
+      ok = mbar_wait_warp(&code_full[grp], (tcount >> 1) & 1) && mbar_wait_warp(&acc_full[ab], (tcount >> 1) & 1);
       ok = named_bar_and(bar_id, S::kGroupThreads, ok);
       if (!ok) break;
       tc_fence_after_sync();
@@ -1278,6 +1279,7 @@ backproject_sr_kernel(const __grid_constant__ TcProblem single, const TcProblem*
           for (int e = 0; e < 16; ++e)
             if (col + e < pn) dbgW[col + e] = w[e];
         }
+        __syncwarp();                                   // what follows in tensor memory is the whole warp's
       };
       {
         uint32_t a0[16], a1[16];
@@ -1307,6 +1309,7 @@ backproject_sr_kernel(const __grid_constant__ TcProblem single, const TcProblem*
     if (!ok && lane == 0) raise_wait_expired(status);
   }
 
+  __syncwarp();                                   // also the warps of which one lane had a role
   tc_fence_before_sync();
   __syncthreads();
   if (CTAS == 2) cluster_sync_all();              // neither CTA leaves while the other may still signal it
