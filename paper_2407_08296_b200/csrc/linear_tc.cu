@@ -512,6 +512,8 @@ int8_linear_kernel(const __grid_constant__ LinArgs a, int32_t* __restrict__ stat
     tc_fence_after_sync();
     tmem_dealloc_pair(tmem_base, 512);
   }
+  __syncwarp();
+  cluster_sync_all();                              // nor while its peer still gives tensor memory back: see tmem_dealloc_pair
 }
 
 constexpr int kDevices = 64, kMaxSplit = 4;

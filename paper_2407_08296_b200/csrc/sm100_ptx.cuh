@@ -261,6 +261,9 @@ __device__ __forceinline__ void tmem_alloc_pair(uint32_t* smem_result, uint32_t 
 __device__ __forceinline__ void tmem_relinquish_pair() {
   asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
 }
+// Both CTAs of the pair perform this together.  A cluster barrier has to follow it: the SM of a CTA that left while its peer was
+// still deallocating could take a CTA of the next launch (which may overlap this one) and allocate there, with cta_group::1
+// perhaps, beside a deallocation that spans both SMs.
 __device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t ncols) {
   asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
 }

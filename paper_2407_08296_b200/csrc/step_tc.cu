@@ -828,6 +828,7 @@ project_adam_kernel(const __grid_constant__ TcProblem single, const TcProblem* _
     tc_fence_after_sync();
     if (CTAS == 2) tmem_dealloc_pair(tmem_base, 2 * BN); else tmem_dealloc(tmem_base, 2 * BN);
   }
+  if (CTAS == 2) { __syncwarp(); cluster_sync_all(); }   // nor while it still gives tensor memory back: see tmem_dealloc_pair
 }
 
 // ============================================================================================
@@ -1317,6 +1318,7 @@ backproject_sr_kernel(const __grid_constant__ TcProblem single, const TcProblem*
     tc_fence_after_sync();
     if (CTAS == 2) tmem_dealloc_pair(tmem_base, 512); else tmem_dealloc(tmem_base, 512);
   }
+  if (CTAS == 2) { __syncwarp(); cluster_sync_all(); }   // nor while it still gives tensor memory back: see tmem_dealloc_pair
 }
 
 // ============================================================================================
