@@ -13,6 +13,16 @@ namespace qg {
 // once every CTA of that launch has called grid_launch_dependents or left.  The kernel has to call grid_dependency_wait
 // before it touches anything an earlier launch may write or read; a launch before it that knows nothing of this (another
 // library's kernel, a copy) is simply waited for.  `cluster`: CTAs per cluster; `overlap` = false: an ordinary launch.
+//
+// What keeps this sound:
+//  - A kernel calls grid_launch_dependents only after its own grid_dependency_wait (or in an ordinary launch), so a launch begins
+//    when the one before the one before it is complete: two are in flight at most, and what a kernel reads through the read-only
+//    path (scales that an earlier step wrote, a new projection) was written by CTAs that had left before this launch began.
+//  - It calls it only when its CTA has its tensor memory.  tcgen05.alloc waits without a limit: a CTA of the later launch that took
+//    an SM's columns first, and then waited for the earlier launch, would never give them back.  No two CTAs that allocate tensor
+//    memory fit an SM together either: each such kernel takes more than half of its shared memory.
+constexpr int kHalfOfSharedMemory = 228 * 1024 / 2;
+
 template <class... Params, class... Args>
 int launch_overlapping(void (*kern)(Params...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, unsigned cluster, bool overlap,
                        Args&&... args) {

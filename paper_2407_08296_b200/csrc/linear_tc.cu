@@ -30,7 +30,7 @@
 #include <atomic>
 #include <cstring>
 
-#include "qg_common.cuh"
+#include "launch.cuh"
 #include "sm100_ptx.cuh"
 #include "tensor_map.cuh"
 
@@ -151,6 +151,7 @@ struct LinSmem {
   static constexpr int kEpiWarps = 4, kConvWarps = 4 * kGroups;
   static constexpr int kThreads = (4 + kEpiWarps + kConvWarps) * 32;
   static_assert(kBytes <= 227 * 1024, "shared memory budget");
+  static_assert(kBytes > kHalfOfSharedMemory, "see launch_overlapping");
 };
 
 __device__ __forceinline__ void raise_expired(int32_t* status) {
@@ -224,7 +225,6 @@ int8_linear_kernel(const __grid_constant__ LinArgs a, int32_t* __restrict__ stat
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 2);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (a.split == 1) grid_launch_dependents();
   if (threadIdx.x == 0) {
     for (int i = 0; i < S::kStages; ++i) {
       mbar_init(&full[i], S::kConvert ? 1 + 2 * 4 : 1);   // the leader's TMA producer, and one group of converter warps per CTA
@@ -241,6 +241,8 @@ int8_linear_kernel(const __grid_constant__ LinArgs a, int32_t* __restrict__ stat
   cluster_sync_all();                              // the other CTAs' barriers exist before anything signals them
   tc_fence_after_sync();
   const uint32_t tmem_base = *tmem_slot;
+  // Whole rounds are an ordinary launch, so everything before them is complete; the shared tiles behind them let nobody begin.
+  if (a.split == 1) grid_launch_dependents();
 
   // tile t -> (m block, n block): consecutive tiles (concurrent pairs) share the n block, i.e. the same
   // columns of B, which for two of the three products is the weight.  `full` and `acc_empty` are the leader's.

@@ -17,8 +17,8 @@ constexpr int kTM = 32, kTN = 256, kTK = 32;
 
 __global__ void __launch_bounds__(256)
 dequant_p_bf16_kernel(qg_qtensor P, uint16_t* __restrict__ out, int64_t ld_out) {
-  ptx::grid_launch_dependents();
   ptx::grid_dependency_wait();
+  ptx::grid_launch_dependents();
   const int ngroups = (int)((P.cols + kGroup - 1) / kGroup);
   const int64_t chunks = P.cols / 8;                 // r % 32 == 0
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;

@@ -262,7 +262,6 @@ project_adam_kernel(const __grid_constant__ TcProblem single, const TcProblem* _
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const TcProblem* probs = SINGLE ? &single : table;
-  grid_launch_dependents();
 
   if (threadIdx.x == 0) {
     // a stage is full once the producer's copies have landed and, in a launch some matrix of which has its A tile
@@ -287,6 +286,7 @@ project_adam_kernel(const __grid_constant__ TcProblem single, const TcProblem* _
   tc_fence_after_sync();
   const uint32_t tmem_base = *tmem_slot;
   grid_dependency_wait();                         // everything up to here overlaps the end of the launch before
+  grid_launch_dependents();                       // the launch before is complete: two are in flight at most
 
   // tile -> (r block, n block) of its problem; consecutive tiles share the n block, so that the G tile
   // one of them brings from HBM serves the others from L2.  A pair takes two adjacent r blocks (this CTA the
@@ -1026,7 +1026,6 @@ backproject_sr_kernel(const __grid_constant__ TcProblem single, const TcProblem*
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const TcProblem* probs = SINGLE ? &single : table;
-  grid_launch_dependents();
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < S::kStages; ++i) { mbar_init(&full[i], 1); mbar_init(&empty[i], 1); }
@@ -1045,6 +1044,7 @@ backproject_sr_kernel(const __grid_constant__ TcProblem single, const TcProblem*
   tc_fence_after_sync();
   const uint32_t tmem_base = *tmem_slot;
   grid_dependency_wait();                         // everything up to here overlaps the end of the launch before
+  grid_launch_dependents();                       // the launch before is complete: two are in flight at most
 
   // tile -> (m block, n block) of its problem; consecutive tiles share the n block of N_b.  A pair takes two
   // adjacent m blocks, this CTA the one of its rank; the leader's `full` barriers count the loads of both CTAs
@@ -1452,6 +1452,7 @@ template <int BN, bool SINGLE, int CTAS, bool S8 = false, int MVS = 0>
 int launch_k1(const TcProblem* single, const TcProblem* table, const TileSchedule& sched, int grid_planned,
               int total_tiles, const StepScalars& sc, int32_t* status, cudaStream_t st, int conv_active) {
   using S = K1Smem<BN, CTAS, MVS>;
+  static_assert(S::kBytes > kHalfOfSharedMemory, "see launch_overlapping");
   auto kern = project_adam_kernel<BN, SINGLE, CTAS, S8, MVS>;
   static bool smem_set[64] = {};
   int rc = set_smem_once(kern, S::kBytes, smem_set);
@@ -1467,6 +1468,7 @@ template <bool SINGLE, int CTAS>
 int launch_k2(const TcProblem* single, const TcProblem* table, const TileSchedule& sched, int grid_planned,
               int total_tiles, const StepScalars& sc, int32_t* status, cudaStream_t st) {
   using S = typename std::conditional<CTAS == 2, K2PairSmem, K2Smem>::type;
+  static_assert(S::kBytes > kHalfOfSharedMemory, "see launch_overlapping");
   auto kern = backproject_sr_kernel<SINGLE, CTAS>;
   static bool smem_set[64] = {};
   int rc = set_smem_once(kern, S::kBytes, smem_set);
@@ -1516,9 +1518,9 @@ constexpr int kDqUnits = 8;
 
 __global__ void __launch_bounds__(256)
 dequant_p_grouped_kernel(const DequantItem* __restrict__ items, const int32_t* __restrict__ block_item) {
-  grid_launch_dependents();
   const DequantItem& it = items[__ldg(block_item + blockIdx.x)];   // host-made map: block -> matrix of the chunk
   grid_dependency_wait();
+  grid_launch_dependents();
   const uint32_t cols = (uint32_t)it.P.cols, rows = (uint32_t)it.P.rows;
   const uint32_t per_row = cols / 8, ngroups = (cols + kGroup - 1) / kGroup, total = rows * per_row;   // r % 32 == 0
   const uint32_t base = (blockIdx.x - (uint32_t)it.block0) * (kDqUnits * 256u) + threadIdx.x;
