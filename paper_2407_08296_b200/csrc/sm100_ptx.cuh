@@ -231,12 +231,30 @@ __device__ __forceinline__ uint32_t mapa_u32(uint32_t local_addr, uint32_t rank)
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(local_addr), "r"(rank));
   return r;
 }
-// An arrival on a barrier of another CTA of the cluster that orders this thread's writes for its own CTA only.  Enough for an
-// operand that the tensor core of THIS SM reads (shared memory behind a proxy fence) whoever issues the MMA, and for an
-// accumulator handed back (tensor memory behind tcgen05.wait::ld).  At cluster scope the arrival holds its thread up for 900
-// to 1300 clocks, until all of its loads and stores, global ones too, are done: LLaMA-7B step as pairs 3510 -> 3460 us.
+// An arrival on a barrier of another CTA of the cluster, and a wait for a barrier that other CTAs arrive on: cluster scope on both
+// sides, which is what orders anything between two CTAs.  The release holds its thread up until all of its loads and stores,
+// global ones too, are done (900 to 1300 clocks in an epilogue).
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
+}
+// The same, ordering this thread's writes for its own CTA only.
 __device__ __forceinline__ void mbar_arrive_remote(uint32_t cluster_addr) {
   asm volatile("mbarrier.arrive.release.cta.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
+}
+// Bounded wait on a barrier of this CTA that is also signalled from the peer CTA (acquire at cluster scope).
+__device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity) {
+  for (uint32_t i = 0; i < kWaitPollLimit; ++i) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(smem_u32(bar)), "r"(parity)
+        : "memory");
+    if (ok) return true;
+  }
+  return false;
 }
 // TMA loads whose completion is counted on a barrier that may live in the peer CTA (no multicast: the data
 // lands in the executing CTA's own shared memory only).

@@ -382,12 +382,16 @@ project_adam_kernel(const __grid_constant__ TcProblem single, const TcProblem* _
         const uint32_t idesc = right ? idesc_right : idesc_left;
         const uint64_t bstep = right ? (32 >> 4) : (2048 >> 4);   // 16 K indices further along B
         const uint32_t ab = tcount & 1;
-        if (!mbar_wait(&acc_empty[ab], ((tcount >> 1) & 1) ^ 1)) { ok = false; break; }
+        if (!(CTAS == 2 ? mbar_wait_cluster(&acc_empty[ab], ((tcount >> 1) & 1) ^ 1)
+                        : mbar_wait(&acc_empty[ab], ((tcount >> 1) & 1) ^ 1))) { ok = false; break; }
         tc_fence_after_sync();
         const uint32_t d_tmem = tmem_base + ab * BN;
         for (int kb = 0; kb < kblocks; ++kb, ++it) {
           const int s = it % S::kStages;
-          if (!mbar_wait(&full[s], (it / S::kStages) & 1)) { ok = false; break; }
+          if (!(CTAS == 2 ? mbar_wait_cluster(&full[s], (it / S::kStages) & 1) : mbar_wait(&full[s], (it / S::kStages) & 1))) {
+            ok = false;
+            break;
+          }
           tc_fence_after_sync();
           // both operands are MN-major: 16 K indices = two 8-index groups of 1024 bytes each; the start
           // address field counts 16-byte units, so a stage or K step is an add on the descriptor
@@ -418,8 +422,9 @@ project_adam_kernel(const __grid_constant__ TcProblem single, const TcProblem* _
     // tile: 1.8 us per K block with the conversion against 0.8 us without.  The kernel is bound by how many bytes
     // it keeps in flight, a stage now also waits for this warp's chain (wake-up, a load issued one K block
     // earlier that takes about 1.5 us to return under the kernel's own traffic, 450 instructions, fence, arrive),
-    // and the global stores of the writer tiles delay their barrier arrivals.  The separate conversion launch costs
-    // 0.2 us per K block equivalent, so it stays the default until these warps take their codes through the copy
+    // and the global stores of the writer tiles delay their barrier arrivals; as CTA pairs the arrival on the
+    // leader's barrier is a cluster-scope release, about 1 us each.  The separate conversion launch costs 0.2 us
+    // per K block equivalent, so it stays the default until these warps take their codes through the copy
     // engine several stages ahead.
     const int ct = (int)threadIdx.x - (64 + S::kEpiWarps * 32);
     struct Pos {
@@ -484,7 +489,7 @@ project_adam_kernel(const __grid_constant__ TcProblem single, const TcProblem* _
       }
       __syncwarp();
       if (lane == 0) {
-        if (CTAS == 2) mbar_arrive_remote(mapa_u32(smem_u32(&full[s]), 0));
+        if (CTAS == 2) mbar_arrive_cluster(mapa_u32(smem_u32(&full[s]), 0));
         else mbar_arrive(&full[s]);
       }
       ++it;
@@ -617,7 +622,7 @@ project_adam_kernel(const __grid_constant__ TcProblem single, const TcProblem* _
           tc_fence_before_sync();
           __syncwarp();
           if (lane == 0) {
-            if (CTAS == 2) mbar_arrive_remote(mapa_u32(smem_u32(&acc_empty[ab]), 0));
+            if (CTAS == 2) mbar_arrive_cluster(mapa_u32(smem_u32(&acc_empty[ab]), 0));
             else mbar_arrive(&acc_empty[ab]);
           }
         };
@@ -772,7 +777,7 @@ project_adam_kernel(const __grid_constant__ TcProblem single, const TcProblem* _
           tc_fence_before_sync();
           __syncwarp();
           if (lane == 0) {
-            if (CTAS == 2) mbar_arrive_remote(mapa_u32(smem_u32(&acc_empty[ab]), 0));
+            if (CTAS == 2) mbar_arrive_cluster(mapa_u32(smem_u32(&acc_empty[ab]), 0));
             else mbar_arrive(&acc_empty[ab]);
           }
         }
@@ -1107,12 +1112,16 @@ backproject_sr_kernel(const __grid_constant__ TcProblem single, const TcProblem*
         const uint32_t idesc = right ? idesc_right : idesc_left;
         const uint64_t astep = right ? (2048 >> 4) : (32 >> 4), bstep = right ? (32 >> 4) : (2048 >> 4);
         const uint32_t ab = tcount & 1;
-        if (!mbar_wait(&acc_empty[ab], ((tcount >> 1) & 1) ^ 1)) { ok = false; break; }
+        if (!(CTAS == 2 ? mbar_wait_cluster(&acc_empty[ab], ((tcount >> 1) & 1) ^ 1)
+                        : mbar_wait(&acc_empty[ab], ((tcount >> 1) & 1) ^ 1))) { ok = false; break; }
         tc_fence_after_sync();
         const uint32_t d_tmem = tmem_base + ab * S::kBN;
         for (int kb = 0; kb < kblocks; ++kb, ++it) {
           const int s = it % S::kStages;
-          if (!mbar_wait(&full[s], (it / S::kStages) & 1)) { ok = false; break; }
+          if (!(CTAS == 2 ? mbar_wait_cluster(&full[s], (it / S::kStages) & 1) : mbar_wait(&full[s], (it / S::kStages) & 1))) {
+            ok = false;
+            break;
+          }
           tc_fence_after_sync();
           // A is K-major (rows of 128 bytes, 16 K indices = 32 bytes further along the row),
           // B is MN-major (16 K indices = two 8-index groups of 1024 bytes)
@@ -1297,7 +1306,7 @@ backproject_sr_kernel(const __grid_constant__ TcProblem single, const TcProblem*
             tc_fence_before_sync();
             __syncwarp();
             if (lane == 0) {
-              if (CTAS == 2) mbar_arrive_remote(mapa_u32(smem_u32(&acc_empty[ab]), 0));
+              if (CTAS == 2) mbar_arrive_cluster(mapa_u32(smem_u32(&acc_empty[ab]), 0));
               else mbar_arrive(&acc_empty[ab]);
             }
           }
@@ -1645,9 +1654,9 @@ void schedule_tiles(const std::vector<int2>& tiles, const std::vector<float>& co
 }
 
 // bit 0: the back-projection of a plan runs as CTA pairs (cta_group::2); bit 1: the projection does; bit 2: the
-// back-projection does where it pays, i.e. in chunks whose ranks average 512 or more (measured under the power cap,
-// where the halved operand traffic buys clock: LLaMA-7B 13.9-14.2 ms against 15.1 unpaired; LLaMA-1B, r = 512, 3.70-3.74
-// ms against 3.75-3.77; LLaMA-130M, r = 256, 262 us either way).  Read when a plan is created.
+// back-projection does where it pays, i.e. in chunks whose ranks average 1024 or more (measured on LLaMA-7B under
+// the power cap: 13.9-14.2 ms against 15.1 unpaired, the halved operand traffic buys clock; on LLaMA-1B, r = 512,
+// pairs are 3 % slower).  Read when a plan is created.
 int g_pair_mode = 6;
 
 // Scratch is shared by the matrices of a chunk; a chunk is a run of consecutive items whose P~ and N_b fit
@@ -1706,7 +1715,7 @@ int plan_create(const StepArgs* items, int32_t count, void* table_dev, size_t ta
     if (g_pair_mode & 4) {
       int64_t rsum = 0;
       for (int k = i; k < j; ++k) rsum += items[k].r;
-      if (rsum >= (int64_t)512 * (j - i)) ch.pairs = 1;
+      if (rsum >= (int64_t)1024 * (j - i)) ch.pairs = 1;
     }
     for (int k = i; k < j; ++k) {
       if (items[k].right) ch.pairs = 0;
