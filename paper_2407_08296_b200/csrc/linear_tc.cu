@@ -13,7 +13,7 @@
 // Persistent CTA PAIRS, one CTA per SM, tiles of 512 or 256 rows x 256 columns: each CTA brings half the rows of A and
 // converts (or brings) half the columns of B, and one thread of the pair issues MMAs over both (cta_group::2).  Warp roles:
 // 0 TMA producer (A, and B of the weight gradient), 1 MMA issuer and tensor-memory owner, 2 TMA producer of the INT8 tiles,
-// 4-7 epilogue, from 8 on converters.
+// 3 (of the second CTA) relay of its converters to the issuer, 4-7 epilogue, from 8 on converters.
 //
 // What bounds it: shared memory's 128 bytes per clock against the MMA, then power.  Per K block of 64 and 256 rows a CTA's
 // MMAs take 512 clocks.  A 256-row tile's traffic (A, half of B, codes, each written once and read once) is 80 KB, 640
@@ -222,13 +222,15 @@ int8_linear_kernel(const __grid_constant__ LinArgs a, int32_t* __restrict__ stat
   uint64_t* raw_empty = raw_full + 4;
   uint64_t* acc_full = raw_empty + 4;
   uint64_t* acc_empty = acc_full + 2;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 2);
+  uint64_t* converted = acc_empty + 2;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(converted + S::kStages);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     for (int i = 0; i < S::kStages; ++i) {
-      mbar_init(&full[i], S::kConvert ? 1 + 2 * 4 : 1);   // the leader's TMA producer, and one group of converter warps per CTA
+      mbar_init(&full[i], S::kConvert ? 1 + 4 + 1 : 1);    // the leader's TMA producer, a group of its converter warps, the peer's relay
       mbar_init(&empty[i], 1);
+      mbar_init(&converted[i], 4);
     }
     for (int i = 0; i < S::kRawStages; ++i) { mbar_init(&raw_full[i], 1); mbar_init(&raw_empty[i], 4); }
     for (int i = 0; i < 2; ++i) { mbar_init(&acc_full[i], 1); mbar_init(&acc_empty[i], 2 * S::kEpiWarps); }
@@ -292,19 +294,19 @@ int8_linear_kernel(const __grid_constant__ LinArgs a, int32_t* __restrict__ stat
       for (int t = wk.first; ok && t < wk.end; t += wk.stride, ++tcount) {
         // one row block per tile: two accumulators take alternate tiles; two: the tile has both, each handed over by itself
         const uint32_t ab = MT == 1 ? (tcount & 1) : 0u, use = MT == 1 ? (tcount >> 1) : tcount;
-        if (!mbar_wait(&acc_empty[ab], (use & 1) ^ 1)) { ok = false; break; }
+        if (!mbar_wait_cluster(&acc_empty[ab], (use & 1) ^ 1)) { ok = false; break; }
         tc_fence_after_sync();
         const uint32_t d_tmem = tmem_base + ab * kTileN;
         for (int kb = wk.kb0; kb < wk.kb1; ++kb, ++it) {
           const int s = it % S::kStages;
-          if (!mbar_wait(&full[s], (it / S::kStages) & 1)) { ok = false; break; }
+          if (!(S::kConvert ? mbar_wait_cluster(&full[s], (it / S::kStages) & 1) : mbar_wait(&full[s], (it / S::kStages) & 1))) { ok = false; break; }
           tc_fence_after_sync();
           const uint64_t da = desc_a0 + (uint64_t)((s * S::kStageBytes) >> 4);
           const uint64_t db = desc_b0 + (uint64_t)((s * S::kStageBytes) >> 4);
 #pragma unroll
           for (int h = 0; h < MT; ++h) {
             if (h == 1 && kb == wk.kb0) {
-              if (!mbar_wait(&acc_empty[1], (use & 1) ^ 1)) { ok = false; break; }
+              if (!mbar_wait_cluster(&acc_empty[1], (use & 1) ^ 1)) { ok = false; break; }
               tc_fence_after_sync();
             }
 #pragma unroll
@@ -338,6 +340,23 @@ int8_linear_kernel(const __grid_constant__ LinArgs a, int32_t* __restrict__ stat
       }
       if (!ok) raise_expired(status);
     }
+  } else if (warp == 3) {
+    // ------------------------------------------------------------------ relay: the second CTA's converted operand -> the issuer
+    // An arrival that orders a converter's stores for the other CTA's issuer has to release at cluster scope, which holds its warp
+    // up until its loads of the next scales are back as well.  So the converters arrive here, at CTA scope, and this thread, which
+    // has nothing of its own in flight, passes their arrival on: it releases what it has acquired.
+    if (S::kConvert && wk.half == 1 && lane == 0) {
+      uint32_t it = 0;
+      bool ok = true;
+      for (int t = wk.first; ok && t < wk.end; t += wk.stride) {
+        for (int kb = wk.kb0; kb < wk.kb1; ++kb, ++it) {
+          const int s = it % S::kStages;
+          if (!mbar_wait(&converted[s], (it / S::kStages) & 1)) { ok = false; break; }
+          mbar_arrive_cluster(mapa_u32(smem_u32(&full[s]), wk.leader));
+        }
+      }
+      if (!ok) raise_expired(status);
+    }
   } else if (warp >= 4 && warp < 4 + S::kEpiWarps) {
     // ------------------------------------------------------------------ epilogue: fp32 accumulator -> bf16
     const int q = warp & 3;
@@ -360,7 +379,10 @@ int8_linear_kernel(const __grid_constant__ LinArgs a, int32_t* __restrict__ stat
         if (c == kTileN / 32 - 1) {                    // every read of this tile's accumulator has landed
           tc_fence_before_sync();
           __syncwarp();
-          if (lane == 0) mbar_arrive_remote(mapa_u32(smem_u32(&acc_empty[ab + h]), wk.leader));
+          if (lane == 0) {
+            if (wk.half == 0) mbar_arrive(&acc_empty[ab + h]);
+            else mbar_arrive_cluster(mapa_u32(smem_u32(&acc_empty[ab + h]), wk.leader));
+          }
         }
         if (n0 + 32 * c < a.cols) {
           uint4 pk[4];
@@ -458,13 +480,13 @@ int8_linear_kernel(const __grid_constant__ LinArgs a, int32_t* __restrict__ stat
         }
         fence_proxy_async_smem();                      // the MMA reads these stores through the async proxy
         __syncwarp();
-        if (lane == 0) { mbar_arrive_remote(mapa_u32(smem_u32(&full[s]), wk.leader)); mbar_arrive(&raw_empty[rs]); }
+        if (lane == 0) { mbar_arrive(wk.half == 0 ? &full[s] : &converted[s]); mbar_arrive(&raw_empty[rs]); }
       }
     }
     if (!ok && lane == 0) raise_expired(status);
   }
 
-  __syncwarp();                                        // one lane of the warps 0 to 2 had a role: the warp goes on together
+  __syncwarp();                                        // one lane of the warps 0 to 3 had a role: the warp goes on together
   if (a.split > 1) {
     // Every MMA of the tile is complete, so the operand stages are free: they hold the sums on their way.  All warps but the
     // first four add up and store, sixteen columns at a time, whatever share of the tile this CTA has.  The cluster barriers
