@@ -275,6 +275,7 @@ int8_linear_kernel(const __grid_constant__ LinArgs a, int32_t* __restrict__ stat
           }
         }
       }
+      ok = ok && mbar_drain<S::kStages>(empty, it);
       if (!ok) raise_expired(status);
     }
   } else if (warp == 1) {

@@ -110,6 +110,7 @@ split_gemm_kernel(const __grid_constant__ SplitArgs a, int32_t* __restrict__ sta
             tma_load_3d(sA + S::kABytes + p * S::kBBytes, &a.mapB, &full[s], 0, p * a.kpad + kb * kBK, n0 / 64);
         }
       }
+      ok = ok && mbar_drain<S::kStages>(empty, it);
       if (!ok) raise_expired(status);
     }
   } else if (warp == 1) {
@@ -285,6 +286,7 @@ gram_kernel(const __grid_constant__ GramArgs a, int nmat, int32_t* __restrict__ 
           }
         }
       }
+      ok = ok && mbar_drain<S::kStages>(empty, it);
       if (!ok) raise_expired(status);
     }
   } else if (warp == 1) {

@@ -54,6 +54,16 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
 // .aligned instructions below).  Lanes that left a loop one by one need not have met again.
 __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity) { return __all_sync(0xFFFFFFFFu, mbar_wait(bar, parity)); }
 
+// The last arrivals on the `empty` barriers of a ring of STAGES stages that was filled `fills` times.  They are commits of the tensor
+// core, which nobody else waits for; a producer does so before its CTA may end, since an arrival that came later would fall on a
+// barrier of whatever CTA has that shared memory by then.
+template <int STAGES>
+__device__ __forceinline__ bool mbar_drain(uint64_t* empty, uint32_t fills) {
+  bool ok = true;
+  for (uint32_t i = fills > STAGES ? fills - STAGES : 0; i < fills; ++i) ok = ok && mbar_wait(&empty[i % STAGES], (i / STAGES) & 1);
+  return ok;
+}
+
 // ----------------------------------------------------------------------------- packed fp32
 // Packed fp32 pairs (one instruction for two lanes of a float2).
 __device__ __forceinline__ float2 mul2(float2 a, float2 b) {

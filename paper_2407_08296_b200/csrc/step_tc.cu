@@ -363,6 +363,7 @@ project_adam_kernel(const __grid_constant__ TcProblem single, const TcProblem* _
           }
         }
       }
+      ok = ok && mbar_drain<S::kStages>(empty, it);
       if (!ok) raise_wait_expired(status);
     }
   } else if (warp == 1) {
@@ -1091,6 +1092,7 @@ backproject_sr_kernel(const __grid_constant__ TcProblem single, const TcProblem*
           }
         }
       }
+      ok = ok && mbar_drain<S::kStages>(empty, it);
       if (!ok) raise_wait_expired(status);
     }
   } else if (warp == 1) {
