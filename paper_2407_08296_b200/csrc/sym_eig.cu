@@ -44,20 +44,26 @@ using ptx::mul2;
 constexpr uint32_t kPollLimit = 1u << 20;
 constexpr int kTriSmem = 225 * 1024;
 
-__device__ __forceinline__ uint4 ld_relaxed_v4(const uint4* p) {
-  uint4 v;
-  asm volatile("ld.relaxed.gpu.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
+// Two values of a step, each with the step's number beside it in ONE 8-byte element: an access of the memory model covers an
+// element, so a reader that sees the number has the value.
+struct __align__(16) Tagged {
+  uint64_t a, b;               // (tag << 32) | bits of the value
+};
+__device__ __forceinline__ Tagged ld_tagged(const Tagged* p) {
+  Tagged v;
+  asm volatile("ld.relaxed.gpu.global.v2.b64 {%0, %1}, [%2];" : "=l"(v.a), "=l"(v.b) : "l"(p) : "memory");
   return v;
 }
-// Two values, each in an 8-byte word with the tag of its step.
-__device__ __forceinline__ void st_relaxed_v4(uint4* p, float a, float b, uint32_t tag) {
-  asm volatile("st.relaxed.gpu.global.v4.u32 [%0], {%1, %2, %3, %4};" ::"l"(p), "r"(__float_as_uint(a)), "r"(tag), "r"(__float_as_uint(b)), "r"(tag)
-               : "memory");
+__device__ __forceinline__ void st_tagged(Tagged* p, float a, float b, uint32_t tag) {
+  const uint64_t high = (uint64_t)tag << 32;
+  asm volatile("st.relaxed.gpu.global.v2.b64 [%0], {%1, %2};" ::"l"(p), "l"(high | __float_as_uint(a)), "l"(high | __float_as_uint(b)) : "memory");
 }
+__device__ __forceinline__ uint32_t tag_of(uint64_t x) { return (uint32_t)(x >> 32); }
+__device__ __forceinline__ float value_of(uint64_t x) { return __uint_as_float((uint32_t)x); }
 
 struct TriArgs {
   Ptrs<float> A, V, tau, d, e;
-  Ptrs<uint4> xchg;
+  Ptrs<Tagged> xchg;
   int N, Np, C;
   int in_smem;               // columns per CTA that shared memory holds
 };
@@ -101,7 +107,7 @@ tridiagonal_kernel(const __grid_constant__ TriArgs a, int32_t* __restrict__ stat
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   float* const A = a.A.p[mat];
   float* const Vg = a.V.p[mat];
-  uint4* const xchg = a.xchg.p[mat];
+  Tagged* const xchg = a.xchg.p[mat];
   const int ncols = (N - cta + C - 1) / C;     // this CTA's columns: cta + l C, l = 0 .. ncols - 1
   const int nr = min(ncols, RC), ns = min(ncols - nr, a.in_smem), ng = ncols - nr - ns;   // registers, shared, global (these retire first)
   const int nc8 = ((N + C - 1) / C + 8) & ~7;  // pitch of the per-column arrays: groups of eight may reach past the end
@@ -157,20 +163,20 @@ tridiagonal_kernel(const __grid_constant__ TriArgs a, int32_t* __restrict__ stat
       // up the words themselves (2048 x 5461: 9.4 ms as it is, 14.3 at once); a lane that waits alone for the rest of its warp
       // adds a trip (10.3).
       const bool wanted = k > 0 && j >= k && j < N;
-      const uint4* const in = xchg + (k & 1) * Np + j;
-      uint4 got = make_uint4(0, 0, 0, 0);
+      const Tagged* const in = xchg + (k & 1) * Np + j;
+      Tagged got{0, 0};
       bool here = !wanted;
       for (uint32_t polls = 0; polls < kPollLimit && !__all_sync(0xFFFFFFFFu, here); ++polls)
         if (!here) {
-          got = ld_relaxed_v4(in);
-          here = got.y == (uint32_t)k && got.w == (uint32_t)k;
+          got = ld_tagged(in);
+          here = tag_of(got.a) == (uint32_t)k && tag_of(got.b) == (uint32_t)k;
         }
       ok = ok && here;
       float p = 0.f;
       if (j >= k && j < N) {
         if (wanted) {
-          p = __uint_as_float(got.x);
-          r[q] = __uint_as_float(got.z);
+          p = value_of(got.a);
+          r[q] = value_of(got.b);
         }
         if (j == k) s_pk = p;
       } else {
@@ -338,7 +344,7 @@ tridiagonal_kernel(const __grid_constant__ TriArgs a, int32_t* __restrict__ stat
       float s = 0.f;
 #pragma unroll
       for (int i = 0; i < WARPS; ++i) s += part[i * 2 * nc8 + l];
-      st_relaxed_v4(xchg + (k1 & 1) * Np + j, s, pivot[l], (uint32_t)k1);
+      st_tagged(xchg + (k1 & 1) * Np + j, s, pivot[l], (uint32_t)k1);
     }
     __syncwarp();
 #pragma unroll
@@ -853,11 +859,11 @@ int launch_sym_eig(const EigBuffers* w, int nb, int64_t N, int64_t r, int32_t* s
   Ptrs<const float> Ac{}, Vc{}, tauc{}, dc{}, ec{}, scalec{}, crossc{};
   Ptrs<double> lam{}, inv{}, plus{}, minus{};
   Ptrs<const double> lamc{}, invc{};
-  Ptrs<uint4> xchg{};
+  Ptrs<Tagged> xchg{};
   for (int i = 0; i < nb; ++i) {
     Ac.p[i] = A.p[i] = w[i].A; Vc.p[i] = V.p[i] = w[i].V; tauc.p[i] = tau.p[i] = w[i].tau;
     dc.p[i] = d.p[i] = w[i].d; ec.p[i] = e.p[i] = w[i].e; Z.p[i] = w[i].Z; scalec.p[i] = scale.p[i] = w[i].scale; crossc.p[i] = cross.p[i] = w[i].cross;
-    lamc.p[i] = lam.p[i] = w[i].lam; invc.p[i] = inv.p[i] = w[i].inv; plus.p[i] = w[i].plus; minus.p[i] = w[i].minus; xchg.p[i] = w[i].xchg;
+    lamc.p[i] = lam.p[i] = w[i].lam; invc.p[i] = inv.p[i] = w[i].inv; plus.p[i] = w[i].plus; minus.p[i] = w[i].minus; xchg.p[i] = (Tagged*)w[i].xchg;
     QG_CUDA_TRY(cudaMemsetAsync(w[i].xchg, 0, (size_t)(2 * Np * 16), st));   // no tag of an earlier call
   }
   eig_scale_factor_kernel<<<nb, 256, 0, st>>>(Ac, (int)N, (int)Np, scale);
