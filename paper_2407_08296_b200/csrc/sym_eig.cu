@@ -636,6 +636,7 @@ back_transform_kernel(const Ptrs<const float> Vb, const Ptrs<const float> taub, 
     for (int i = 0; i < kBackStages; ++i) ptx::mbar_init(&landed[i], 1);
     ptx::fence_mbar_init();
   }
+  ptx::fence_proxy_async_smem();                    // these stores come before the copies that go over most of the ring
   auto fetch = [&](int step) {                      // one thread: reflectors k = N - 1 - 2 step and k - 1, rows k .. on in whole groups
     const int k = N - 1 - 2 * step;
     if (tid != 0 || k < 0) return;
