@@ -946,7 +946,7 @@ static int refresh_direct(const RefreshJob* jobs, const Batch& bt, int64_t m, in
   }
   int rc = launch_gram(G, nb, ldg, transposed != long_side, s, l, A, eig_pitch(s), status, st);
   if (rc != QG_OK) return rc;
-  rc = launch_sym_eig(eig, nb, s, re, status, st);
+  rc = launch_sym_eig(eig, nb, s, re, r, status, st);
   if (rc != QG_OK) return rc;
   const Ptrs<const float> V = bt.tab<const float>([](const RefreshWs& x) { return x.eig.Z; });
   if (!long_side) return finish_vectors(jobs, bt, V, re, m, r, false, st);

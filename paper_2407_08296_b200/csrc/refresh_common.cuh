@@ -39,9 +39,9 @@ struct EigBuffers {
 };
 size_t carve_eig(void* base, int64_t N, int64_t r, EigBuffers* out);
 // On return (stream order) Z[i][j] holds the eigenvector of the j-th largest eigenvalue, j < r, of every matrix.
-// QG_DEV_BAD_FACTOR is raised in *status where the r-th eigenvalue is so small against the first that its vector is lost in
-// rounding.
-int launch_sym_eig(const EigBuffers* w, int nb, int64_t N, int64_t r, int32_t* status, cudaStream_t st);
+// QG_DEV_BAD_FACTOR is raised in *status where the `wanted`-th eigenvalue (wanted <= r) is so small against the first that its
+// vector is lost in rounding.
+int launch_sym_eig(const EigBuffers* w, int nb, int64_t N, int64_t r, int64_t wanted, int32_t* status, cudaStream_t st);
 
 // ---- refresh_tc.cu
 // A[i] (N x N fp32, pitch lda) = X X^T for every matrix of a batch; X(i, k) = G[i * ldg + k] (N rows of K), or, if `columns`,

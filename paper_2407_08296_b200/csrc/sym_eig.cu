@@ -456,10 +456,11 @@ eigenvalue_kernel(const Ptrs<const float> db, const Ptrs<const float> eb, int N,
 
 // Whether binary32 resolved the vectors: A and its reduction carry an error of some units in the last place of the largest
 // eigenvalue, and neighbours in the bulk of a gradient's spectrum lie about lambda / N apart.  Below this bound the subspace
-// can be off by more than 1e-2 rad (768 rows: lambda_r / lambda_1 = 3e-6 gave 3.5e-2).
-__global__ void resolved_kernel(const Ptrs<const double> lamb, int N, int r, int32_t* __restrict__ status) {
+// can be off by more than 1e-2 rad (768 rows: lambda_r / lambda_1 = 3e-6 gave 3.5e-2).  `wanted`: of the vectors computed, those the
+// caller asked for.
+__global__ void resolved_kernel(const Ptrs<const double> lamb, int N, int wanted, int32_t* __restrict__ status) {
   const double* lam = lamb.p[blockIdx.x];
-  if (!(lam[r - 1] >= 0.1 * N * 0x1p-24 * lam[0]) && status) atomicOr(status, QG_DEV_BAD_FACTOR);
+  if (!(lam[wanted - 1] >= 0.1 * N * 0x1p-24 * lam[0]) && status) atomicOr(status, QG_DEV_BAD_FACTOR);
 }
 
 // ------------------------------------------------------------------------------------------ 3. eigenvectors of T
@@ -853,8 +854,8 @@ size_t carve_eig(void* base, int64_t N, int64_t r, EigBuffers* out) {
   return off;
 }
 
-int launch_sym_eig(const EigBuffers* w, int nb, int64_t N, int64_t r, int32_t* status, cudaStream_t st) {
-  if (N < 2 || N > kEigMax || r < 1 || r > N || nb < 1 || nb > kMaxBatch) return QG_UNSUPPORTED_SHAPE;
+int launch_sym_eig(const EigBuffers* w, int nb, int64_t N, int64_t r, int64_t wanted, int32_t* status, cudaStream_t st) {
+  if (N < 2 || N > kEigMax || r < 1 || r > N || wanted < 1 || wanted > r || nb < 1 || nb > kMaxBatch) return QG_UNSUPPORTED_SHAPE;
   const int64_t Np = eig_pitch(N);
   Ptrs<float> A{}, V{}, tau{}, d{}, e{}, Z{}, scale{}, cross{};
   Ptrs<const float> Ac{}, Vc{}, tauc{}, dc{}, ec{}, scalec{}, crossc{};
@@ -913,7 +914,7 @@ int launch_sym_eig(const EigBuffers* w, int nb, int64_t N, int64_t r, int32_t* s
     eigenvalue_kernel<<<dim3((unsigned)ceil_div(r, kSturmWarps), (unsigned)nb), kSturmWarps * 32, (size_t)N * 16, st>>>(dc, ec, (int)N, (int)r, lam);
     QG_LAUNCH_CHECK();
   }
-  resolved_kernel<<<nb, 1, 0, st>>>(lamc, (int)N, (int)r, status);
+  resolved_kernel<<<nb, 1, 0, st>>>(lamc, (int)N, (int)wanted, status);
   QG_LAUNCH_CHECK();
   {
     static bool done[kDevices] = {};

@@ -80,3 +80,27 @@ def test_batches_of_odd_gradients_from_both_sides(m, n, r, side):
     assert int(status.item()) == 0
     for it in items[::3]:
         _check(it["G"], it["P_fp32"], side)
+
+
+def _with_singular_values(m, n, values, seed):
+    """A bf16 gradient with these singular values (and what rounding to bf16 adds: about 1e-3 of its size, spread over all of them)."""
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(seed)
+    u = torch.linalg.qr(torch.randn(m, len(values), device="cuda", dtype=torch.float64, generator=gen))[0]
+    v = torch.linalg.qr(torch.randn(n, len(values), device="cuda", dtype=torch.float64, generator=gen))[0]
+    G = B.zeros_matrix(m, n, torch.bfloat16)
+    G.copy_(((u * values) @ v.T).float())
+    return G
+
+
+def test_vectors_computed_beside_those_wanted_do_not_raise_the_flag():
+    # vectors of the long side are computed in whole 64s: 96 wanted, 128 computed, and the spectrum ends with the 96th
+    m, n, r = 1025, 768, 96
+    G = _with_singular_values(m, n, torch.linspace(1.0, 0.5, r, device="cuda", dtype=torch.float64), seed=3)
+    P = torch.zeros((m, r), device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    B.refresh_subspace(G, r, P_fp32=P, status=status)
+    assert int(status.item()) == 0
+    u = torch.linalg.svd(G.double(), full_matrices=False)[0][:, :r]
+    # the subspace is separated by a gap of half the spectrum: it is resolved to some units in the last place of binary32
+    assert float((u - P.double() @ (P.double().T @ u)).norm(dim=0).max()) <= 768 * 2.0 ** -24 / 0.25
