@@ -241,10 +241,10 @@ tridiagonal_kernel(const __grid_constant__ TriArgs a, int32_t* __restrict__ stat
     float beta = alpha, scl = 0.f;
     tau = 0.f;
     if (sig > 1e-36f) {
-      const float len2 = fmaf(alpha, alpha, sig);
-      beta = -copysignf(len2 * rsqrtf(len2), alpha);
-      tau = __fdividef(beta - alpha, beta);
-      scl = __fdividef(1.f, alpha - beta);
+      // correctly rounded, not the approximate forms: tau and scl have to be those of one reflector to the last bits
+      beta = -copysignf(sqrtf(fmaf(alpha, alpha, sig)), alpha);
+      tau = (beta - alpha) / beta;
+      scl = 1.f / (alpha - beta);
     }
 #pragma unroll
     for (int q = 0; q < NQ; ++q) {
