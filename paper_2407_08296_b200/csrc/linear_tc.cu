@@ -13,7 +13,7 @@
 // Persistent CTA PAIRS, one CTA per SM, tiles of 512 or 256 rows x 256 columns: each CTA brings half the rows of A and
 // converts (or brings) half the columns of B, and one thread of the pair issues MMAs over both (cta_group::2).  Warp roles:
 // 0 TMA producer (A, and B of the weight gradient), 1 MMA issuer and tensor-memory owner, 2 TMA producer of the INT8 tiles,
-// 3 (of the second CTA) relay of its converters to the issuer, 4-7 epilogue, from 8 on converters.
+// 4-7 epilogue, from 8 on converters; 3 and the last two (of the second CTA) relay its converters' arrivals to the issuer.
 //
 // What bounds it: shared memory's 128 bytes per clock against the MMA, then power.  Per K block of 64 and 256 rows a CTA's
 // MMAs take 512 clocks.  A 256-row tile's traffic (A, half of B, codes, each written once and read once) is 80 KB, 640
@@ -83,7 +83,7 @@ struct Walk {
   }
 };
 
-// Every second K block of a pair's tiles, for a group of converter warps.
+// The K blocks of a pair's tiles one after the other, for warps that take them in turn.
 struct BlockWalk {
   const Walk& w;
   int t, kb;
@@ -149,7 +149,8 @@ struct LinSmem {
   static constexpr int kGroups = MODE == kWeightGrad ? 2 : 3;   // of four converter warps (of no use but for the sums of a split tile
                                                                // where nothing is converted)
   static constexpr int kEpiWarps = 4, kConvWarps = 4 * kGroups;
-  static constexpr int kThreads = (4 + kEpiWarps + kConvWarps) * 32;
+  static constexpr int kRelays = kConvert ? 3 : 0;             // warp 3 and those past the converters
+  static constexpr int kThreads = (4 + kEpiWarps + kConvWarps + (kConvert ? kRelays - 1 : 0)) * 32;
   static_assert(kBytes <= 227 * 1024, "shared memory budget");
   static_assert(kBytes > kHalfOfSharedMemory, "see launch_overlapping");
 };
@@ -341,20 +342,21 @@ int8_linear_kernel(const __grid_constant__ LinArgs a, int32_t* __restrict__ stat
       }
       if (!ok) raise_expired(status);
     }
-  } else if (warp == 3) {
-    // ------------------------------------------------------------------ relay: the second CTA's converted operand -> the issuer
-    // An arrival that orders a converter's stores for the other CTA's issuer has to release at cluster scope, which holds its warp
-    // up until its loads of the next scales are back as well.  So the converters arrive here, at CTA scope, and this thread, which
-    // has nothing of its own in flight, passes their arrival on: it releases what it has acquired.
+  } else if (warp == 3 || warp >= 4 + S::kEpiWarps + S::kConvWarps) {
+    // ------------------------------------------------------------------ relays: the second CTA's converted operand -> the issuer
+    // An arrival that orders a converter's stores for the other CTA's issuer has to release at cluster scope, which takes some 600
+    // clocks or more (a converter also waits for its loads of the next scales then).  So the converters arrive at CTA scope on a
+    // barrier of their own CTA, and threads that have nothing else to do pass their arrivals on: they release what they have
+    // acquired.  One such thread would be the limit, three take the K blocks in turn.  Forward 8192 x 2048 x 5461 / input gradient
+    // 3001 x 11008 x 4096: the converters at cluster scope 159 / 216 us, one relay 179 / 249, three 145 / 204.
+    const int relay = warp == 3 ? 0 : warp - (4 + S::kEpiWarps + S::kConvWarps) + 1;
     if (S::kConvert && wk.half == 1 && lane == 0) {
-      uint32_t it = 0;
+      uint32_t it = relay;
       bool ok = true;
-      for (int t = wk.first; ok && t < wk.end; t += wk.stride) {
-        for (int kb = wk.kb0; kb < wk.kb1; ++kb, ++it) {
-          const int s = it % S::kStages;
-          if (!mbar_wait(&converted[s], (it / S::kStages) & 1)) { ok = false; break; }
-          mbar_arrive_cluster(mapa_u32(smem_u32(&full[s]), wk.leader));
-        }
+      for (BlockWalk bw(wk, relay); ok && bw.valid(); bw.advance(S::kRelays), it += S::kRelays) {
+        const int s = it % S::kStages;
+        ok = mbar_wait(&converted[s], (it / S::kStages) & 1);
+        if (ok) mbar_arrive_cluster(mapa_u32(smem_u32(&full[s]), wk.leader));
       }
       if (!ok) raise_expired(status);
     }
@@ -412,7 +414,7 @@ int8_linear_kernel(const __grid_constant__ LinArgs a, int32_t* __restrict__ stat
       }
     }
     if (!ok && lane == 0) raise_expired(status);
-  } else if (S::kConvert && warp >= 8) {
+  } else if (S::kConvert && warp >= 8) {   // (up to the relays above)
     // ------------------------------------------------------------------ converters: INT8 tile -> bf16 operand
     // Groups of four warps take K blocks in turn, so that the chain of one block (wait, load, convert, store, fence, arrive:
     // 900 to 1600 clocks) overlaps those of the next: 2 -> 3 groups, input gradient 3001 x 11008 x 4096, 256-row tiles, 315 ->
@@ -481,16 +483,16 @@ int8_linear_kernel(const __grid_constant__ LinArgs a, int32_t* __restrict__ stat
         }
         fence_proxy_async_smem();                      // the MMA reads these stores through the async proxy
         __syncwarp();
-        if (lane == 0) { mbar_arrive(wk.half == 0 ? &full[s] : &converted[s]); mbar_arrive(&raw_empty[rs]); }
+        if (lane == 0) { mbar_arrive(&raw_empty[rs]); mbar_arrive(wk.half == 0 ? &full[s] : &converted[s]); }
       }
     }
     if (!ok && lane == 0) raise_expired(status);
   }
 
-  __syncwarp();                                        // one lane of the warps 0 to 3 had a role: the warp goes on together
+  __syncwarp();                                        // also the warps of which one lane had a role
   if (a.split > 1) {
-    // Every MMA of the tile is complete, so the operand stages are free: they hold the sums on their way.  All warps but the
-    // first four add up and store, sixteen columns at a time, whatever share of the tile this CTA has.  The cluster barriers
+    // Every MMA of the tile is complete, so the operand stages are free: they hold the sums on their way.  The
+    // epilogue warps and the converters add up and store, sixteen columns at a time, whatever share of the tile this CTA has.  The cluster barriers
     // count warps: only stores are under a condition of the lane, and every warp joins before each of them.
     const int q = warp & 3, row = q * 32 + lane;
     const int m0 = (wk.first % a.mblocks) * (MT * 2 * kTileM) + (int)wk.half * kTileM, n0 = (wk.first / a.mblocks) * kTileN;
@@ -508,9 +510,9 @@ int8_linear_kernel(const __grid_constant__ LinArgs a, int32_t* __restrict__ stat
       }
       __syncwarp();
       cluster_sync_all();
-      if (some && warp >= 4) {
+      if (some && warp >= 4 && warp < 4 + S::kEpiWarps + S::kConvWarps) {
 #pragma unroll 1
-        for (int j = (int)wk.part + a.split * ((warp - 4) >> 2); j < kTileN / 16 && n0 + 16 * j < a.cols; j += a.split * (S::kThreads / 128 - 1)) {
+        for (int j = (int)wk.part + a.split * ((warp - 4) >> 2); j < kTileN / 16 && n0 + 16 * j < a.cols; j += a.split * (1 + S::kGroups)) {
           uint32_t pk[8];
           sum_columns16(stage_base, j, row, wk.half, a.split, pk);
           const int gr = m0 + h * 2 * kTileM + row, col = n0 + 16 * j;
