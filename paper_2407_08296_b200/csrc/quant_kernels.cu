@@ -27,12 +27,12 @@ __device__ __forceinline__ bool stream_unit(int64_t rows, int runs, int64_t& row
 
 __device__ __forceinline__ float redux_min(float v) {
   float r;
-  asm("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+  asm volatile("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
   return r;
 }
 __device__ __forceinline__ float redux_max(float v) {
   float r;
-  asm("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+  asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
   return r;
 }
 
@@ -75,7 +75,9 @@ quantize_rtn_kernel(const float* __restrict__ src, int64_t ld_src, int64_t rows,
     mx = redux_max(mx);
     const GroupParams gp = group_params<BITS>(mn, mx);
     // rint(t) + z as integers: adding 1.5 * 2^23 rounds t to the nearest integer, ties to even, and leaves it in the low
-    // mantissa bits; exact while |t| < 2^22, i.e. for all of a group whose zero point is below 2^20
+    // mantissa bits; exact while |t| < 2^22, i.e. for all of a group whose zero point is below 2^20 and whose scale comes from
+    // its extent.  Where it does not (an infinity, an extent past binary32's largest) t may be anything: above 2^22 the sum
+    // only grows and the code is the largest; below -2^21, and for a NaN, it is the smallest, as fmaxf makes it here and there.
     const bool small = fabsf(gp.z) < 0x1p20f;
     const int iz = small ? (int)gp.z - 0x4B400000 : 0;
     if (lane == 0) {
@@ -91,7 +93,7 @@ quantize_rtn_kernel(const float* __restrict__ src, int64_t ld_src, int64_t rows,
       for (int e = 0; e < 4; ++e) {
         int q;
         if (small) {
-          q = __float_as_int(__fadd_rn(__fmul_rn(v[i][e], gp.inv), 12582912.0f)) + iz;
+          q = __float_as_int(__fadd_rn(fmaxf(__fmul_rn(v[i][e], gp.inv), -0x1p21f), 12582912.0f)) + iz;
           q = min(max(q, -(1 << (BITS - 1))), (1 << (BITS - 1)) - 1);
         } else {
           q = (int)rtn_code<BITS>(v[i][e], gp);
