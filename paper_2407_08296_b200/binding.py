@@ -207,8 +207,8 @@ class QTensor:
         codes = torch.empty((rows, ld // per_byte), dtype=torch.int8 if bits == 8 else torch.uint8, device=device)
         if ld != cols:
             codes[:, cols // per_byte:].fill_({8: 0, 4: 0x88, 2: 0xAA}[bits])
-        scales, zeros = torch.empty((2, rows, ng), dtype=torch.float32, device=device)
-        return QTensor(codes, scales, zeros, rows, cols, ld, bits)
+        return QTensor(codes, torch.empty((rows, ng), dtype=torch.float32, device=device),
+                       torch.empty((rows, ng), dtype=torch.float32, device=device), rows, cols, ld, bits)
 
     def c_struct(self) -> _CQTensor:
         return _CQTensor(_ptr(self.codes), _ptr(self.scales), _ptr(self.zeros), self.rows, self.cols, self.ld,

@@ -121,3 +121,15 @@ def test_wait_expiry_aid_validates_on_the_host():
     assert L.qgalore_debug_expire_wait(0, 0x1000, None, None) == B.QG_INVALID_ARGUMENT
     assert L.qgalore_debug_expire_wait(8, None, None, None) == B.QG_INVALID_ARGUMENT
     assert L.qgalore_debug_expire_wait(8, 0x1002, None, None) == B.QG_MISALIGNED
+
+
+@pytest.mark.parametrize("bits", [2, 4, 8])
+def test_a_quantized_matrix_has_a_storage_of_its_own_for_each_part(bits):
+    # the one a quantize call makes for itself: its scales can be saved, resized or freed without its zero points
+    q = B.QTensor._to_be_written(3, 300, bits, "cpu")
+    parts = [q.codes, q.scales, q.zeros]
+    assert len({t.untyped_storage().data_ptr() for t in parts}) == 3
+    for t in parts:
+        assert t.untyped_storage().nbytes() == t.numel() * t.element_size()
+    like = B.QTensor.empty(3, 300, bits, "cpu")
+    assert [(t.shape, t.stride(), t.dtype) for t in parts] == [(t.shape, t.stride(), t.dtype) for t in (like.codes, like.scales, like.zeros)]
