@@ -51,9 +51,10 @@ constexpr int kCoopDevices = 64;
 
 // Test aid: 0 keeps every product of the refresh on the CUDA cores.
 int g_refresh_tc = 1;
-// Test aid: 0 takes the iterative route for every shape, and rotates the rows of its Rayleigh-Ritz matrix pair by pair
-// through L2.
+// Test aid: 0 rotates the rows of the Rayleigh-Ritz matrix pair by pair through L2 for every shape.
 int g_jacobi_blocks = 1;
+// Test aid: 0 takes the iterative route for every shape.
+int g_refresh_direct = 1;
 
 constexpr int kPanel = 64;    // columns orthonormalised together
 constexpr int kMaxSweeps = 32;
@@ -1072,7 +1073,7 @@ static int refresh_iterative(const RefreshJob* jobs, const Batch& bt, int64_t m,
 // 2048 x 2048, b = 256 9.3 ms at 0.2 rad against 9.4 ms at 2e-5; 1024 x 2048, b = 64 2.5 ms against 4.
 static bool direct_route(int64_t m, int64_t n, int64_t b) {
   const int64_t s = m < n ? m : n;
-  return g_jacobi_blocks && s <= kEigMax && s <= 8 * b;
+  return g_refresh_direct && s <= kEigMax && s <= 8 * b;
 }
 
 // One batch (at most kMaxBatch matrices of one shape).
@@ -1112,6 +1113,7 @@ int launch_refresh_batched(const RefreshJob* jobs, int count, int64_t m, int64_t
 
 int set_refresh_tc(int on) { g_refresh_tc = on ? 1 : 0; return QG_OK; }
 int set_jacobi_blocks(int on) { g_jacobi_blocks = on ? 1 : 0; return QG_OK; }
+int set_refresh_direct(int on) { g_refresh_direct = on ? 1 : 0; return QG_OK; }
 
 int launch_refresh(const uint16_t* G, int64_t ldg, int64_t m, int64_t n, int64_t r, int64_t b, int iters, int sweeps,
                    uint64_t seed, const qg_qtensor* P_new, float* P_fp32, void* ws, size_t ws_bytes, int32_t* status,

@@ -116,13 +116,26 @@ def test_refresh_subspace_matches_exact_svd(m, n, r):
 
 def test_refresh_with_the_row_by_row_eigen_iteration():
     # blocks wider than 2048 columns do not fit the block form of the Jacobi iteration and take the row-by-row form;
-    # here the same form is selected on a small shape
+    # here the same form is selected on a small shape, of the iterative route
     B.debug_set_jacobi_blocks(False)
+    B.debug_set_refresh_direct(False)
     try:
         run_refresh_case(768, 768, 256, seed=1024)
         run_refresh_case(512, 1376, 128, seed=640)
     finally:
         B.debug_set_jacobi_blocks(True)
+        B.debug_set_refresh_direct(True)
+
+
+def test_refresh_by_the_iterative_route():
+    # shapes that the direct route would take, by the other one: the block form of the Jacobi iteration at 512 and 256 columns
+    B.debug_set_refresh_direct(False)
+    try:
+        run_refresh_case(768, 768, 256, seed=1024)
+        run_refresh_case(512, 1376, 128, seed=640)
+        run_refresh_case(1376, 512, 128, seed=641)
+    finally:
+        B.debug_set_refresh_direct(True)
 
 
 def test_refresh_reports_similarity_with_previous_projection():

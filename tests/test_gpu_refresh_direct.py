@@ -1,6 +1,7 @@
 """The direct route of the subspace refresh where its kernels change: the row counts at which the tridiagonal reduction and
 the back-transformation take another instance, a batch that is reduced in several launches, vectors on the long side,
-odd extents, and gradients whose eigenvalues coincide."""
+odd extents, gradients whose eigenvalues coincide, spectra on both sides of what it resolves, and the shapes it leaves to the
+iterative route."""
 import pytest
 import torch
 
@@ -104,3 +105,19 @@ def test_vectors_computed_beside_those_wanted_do_not_raise_the_flag():
     u = torch.linalg.svd(G.double(), full_matrices=False)[0][:, :r]
     # the subspace is separated by a gap of half the spectrum: it is resolved to some units in the last place of binary32
     assert float((u - P.double() @ (P.double().T @ u)).norm(dim=0).max()) <= 768 * 2.0 ** -24 / 0.25
+
+
+# Shapes that take the iterative route by themselves, one for each block form of its eigen-iteration: a block that is a small part
+# of the short side (64 of 1024 columns: rows of up to 1024), and a short side of more than 4096 rows (a block of 1088).  The
+# spectrum falls by ten behind the r-th vector, so that twelve iterations leave 10^-24 of what lies behind it.
+@pytest.mark.parametrize("m,n,r", [(1024, 1100, 32), (4224, 4160, 544)])
+def test_shapes_of_the_iterative_route(m, n, r):
+    s = min(m, n)
+    values = torch.full((s,), 0.05, device="cuda", dtype=torch.float64)
+    values[:r] = torch.linspace(1.0, 0.5, r, device="cuda", dtype=torch.float64)
+    G = _with_singular_values(m, n, values, seed=r)
+    P = torch.zeros((m, r), device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    B.refresh_subspace(G, r, P_fp32=P, status=status, seed=5)
+    assert int(status.item()) == 0
+    _check(G, P, "left")
