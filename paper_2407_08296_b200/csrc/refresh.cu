@@ -10,7 +10,9 @@
 // Its error is that of a symmetric eigenproblem in binary32: measured against an exact SVD the subspace is off by 4e-5 ..
 // 3e-4 rad on rank-32 signals with noise at 1e-3 (the iterative route: 1e-4 .. 5e-3, and up to 0.4 at r = s / 8, where its
 // block of 2 r columns does not converge in 12 iterations).  It grows with lambda_1 / lambda_r; where that leaves the r-th
-// vector unresolved QG_DEV_BAD_FACTOR is raised (the iterative route met a bad pivot there and returned NaN).
+// vector unresolved QG_DEV_BAD_FACTOR is raised, beside vectors that are orthonormal all the same.  (The iterative route meets a
+// bad pivot there and returns NaN, and does so much earlier: 512 x 768, r = 128, geometric spectra from sigma_r / sigma_1 = 3e-2
+// down, where the direct one is off by 4e-5 rad, 1.7e-3 at 3e-3 and, flagged, 1.5e-2 at 1e-3.)
 // Time (one matrix, then a batch of eight, per matrix): 768 x 2048 r 256 17.2 -> 2.4 ms; 1024 x 1024 r 256 x 8 3.7 -> 0.80;
 // 2048 x 5461 r 512 42.8 -> 9.4 and 15.3 -> 4.5; 4096 x 4608 r 512 46.
 //

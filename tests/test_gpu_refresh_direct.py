@@ -121,3 +121,22 @@ def test_shapes_of_the_iterative_route(m, n, r):
     B.refresh_subspace(G, r, P_fp32=P, status=status, seed=5)
     assert int(status.item()) == 0
     _check(G, P, "left")
+
+
+# The flag is raised where the r-th eigenvalue is below 0.1 * 768 * 2^-24 of the first, a singular value of 2.1e-3 of the first.
+# Above it the subspace is the exact one's to the 1e-2 rad asked of every refresh; below, the vectors are still orthonormal.
+@pytest.mark.parametrize("ratio,flag", [(1e-2, 0), (3.2e-3, 0), (1.5e-3, B.QG_DEV_BAD_FACTOR), (5e-4, B.QG_DEV_BAD_FACTOR)])
+def test_spectra_on_both_sides_of_what_is_resolved(ratio, flag):
+    m, n, r = 768, 1100, 128
+    values = torch.full((m,), 0.3 * ratio, device="cuda", dtype=torch.float64)
+    values[:r] = ratio ** (torch.arange(r, device="cuda", dtype=torch.float64) / (r - 1))
+    G = _with_singular_values(m, n, values, seed=9)
+    P = torch.zeros((m, r), device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    B.refresh_subspace(G, r, P_fp32=P, status=status)
+    assert int(status.item()) == flag
+    Z = P.double()
+    assert float((Z.T @ Z - torch.eye(r, device="cuda")).abs().max()) <= 768 * 2.0 ** -24
+    if flag == 0:
+        u = torch.linalg.svd(G.double(), full_matrices=False)[0][:, :r]
+        assert float(torch.linalg.matrix_norm(u - Z @ (Z.T @ u), 2)) < 1e-2
