@@ -212,10 +212,10 @@ QG_API int qgalore_plan_step_timed(const qg_plan* plan, const qg_hyper* h, int32
                             float* kernel_ms, int32_t* kernel_launches);
 
 /* --- Sec. 3.5 "obtain the projection matrix using SVD" + Sec. 3.3 INT4 storage ------------
- * Top-r left singular vectors of G (bf16, m x n, pitch ldg), then Quant_4 into P_new.  Where the short side s = min(m, n)
- * has at most 4096 rows and s <= 8 b, b = r + oversample_cols: the r leading eigenvectors of the Gram matrix of the short
- * side (tridiagonal reduction in binary32, eigenvalues and their vectors in binary64), and G times them for vectors on the
- * long side; iters and seed do not enter.  Else: block subspace iteration on G G^T with a block of b columns (`iters`
+ * Top-r left singular vectors of G (bf16, m x n, pitch ldg), then Quant_4 into P_new.  With s = min(m, n) and b = r +
+ * oversample_cols, where s <= 8 b (s up to 768), 6 b (up to 1536), 4 b (up to 2048) or 2.5 b (up to 4096): the r leading
+ * eigenvectors of the Gram matrix of the short side (tridiagonal reduction in binary32, eigenvalues and their vectors in
+ * binary64), and G times them for vectors on the long side; iters and seed do not enter.  Else: block subspace iteration on G G^T with a block of b columns (`iters`
  * multiplications by G G^T, each followed by a block Gram-Schmidt orthonormalisation) and a Rayleigh-Ritz step
  * (eigenvectors of the projected b x b matrix by a Jacobi iteration on binary32 rows with binary64 sums), the random start
  * block drawn from Philox keyed by `seed`.  Each column carries the sign that makes its

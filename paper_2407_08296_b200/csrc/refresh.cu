@@ -1,7 +1,7 @@
 // Subspace refresh (Sec. 3.5: "obtain the projection matrix using SVD"; Sec. 3.3: INT4 storage): the top-r left singular
 // vectors of the gradient G (m x n, bf16), without a full SVD, by one of two routes.
 //
-// Direct, where the short side has at most kEigMax rows and the block is not a small part of it:
+// Direct, where that is the faster (direct_shape):
 //
 //   A = G G^T or G^T G, whichever is smaller (refresh_tc.cu: every product of two bfloat16 values is exact, sums in fp32)
 //   X <- its r leading eigenvectors (sym_eig.cu: tridiagonal reduction, bisection, twisted factorisations)
@@ -824,6 +824,19 @@ struct RefreshWs {
   int32_t* done;
 };
 
+// The route of a shape.  Direct: the whole of the short side's Gram matrix is reduced, 3 us a row up to 1024 rows, 5 at 2048, 11 at
+// 4096, and from 2048 rows on a batch gains little, since few of its matrices fit the SMs together.  Iterative: the cost goes
+// with the block, and a batch shares its many small launches.  The line lies where the direct one is the faster both alone and in
+// batches of eight (it decides on the shape only, so that a matrix gets the same vectors in either).  Measured, ms per matrix
+// alone / in eights, direct and iterative: 768 x 768 b 128 2.4 / 0.40 and 3.9 / 0.95; 1024 x 1024 b 128 4.8 / 0.82 and 4.1 / 1.1, b
+// 256 4.8 / 0.85 and 7.9 / 1.7; 1536 x 1536 b 192 6.4 / 2.1 and 6.3 / 1.7, b 384 6.3 / 2.2 and 13 / 3.1; 2048 x 2048 b 256 10.4 /
+// 4.5 and 9.1 / 2.3, b 512 10.4 / 4.5 and 18 / 4.5; 3072 x 3072 b 768 23 / 19.5 and 31 / 11.3, b 1536 22 / 21 and 73 / 39; 4096 x
+// 4096 b 1024 47 / 44 and 47 / 19, b 2048 47 / 45 and 119 / 74.
+bool direct_shape(int64_t m, int64_t n, int64_t b) {
+  const int64_t s = m < n ? m : n;
+  return s <= 768 ? s <= 8 * b : s <= 1536 ? s <= 6 * b : s <= 2048 ? s <= 4 * b : s <= kEigMax && 2 * s <= 5 * b;
+}
+
 // Scratch of one matrix (left singular vectors of X, m x n; a block of b columns, at most as many vectors).
 size_t carve_refresh(void* base, int64_t m, int64_t n, int64_t b, RefreshWs* w) {
   size_t off = 0;
@@ -1070,13 +1083,6 @@ static int refresh_iterative(const RefreshJob* jobs, const Batch& bt, int64_t m,
   return finish_vectors(jobs, bt, QG_TAB(const float, P32), r, m, r, false, st);
 }
 
-// The route of a shape.  Direct: the whole of the short side's Gram matrix is reduced, 3 us a row up to 1024 rows, 4.5
-// at 2048, 11 at 4096.  Iterative: the cost goes with the block, whose accuracy at a small part of the spectrum is poor (above):
-// 2048 x 2048, b = 256 9.3 ms at 0.2 rad against 9.4 ms at 2e-5; 1024 x 2048, b = 64 2.5 ms against 4.
-static bool direct_route(int64_t m, int64_t n, int64_t b) {
-  const int64_t s = m < n ? m : n;
-  return g_refresh_direct && s <= kEigMax && s <= 8 * b;
-}
 
 // One batch (at most kMaxBatch matrices of one shape).
 static int refresh_batch(const RefreshJob* jobs, int nb, int64_t m, int64_t n, int64_t r, int64_t b, int iters, int sweeps,
@@ -1087,7 +1093,7 @@ static int refresh_batch(const RefreshJob* jobs, int nb, int64_t m, int64_t n, i
     carve_refresh(ws + (size_t)i * ws_stride, m, n, b, &bt.w[i]);
     if (jobs[i].ldg != jobs[0].ldg) return QG_INVALID_ARGUMENT;          // one pitch per batch (the caller groups by it)
   }
-  int rc = direct_route(m, n, b) ? refresh_direct(jobs, bt, m, n, r, status, st, transposed)
+  int rc = g_refresh_direct && direct_shape(m, n, b) ? refresh_direct(jobs, bt, m, n, r, status, st, transposed)
                                  : refresh_iterative(jobs, bt, m, n, r, b, iters, sweeps, status, st, transposed);
   if (rc != QG_OK) return rc;
   for (int i = 0; i < nb; ++i) {
