@@ -815,6 +815,7 @@ struct RefreshWs {
   EigBuffers eig;  // of the Gram matrix of the short side
   float* XV;       // X V, for vectors on the long side
   uint16_t* planes_v;
+  float* P32_direct;
   // iterative route (in the same memory)
   float *Q, *Y, *Z, *Wp, *Cb, *S, *Linv, *Xsel;
   void* part;      // partial sums of sliced products
@@ -842,16 +843,26 @@ size_t carve_refresh(void* base, int64_t m, int64_t n, int64_t b, RefreshWs* w) 
   size_t off = 0;
   auto take = [&](size_t bytes) { void* p = base ? (char*)base + off : nullptr; off += (size_t)round_up((int64_t)bytes, 256); return p; };
   RefreshWs t{};
-  t.P32 = (float*)take((size_t)m * b * 4);
-  const size_t routes = off;
   const int64_t s = m < n ? m : n;
-  if (s <= kEigMax) {
+  if (direct_shape(m, n, b)) {
     take(carve_eig(base ? (char*)base + off : nullptr, s, b, &t.eig));
-    t.XV = (float*)take((size_t)m * b * 4);
-    t.planes_v = (uint16_t*)take(split_planes_bytes(s, b));
+    // what comes after the eigenvectors goes over A and V, where it fits
+    size_t used = 0;
+    auto over = [&](size_t bytes) -> void* {
+      const size_t at = used, whole = (size_t)(2 * s * eig_pitch(s)) * 4;
+      if (at + bytes > whole) return take(bytes);
+      used += (size_t)round_up((int64_t)bytes, 256);
+      return base ? (char*)t.eig.A + at : nullptr;
+    };
+    t.P32_direct = (float*)over((size_t)m * b * 4);
+    if (m > s) {
+      t.XV = (float*)over((size_t)m * b * 4);
+      t.planes_v = (uint16_t*)over(split_planes_bytes(s, b));
+    }
   }
   const size_t direct = off;
-  off = routes;
+  off = 0;
+  t.P32 = (float*)take((size_t)m * b * 4);
   t.T = (float*)take((size_t)b * b * 4);
   t.lam = (double*)take((size_t)b * 8);
   t.off = (double*)take(kMaxSweeps * 8);     // largest normalised inner product of each sweep
@@ -1093,8 +1104,10 @@ static int refresh_batch(const RefreshJob* jobs, int nb, int64_t m, int64_t n, i
     carve_refresh(ws + (size_t)i * ws_stride, m, n, b, &bt.w[i]);
     if (jobs[i].ldg != jobs[0].ldg) return QG_INVALID_ARGUMENT;          // one pitch per batch (the caller groups by it)
   }
-  int rc = g_refresh_direct && direct_shape(m, n, b) ? refresh_direct(jobs, bt, m, n, r, status, st, transposed)
-                                 : refresh_iterative(jobs, bt, m, n, r, b, iters, sweeps, status, st, transposed);
+  const bool direct = g_refresh_direct && direct_shape(m, n, b);
+  for (int i = 0; direct && i < nb; ++i) bt.w[i].P32 = bt.w[i].P32_direct;
+  int rc = direct ? refresh_direct(jobs, bt, m, n, r, status, st, transposed)
+                  : refresh_iterative(jobs, bt, m, n, r, b, iters, sweeps, status, st, transposed);
   if (rc != QG_OK) return rc;
   for (int i = 0; i < nb; ++i) {
     rc = launch_quantize_rtn(jobs[i].P_new->bits, bt.w[i].P32, m, r, r, jobs[i].P_new, st);

@@ -25,7 +25,7 @@ int launch_cooperative(const void* kern, unsigned grid, unsigned block, void** a
 constexpr int64_t kEigMax = 4096;
 inline int64_t eig_pitch(int64_t N) { return round_up(N, 128); }   // row pitch of A and V (floats)
 
-// Buffers of one matrix, carved by carve_eig.
+// Buffers of one matrix, carved by carve_eig: A and V first, back to back.  After launch_sym_eig all but Z is free for use.
 struct EigBuffers {
   float* A;            // N rows of eig_pitch(N) floats, symmetric: the matrix, destroyed
   float* V;            // same extents: row k holds Householder vector v_k
@@ -33,7 +33,7 @@ struct EigBuffers {
   float* cross;        // N floats: v_k . v_{k-1}
   float* scale;        // the power of two A is scaled by
   double *lam, *inv;   // r doubles each: the leading eigenvalues (of the scaled matrix), 1 / norm of the vectors of step 3
-  double *plus, *minus;  // N x r doubles each: pivots of the two factorisations of step 3
+  double *plus, *minus;  // the pivots of the two factorisations of step 3 for some of the vectors (plus over A)
   float* Z;            // N x r (pitch r): eigenvectors of the tridiagonal matrix, then of A
   uint4* xchg;         // 2 x eig_pitch(N): exchange between the CTAs of a matrix
 };

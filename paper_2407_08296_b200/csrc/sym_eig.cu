@@ -472,7 +472,7 @@ constexpr double kPivotFloor = 1e-280;
 __device__ __forceinline__ double guarded(double q) { return fabs(q) < kPivotFloor ? copysign(kPivotFloor, q) : q; }
 
 __global__ void __launch_bounds__(64)
-tridiagonal_vectors_kernel(const Ptrs<const float> db, const Ptrs<const float> eb, int N, int r, const Ptrs<const double> lamb,
+tridiagonal_vectors_kernel(const Ptrs<const float> db, const Ptrs<const float> eb, int N, int t0, int count, int r, const Ptrs<const double> lamb,
                            const Ptrs<double> plusb, const Ptrs<double> minusb, const Ptrs<float> Zb, const Ptrs<double> invb) {
   extern __shared__ double vec_smem[];
   __shared__ double s_best[2][32], s_sum[32];
@@ -485,11 +485,11 @@ tridiagonal_vectors_kernel(const Ptrs<const float> db, const Ptrs<const float> e
     e[i] = i + 1 < N ? eb.p[mat][i] : 0.f;
   }
   __syncthreads();
-  const int t = blockIdx.x * 32 + lane;
-  const bool live = t < r;
-  const double lam = live ? lamb.p[mat][t] : 0.0;
-  double* plus = plusb.p[mat] + min(t, r - 1);      // D+_i, D-_i
-  double* minus = minusb.p[mat] + min(t, r - 1);
+  const int t = blockIdx.x * 32 + lane;             // of the vectors t0 .. t0 + count - 1 (of r), whose pivots have pitch count
+  const bool live = t < count;
+  const double lam = live ? lamb.p[mat][t0 + t] : 0.0;
+  double* plus = plusb.p[mat] + min(t, count - 1);  // D+_i, D-_i
+  double* minus = minusb.p[mat] + min(t, count - 1);
   if (live && side == 0) {
     double q = guarded(d[0] - lam);
     plus[0] = q;
@@ -497,16 +497,16 @@ tridiagonal_vectors_kernel(const Ptrs<const float> db, const Ptrs<const float> e
     for (int i = 1; i < N; ++i) {
       const double ei = e[i - 1];
       q = guarded((d[i] - lam) - ei * (ei / q));
-      plus[(int64_t)i * r] = q;
+      plus[(int64_t)i * count] = q;
     }
   } else if (live) {
     double q = guarded(d[N - 1] - lam);
-    minus[(int64_t)(N - 1) * r] = q;
+    minus[(int64_t)(N - 1) * count] = q;
 #pragma unroll 4
     for (int i = N - 2; i >= 0; --i) {
       const double ei = e[i];
       q = guarded((d[i] - lam) - ei * (ei / q));
-      minus[(int64_t)i * r] = q;
+      minus[(int64_t)i * count] = q;
     }
   }
   __syncthreads();
@@ -522,8 +522,8 @@ tridiagonal_vectors_kernel(const Ptrs<const float> db, const Ptrs<const float> e
 #pragma unroll
         for (int u = 0; u < kBatch; ++u) {
           const int64_t i = min(b + u, N - 1);
-          p[u] = plus[i * r];
-          m[u] = minus[i * r];
+          p[u] = plus[i * count];
+          m[u] = minus[i * count];
         }
 #pragma unroll
         for (int u = 0; u < kBatch; ++u) {
@@ -537,13 +537,13 @@ tridiagonal_vectors_kernel(const Ptrs<const float> db, const Ptrs<const float> e
   }
   __syncthreads();
   const int twist = s_best[1][lane] < s_best[0][lane] ? s_at[1][lane] : s_at[0][lane];
-  float* Z = Zb.p[mat] + min(t, r - 1);
+  float* Z = Zb.p[mat] + t0 + min(t, count - 1);
   double z = 1.0, sum = 0.0;
   if (live && side == 0) {                          // z_i = -(e_i / D+_i) z_{i+1} above the twist
     for (int b = twist - 1; b >= 0; b -= kBatch) {
       double l[kBatch];
 #pragma unroll
-      for (int u = 0; u < kBatch; ++u) { const int64_t i = max(b - u, 0); l[u] = plus[i * r]; }
+      for (int u = 0; u < kBatch; ++u) { const int64_t i = max(b - u, 0); l[u] = plus[i * count]; }
 #pragma unroll
       for (int u = 0; u < kBatch; ++u) l[u] = (double)e[max(b - u, 0)] / l[u];
 #pragma unroll
@@ -560,7 +560,7 @@ tridiagonal_vectors_kernel(const Ptrs<const float> db, const Ptrs<const float> e
     for (int b = twist + 1; b < N; b += kBatch) {
       double l[kBatch];
 #pragma unroll
-      for (int u = 0; u < kBatch; ++u) { const int64_t i = min(b + u, N - 1); l[u] = minus[i * r]; }
+      for (int u = 0; u < kBatch; ++u) { const int64_t i = min(b + u, N - 1); l[u] = minus[i * count]; }
 #pragma unroll
       for (int u = 0; u < kBatch; ++u) l[u] = (double)e[min(b + u, N - 1) - 1] / l[u];
 #pragma unroll
@@ -573,7 +573,7 @@ tridiagonal_vectors_kernel(const Ptrs<const float> db, const Ptrs<const float> e
     }
   }
   __syncthreads();
-  if (live && side == 1) invb.p[mat][t] = 1.0 / sqrt(s_sum[lane] + sum);
+  if (live && side == 1) invb.p[mat][t0 + t] = 1.0 / sqrt(s_sum[lane] + sum);
 }
 
 // ------------------------------------------------------------------------------------------ 4. X = H Z
@@ -832,6 +832,10 @@ int launch_cooperative(const void* kern, unsigned grid, unsigned block, void** a
   return QG_OK;
 }
 
+// The vectors of a launch of step 3: as many as have their D+ where A was; half of that for large matrices, whose scratch matters
+// (a refresh asks for a quarter of the vectors there are as a rule, so that either is one launch).
+static int64_t vectors_at_once(int64_t N, int64_t r) { return std::min(r, eig_pitch(N) / (N <= 2048 ? 2 : 4)); }
+
 size_t carve_eig(void* base, int64_t N, int64_t r, EigBuffers* out) {
   size_t off = 0;
   auto take = [&](size_t bytes) { void* p = base ? (char*)base + off : nullptr; off += (size_t)round_up((int64_t)bytes, 256); return p; };
@@ -846,8 +850,8 @@ size_t carve_eig(void* base, int64_t N, int64_t r, EigBuffers* out) {
   w.scale = (float*)take(4);
   w.lam = (double*)take((size_t)(r * 8));
   w.inv = (double*)take((size_t)(r * 8));
-  w.plus = (double*)take((size_t)(N * r * 8));
-  w.minus = (double*)take((size_t)(N * r * 8));
+  w.minus = (double*)take((size_t)(N * vectors_at_once(N, r) * 8));
+  w.plus = (double*)w.A;                            // done with when the pivots come
   w.Z = (float*)take((size_t)(N * r * 4));
   w.xchg = (uint4*)take((size_t)(2 * Np * 16));
   if (out) *out = w;
@@ -921,8 +925,13 @@ int launch_sym_eig(const EigBuffers* w, int nb, int64_t N, int64_t r, int64_t wa
     const int rc = opt_in(tridiagonal_vectors_kernel, (int)kEigMax * 12, done);
     if (rc != QG_OK) return rc;
   }
-  tridiagonal_vectors_kernel<<<dim3((unsigned)ceil_div(r, 32), (unsigned)nb), 64, (size_t)N * 12, st>>>(dc, ec, (int)N, (int)r, lamc, plus, minus, Z, inv);
-  QG_LAUNCH_CHECK();
+  const int64_t at_once = vectors_at_once(N, r);
+  for (int64_t t0 = 0; t0 < r; t0 += at_once) {
+    const int64_t count = std::min(at_once, r - t0);
+    tridiagonal_vectors_kernel<<<dim3((unsigned)ceil_div(count, 32), (unsigned)nb), 64, (size_t)N * 12, st>>>(dc, ec, (int)N, (int)t0, (int)count, (int)r, lamc, plus, minus,
+                                                                                                             Z, inv);
+    QG_LAUNCH_CHECK();
+  }
   reflector_pairs_kernel<<<dim3((unsigned)ceil_div(N, 8), (unsigned)nb), 128, 0, st>>>(Vc, (int)N, (int)Np, cross);
   QG_LAUNCH_CHECK();
   const bool few = nb * r <= 4 * sms;                // a CTA of two warps per SM

@@ -133,3 +133,12 @@ def test_a_quantized_matrix_has_a_storage_of_its_own_for_each_part(bits):
         assert t.untyped_storage().nbytes() == t.numel() * t.element_size()
     like = B.QTensor.empty(3, 300, bits, "cpu")
     assert [(t.shape, t.stride(), t.dtype) for t in parts] == [(t.shape, t.stride(), t.dtype) for t in (like.codes, like.scales, like.zeros)]
+
+
+def test_refresh_scratch_is_that_of_the_iterative_route():
+    # both routes work in the same scratch; programs that hold a fixed one sized it by the iterative route: the block three times on
+    # its own side and once on the other, two b x b matrices, the bfloat16 planes of an iterate, panels, 32 MB of partial sums
+    for m, n, b in [(64, 64, 64), (768, 2048, 512), (2048, 768, 512), (2048, 2048, 256), (3000, 8000, 768), (4096, 4096, 512), (4096, 4096, 2048),
+                    (4096, 11008, 2048), (11008, 4096, 2048), (3753, 3708, 1728), (4028, 4007, 1664), (20000, 700, 640), (4096, 4096, 4096)]:
+        most = 12 * m * b + 4 * n * b + 8 * b * b + 6 * ((max(m, n) + 63) // 64 * 64) * b + 256 * (m + b) + (33 << 20)
+        assert B.workspace_bytes(B.QG_OP_REFRESH, m, n, b) <= most, (m, n, b)

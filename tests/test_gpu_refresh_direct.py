@@ -152,3 +152,15 @@ def test_route_of_a_shape(s, b, direct):
     for seed in range(2):
         B.refresh_subspace(G, r, oversample_cols=b - r, seed=seed, P_fp32=P[seed])
     assert torch.equal(P[0], P[1]) == direct
+
+
+# More vectors than one launch finds, whose pivots lie over the matrix that has been reduced: more than half of the short side's, or
+# a quarter from 2049 rows on; vectors of the long side and their product go there as well.
+@pytest.mark.parametrize("m,n,r", [(512, 640, 320), (700, 512, 416), (2304, 2310, 640)])
+def test_vectors_found_in_several_launches(m, n, r):
+    G = _gradient(m, n, seed=r)
+    P = torch.zeros((m, r), device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    B.refresh_subspace(G, r, P_fp32=P, status=status)
+    assert int(status.item()) == 0
+    _check(G, P, "left")
