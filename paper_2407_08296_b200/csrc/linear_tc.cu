@@ -31,21 +31,13 @@
 #include <cstring>
 
 #include "launch.cuh"
-#include "sm100_ptx.cuh"
-#include "tensor_map.cuh"
+#include "linear_common.cuh"
 
 namespace qg {
 
-using namespace ptx;
+using namespace linear;
 
 namespace {
-
-constexpr int kBK = 64;        // K extent of a pipeline stage
-constexpr int kTileM = 128;    // accumulator rows (TMEM lanes)
-constexpr int kTileN = 256;    // accumulator columns; a multiple of the quantization group along n
-constexpr int kSlab = 64 * kBK * 2;   // one 64-wide MN-major slab of a stage: 64 K rows of 128 bytes
-
-enum : int { kForward = 0, kInputGrad = 1, kWeightGrad = 2 };
 
 struct LinArgs {
   CUtensorMap mapA;            // bf16 activations: K-major 2-D (X of the forward product, where it is the MMA's B
@@ -155,57 +147,11 @@ struct LinSmem {
   static_assert(kBytes > kHalfOfSharedMemory, "see launch_overlapping");
 };
 
-__device__ __forceinline__ void raise_expired(int32_t* status) {
-  if (status) atomicOr(status, QG_DEV_WAIT_EXPIRED);
-}
-
-// Four lanes 4 g .. 4 g + 3 hold a row of four 16-byte pieces each; afterwards lane 4 g + j holds piece j of all four rows, so
-// that they store 64 contiguous bytes of one row together.  (A row per lane is 32 half-filled sectors per instruction: input
-// gradient 8192 x 2048 x 5461 160 -> 147 us, forward 4690 x 4254 x 128 38 -> 27.)
-__device__ __forceinline__ void quad_transpose(uint4 (&p)[4], int lane) {
-#pragma unroll
-  for (int bit = 1; bit <= 2; bit <<= 1) {
-    const bool up = lane & bit;
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      if (c & bit) continue;
-      uint4 &lo = p[c], &hi = p[c | bit];
-      const uint4 out = up ? lo : hi;
-      const uint4 in = make_uint4(__shfl_xor_sync(0xFFFFFFFFu, out.x, bit), __shfl_xor_sync(0xFFFFFFFFu, out.y, bit),
-                                  __shfl_xor_sync(0xFFFFFFFFu, out.z, bit), __shfl_xor_sync(0xFFFFFFFFu, out.w, bit));
-      if (up) lo = in; else hi = in;
-    }
-  }
-}
-
 // A load that stays where it is written (the compiler moves others down to their first use).
 __device__ __forceinline__ float ld_early(const float* p) {
   float v;
   asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(v) : "l"(p));
   return v;
-}
-
-// Sixteen INT8 codes (one 16-byte word) -> sixteen bfloat16 of (q - z) * s, as two 16-byte words.
-// bias = 2^23 + 128 + z: the code byte with its sign bit flipped is q + 128, placed in the low mantissa
-// byte of 2^23 it reads as the float 2^23 + 128 + q, and subtracting bias leaves q - z exactly; one
-// binary32 multiplication and one rounding to bfloat16 follow, the same two roundings as the definition.
-__device__ __forceinline__ void dequant16(const uint4 codes, float bias, float s, uint4& lo, uint4& hi) {
-  const uint32_t w[4] = {codes.x ^ 0x80808080u, codes.y ^ 0x80808080u, codes.z ^ 0x80808080u, codes.w ^ 0x80808080u};
-  const float2 nb = make_float2(-bias, -bias), s2 = make_float2(s, s);
-  uint32_t out[8];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const float2 a = make_float2(__uint_as_float(__byte_perm(w[i], 0x4B000000u, 0x7440)),
-                                 __uint_as_float(__byte_perm(w[i], 0x4B000000u, 0x7441)));
-    const float2 b = make_float2(__uint_as_float(__byte_perm(w[i], 0x4B000000u, 0x7442)),
-                                 __uint_as_float(__byte_perm(w[i], 0x4B000000u, 0x7443)));
-    const float2 va = mul2(add2(a, nb), s2), vb = mul2(add2(b, nb), s2);
-    __nv_bfloat162 pa = __floats2bfloat162_rn(va.x, va.y), pb = __floats2bfloat162_rn(vb.x, vb.y);
-    out[2 * i] = *reinterpret_cast<uint32_t*>(&pa);
-    out[2 * i + 1] = *reinterpret_cast<uint32_t*>(&pb);
-  }
-  lo = make_uint4(out[0], out[1], out[2], out[3]);
-  hi = make_uint4(out[4], out[5], out[6], out[7]);
 }
 
 template <int MODE, int MT>
@@ -387,29 +333,7 @@ int8_linear_kernel(const __grid_constant__ LinArgs a, int32_t* __restrict__ stat
             else mbar_arrive_cluster(mapa_u32(smem_u32(&acc_empty[ab + h]), wk.leader));
           }
         }
-        if (n0 + 32 * c < a.cols) {
-          uint4 pk[4];
-#pragma unroll
-          for (int i = 0; i < 16; ++i) {
-            __nv_bfloat162 h2 = __floats2bfloat162_rn(__uint_as_float(v[2 * i]), __uint_as_float(v[2 * i + 1]));
-            reinterpret_cast<uint32_t*>(pk)[i] = *reinterpret_cast<uint32_t*>(&h2);
-          }
-          quad_transpose(pk, lane);                    // pk[i]: columns 8 (lane % 4) .. + 7 of row 4 (lane / 4) + i
-          const int col = n0 + 32 * c + 8 * (lane & 3);
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const int row = m0 + h * 2 * kTileM + q * 32 + (lane & ~3) + i;
-            uint16_t* d = a.D + (int64_t)row * a.ldd + col;
-            if (row < a.rows && col + 8 <= a.cols) {
-              *reinterpret_cast<uint4*>(d) = pk[i];
-            } else if (row < a.rows && col < a.cols) {
-              const uint32_t u[4] = {pk[i].x, pk[i].y, pk[i].z, pk[i].w};
-#pragma unroll
-              for (int e = 0; e < 8; ++e)
-                if (col + e < a.cols) d[e] = (uint16_t)((e & 1) ? (u[e >> 1] >> 16) : (u[e >> 1] & 0xFFFFu));
-            }
-          }
-        }
+        if (n0 + 32 * c < a.cols) store_piece(a.D, a.ldd, a.rows, a.cols, m0 + h * 2 * kTileM + q * 32, n0 + 32 * c, lane, v);
         __syncwarp();                                  // the next loads from tensor memory are the whole warp's
       }
     }
@@ -446,7 +370,7 @@ int8_linear_kernel(const __grid_constant__ LinArgs a, int32_t* __restrict__ stat
         bw.advance(S::kGroups);
         fetch(bw);
         const int rs = it % S::kRawStages, s = it % S::kStages;
-        ok = mbar_wait_warp(&raw_full[rs], (it / S::kRawStages) & 1) && mbar_wait_warp(&empty[s], ((it / S::kStages) & 1) ^ 1);
+        ok = __all_sync(0xFFFFFFFFu, mbar_wait(&raw_full[rs], (it / S::kRawStages) & 1) && mbar_wait(&empty[s], ((it / S::kStages) & 1) ^ 1));
         if (!ok) break;
         const uint8_t* raw = raw_base + rs * S::kRawBytes;
         uint8_t* sB = stage_base + s * S::kStageBytes + S::kABytes;
@@ -646,9 +570,35 @@ int launch_rounds(LinArgs a, const Rounds& r, int32_t* status, cudaStream_t st) 
   return r.rest > 0 ? launch(r.whole, r.whole + r.rest, r.split, r.rest, r.whole > 0) : QG_OK;
 }
 
-// One or two row blocks per tile, whichever is estimated to take less time.
+// Whether single CTAs (linear_single.cu) take the forward product or the weight gradient in less time than the pairs' plan `r`.  Both
+// in microseconds, fitted to 107 products of 17 .. 8192 tokens and 163 .. 11008 rows and columns, device time: what a launch
+// takes from begin to end, K blocks, what a further round adds, and a second launch that has to wait for whole clusters of free SMs.
+// The pairs have to be the faster by more than the fit is off by.  Pairs and single CTAs, T x m x n: forward 256 x 512 x 512 14.4
+// and 12.3, 1024 x 1024 x 1024 16.5 and 16.4, 256 x 2048 x 2048 18.5 and 22.6, 8192 x 4096 x 512 57 and 49, 8192 x 2048 x 2048 71 and 84;
+// weight gradient 256 x 1024 x 1024 10.3 and 8.2, 1024 x 2048 x 2048 14.5 and 12.4, 4096 x 512 x 512 18.5 and 24.8, 8192 x 768 x 2048 34
+// and 52.  (The input gradient by single CTAs was slower throughout.)
 template <int MODE>
-int launch_product(const LinArgs& a, int32_t* status, cudaStream_t st) {
+bool single_pays(const LinArgs& a, const Rounds& r, int mt) {
+  const double kb = (a.K + kBK - 1) / kBK;
+  const int across = MODE == kForward ? a.cols : a.rows, along = MODE == kForward ? a.rows : a.cols;   // forward is computed transposed
+  const int64_t tiles = (int64_t)((across + kTileM - 1) / kTileM) * ((along + kTileN - 1) / kTileN);
+  if (tiles > (int64_t)1 << 30) return false;                        // the tile index is an int
+  const double more = (double)((tiles - 1) / (2 * r.pairs)), pairs_more = (r.whole + r.pairs - 1) / r.pairs - 1.0;
+  const bool two_launches = r.whole > 0 && r.rest > 0;
+  if (MODE == kForward) {
+    const double single = 8.5 + 0.43 * kb + more * std::max(0.48 * kb + 2.0, 4.0);
+    const double pairs = 11.7 + (mt == 1 ? 0.33 * r.time + 3.0 * std::max(pairs_more, 0.0) : 0.45 * r.time) + (two_launches ? 9.0 : 0.0);
+    return pairs >= 0.96 * single;
+  }
+  const double single = 8.0 + 0.27 * kb * (more + 1.0) + 1.6 * more;
+  const double pairs = 10.0 + 0.27 * r.time + std::max(pairs_more, 0.0) * std::max(2.4 - 0.27 * kb, 0.0) + (two_launches ? 8.0 : 0.0);
+  return pairs >= 0.94 * single;
+}
+
+// One or two row blocks per tile, or single CTAs (`by_single_ctas` launches them), whichever is estimated to take less time.
+// `operands` fills in what the pairs read from.
+template <int MODE, class Operands, class Single>
+int launch_product(const LinArgs& a, int32_t* status, cudaStream_t st, Operands operands, Single by_single_ctas) {
   int dev = 0;
   QG_CUDA_TRY(cudaGetDevice(&dev));
   if (dev < 0 || dev >= kDevices) return QG_UNSUPPORTED_SHAPE;
@@ -656,7 +606,10 @@ int launch_product(const LinArgs& a, int32_t* status, cudaStream_t st) {
   int rc = plan_rounds<MODE, 1>(a, dev, one);
   if (rc == QG_OK) rc = plan_rounds<MODE, 2>(a, dev, two);
   if (rc != QG_OK) return rc;
-  return two.time < one.time ? launch_rounds<MODE, 2>(a, two, status, st) : launch_rounds<MODE, 1>(a, one, status, st);
+  const bool tall = two.time < one.time;
+  if (MODE != kInputGrad && single_pays<MODE>(a, tall ? two : one, tall ? 2 : 1)) return by_single_ctas();
+  if (!operands()) return QG_CUDA_ERROR;
+  return tall ? launch_rounds<MODE, 2>(a, two, status, st) : launch_rounds<MODE, 1>(a, one, status, st);
 }
 
 }  // namespace
@@ -669,35 +622,28 @@ int launch_int8_linear(int mode, const uint16_t* act, int64_t ld_act, const uint
   memset(&a, 0, sizeof(a));
   a.D = D;
   a.ldd = ldd;
-  bool ok = true;
-  if (mode == kWeightGrad) {
-    // act = dY (T x m), act2 = X (T x n); both enter as 64-wide column slabs, K = T runs down the rows
-    ok &= make_map_chunked(&a.mapA, act, T, (m + 63) / 64, ld_act, kBK, 2);
-    ok &= make_map_chunked(&a.mapB, act2, T, (n + 63) / 64, ld_act2, kBK, 2);
-    a.rows = (int32_t)m; a.cols = (int32_t)n; a.K = (int32_t)T;
-  } else {
+  a.rows = (int32_t)(mode == kWeightGrad ? m : T);
+  a.cols = (int32_t)(mode == kForward ? m : n);
+  a.K = (int32_t)(mode == kForward ? n : mode == kInputGrad ? m : T);
+  a.nblocks = (a.cols + kTileN - 1) / kTileN;
+  if ((int64_t)((a.rows + 2 * kTileM - 1) / (2 * kTileM)) * a.nblocks > (int64_t)1 << 30) return QG_UNSUPPORTED_SHAPE;   // the tile index is an int
+  const auto operands = [&] {
+    if (mode == kWeightGrad)
+      // act = dY (T x m), act2 = X (T x n); both enter as 64-wide column slabs, K = T runs down the rows
+      return make_map_chunked(&a.mapA, act, T, (m + 63) / 64, ld_act, kBK, 2) && make_map_chunked(&a.mapB, act2, T, (n + 63) / 64, ld_act2, kBK, 2);
     a.scales = W->scales;
     a.zeros = W->zeros;
     a.ngroups = (int32_t)((n + kGroup - 1) / kGroup);
     a.w_rows = (int32_t)m;
-    if (mode == kForward) {
-      // act = X (T x n)
-      ok &= make_map(&a.mapA, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, act, n, T, ld_act, kBK, kTileM, CU_TENSOR_MAP_SWIZZLE_128B);
-      ok &= make_map(&a.mapB, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, W->codes, n, m, W->ld, kBK, kTileN / 2, CU_TENSOR_MAP_SWIZZLE_64B);
-      a.rows = (int32_t)T; a.cols = (int32_t)m; a.K = (int32_t)n;
-    } else {
-      // act = dY (T x m)
-      ok &= make_map(&a.mapA, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, act, m, T, ld_act, kBK, kTileM, CU_TENSOR_MAP_SWIZZLE_128B);
-      ok &= make_map(&a.mapB, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, W->codes, n, m, W->ld, kTileN / 2, kBK, CU_TENSOR_MAP_SWIZZLE_NONE);
-      a.rows = (int32_t)T; a.cols = (int32_t)n; a.K = (int32_t)m;
-    }
-  }
-  if (!ok) return QG_CUDA_ERROR;
-  a.nblocks = (a.cols + kTileN - 1) / kTileN;
-  if ((int64_t)((a.rows + 2 * kTileM - 1) / (2 * kTileM)) * a.nblocks > (int64_t)1 << 30) return QG_UNSUPPORTED_SHAPE;   // the tile index is an int
-  if (mode == kForward) return launch_product<kForward>(a, status, st);
-  if (mode == kInputGrad) return launch_product<kInputGrad>(a, status, st);
-  return launch_product<kWeightGrad>(a, status, st);
+    // act = X (T x n) or dY (T x m)
+    return make_map(&a.mapA, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, act, a.K, T, ld_act, kBK, kTileM, CU_TENSOR_MAP_SWIZZLE_128B) &&
+           (mode == kForward ? make_map(&a.mapB, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, W->codes, n, m, W->ld, kBK, kTileN / 2, CU_TENSOR_MAP_SWIZZLE_64B)
+                             : make_map(&a.mapB, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, W->codes, n, m, W->ld, kTileN / 2, kBK, CU_TENSOR_MAP_SWIZZLE_NONE));
+  };
+  const auto single = [&] { return launch_single(mode, act, ld_act, act2, ld_act2, W, T, m, n, D, ldd, status, st); };
+  if (mode == kForward) return launch_product<kForward>(a, status, st, operands, single);
+  if (mode == kInputGrad) return launch_product<kInputGrad>(a, status, st, operands, single);
+  return launch_product<kWeightGrad>(a, status, st, operands, single);
 }
 
 }  // namespace qg

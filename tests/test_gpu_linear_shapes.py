@@ -72,3 +72,19 @@ def test_products_whose_tiles_are_split_along_k(T, m, n):
 @pytest.mark.parametrize("T,m,n", [(1337, 4096, 4096), (3001, 11008, 4096)])
 def test_split_products_whose_rows_end_inside_a_warp(T, m, n):
     test_products_whose_tiles_are_split_along_k(T, m, n)
+
+
+# By the estimates that choose between CTA pairs and single CTAs: the forward product by single CTAs in one round (a K of less than
+# a block, columns and rows that end inside a tile) and in several, the weight gradient by single CTAs in one and several rounds,
+# and by pairs with 512 rows a tile.
+@pytest.mark.parametrize("T,m,n", [(17, 129, 40), (255, 1000, 513), (2000, 4300, 300), (5461, 2049, 130), (8200, 4100, 600), (700, 3000, 4000)])
+def test_products_by_single_ctas(T, m, n):
+    test_products_whose_tiles_are_split_along_k(T, m, n)
+
+
+# By the same estimates, the forms of the pairs' kernel: 256 and 512 rows a tile, whole rounds, whole rounds and a shared remainder, and
+# tiles that are all shared; first as the forward product takes them, then as the weight gradient does.
+@pytest.mark.parametrize("T,m,n", [(261, 5827, 2734), (289, 9710, 2155), (12599, 267, 1920), (272, 4855, 6738), (15229, 516, 3740),
+                                   (525, 9887, 828), (2014, 244, 228), (4811, 9965, 267), (8947, 261, 4777), (3927, 3591, 9274), (12426, 8853, 1057)])
+def test_products_in_each_form_of_the_pairs(T, m, n):
+    test_products_whose_tiles_are_split_along_k(T, m, n)
