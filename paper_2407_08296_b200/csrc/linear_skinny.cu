@@ -151,7 +151,7 @@ int launch(const SkinnyArgs& a, cudaStream_t st) {
 int launch_int8_linear_skinny(const uint16_t* X, int64_t ldx, const qg_qtensor* W, int64_t T, uint16_t* Y, int64_t ldy, cudaStream_t st) {
   const SkinnyArgs a{X, ldx, (const int8_t*)W->codes, W->ld, W->scales, W->zeros, Y, ldy, (int32_t)T, (int32_t)W->rows,
                      (int32_t)W->cols, (int32_t)ceil_div(W->cols, kGroup)};
-  const int warps = a.ngroups <= 4 ? 4 : ceil_div(a.m, 16) <= 148 && a.ngroups >= 16 ? 16 : 8;
+  const int warps = a.ngroups <= 4 ? 4 : ceil_div(a.m, 16) <= sm_count() && a.ngroups >= 16 ? 16 : 8;
   if (T <= 8) return warps == 4 ? launch<1, 4>(a, st) : warps == 8 ? launch<1, 8>(a, st) : launch<1, 16>(a, st);
   return warps == 4 ? launch<2, 4>(a, st) : warps == 8 ? launch<2, 8>(a, st) : launch<2, 16>(a, st);
 }

@@ -19,12 +19,10 @@
 // MMAs take 512 clocks.  A 256-row tile's traffic (A, half of B, codes, each written once and read once) is 80 KB, 640
 // clocks, with a converted operand and 64 KB, 512 clocks, without; a 512-row tile uses B twice: 64 KB and 56 KB per 256 rows,
 // and half the conversions.  (Single CTAs with tiles of 128 or 256 rows: 96 to 128 KB.)  A 256-row tile leaves tensor memory
-// room for a second accumulator, so that its epilogue overlaps the next tile.  Measured, clocks per K block and 256 rows:
-// 765 to 910 converted, 545 to 570 not; 512-row tiles 560 to 710 and 523, at the 1.45 to 1.6 GHz that the power limit leaves.
-// Kernel time of single CTAs -> pairs, T x m x n: forward 8192 x 2048 x 5461 163 -> 133 us, 3001 x 11008 x 4096 230 -> 205;
-// input gradient 215 -> 154, 265 -> 181; weight gradient 138 -> 124, 202 -> 175.
-// (The forward product with W~ as the A operand in tensor memory moves 48 KB per block, but takes some 830 clocks whatever the
-// tile's columns: the MMA's load of A from there does not overlap.  176 us.)
+// room for a second accumulator, so that its epilogue overlaps the next tile.  The tensor pipe is busy 69 to 82 % of the active
+// clocks with a converted operand (8192 rows), 90 % without.  Time by single CTAs -> by pairs, T x m x n: forward 8192 x 2048 x 5461
+// 175 -> 144 us, 3001 x 11008 x 4096 240 -> 209; input gradient 210 -> 150, 365 -> 203; weight gradient 155 -> 132, 217 -> 194.
+// Short products stay with single CTAs (linear_single.cu; see single_pays).
 // Every barrier wait is bounded; a wait that runs out raises QG_DEV_WAIT_EXPIRED and the role stops.
 #include <algorithm>
 #include <atomic>
@@ -40,15 +38,15 @@ using namespace linear;
 namespace {
 
 struct LinArgs {
-  CUtensorMap mapA;            // bf16 activations: K-major 2-D (X of the forward product, where it is the MMA's B
-                               // operand; dY of the input gradient) or chunked 3-D (dY of the weight gradient)
+  CUtensorMap mapA;            // bf16 activations: K-major 2-D (X of the forward product, dY of the input gradient) or
+                               // chunked 3-D (dY of the weight gradient)
   CUtensorMap mapB;            // INT8 codes of W (2-D, bytes) or, for the weight gradient, X chunked 3-D
   const float* scales;         // of W: [w_rows][ngroups]
   const float* zeros;
   int32_t ngroups, w_rows;
   uint16_t* D;                 // bf16 output, row-major
   int64_t ldd;
-  int32_t rows, cols, K;       // accumulator extents (forward: rows of W x rows of X) and contraction length
+  int32_t rows, cols, K;       // accumulator extents and contraction length
   int32_t mblocks, nblocks;
   int32_t tile0, tile_end;     // the tiles of this launch
   int32_t split;               // 1: persistent pairs walk the tiles; else one cluster of `split` pairs per tile, see Walk
@@ -341,8 +339,8 @@ int8_linear_kernel(const __grid_constant__ LinArgs a, int32_t* __restrict__ stat
   } else if (S::kConvert && warp >= 8) {   // (up to the relays above)
     // ------------------------------------------------------------------ converters: INT8 tile -> bf16 operand
     // Groups of four warps take K blocks in turn, so that the chain of one block (wait, load, convert, store, fence, arrive:
-    // 900 to 1600 clocks) overlaps those of the next: 2 -> 3 groups, input gradient 3001 x 11008 x 4096, 256-row tiles, 315 ->
-    // 248 us; four are no better.  The scales are loaded a block ahead.
+    // 900 to 1600 clocks) overlaps those of the next: with two groups the input gradient 3001 x 11008 x 4096 took a quarter
+    // longer; four are no better.  The scales are loaded a block ahead.
     const int grp = (warp - 8) >> 2, lt = threadIdx.x & 127;
     uint32_t it = grp;
     bool ok = true;
@@ -492,10 +490,9 @@ int resident_clusters(int split, int dev) {
 
 // CTA pairs that share a tile of the last, unfilled round (`tiles` of them for `pairs` pairs): as many as keep every tile's
 // cluster resident, each with at least four K blocks.  1 (the round as it is) where that saves fewer than `saves` K blocks:
-// adding up the accumulators takes 4 to 8 us, a K block 0.35 (weight gradient, 1024 x 1376 x 512: 12.6 us as it is, 14.5
-// shared) to 0.5 us (input gradient 18 x 1137 x 163: 16.5 and 12.6).
-// Measured, against whole tiles by single CTAs: forward 310 x 1159 x 5993 53 -> 27 us, 512 x 2048 x 5461 51 -> 31; input
-// gradient 904 x 6535 x 4003 120 -> 57, 64 x 4096 x 4096 74 -> 27; weight gradient 2000 x 600 x 900 22 -> 18.
+// adding up the accumulators takes 4 to 8 us, a K block 0.27 (weight gradient) to 0.5 us.  Measured, a pair to each tile and
+// shared, 256 rows: forward 310 x 1159 x 5993 52 -> 30 us, 512 x 2048 x 5461 61 -> 36, 64 x 4096 x 4096 38 -> 24; input gradient 64 x 4096
+// x 4096 38 -> 24, 18 x 1137 x 163 18 -> 16; weight gradient 2000 x 600 x 900 24 -> 20.
 template <auto KERN, int THREADS, int SMEM>
 int choose_split(int tiles, int kblocks, int pairs, int saves, int dev) {
   int split = tiles > 0 ? pairs / tiles : 1;
@@ -528,11 +525,11 @@ int plan_rounds(const LinArgs& a, int dev, Rounds& r) {
   r.rest = total % r.pairs;
   r.split = choose_split<kern, S::kThreads, S::kBytes>(r.rest, kblocks, r.pairs, MODE == kWeightGrad ? 16 : 8, dev);
   r.whole = total - r.rest;
-  // A K block of a 512-row tile takes 1.57 of a 256-row tile's time with a converted operand (16384 x 4096 x 4096 forward 498
-  // us for 14 rounds, 382 for 7), 1.9 without (365 and 344, weight gradient); its epilogue, which nothing overlaps, and the
-  // sums of a split tile count as 6 and 12 blocks per 256 rows.  So small products keep 256 rows (512 x 2048 x 5461 forward
-  // 29 us against 37, 2000 x 600 x 900 21 against 29) and all weight gradients but the largest (8192 x 2048 x 5461 124 against
-  // 134).
+  // A K block of a 512-row tile takes 1.9 of a 256-row tile's time without a converted operand and 1.57 with one, as fitted to
+  // products of few rounds; where 512 rows are taken for their rounds it is less (16384 x 4096 x 4096 forward 652 us for 14
+  // rounds, 437 for 7).  Its epilogue, which nothing overlaps, and the sums of a split tile count as 6 and 12 blocks per 256
+  // rows.  So small products keep 256 rows (512 x 2048 x 5461 forward 36 us against 46, 2000 x 600 x 900 22 against 30), and weight
+  // gradients but for a few (904 x 6535 x 4003 42 against 53).
   const double block = MT == 1 ? 1.0 : MODE == kWeightGrad ? 1.9 : 1.57, tile = MT == 1 ? 0 : 6, sums = r.split > 1 ? MT * 12 : 0;
   r.time = (r.whole / r.pairs) * (kblocks * block + tile) + (r.rest ? (kblocks + r.split - 1) / r.split * block + tile + sums : 0);
   if (r.split == 1) { r.whole = total; r.rest = 0; }

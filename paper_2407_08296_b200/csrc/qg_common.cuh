@@ -21,6 +21,7 @@ constexpr int kGroup = 256;  // Sec. 3.1: block size 256
 // ----------------------------------------------------------------------------- host plumbing
 void note_cuda_error(cudaError_t e, const char* where);
 void count_launch(int n = 1);
+int sm_count();              // SMs of the device that is current at the first call
 
 #define QG_CUDA_TRY(expr)                                  \
   do {                                                     \

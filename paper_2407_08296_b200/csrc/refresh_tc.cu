@@ -417,15 +417,6 @@ split_planes_kernel(const float* __restrict__ B, int64_t ldb, int K, int N, int 
     *reinterpret_cast<uint4*>(planes + ((int64_t)p * kpad + row) * N + c0) = make_uint4(out[p][0], out[p][1], out[p][2], out[p][3]);
 }
 
-int split_sm_count() {
-  static int n = [] {
-    int dev = 0, v = 148;
-    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
-    return v > 0 ? v : 148;
-  }();
-  return n;
-}
-
 }  // namespace
 
 int launch_gram(const uint16_t* const* G, int nmat, int64_t ldg, bool columns, int64_t N, int64_t K, float* const* A, int64_t lda,
@@ -445,7 +436,7 @@ int launch_gram(const uint16_t* const* G, int nmat, int64_t ldg, bool columns, i
   a.lda = lda; a.N = (int32_t)N; a.K = (int32_t)K;
   const int mblocks = (int)ceil_div(N, kTileM);
   for (int mb = 0; mb < mblocks; ++mb) a.tiles += mb / 2 + 1;
-  const int total = a.tiles * nmat, grid = total < split_sm_count() ? total : split_sm_count();
+  const int total = a.tiles * nmat, grid = total < sm_count() ? total : sm_count();
   static bool smem_set[2][64] = {};
   int dev = 0;
   QG_CUDA_TRY(cudaGetDevice(&dev));
@@ -500,7 +491,7 @@ int launch_split_gemm(const uint16_t* A, int64_t sa_m, int64_t sa_k, const float
   a.mblocks = (int32_t)ceil_div(M, kTileM);
   a.nblocks = (int32_t)ceil_div(N, kTileN);
   const int total = a.mblocks * a.nblocks;
-  const int grid = total < split_sm_count() ? total : split_sm_count();
+  const int grid = total < sm_count() ? total : sm_count();
   static bool smem_set[2][64] = {};
   int dev = 0;
   QG_CUDA_TRY(cudaGetDevice(&dev));

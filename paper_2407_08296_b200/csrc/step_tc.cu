@@ -1427,15 +1427,6 @@ int fill_problem(const StepArgs& a, const TcScratch& w, TcProblem* p, int bn) {
   return QG_OK;
 }
 
-int sm_count() {
-  static int n = [] {
-    int dev = 0, v = 148;
-    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
-    return v > 0 ? v : 148;
-  }();
-  return n;
-}
-
 // Opts a kernel instance into its dynamic shared memory, once per device and instance (`done` is the calling
 // launcher's own flag array, one launcher per instance).
 template <class K>

@@ -8,8 +8,8 @@
 // The reduction is a chain of N dependent steps whatever runs it, so it is laid out for the shortest step: the matrix
 // stays on the SMs (columns dealt out to the CTAs, in registers and shared memory), one pass over it per step applies the
 // previous rank-2 update and multiplies by the new Householder vector, and ONE exchange through L2 per step carries what
-// every CTA needs of the others.  That exchange has no barrier: every value travels in a word of its own with the step's
-// number beside it, and the reader polls the word itself.
+// every CTA needs of the others.  That exchange has no barrier: every value travels in a 64-bit word of its own together with
+// the step's number, and the reader polls the word itself.
 #include <algorithm>
 #include <cmath>
 #include <mutex>
@@ -38,7 +38,7 @@ using ptx::mul2;
 // What bounds a step is latency: the trip through L2, two CTA barriers and the reductions.  |x|^2 is therefore taken
 // from sums over R - tau P and v that are reduced together with P . v (one barrier less); where the two terms of x
 // cancel the sum is taken again over x itself.
-// A thread keeps rows tid + 512 q of every column, the last columns in registers, those before in shared memory and,
+// A thread keeps rows tid + THREADS q of every column, the last columns in registers, those before in shared memory and,
 // past that, in global memory (L2): the row's v, w, v' are then registers too, and the pass reads nothing but two
 // scalars per column.
 constexpr uint32_t kPollLimit = 1u << 20;
@@ -158,10 +158,9 @@ tridiagonal_kernel(const __grid_constant__ TriArgs a, int32_t* __restrict__ stat
 #pragma unroll
     for (int q = 0; q < NQ; ++q) {
       const int j = tid + q * THREADS;
-      // The whole warp stays in the loop: lanes that left it one by one would run on by themselves, and a CTA barrier counts a
-      // warp as arrived with the first of them.  Row after row: with all of a thread's words asked for at once the polls hold
-      // up the words themselves (2048 x 5461: 9.4 ms as it is, 14.3 at once); a lane that waits alone for the rest of its warp
-      // adds a trip (10.3).
+      // The whole warp stays in the loop, so that what follows is executed once and not by parts of it, and reaches the barrier
+      // together.  Row after row: with all of a thread's words asked for at once the polls hold up the words themselves (2048 x
+      // 5461: 9.4 ms as it is, 14.3 at once); a lane that waits alone for the rest of its warp adds a trip (10.3).
       const bool wanted = k > 0 && j >= k && j < N;
       const Tagged* const in = xchg + (k & 1) * Np + j;
       Tagged got{0, 0};
@@ -767,15 +766,6 @@ back_transform_kernel(const Ptrs<const float> Vb, const Ptrs<const float> taub, 
 constexpr int kDevices = 64;
 std::mutex g_coop_mutex;
 cudaEvent_t g_coop_done[kDevices] = {};        // completion of the last cooperative launch, per device ordinal
-
-int sm_count() {
-  static int n = [] {
-    int dev = 0, v = 148;
-    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
-    return v > 0 ? v : 148;
-  }();
-  return n;
-}
 
 // Opts a kernel instance into its dynamic shared memory, once per device and instance.
 template <class K>
