@@ -426,7 +426,7 @@ def test_projection_dequantized_inside_the_kernel_equals_the_separate_launch():
             torch.cuda.synchronize()
             results[fused] = items + singles
     finally:
-        B.debug_set_fused_dequant(True)
+        B.debug_set_fused_dequant(False)                            # the default
     for a, b in zip(results[True], results[False]):
         assert torch.equal(a["W"].codes, b["W"].codes) and torch.equal(a["W"].scales, b["W"].scales)
         assert torch.equal(a["W"].zeros, b["W"].zeros) and torch.equal(a["M"], b["M"]) and torch.equal(a["V"], b["V"])
