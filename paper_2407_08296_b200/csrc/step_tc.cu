@@ -1441,10 +1441,11 @@ int set_smem_once(K kernel, int bytes, bool* done) {
 }
 
 // Whether a launch of the step overlaps the one before it.  Short launches are latency: 512 x 1376 at r = 128 28.7 -> 22.7 us
-// per step, 5461 x 2048 at r = 512 67.6 -> 63.2, the first pass over a LLaMA-130M stack (5 tiles per CTA) 285 -> 267.  Long
-// ones run at the power cap, where closing a gap saves nothing and waiting CTAs cost a little: a LLaMA-1B stack (30 tiles
-// per CTA) 3.68-3.70 ms a step with ordinary launches, 3.73-3.79 with overlapping ones.
-bool overlaps(int64_t tiles, int64_t grid) { return tiles <= 8 * grid; }
+// per step, 5461 x 2048 at r = 512 67.6 -> 63.2, two LLaMA-130M layers at r = 192 60.3 -> 58.1.  Long ones run at the power cap,
+// where closing a gap saves nothing and waiting CTAs cost a little: four layers of 1603 / 4269 columns at r = 384 (the projection
+// 5.6 tiles per CTA) 390 us a step with ordinary launches, 394 with overlapping ones; a LLaMA-1B stack (30 tiles per CTA)
+// 3.68-3.70 and 3.73-3.79 ms.
+bool overlaps(int64_t tiles, int64_t grid) { return tiles <= 5 * grid; }
 
 // The projection's column-tile width: 256 halves the operand traffic per flop of the 128-wide tile,
 // but only pays once there are enough tiles to occupy every SM.

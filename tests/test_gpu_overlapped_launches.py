@@ -30,15 +30,38 @@ def _run(base, pair_mode, wait, workspace_bytes=None):
     return items
 
 
-# Five LLaMA-130M layers are one chunk whose projection runs in pairs (310 tiles, ranks of whole 256s) and whose
-# back-projection does not (1080 tiles), both short enough to overlap the launch before them; a workspace of a few matrices makes several such
-# chunks a step; mode 3 has both in pairs.
-@pytest.mark.parametrize("pair_mode,matrices", [(6, None), (6, 12), (3, None), (1, 12)])
-def test_steps_behind_one_another_equal_steps_one_by_one(pair_mode, matrices):
-    _, base = build_stack("llama130m", torch.device("cuda", 0), seed=7, layers=5)
-    ws = None if matrices is None else matrices * B.workspace_bytes(B.QG_OP_PROJECT_STEP, 2048, 768, 256)
+def _matrices(count, m, n, r):
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(11)
+    items = []
+    for k in range(count):
+        G = B.zeros_matrix(m, n, torch.bfloat16)
+        G.copy_(1e-3 * torch.randn(m, n, device="cuda", generator=gen))
+        w, p = B.zeros_matrix(m, n, torch.float32), B.zeros_matrix(m, r, torch.float32)
+        w.copy_(0.02 * torch.randn(m, n, device="cuda", generator=gen))
+        p.copy_(torch.randn(m, r, device="cuda", generator=gen) / m ** 0.5)
+        items.append({"G": G, "P": B.quantize_int4(p), "W": B.quantize_int8(w), "M": B.zeros_matrix(r, n, torch.float32),
+                      "V": B.zeros_matrix(r, n, torch.float32), "seed": k})
+    return items
+
+
+# Twelve matrices of 768 x 2048 at rank 512 are one chunk whose projection runs in pairs (384 tiles, a rank of whole 256s) and whose
+# back-projection does not (576 tiles), both short enough to overlap the launch before them (five tiles a CTA); a workspace of a few
+# of them makes chunks of single CTAs only; mode 3 has both in pairs, mode 1 the back-projection.
+@pytest.mark.parametrize("pair_mode,at_once", [(6, 12), (6, 4), (3, 12), (1, 4)])
+def test_steps_behind_one_another_equal_steps_one_by_one(pair_mode, at_once):
+    base = _matrices(12, 768, 2048, 512)
+    ws = (at_once + 1) * B.workspace_bytes(B.QG_OP_PROJECT_STEP, 768, 2048, 512)
     got, want = _run(base, pair_mode, False, ws), _run(base, 0, True)
     for a, b in zip(got, want):
         assert torch.equal(a["W"].codes, b["W"].codes)
         assert torch.equal(a["W"].scales, b["W"].scales) and torch.equal(a["W"].zeros, b["W"].zeros)
+        assert torch.equal(a["M"], b["M"]) and torch.equal(a["V"], b["V"])
+
+
+def test_a_stack_stepped_without_waiting_equals_steps_one_by_one():
+    _, base = build_stack("llama130m", torch.device("cuda", 0), seed=7, layers=5)
+    got, want = _run(base, 6, False), _run(base, 0, True)
+    for a, b in zip(got, want):
+        assert torch.equal(a["W"].codes, b["W"].codes) and torch.equal(a["W"].scales, b["W"].scales)
         assert torch.equal(a["M"], b["M"]) and torch.equal(a["V"], b["V"])
