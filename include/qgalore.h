@@ -213,7 +213,7 @@ QG_API int qgalore_plan_step_timed(const qg_plan* plan, const qg_hyper* h, int32
 
 /* --- Sec. 3.5 "obtain the projection matrix using SVD" + Sec. 3.3 INT4 storage ------------
  * Top-r left singular vectors of G (bf16, m x n, pitch ldg), then Quant_4 into P_new.  With s = min(m, n) and b = r +
- * oversample_cols, where s <= 8 b (s up to 768), 6 b (up to 1536), 4 b (up to 2048) or 2.5 b (up to 4096): the r leading
+ * oversample_cols, where s <= 8 b (s up to 768), 6 b (up to 1536) or 4 b (up to 4096): the r leading
  * eigenvectors of the Gram matrix of the short side (tridiagonal reduction in binary32, eigenvalues and their vectors in
  * binary64), and G times them for vectors on the long side; iters and seed do not enter.  Else: block subspace iteration on G G^T with a block of b columns (`iters`
  * multiplications by G G^T, each followed by a block Gram-Schmidt orthonormalisation) and a Rayleigh-Ritz step
@@ -224,7 +224,8 @@ QG_API int qgalore_plan_step_timed(const qg_plan* plan, const qg_hyper* h, int32
  *   P_fp32     optional (may be NULL): m x r fp32, pitch r, receives the vectors before quantization
  *   P_prev, sim_dev  if both given, the similarity of Sec. 3.2 between P_prev and P_new over the leading
  *              sim_cols columns (<= 0: all) is written to *sim_dev
- *   workspace  qgalore_workspace_bytes(QG_OP_REFRESH, m, n, b) bytes, 256-byte aligned
+ *   workspace  qgalore_workspace_bytes(QG_OP_REFRESH, m, n, b) bytes, 256-byte aligned (with less, down to what the iteration
+ *              takes, the iteration is what runs)
  *   status_dev optional; receives QG_DEV_NOT_CONVERGED / QG_DEV_BAD_FACTOR
  * Shape rules: r % 32 == 0, b % 64 == 0, b <= min(m, n), b <= 4096.  Typical use: b = 2 r, iters = 12.
  * The Adam moments and the step count are not touched. */

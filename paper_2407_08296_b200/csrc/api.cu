@@ -1,5 +1,6 @@
 // extern "C" boundary of the Q-GaLore library: argument validation, scalar preparation and
 // dispatch to the kernels.  Nothing here allocates or synchronises.
+#include <algorithm>
 #include <atomic>
 #include <cmath>
 #include <cstdio>
@@ -36,6 +37,7 @@ int launch_refresh(const uint16_t* G, int64_t ldg, int64_t m, int64_t n, int64_t
                    uint64_t seed, const qg_qtensor* P_new, float* P_fp32, void* ws, size_t ws_bytes, int32_t* status,
                    cudaStream_t st, bool transposed);
 size_t refresh_workspace_bytes(int64_t m, int64_t n, int64_t b);
+size_t refresh_least_workspace_bytes(int64_t m, int64_t n, int64_t b);
 int launch_refresh_batched(const RefreshJob* jobs, int count, int64_t m, int64_t n, int64_t r, int64_t b, int iters, int sweeps,
                            void* ws, size_t ws_bytes, int32_t* status, cudaStream_t st, bool transposed);
 struct Plan;
@@ -399,7 +401,7 @@ static int refresh_impl(const qg_refresh_item* items, int32_t count, int64_t m, 
     if (it.sim_dev && !aligned4(it.sim_dev)) return QG_MISALIGNED;
     jobs[(size_t)i] = RefreshJob{it.G, it.ldg, it.seed, &it.P_new, it.P_fp32};
   }
-  if (workspace_bytes < qgalore_workspace_bytes(QG_OP_REFRESH, pm, pn, b)) return QG_WORKSPACE_TOO_SMALL;
+  if (workspace_bytes < std::max(refresh_least_workspace_bytes(pm, pn, b), similarity_workspace_bytes(pm, b))) return QG_WORKSPACE_TOO_SMALL;
   constexpr int kJacobiSweeps = 12;
   int rc = launch_refresh_batched(jobs.data(), count, pm, pn, r, b, iters, kJacobiSweeps, workspace, workspace_bytes, status_dev,
                                   (cudaStream_t)stream, right);

@@ -1,7 +1,7 @@
 // Subspace refresh (Sec. 3.5: "obtain the projection matrix using SVD"; Sec. 3.3: INT4 storage): the top-r left singular
 // vectors of the gradient G (m x n, bf16), without a full SVD, by one of two routes.
 //
-// Direct, where that is the faster (direct_shape):
+// Direct, where that is no slower for a matrix alone (direct_shape):
 //
 //   A = G G^T or G^T G, whichever is smaller (refresh_tc.cu: every product of two bfloat16 values is exact, sums in fp32)
 //   X <- its r leading eigenvectors (sym_eig.cu: tridiagonal reduction, bisection, twisted factorisations)
@@ -35,6 +35,7 @@
 // (Quant_4).  Several matrices of one shape are refreshed together (a "batch", up to kMaxBatch): every launch carries a
 // matrix index beside its tile index and reads its operands from small pointer tables passed by value, so launches and
 // barriers are paid once per batch instead of once per matrix.
+#include <algorithm>
 #include <cmath>
 
 #include "refresh_common.cuh"
@@ -815,7 +816,6 @@ struct RefreshWs {
   EigBuffers eig;  // of the Gram matrix of the short side
   float* XV;       // X V, for vectors on the long side
   uint16_t* planes_v;
-  float* P32_direct;
   // iterative route (in the same memory)
   float *Q, *Y, *Z, *Wp, *Cb, *S, *Linv, *Xsel;
   void* part;      // partial sums of sliced products
@@ -827,24 +827,26 @@ struct RefreshWs {
 
 // The route of a shape.  Direct: the whole of the short side's Gram matrix is reduced, 3 us a row up to 1024 rows, 5 at 2048, 11 at
 // 4096, and from 2048 rows on a batch gains little, since few of its matrices fit the SMs together.  Iterative: the cost goes
-// with the block, and a batch shares its many small launches.  The line lies where the direct one is the faster both alone and in
-// batches of eight (it decides on the shape only, so that a matrix gets the same vectors in either).  Measured, ms per matrix
+// with the block, and a batch shares its many small launches; but where the r-th singular value lies in a bulk, a block of 2 r
+// columns has not converged after 12 iterations unless it is some half of the short side (0.2 .. 0.4 rad at r = s / 8).  So the
+// line lies where the direct one is no slower for a matrix alone, and for blocks of a quarter of the short side it is taken in
+// batches as well, slower or not (the shape decides, so that a matrix gets the same vectors in either).  Measured, ms per matrix
 // alone / in eights, direct and iterative: 768 x 768 b 128 2.4 / 0.40 and 3.9 / 0.95; 1024 x 1024 b 128 4.8 / 0.82 and 4.1 / 1.1, b
 // 256 4.8 / 0.85 and 7.9 / 1.7; 1536 x 1536 b 192 6.4 / 2.1 and 6.3 / 1.7, b 384 6.3 / 2.2 and 13 / 3.1; 2048 x 2048 b 256 10.4 /
-// 4.5 and 9.1 / 2.3, b 512 10.4 / 4.5 and 18 / 4.5; 3072 x 3072 b 768 23 / 19.5 and 31 / 11.3, b 1536 22 / 21 and 73 / 39; 4096 x
-// 4096 b 1024 47 / 44 and 47 / 19, b 2048 47 / 45 and 119 / 74.
+// 4.5 and 9.1 / 2.3, b 512 10.4 / 4.5 and 18 / 4.5; 3072 x 3072 b 384 23 / 19 and 16 / 4.5, b 768 23 / 19.5 and 31 / 11.3; 4096 x 4096 b
+// 512 47 / 42 and 22 / 7.1, b 1024 47 / 44 and 47 / 19, b 2048 47 / 45 and 119 / 74.
 bool direct_shape(int64_t m, int64_t n, int64_t b) {
   const int64_t s = m < n ? m : n;
-  return s <= 768 ? s <= 8 * b : s <= 1536 ? s <= 6 * b : s <= 2048 ? s <= 4 * b : s <= kEigMax && 2 * s <= 5 * b;
+  return s <= 768 ? s <= 8 * b : s <= 1536 ? s <= 6 * b : s <= kEigMax && s <= 4 * b;
 }
 
-// Scratch of one matrix (left singular vectors of X, m x n; a block of b columns, at most as many vectors).
-size_t carve_refresh(void* base, int64_t m, int64_t n, int64_t b, RefreshWs* w) {
+// Scratch of one matrix (left singular vectors of X, m x n; a block of b columns, at most as many vectors) by either route.
+size_t carve_refresh(void* base, int64_t m, int64_t n, int64_t b, bool direct, RefreshWs* w) {
   size_t off = 0;
   auto take = [&](size_t bytes) { void* p = base ? (char*)base + off : nullptr; off += (size_t)round_up((int64_t)bytes, 256); return p; };
   RefreshWs t{};
   const int64_t s = m < n ? m : n;
-  if (direct_shape(m, n, b)) {
+  if (direct) {
     take(carve_eig(base ? (char*)base + off : nullptr, s, b, &t.eig));
     // what comes after the eigenvectors goes over A and V, where it fits
     size_t used = 0;
@@ -854,14 +856,14 @@ size_t carve_refresh(void* base, int64_t m, int64_t n, int64_t b, RefreshWs* w) 
       used += (size_t)round_up((int64_t)bytes, 256);
       return base ? (char*)t.eig.A + at : nullptr;
     };
-    t.P32_direct = (float*)over((size_t)m * b * 4);
+    t.P32 = (float*)over((size_t)m * b * 4);
     if (m > s) {
       t.XV = (float*)over((size_t)m * b * 4);
       t.planes_v = (uint16_t*)over(split_planes_bytes(s, b));
     }
+    if (w) *w = t;
+    return off;
   }
-  const size_t direct = off;
-  off = 0;
   t.P32 = (float*)take((size_t)m * b * 4);
   t.T = (float*)take((size_t)b * b * 4);
   t.lam = (double*)take((size_t)b * 8);
@@ -878,7 +880,7 @@ size_t carve_refresh(void* base, int64_t m, int64_t n, int64_t b, RefreshWs* w) 
   t.part = take((size_t)kSplitScratch);
   t.planes = (uint16_t*)take(split_planes_bytes(m > n ? m : n, b));
   if (w) *w = t;
-  return off > direct ? off : direct;
+  return off;
 }
 
 // The workspaces of the matrices of one batch, and pointer tables into them.
@@ -942,7 +944,12 @@ int orthonormalize(const Batch& bt, int64_t m, int64_t b, int32_t* status, cudaS
 
 }  // namespace
 
-size_t refresh_workspace_bytes(int64_t m, int64_t n, int64_t b) { return carve_refresh(nullptr, m, n, b, nullptr); }
+// What a matrix is refreshed in at least, by the iterative route, and what it is given to take the route of its shape: more where
+// the matrix and its reflectors alone are more than that (from 2600 rows on, with blocks of a quarter of them).
+size_t refresh_least_workspace_bytes(int64_t m, int64_t n, int64_t b) { return carve_refresh(nullptr, m, n, b, false, nullptr); }
+size_t refresh_workspace_bytes(int64_t m, int64_t n, int64_t b) {
+  return std::max(refresh_least_workspace_bytes(m, n, b), direct_shape(m, n, b) ? carve_refresh(nullptr, m, n, b, true, nullptr) : 0);
+}
 
 // Unit length (if asked for) and sign of the vectors in S (pitch lds): P32, P_fp32.
 static int finish_vectors(const RefreshJob* jobs, const Batch& bt, const Ptrs<const float>& S, int64_t lds, int64_t rows, int64_t r,
@@ -1096,16 +1103,14 @@ static int refresh_iterative(const RefreshJob* jobs, const Batch& bt, int64_t m,
 
 
 // One batch (at most kMaxBatch matrices of one shape).
-static int refresh_batch(const RefreshJob* jobs, int nb, int64_t m, int64_t n, int64_t r, int64_t b, int iters, int sweeps,
+static int refresh_batch(const RefreshJob* jobs, int nb, int64_t m, int64_t n, int64_t r, int64_t b, int iters, int sweeps, bool direct,
                          char* ws, size_t ws_stride, int32_t* status, cudaStream_t st, bool transposed) {
   Batch bt{};
   bt.nb = nb;
   for (int i = 0; i < nb; ++i) {
-    carve_refresh(ws + (size_t)i * ws_stride, m, n, b, &bt.w[i]);
+    carve_refresh(ws + (size_t)i * ws_stride, m, n, b, direct, &bt.w[i]);
     if (jobs[i].ldg != jobs[0].ldg) return QG_INVALID_ARGUMENT;          // one pitch per batch (the caller groups by it)
   }
-  const bool direct = g_refresh_direct && direct_shape(m, n, b);
-  for (int i = 0; direct && i < nb; ++i) bt.w[i].P32 = bt.w[i].P32_direct;
   int rc = direct ? refresh_direct(jobs, bt, m, n, r, status, st, transposed)
                   : refresh_iterative(jobs, bt, m, n, r, b, iters, sweeps, status, st, transposed);
   if (rc != QG_OK) return rc;
@@ -1116,16 +1121,18 @@ static int refresh_batch(const RefreshJob* jobs, int nb, int64_t m, int64_t n, i
   return QG_OK;
 }
 
-// `count` matrices of one shape, in batches of as many as the workspace holds (at most kMaxBatch).
+// `count` matrices of one shape, in batches of as many as the workspace holds (at most kMaxBatch).  A workspace that is only large
+// enough for the iterative route gets that one.
 int launch_refresh_batched(const RefreshJob* jobs, int count, int64_t m, int64_t n, int64_t r, int64_t b, int iters, int sweeps,
                            void* ws, size_t ws_bytes, int32_t* status, cudaStream_t st, bool transposed) {
-  const size_t stride = refresh_workspace_bytes(m, n, b);
+  if (ws_bytes < refresh_least_workspace_bytes(m, n, b)) return QG_WORKSPACE_TOO_SMALL;
+  const bool direct = g_refresh_direct && direct_shape(m, n, b) && ws_bytes >= refresh_workspace_bytes(m, n, b);
+  const size_t stride = direct ? refresh_workspace_bytes(m, n, b) : refresh_least_workspace_bytes(m, n, b);
   int64_t fit = (int64_t)(ws_bytes / stride);
-  if (fit < 1) return QG_WORKSPACE_TOO_SMALL;
   if (fit > kMaxBatch) fit = kMaxBatch;
   for (int first = 0; first < count; first += (int)fit) {
     const int nb = count - first < (int)fit ? count - first : (int)fit;
-    const int rc = refresh_batch(jobs + first, nb, m, n, r, b, iters, sweeps, reinterpret_cast<char*>(ws), stride, status, st,
+    const int rc = refresh_batch(jobs + first, nb, m, n, r, b, iters, sweeps, direct, reinterpret_cast<char*>(ws), stride, status, st,
                                  transposed);
     if (rc != QG_OK) return rc;
   }

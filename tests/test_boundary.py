@@ -136,7 +136,8 @@ def test_a_quantized_matrix_has_a_storage_of_its_own_for_each_part(bits):
 
 
 def test_refresh_scratch_is_that_of_the_iterative_route():
-    # both routes work in the same scratch; programs that hold a fixed one sized it by the iterative route: the block three times on
+    # both routes work in the same scratch (but for blocks of a quarter of some thousand rows, where the smaller one is accepted as
+    # well); programs that hold a fixed one sized it by the iterative route: the block three times on
     # its own side and once on the other, two b x b matrices, the bfloat16 planes of an iterate, panels, 32 MB of partial sums
     for m, n, b in [(64, 64, 64), (768, 2048, 512), (2048, 768, 512), (2048, 2048, 256), (3000, 8000, 768), (4096, 4096, 512), (4096, 4096, 2048),
                     (4096, 11008, 2048), (11008, 4096, 2048), (3753, 3708, 1728), (4028, 4007, 1664), (20000, 700, 640), (4096, 4096, 4096)]:

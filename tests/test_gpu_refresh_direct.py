@@ -37,7 +37,7 @@ def _check(G, P, side):
 
 
 @pytest.mark.parametrize("m,n,r,side", [(64, 700, 32, "left"), (130, 128, 32, "left"), (511, 640, 64, "left"), (513, 1025, 128, "left"),
-                                        (1025, 1030, 160, "right"), (1100, 769, 96, "left"), (2049, 2100, 416, "left"), (2500, 2047, 256, "left")])
+                                        (1025, 1030, 160, "right"), (1100, 769, 96, "left"), (2049, 2100, 288, "left"), (2500, 2047, 256, "left")])
 def test_vectors_are_those_of_a_nearby_matrix(m, n, r, side):
     G = _gradient(m, n, seed=m)
     P = torch.zeros((m if side == "left" else n, r), device="cuda")
@@ -145,7 +145,7 @@ def test_spectra_on_both_sides_of_what_is_resolved(ratio, flag):
 # The route is decided by the shape: on either side of its line for each range of short sides.  The seed of the start block enters
 # the iterative route only.
 @pytest.mark.parametrize("s,b,direct", [(768, 128, True), (768, 64, False), (1024, 128, False), (1088, 192, True), (1536, 256, True), (1600, 256, False),
-                                        (2048, 512, True), (2112, 768, False), (2112, 896, True)])
+                                        (2048, 512, True), (2112, 512, False), (2112, 576, True)])
 def test_route_of_a_shape(s, b, direct):
     G, r = _gradient(s, s + 8, seed=1), 32
     P = [torch.zeros((s, r), device="cuda") for _ in range(2)]
@@ -164,3 +164,23 @@ def test_vectors_found_in_several_launches(m, n, r):
     B.refresh_subspace(G, r, P_fp32=P, status=status)
     assert int(status.item()) == 0
     _check(G, P, "left")
+
+
+def test_a_workspace_of_the_iterative_route_gets_that_route():
+    # the direct route asks for more than the iterative one here; a caller with a workspace of the smaller size is served by it
+    s, b, r = 3072, 768, 384
+    G = _gradient(s, s, seed=2)
+    enough = 12 * s * b + 4 * s * b + 8 * b * b + 6 * s * b + 256 * (s + b) + (33 << 20)
+    assert enough < B.workspace_bytes(B.QG_OP_REFRESH, s, s, b)
+    P = [torch.zeros((s, r), device="cuda") for _ in range(3)]
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    ws = torch.empty(enough, dtype=torch.uint8, device="cuda")
+    B.refresh_subspace(G, r, oversample_cols=b - r, P_fp32=P[0], workspace=ws, status=status)
+    B.debug_set_refresh_direct(False)
+    try:
+        B.refresh_subspace(G, r, oversample_cols=b - r, P_fp32=P[1], status=status)
+    finally:
+        B.debug_set_refresh_direct(True)
+    B.refresh_subspace(G, r, oversample_cols=b - r, P_fp32=P[2], status=status)
+    assert int(status.item()) == 0
+    assert torch.equal(P[0], P[1]) and not torch.equal(P[0], P[2])
